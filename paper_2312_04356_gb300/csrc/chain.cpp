@@ -35,6 +35,58 @@ u64 invmod(u64 a, u64 q) { return powmod(a, q - 2, q); }
 
 u64 shoup(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }
 
+void ntt_pair(u64 w, u64 q, bool fold, u64* out2) {
+    if (!fold) {
+        out2[0] = w;
+        out2[1] = shoup(w, q);
+        return;
+    }
+    const u64 v[2] = {w, mulmod(w, (1ull << 32) % q, q)};
+    for (int i = 0; i < 2; ++i) {
+        const int64_t s = v[i] > q / 2 ? (int64_t)v[i] - (int64_t)q : (int64_t)v[i];   // balanced
+        const int32_t lo = (int32_t)(uint32_t)(u64)s;                                  // signed low digit
+        const int64_t hi = (s - lo) / ((int64_t)1 << 32);
+        out2[i] = (u64)(uint32_t)lo | ((u64)(uint32_t)(int32_t)hi << 32);
+    }
+}
+
+int ntt_tw_pos(int idx, int logn) {
+    if (logn != 16 || idx < 2) return idx;
+    int sg = 0;
+    while ((idx >> sg) > 1) ++sg;                           // stage: idx in [2^sg, 2^(sg+1))
+    const int u = sg & 7;                                   // local stage of its pass
+    if (u <= 4) return idx;
+    const int j = idx & ((1 << u) - 1);
+    return (idx - j) | ((j & ((1 << (u - 4)) - 1)) << 4) | (j >> (u - 4));
+}
+
+// Which primes qualify, and the constants (fold.cuh; the ranges are those stated at ArFold in ntt.cu)
+bool fold_consts(u64 q, FoldMod& f) {
+    f = FoldMod{};
+    int K = 1;
+    while (K < 62 && (q >> K) > 1) ++K;                                  // 2^K <= q < 2^(K+1)
+    if (K < 62 && (((u64)2 << K) - q) < q - ((u64)1 << K)) ++K;          // the nearer power
+    if (K < 33 || K > 60) return false;
+    const int64_t e = (int64_t)((u64)1 << K) - (int64_t)q;
+    const u128 ae = (u128)(e < 0 ? -e : e);
+    if (ae >= (1u << 26)) return false;
+    const u128 R = ((u128)1 << K) + (ae << 31), lim = ((u128)7 << 60);   // |values| <= 7 2^60
+    // folded value of any word, and the two classes' largest lazy value
+    const u128 opened = ((u128)1 << K) + (ae << (63 - K));
+    const bool big = 17 * R > ((u128)1 << 62);
+    const u128 top = big ? opened + 4 * R : 4 * (u128)q + 16 * R;        // forward
+    const u128 inv = big ? 4 * (R > opened ? R : opened) : 16 * (R > opened ? R : opened);
+    if (top > lim || inv > lim) return false;
+    if ((big ? ((u128)8 << (60 - K)) : (top >> K) + 1) * ae >= q) return false;   // canonical after one fold
+    // |x0 W0 + x1 W1| <= (2^31 + |x1|) q / 2 < 2^(K + 31)
+    if ((((u128)1 << 31) + (lim >> 32) + 2) * q >= ((u128)1 << (K + 32))) return false;
+    f.kc = (unsigned)(K - 32);
+    f.mask = (unsigned)(((u64)1 << (K - 32)) - 1);
+    f.e = (int)e;
+    f.big = big ? 1 : 0;
+    return true;
+}
+
 u64 from_signed(int64_t v, u64 q) {
     if (v >= 0) return (u64)v % q;
     u64 m = ((u64)(-(v + 1)) + 1) % q;

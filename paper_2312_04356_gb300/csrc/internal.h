@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "ckks.h"
+#include "fold.cuh"
 #include "modarith.cuh"
 
 typedef std::complex<double> cplx;
@@ -36,9 +37,12 @@ struct CkksError {
 // Per-prime constants, indexed by global prime id (q_0..q_L, then p_0..p_{np-1}).
 struct DevPrime {
     DevMod m;
-    const ulonglong2* tw;    // (psi^rev(k), Shoup companion), k < N   (forward, Cooley-Tukey)
-    const ulonglong2* itw;   // (psi^-rev(k), Shoup companion)          (inverse, Gentleman-Sande)
-    u64 n_inv, n_inv_p;
+    FoldMod f;
+    // transform constants as the pairs of hostmath::ntt_pair
+    const ulonglong2* tw;    // psi^rev(k), k < N   (forward, Cooley-Tukey)
+    const ulonglong2* itw;   // psi^-rev(k)          (inverse, Gentleman-Sande)
+    ulonglong2 n_inv;
+    u64 im, im_p;            // psi^(N/2) and its Shoup companion
     u64 r64, r64p;           // 2^64 mod q and its Shoup companion (128-bit lazy sums)
     u64 inv64;               // floor(2^64 / q): Shoup companion of 1, reduces any 64-bit word
 };
@@ -57,7 +61,7 @@ struct ConvTab {
     // p_m - (prod q_i mod p_m) [nout] followed by its Shoup companions [nout]
     u64* d_inv_q = nullptr;
     u64* d_corr = nullptr;
-    // N^{-1} qhat_i^{-1} mod q_i and its Shoup companion, [nin][2]: the factor an inverse NTT
+    // N^{-1} qhat_i^{-1} mod q_i as pairs (hostmath::ntt_pair), [nin][2]: the factor an inverse NTT
     // ends with when its output feeds this conversion directly (prescaled inputs)
     u64* d_iscale = nullptr;
     // tensor-core form (kern::base_convert_jobs with ctx->conv_tc): the table split into 8-bit
@@ -104,6 +108,7 @@ struct ckks_ctx {
     ckks_params P;
     int logn = 0, n = 0, nq = 0, L = 0, alpha = 0, np = 0, nall = 0, n_circuit = 0;
     bool mods_below_2_60 = false;    // every modulus < 2^60 (enables the split base conversion)
+    bool fold = false;               // every modulus qualifies for fold.cuh
     std::vector<u64> q, p, psi;      // psi indexed by prime id
     std::vector<u64> mod_of;         // modulus by prime id
     std::vector<double> delta;
@@ -145,7 +150,7 @@ struct ckks_ctx {
     std::vector<int*> d_modup_off, d_modup_pid;
     std::vector<int> modup_nrows;
     // per level: for each of the l + 1 rows of a ModUp input, N^{-1} qhat^{-1} of its digit's
-    // conversion (Shoup pairs, [l+1][2]), the inverse NTT's final factor for prescaled inputs
+    // conversion (pairs, [l+1][2]), the inverse NTT's final factor for prescaled inputs
     std::vector<u64*> d_modup_iscale;
     std::map<std::pair<int, int>, std::unique_ptr<ConvTab>> modup_tabs;  // (level, digit)
     std::map<int, std::unique_ptr<ConvTab>> moddown_tabs;               // level
@@ -453,6 +458,13 @@ u64 mulmod(u64 a, u64 b, u64 q);
 u64 powmod(u64 a, u64 e, u64 q);
 u64 invmod(u64 a, u64 q);
 u64 shoup(u64 w, u64 q);
+// the folding constants of q; false (and zeros) when q is not next to a power of two
+bool fold_consts(u64 q, FoldMod& f);
+// a transform constant w as the kernels take it: fold.cuh's packed digits, else w and its Shoup companion
+void ntt_pair(u64 w, u64 q, bool fold, u64* out2);
+// position of twiddle idx (2^stage + group) in a prime's table: in order, but for N = 2^16 the last
+// four stages of each eight-stage pass are transposed within a sub-problem (ntt.cu)
+int ntt_tw_pos(int idx, int logn);
 u64 from_signed(int64_t v, u64 q);
 DevMod make_mod(u64 q);
 bool is_prime(u64 n);

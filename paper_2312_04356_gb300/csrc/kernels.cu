@@ -1,4 +1,5 @@
-// Device kernels of the RNS-CKKS hot path and their launchers.
+// Device kernels of the RNS-CKKS hot path (all but the transforms, ntt.cu, and the tensor-core base
+// conversion, convert_tc.cu) and their launchers.
 //
 // Layout: a polynomial is [limb][N] uint64, limb k of an array of several
 // polynomials uses the prime with global id ids[k % lpp].  One CTA row of the
@@ -6,9 +7,6 @@
 #include "launch.cuh"
 
 #include <atomic>
-
-#include <cooperative_groups.h>
-namespace cg = cooperative_groups;
 
 // ------------------------------------------------------------ DevBuf -------
 thread_local const DevAlloc* tl_alloc = nullptr;
@@ -133,616 +131,6 @@ constexpr int EWV_VEC = 4;
         else                                                                                 \
             klaunch(c, K<1>, ewv_grid(c->n, (nl), 1), EW_THREADS, 0, __VA_ARGS__);        \
     } while (0)
-
-// ------------------------------------------------------------------ NTT ----
-// One pass covers `c` consecutive butterfly stages s0..s0+c-1 (stage s: 2^s groups,
-// stride t = N >> (s+1)).  Over those stages only index bits log2(T1)..log2(T0) move
-// (T0 = N >> (s0+1), T1 = N >> (s0+c)), so the limb splits into independent
-// sub-problems of 2^c elements j = hi*2T0 + k*T1 + lo.  A CTA stages SUB of them
-// (4096 elements) in shared memory, runs the c stages, and writes them back.
-constexpr int NTT_THREADS = 256;
-
-template <bool INV>
-__global__ void __launch_bounds__(NTT_THREADS)
-    k_ntt_pass(u64* __restrict__ data, const DevPrime* __restrict__ primes, const int* __restrict__ ids, int lpp,
-               size_t pstride, int logn, int s0, int c, int logsub, int scale_out, const u64* __restrict__ osc) {
-    griddep_entry();
-    extern __shared__ u64 sm[];
-    const int limb = blockIdx.y;
-    const DevPrime* P = primes + ids[limb % lpp];
-    const u64 q = P->m.q;
-    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(limb % lpp) << logn);
-    const int span = 1 << c;
-    const int SUB = 1 << logsub;
-    const int stride = SUB > 1 ? SUB + 1 : 1;
-    const int logT1 = logn - s0 - c;
-    const int T1 = 1 << logT1;
-    const int log2T0 = logn - s0;
-    const int sid0 = blockIdx.x * SUB;
-    const int total = SUB << c;
-
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        int s, k;
-        if (T1 == 1) {
-            s = e >> c;
-            k = e & (span - 1);
-        } else {
-            k = e >> logsub;
-            s = e & (SUB - 1);
-        }
-        int sid = sid0 + s;
-        size_t j = ((size_t)(sid >> logT1) << log2T0) + ((size_t)k << logT1) + (sid & (T1 - 1));
-        sm[k * stride + s] = a[j];
-    }
-    __syncthreads();
-
-    const int nbf = total >> 1;
-    for (int u = 0; u < c; ++u) {
-        const int uu = INV ? (c - 1 - u) : u;
-        const int sg = s0 + uu;               // global stage
-        const int lt = c - 1 - uu;            // log2 of the local stride
-        const int tk = 1 << lt;
-        for (int e = threadIdx.x; e < nbf; e += blockDim.x) {
-            const int s = e & (SUB - 1);
-            const int b = e >> logsub;
-            const int k = ((b >> lt) << (lt + 1)) | (b & (tk - 1));
-            const int sid = sid0 + s;
-            const size_t j = ((size_t)(sid >> logT1) << log2T0) + ((size_t)k << logT1) + (sid & (T1 - 1));
-            const int widx = (1 << sg) + (int)(j >> (logn - sg));
-            u64* px = sm + k * stride + s;
-            u64* py = sm + (k + tk) * stride + s;
-            const u64 x = *px, y = *py;
-            if (!INV) {
-                const ulonglong2 w = P->tw[widx];
-                const u64 v = mul_shoup(y, w.x, w.y, q);
-                *px = add_mod(x, v, q);
-                *py = sub_mod(x, v, q);
-            } else {
-                *px = add_mod(x, y, q);
-                const ulonglong2 w = P->itw[widx];
-                *py = mul_shoup(sub_mod(x, y, q), w.x, w.y, q);
-            }
-        }
-        __syncthreads();
-    }
-
-    // the inverse transform's final factor: N^{-1}, or per row a caller-given (w, w') Shoup pair
-    const u64 ninv = osc ? osc[2 * (limb % lpp)] : P->n_inv, ninvp = osc ? osc[2 * (limb % lpp) + 1] : P->n_inv_p;
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        int s, k;
-        if (T1 == 1) {
-            s = e >> c;
-            k = e & (span - 1);
-        } else {
-            k = e >> logsub;
-            s = e & (SUB - 1);
-        }
-        int sid = sid0 + s;
-        size_t j = ((size_t)(sid >> logT1) << log2T0) + ((size_t)k << logT1) + (sid & (T1 - 1));
-        u64 v = sm[k * stride + s];
-        if (scale_out) v = mul_shoup(v, ninv, ninvp, q);
-        a[j] = v;
-    }
-}
-
-// ---- fast path for N = 2^16: two passes of 8 stages, each as two radix-16 rounds ----
-// A pass works on 256-element sub-problems (k = 0..255), 16 threads per sub-problem,
-// 16 values per thread in registers.  Round A covers local stages u = 0..3 on the
-// elements k = t + 16 i, round B covers u = 4..7 on k = 16 t + i; one shared-memory
-// exchange separates them.  Butterflies are Harvey's lazy forms: forward values stay in
-// [0, 4q), inverse values in [0, 2q); the last forward pass and the N^{-1} scaling
-// return canonical residues.  Twiddle of local stage u for element k of sub-problem hi:
-// index 2^(s0+u) + hi 2^u + (k >> (8 - u)).
-constexpr int F_STRIDE = 273;             // shared words per sub-problem: 256 + 16 pad, odd
-__device__ __forceinline__ int f_slot(int sp, int k) { return sp * F_STRIDE + k + (k >> 4); }
-
-// Forward butterflies reduce the upper input only on odd local stages (threshold 4q): an
-// uncorrected stage maps inputs in [0, b q) to [0, (b + 2) q), a corrected one (valid for
-// b <= 8) to [0, 6q).  From canonical inputs the values stay below 8q, which fits in 64
-// bits for every prime below 2^61; each pass ends in [0, 6q).
-template <bool CORR>
-__device__ __forceinline__ void ct_bfly(u64& x, u64& y, u64 w, u64 wp, u64 q, u64 q2, u64 q4) {
-    if (CORR && x >= q4) x -= q4;
-    const u64 t = y * w - __umul64hi(y, wp) * q;   // [0, 2q)
-    y = x - t + q2;
-    x = x + t;
-}
-__device__ __forceinline__ void gs_bfly(u64& x, u64& y, u64 w, u64 wp, u64 q, u64 q2) {
-    u64 s = x + y;
-    if (s >= q2) s -= q2;
-    const u64 d = x - y + q2;
-    y = d * w - __umul64hi(d, wp) * q;             // [0, 2q)
-    x = s;
-}
-
-// forward round over 4 local stages u0..u0+3; element i of the thread has index k(i);
-// tw index offset for lower element i at stage u: base_u + (k(i) >> (8 - u))
-template <bool ROUND_B>
-__device__ __forceinline__ void fwd_round(u64 (&x)[16], int t, int hi, int s0, const DevPrime* __restrict__ P,
-                                          u64 q, u64 q2) {
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int u = (ROUND_B ? 4 : 0) + s;
-        const int is = 8 >> s;
-        const int base = (1 << (s0 + u)) + (hi << u);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (i & is) continue;
-            const int idx = ROUND_B ? base + (t << s) + (i >> (4 - s)) : base + (i >> (4 - s));
-            const ulonglong2 w = __ldg(P->tw + idx);
-            if (u & 1)
-                ct_bfly<true>(x[i], x[i + is], w.x, w.y, q, q2, 2 * q2);
-            else
-                ct_bfly<false>(x[i], x[i + is], w.x, w.y, q, q2, 2 * q2);
-        }
-    }
-}
-
-template <bool ROUND_B>
-__device__ __forceinline__ void inv_round(u64 (&x)[16], int t, int hi, int s0, const DevPrime* __restrict__ P,
-                                          u64 q, u64 q2) {
-#pragma unroll
-    for (int s = 3; s >= 0; --s) {
-        const int u = (ROUND_B ? 4 : 0) + s;
-        const int is = 8 >> s;
-        const int base = (1 << (s0 + u)) + (hi << u);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (i & is) continue;
-            const int idx = ROUND_B ? base + (t << s) + (i >> (4 - s)) : base + (i >> (4 - s));
-            const ulonglong2 w = __ldg(P->itw + idx);
-            gs_bfly(x[i], x[i + is], w.x, w.y, q, q2);
-        }
-    }
-}
-
-// Input of the inverse transform's first pass when it is not the data array itself (SRC
-// kernels): row k reads src + (k / lpp) * src_pstride + (k % lpp) N and the result goes to the
-// data array, so the input is left as it is (no copy before an out-of-place transform).
-// ow != 0 replaces the final factor N^{-1} by the Shoup pair (ow, owp), e.g. k N^{-1} to
-// multiply the result by the integer k.
-struct NttSrc {
-    const u64* src;
-    size_t src_pstride;
-    u64 ow, owp;
-};
-
-// COL: sub-problems are columns (s0 = 0, T1 = 256, element j = k*256 + lo), threads with
-//      consecutive tid take consecutive columns.  ROW: sub-problems are contiguous rows
-//      (s0 = 8, T1 = 1, j = hi*256 + k), consecutive tid take consecutive k.
-template <bool COL, bool INV, int SUBS, int MINB, bool SRC = false>
-__global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ data, const DevPrime* __restrict__ primes,
-                                                    const int* __restrict__ ids, int lpp, size_t pstride,
-                                                    const int* __restrict__ loff, const u64* __restrict__ osc,
-                                                    NttSrc io) {
-    static_assert(!SRC || (INV && !COL), "only the inverse transform's first pass reads a separate source");
-    griddep_entry();
-    __shared__ u64 sm[SUBS * F_STRIDE];
-    const int limb = blockIdx.y;
-    const int r = limb % lpp;
-    const DevPrime* P = primes + ids[r];
-    const u64 q = P->m.q, q2 = 2 * q;
-    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(loff ? loff[r] : r) << 16);
-    const int tid = threadIdx.x;
-    const int sp = COL ? (tid % SUBS) : (tid >> 4);
-    const int t = COL ? (tid / SUBS) : (tid & 15);
-    const int sub = blockIdx.x * SUBS + sp;            // global sub-problem: column lo or row hi
-    const int s0 = COL ? 0 : 8;
-    const int hi = COL ? 0 : sub;
-    u64 x[16];
-    auto gidx = [&](int k) -> size_t { return COL ? ((size_t)k << 8) + sub : ((size_t)sub << 8) + k; };
-
-    if (!INV) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = a[gidx(t + 16 * i)];
-        fwd_round<false>(x, t, hi, s0, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(sp, t + 16 * i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(sp, 16 * t + i)];
-        fwd_round<true>(x, t, hi, s0, P, q, q2);
-        if (COL) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(16 * t + i)] = x[i];     // lazy, [0, 6q)
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                u64 v = x[i];
-                if (v >= 2 * q2) v -= 2 * q2;
-                if (v >= q2) v -= q2;
-                if (v >= q) v -= q;
-                x[i] = v;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) sm[f_slot(sp, 16 * t + i)] = x[i];
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = sm[f_slot(sp, t + 16 * i)];
-        }
-    } else {
-        if (COL) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = a[gidx(16 * t + i)];
-        } else {
-            const u64* sr = SRC ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << 16) : a;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) sm[f_slot(sp, t + 16 * i)] = sr[gidx(t + 16 * i)];
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(sp, 16 * t + i)];
-            __syncthreads();
-        }
-        inv_round<true>(x, t, hi, s0, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(sp, 16 * t + i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(sp, t + 16 * i)];
-        inv_round<false>(x, t, hi, s0, P, q, q2);
-        if (COL) {
-            const u64 ni = io.ow ? io.ow : osc ? osc[2 * r] : P->n_inv;
-            const u64 nip = io.ow ? io.owp : osc ? osc[2 * r + 1] : P->n_inv_p;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = mul_shoup(x[i], ni, nip, q);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = x[i];     // lazy, [0, 2q)
-        }
-    }
-}
-
-// ---- the same pass with 4 values per thread: four radix-4 register rounds (local stages
-// 2r, 2r+1), three shared-memory exchanges, 64 threads per sub-problem and 4 sub-problems
-// per 256-thread CTA: four times the threads of k_ntt16, for launches over few limbs.
-// In round r thread t holds k0 + {0, e, d, d + e} (d = 128 >> 2r, e = d / 2), k0 = t with
-// zero bits inserted at the positions of d and e.  Butterflies, twiddle indices and the
-// lazy bounds are those of k_ntt16, so both kernels return the same residues.
-__device__ __forceinline__ int ins0(int t, int p) { return ((t >> p) << (p + 1)) | (t & ((1 << p) - 1)); }
-
-template <bool COL, bool INV, bool SRC = false>
-__global__ void __launch_bounds__(256) k_ntt16s(u64* __restrict__ data, const DevPrime* __restrict__ primes,
-                                                const int* __restrict__ ids, int lpp, size_t pstride,
-                                                const int* __restrict__ loff, const u64* __restrict__ osc,
-                                                NttSrc io) {
-    static_assert(!SRC || (INV && !COL), "only the inverse transform's first pass reads a separate source");
-    griddep_entry();
-    __shared__ u64 sm[4 * F_STRIDE];
-    const int limb = blockIdx.y;
-    const int r = limb % lpp;
-    const DevPrime* P = primes + ids[r];
-    const u64 q = P->m.q, q2 = 2 * q;
-    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(loff ? loff[r] : r) << 16);
-    const int tid = threadIdx.x;
-    const int sp = COL ? (tid & 3) : (tid >> 6);
-    const int t = COL ? (tid >> 2) : (tid & 63);
-    const int sub = blockIdx.x * 4 + sp;
-    const int s0 = COL ? 0 : 8;
-    const int hi = COL ? 0 : sub;
-    auto gidx = [&](int k) -> size_t { return COL ? ((size_t)k << 8) + sub : ((size_t)sub << 8) + k; };
-    u64 x[4];
-    int k0 = 0;
-    if (!INV) {
-#pragma unroll
-        for (int rr = 0; rr < 4; ++rr) {
-            const int u = 2 * rr, d = 128 >> u, e = d >> 1;
-            k0 = ins0(ins0(t, 6 - u), 7 - u);
-            const int ks[4] = {k0, k0 + e, k0 + d, k0 + d + e};
-            if (rr == 0) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = a[gidx(ks[i])];
-            } else {
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = sm[f_slot(sp, ks[i])];
-            }
-            // stage u (odd/even correction as in k_ntt16): pairs (0, 2), (1, 3), one twiddle
-            {
-                const ulonglong2 w = __ldg(P->tw + (1 << (s0 + u)) + (hi << u) + (k0 >> (8 - u)));
-                ct_bfly<false>(x[0], x[2], w.x, w.y, q, q2, 2 * q2);
-                ct_bfly<false>(x[1], x[3], w.x, w.y, q, q2, 2 * q2);
-            }
-            // stage u + 1 (odd): pairs (0, 1), (2, 3)
-            {
-                const int base = (1 << (s0 + u + 1)) + (hi << (u + 1));
-                const ulonglong2 w0 = __ldg(P->tw + base + (k0 >> (7 - u)));
-                const ulonglong2 w1 = __ldg(P->tw + base + ((k0 + d) >> (7 - u)));
-                ct_bfly<true>(x[0], x[1], w0.x, w0.y, q, q2, 2 * q2);
-                ct_bfly<true>(x[2], x[3], w1.x, w1.y, q, q2, 2 * q2);
-            }
-            if (rr < 3) {
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) sm[f_slot(sp, ks[i])] = x[i];
-            } else if (COL) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[gidx(ks[i])] = x[i];     // lazy, [0, 6q)
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    u64 v = x[i];
-                    if (v >= 2 * q2) v -= 2 * q2;
-                    if (v >= q2) v -= q2;
-                    if (v >= q) v -= q;
-                    a[gidx(ks[i])] = v;
-                }
-            }
-        }
-    } else {
-#pragma unroll
-        for (int rr = 3; rr >= 0; --rr) {
-            const int u = 2 * rr, d = 128 >> u, e = d >> 1;
-            k0 = ins0(ins0(t, 6 - u), 7 - u);
-            const int ks[4] = {k0, k0 + e, k0 + d, k0 + d + e};
-            if (rr == 3) {
-                const u64* sr = SRC ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << 16) : a;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = sr[gidx(ks[i])];
-            } else {
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = sm[f_slot(sp, ks[i])];
-            }
-            // stage u + 1 first: pairs (0, 1), (2, 3)
-            {
-                const int base = (1 << (s0 + u + 1)) + (hi << (u + 1));
-                const ulonglong2 w0 = __ldg(P->itw + base + (k0 >> (7 - u)));
-                const ulonglong2 w1 = __ldg(P->itw + base + ((k0 + d) >> (7 - u)));
-                gs_bfly(x[0], x[1], w0.x, w0.y, q, q2);
-                gs_bfly(x[2], x[3], w1.x, w1.y, q, q2);
-            }
-            // stage u: pairs (0, 2), (1, 3)
-            {
-                const ulonglong2 w = __ldg(P->itw + (1 << (s0 + u)) + (hi << u) + (k0 >> (8 - u)));
-                gs_bfly(x[0], x[2], w.x, w.y, q, q2);
-                gs_bfly(x[1], x[3], w.x, w.y, q, q2);
-            }
-            if (rr > 0) {
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) sm[f_slot(sp, ks[i])] = x[i];
-            } else if (COL) {
-                const u64 ni = io.ow ? io.ow : osc ? osc[2 * r] : P->n_inv;
-                const u64 nip = io.ow ? io.owp : osc ? osc[2 * r + 1] : P->n_inv_p;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[gidx(ks[i])] = mul_shoup(x[i], ni, nip, q);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[gidx(ks[i])] = x[i];     // lazy, [0, 2q)
-            }
-        }
-    }
-}
-
-// ---- the whole N = 2^16 transform in one launch: a cluster of 8 CTAs per limb (512 threads
-// each, 16 values per thread).  Forward: CTA r runs stages 0-7 on columns 32r .. 32r+31 (the
-// COL pass of k_ntt16 with 32 sub-problems), writes them to its shared memory as [row][32],
-// and after a cluster barrier reads rows 32r .. 32r+31 from all eight CTAs through
-// distributed shared memory for stages 8-15 (the ROW pass).  Inverse: the same in reverse
-// order.  Butterflies, twiddles and lazy bounds are those of k_ntt16, so the residues are
-// identical; the data makes one trip through HBM instead of two.  Every thread of every CTA
-// reaches both cluster barriers (no early exit), and the second barrier keeps each CTA's
-// shared memory alive until the other CTAs have read it.
-constexpr int CL_SUBS = 32, CL_THREADS = 512, CL_SMEM_WORDS = CL_SUBS * F_STRIDE;
-
-template <bool INV>
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(CL_THREADS, 2)
-    k_ntt_cl(u64* __restrict__ data, const DevPrime* __restrict__ primes, const int* __restrict__ ids, int lpp,
-             size_t pstride, const int* __restrict__ loff, const u64* __restrict__ osc, NttSrc io) {
-    griddep_entry();
-    extern __shared__ u64 sm[];
-    cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank();
-    const int limb = blockIdx.y;
-    const int r = limb % lpp;
-    const DevPrime* P = primes + ids[r];
-    const u64 q = P->m.q, q2 = 2 * q;
-    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(loff ? loff[r] : r) << 16);
-    const int tid = threadIdx.x;
-    // COL mapping: column 32 rank + spc, elements (rows) t + 16 i / 16 t + i
-    const int spc = tid % CL_SUBS, tc = tid / CL_SUBS, col = CL_SUBS * rank + spc;
-    // ROW mapping: row 32 rank + spr, elements (columns) t + 16 i / 16 t + i
-    const int spr = tid >> 4, tr = tid & 15, row = CL_SUBS * rank + spr;
-    u64 x[16];
-    if (!INV) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = a[((size_t)(tc + 16 * i) << 8) + col];
-        fwd_round<false>(x, tc, 0, 0, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(spc, tc + 16 * i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(spc, 16 * tc + i)];
-        fwd_round<true>(x, tc, 0, 0, P, q, q2);                      // column col, rows 16 tc + i
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[(16 * tc + i) * CL_SUBS + spc] = x[i];
-        cl.sync();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {                               // column tr + 16 i of row `row`
-            const u64* src = cl.map_shared_rank(sm, i >> 1);
-            x[i] = src[row * CL_SUBS + tr + 16 * (i & 1)];
-        }
-        cl.sync();
-        fwd_round<false>(x, tr, row, 8, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(spr, tr + 16 * i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(spr, 16 * tr + i)];
-        fwd_round<true>(x, tr, row, 8, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            u64 v = x[i];
-            if (v >= 2 * q2) v -= 2 * q2;
-            if (v >= q2) v -= q2;
-            if (v >= q) v -= q;
-            x[i] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(spr, 16 * tr + i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) a[((size_t)row << 8) + tr + 16 * i] = sm[f_slot(spr, tr + 16 * i)];
-    } else {
-        const u64* sr = io.src ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << 16) : a;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(spr, tr + 16 * i)] = sr[((size_t)row << 8) + tr + 16 * i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(spr, 16 * tr + i)];
-        __syncthreads();
-        inv_round<true>(x, tr, row, 8, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(spr, 16 * tr + i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(spr, tr + 16 * i)];
-        inv_round<false>(x, tr, row, 8, P, q, q2);                   // row `row`, columns tr + 16 i
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[spr * 256 + tr + 16 * i] = x[i];
-        cl.sync();
-        {
-            const u64* src = cl.map_shared_rank(sm, tc >> 1);          // rows 16 tc + i live there
-#pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = src[(16 * (tc & 1) + i) * 256 + col];
-        }
-        cl.sync();
-        inv_round<true>(x, tc, 0, 0, P, q, q2);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) sm[f_slot(spc, 16 * tc + i)] = x[i];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = sm[f_slot(spc, tc + 16 * i)];
-        inv_round<false>(x, tc, 0, 0, P, q, q2);
-        const u64 ni = io.ow ? io.ow : osc ? osc[2 * r] : P->n_inv;
-        const u64 nip = io.ow ? io.owp : osc ? osc[2 * r + 1] : P->n_inv_p;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) a[((size_t)(tc + 16 * i) << 8) + col] = mul_shoup(x[i], ni, nip, q);
-    }
-}
-
-// few limbs: 64-thread CTAs (4 sub-problems) so that the grid still covers the SMs
-// Variants (identical results): CTA of 16 or 4 sub-problems, register budget for 3 or 4
-// resident 256-thread CTAs per SM.  ckks_autotune times them per limb-count class; the
-// default (no tuning) is 16 sub-problems at >= 16 limbs, else 4, 80 registers.
-enum NttVariant {
-    NTT_V16_R80 = 0, NTT_V16_R64 = 1, NTT_V4_R80 = 2, NTT_V4_R64 = 3, NTT_X4 = 4, NTT_CL = 5, NTT_NVARIANTS = 6
-};
-
-template <bool COL, bool INV, bool SRC = false>
-void launch_ntt16_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const int* ids, int lpp,
-                          size_t pstride, const int* loff, const u64* osc, const NttSrc& io) {
-    switch (v) {
-        case NTT_V16_R80:
-            klaunch(cx, k_ntt16<COL, INV, 16, 3, SRC>, dim3(256 / 16, nlimbs), 256, 0,
-                    data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-            break;
-        case NTT_V16_R64:
-            klaunch(cx, k_ntt16<COL, INV, 16, 4, SRC>, dim3(256 / 16, nlimbs), 256, 0,
-                    data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-            break;
-        case NTT_V4_R80:
-            klaunch(cx, k_ntt16<COL, INV, 4, 8, SRC>, dim3(256 / 4, nlimbs), 64, 0,
-                    data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-            break;
-        case NTT_V4_R64:
-            klaunch(cx, k_ntt16<COL, INV, 4, 12, SRC>, dim3(256 / 4, nlimbs), 64, 0,
-                    data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-            break;
-        default:
-            klaunch(cx, k_ntt16s<COL, INV, SRC>, dim3(256 / 4, nlimbs), 256, 0,
-                    data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-            break;
-    }
-}
-
-inline int ntt_class(int nlimbs) {
-    int c = 0;
-    while (c < 7 && (2 << c) <= nlimbs) ++c;   // classes: 1, 2-3, 4-7, 8-15, 16-31, 32-63, 64-127, >=128
-    return c;
-}
-
-template <bool INV>
-void launch_ntt_cl(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
-                   const int* loff, const u64* osc, const NttSrc& io) {
-    static std::atomic<unsigned> done{0};
-    allow_dynamic_smem((const void*)k_ntt_cl<INV>, CL_SMEM_WORDS * (int)sizeof(u64), done);
-    klaunch(cx, k_ntt_cl<INV>, dim3(8, nlimbs), CL_THREADS, CL_SMEM_WORDS * sizeof(u64),
-            data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-}
-
-// One whole N = 2^16 transform with variant v: the cluster kernel, or the two passes (forward:
-// COL then ROW; inverse: ROW then COL).  Algorithmic bytes: one read and one write of the
-// limbs per transform, split evenly over the two passes.
-// (io: a separate source of the inverse's first pass and an output factor, as NttSrc
-// describes)
-template <bool INV>
-void launch_ntt_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
-                        const int* loff, const u64* osc = nullptr, const NttSrc& io = NttSrc{}) {
-    const char* nm = INV ? "ntt_inv" : "ntt_fwd";
-    const double bytes = 2.0 * nlimbs * cx->n * 8.0;
-    CK_CHECK(INV || !io.src, CKKS_EINVAL, "only the inverse transform reads a separate source");
-    if (v == NTT_CL) {
-        KTimer kt_(cx, nm, bytes);
-        launch_ntt_cl<INV>(cx, data, nlimbs, ids, lpp, pstride, loff, osc, io);
-        return;
-    }
-    {
-        KTimer kt_(cx, nm, bytes / 2);
-        if (INV && io.src)     // the inverse's first pass is the ROW pass
-            launch_ntt16_variant<false, true, true>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
-        else
-            launch_ntt16_variant<!INV, INV>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
-    }
-    {
-        KTimer kt_(cx, nm, bytes / 2);
-        launch_ntt16_variant<INV, INV>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
-    }
-}
-
-// the variant that transforms of nlimbs limbs use: the tuned one of their size class, else
-// 16 sub-problems per CTA from 16 limbs on and 4 below
-inline int ntt_pick(const ckks_ctx* cx, int nlimbs) {
-    const int v = cx->ntt_choice[ntt_class(nlimbs)];
-    return v >= 0 ? v : nlimbs >= 16 ? NTT_V16_R80 : NTT_V4_R80;
-}
-
-template <bool INV>
-void launch_ntt_transform(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
-                          const int* loff = nullptr, const u64* osc = nullptr, const NttSrc& io = NttSrc{}) {
-    launch_ntt_variant<INV>(cx, ntt_pick(cx, nlimbs), data, nlimbs, ids, lpp, pstride, loff, osc, io);
-}
-
-struct PassPlan {
-    int s0, c;
-};
-
-inline std::vector<PassPlan> ntt_passes(int logn) {
-    if (logn <= 12) return {{0, logn}};
-    return {{0, logn - 8}, {logn - 8, 8}};
-}
-
-template <bool INV>
-void launch_pass(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride, PassPlan p,
-                 int scale_out, const u64* osc = nullptr) {
-    const int logn = cx->logn;
-    int logsub = 12 - p.c;
-    if (logsub < 0) logsub = 0;
-    if (logsub > logn - p.c) logsub = logn - p.c;
-    const int SUB = 1 << logsub;
-    const int tiles = (1 << (logn - p.c)) / SUB;
-    const int stride = SUB > 1 ? SUB + 1 : 1;
-    const size_t smem = (size_t)stride * (1 << p.c) * sizeof(u64);
-    dim3 grid(tiles, nlimbs);
-    { KTimer kt_(cx, INV ? "ntt_inv" : "ntt_fwd", 2.0 * nlimbs * cx->n * 8.0 * p.c / logn);
-    klaunch(cx, k_ntt_pass<INV>, grid, NTT_THREADS, smem, data, cx->d_primes, ids, lpp, pstride, logn, p.s0, p.c,
-            logsub, scale_out, osc);
-    }
-}
 
 // ----------------------------------------------------------- elementwise ----
 // One thread per V consecutive words of a limb (V = 2 or 4: 16-byte loads and stores, used
@@ -1027,8 +415,8 @@ __global__ void k_imult(const u64* a, u64* o, const DevPrime* P, const int* ids,
     const DevPrime* pr = P + ids[limb % lpp];
     const u64 q = pr->m.q;
     // X^{N/2} at psi^(2r+1): psi^{N/2} when r is even, -psi^{N/2} when r is odd;
-    // psi^{N/2} = tw[1] since rev(1) = N/2
-    const u64 w = pr->tw[1].x, wp = pr->tw[1].y;
+    // psi^{N/2} is the prime's im
+    const u64 w = pr->im, wp = pr->im_p;
     const size_t off = (size_t)limb << logn;
     EW_LOOP(1 << logn) {
         u64 v = mul_shoup(a[off + j], w, wp, q);
@@ -1595,69 +983,6 @@ namespace kern {
 
 #define LAUNCH_CHECK() CUDA_CHECK(cudaGetLastError())
 
-void ntt_forward(const ckks_ctx* c, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride) {
-    if (nlimbs <= 0) return;
-    if (pstride == 0) pstride = (size_t)lpp * c->n;
-    if (c->logn == 16) {
-        launch_ntt_transform<false>(c, data, nlimbs, ids, lpp, pstride);
-        LAUNCH_CHECK();
-        return;
-    }
-    for (const PassPlan& p : ntt_passes(c->logn)) launch_pass<false>(c, data, nlimbs, ids, lpp, pstride, p, 0);
-    LAUNCH_CHECK();
-}
-
-// Time every NTT variant (forward + inverse) on scratch limbs of each size class and keep the
-// fastest per class in ctx->ntt_choice.  Results are identical for every variant.
-void autotune_ntt(ckks_ctx* c, int reps) {
-    if (c->logn != 16) return;
-    const int sizes[8] = {1, 2, 7, 14, 24, 48, 96, 192};
-    DevBuf buf((size_t)192 << 16, c->stream);
-    CUDA_CHECK(cudaMemsetAsync(buf.ptr, 0, ((size_t)192 << 16) * 8, c->stream));
-    std::vector<int> ids(192);
-    for (int i = 0; i < 192; ++i) ids[i] = i % c->nall;
-    DevBuf dids(96, c->stream);
-    CUDA_CHECK(cudaMemcpyAsync(dids.ptr, ids.data(), 192 * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    for (int k = 0; k < 8; ++k) {
-        const int nl = sizes[k];
-        float best = 1e30f;
-        int bestv = -1;
-        for (int v = 0; v < NTT_NVARIANTS; ++v) {
-            for (int w = 0; w < 2; ++w) {   // warm up, then time
-                cudaEventRecord(e0, c->stream);
-                for (int r = 0; r < reps; ++r) {
-                    const int* d = (const int*)dids.ptr;
-                    launch_ntt_variant<false>(c, v, buf.ptr, nl, d, nl, (size_t)nl << 16, nullptr);
-                    launch_ntt_variant<true>(c, v, buf.ptr, nl, d, nl, (size_t)nl << 16, nullptr);
-                }
-                cudaEventRecord(e1, c->stream);
-                CUDA_CHECK(cudaEventSynchronize(e1));
-            }
-            float ms = 0;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
-                best = ms;
-                bestv = v;
-            }
-        }
-        c->ntt_choice[k] = bestv;
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    LAUNCH_CHECK();
-}
-
-void ntt_forward_list(const ckks_ctx* c, u64* data, int nlimbs, const int* off, const int* ids, int nb,
-                      size_t bstride) {
-    if (nlimbs <= 0 || nb <= 0) return;
-    CK_CHECK(c->logn == 16, CKKS_EINVAL, "limb-list NTT needs N = 2^16");
-    launch_ntt_transform<false>(c, data, nlimbs * nb, ids, nlimbs, bstride, off);
-    LAUNCH_CHECK();
-}
-
 template <int V>
 static void launch_bsgs_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int* ids, const KsBatch& bt) {
     const dim3 grid = ewv_grid(c->n, 2 * nl * bt.nb, V);
@@ -1762,53 +1087,6 @@ void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* 
         launch_bsgs_async(c, t, D, c0, c1, nl, next, ext_ids, s, sp, bt);
     }
     LAUNCH_CHECK();
-}
-
-void ntt_inverse(const ckks_ctx* c, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride, const u64* osc) {
-    if (nlimbs <= 0) return;
-    if (pstride == 0) pstride = (size_t)lpp * c->n;
-    if (c->logn == 16) {
-        launch_ntt_transform<true>(c, data, nlimbs, ids, lpp, pstride, nullptr, osc);
-        LAUNCH_CHECK();
-        return;
-    }
-    std::vector<PassPlan> ps = ntt_passes(c->logn);
-    for (int i = (int)ps.size() - 1; i >= 0; --i)
-        launch_pass<true>(c, data, nlimbs, ids, lpp, pstride, ps[i], ps[i].s0 == 0 ? 1 : 0,
-                          ps[i].s0 == 0 ? osc : nullptr);
-    LAUNCH_CHECK();
-}
-
-void ntt_inverse_from(const ckks_ctx* c, const u64* src, size_t src_pstride, u64* data, int nlimbs, const int* ids,
-                      int lpp, size_t pstride, const u64* osc, u64 kres, int k_id) {
-    if (nlimbs <= 0) return;
-    if (pstride == 0) pstride = (size_t)lpp * c->n;
-    const bool scaled = k_id >= 0 && kres != 1;
-    CK_CHECK(nlimbs % lpp == 0, CKKS_EINVAL, "whole polynomials only");
-    CK_CHECK(!scaled || (lpp == 1 && osc == nullptr && pstride == c->n), CKKS_EINVAL,
-             "an integer factor needs one contiguous row per polynomial and no output scale table");
-    if (c->logn == 16) {
-        NttSrc io{src, src_pstride, 0, 0};
-        if (scaled) {
-            const u64 q = c->mod_of[k_id];
-            io.ow = hostmath::mulmod(kres, hostmath::invmod((u64)c->n % q, q), q);
-            io.owp = hostmath::shoup(io.ow, q);
-        }
-        launch_ntt_transform<true>(c, data, nlimbs, ids, lpp, pstride, nullptr, osc, io);
-        LAUNCH_CHECK();
-        return;
-    }
-    // the smaller rings: copy (and scale), then transform in place
-    if (scaled) {
-        ScalarVec sv;
-        sv.v[0] = kres;
-        sv.vp[0] = hostmath::shoup(kres, c->mod_of[k_id]);
-        mul_scalar_v(c, src, sv, data, nlimbs, ids, 1, src_pstride);
-    } else {
-        CUDA_CHECK(cudaMemcpy2DAsync(data, pstride * 8, src, src_pstride * 8, (size_t)lpp * c->n * 8, nlimbs / lpp,
-                                     cudaMemcpyDeviceToDevice, c->stream));
-    }
-    ntt_inverse(c, data, nlimbs, ids, lpp, pstride, osc);
 }
 
 void add(const ckks_ctx* c, const u64* a, const u64* b, u64* o, int nl, const int* ids, int lpp) {

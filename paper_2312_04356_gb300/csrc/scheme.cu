@@ -99,8 +99,7 @@ static std::unique_ptr<ConvTab> make_conv_tab(ckks_ctx* c, const std::vector<int
     std::vector<u64> isc(2 * t->nin);
     for (int i = 0; i < t->nin; ++i) {
         const u64 qi = c->mod_of[in_ids[i]];
-        isc[2 * i] = mulmod(invmod((u64)c->n % qi, qi), qinv[i], qi);
-        isc[2 * i + 1] = shoup(isc[2 * i], qi);
+        ntt_pair(mulmod(invmod((u64)c->n % qi, qi), qinv[i], qi), qi, c->fold, &isc[2 * i]);
     }
     t->d_iscale = dev_upload_persistent(isc);
     std::vector<int> ids_rows = out_ids;
@@ -251,8 +250,10 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
     c->mod_of = c->q;
     c->mod_of.insert(c->mod_of.end(), c->p.begin(), c->p.end());
     c->mods_below_2_60 = std::all_of(c->mod_of.begin(), c->mod_of.end(), [](u64 m) { return m < (1ull << 60); });
+    FoldMod fm;
+    c->fold = std::all_of(c->mod_of.begin(), c->mod_of.end(), [&](u64 m) { return fold_consts(m, fm); });
     const int n = c->n, logn = c->logn;
-    // twiddle tables: per prime 2 arrays of N (value, Shoup companion) pairs
+    // twiddle tables: per prime 2 arrays of N pairs
     std::vector<u64> tables((size_t)c->nall * 4 * n);
     std::vector<DevPrime> primes(c->nall);
     c->psi.resize(c->nall);
@@ -273,18 +274,21 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
         u64* base = tables.data() + (size_t)id * 4 * n;
         for (int k = 0; k < n; ++k) {
             unsigned r = brev_host(k, logn);
-            base[2 * k] = pw[r];
-            base[2 * k + 1] = shoup(pw[r], qq);
-            base[2 * n + 2 * k] = ipw[r];
-            base[2 * n + 2 * k + 1] = shoup(ipw[r], qq);
+            const size_t at = 2 * (size_t)ntt_tw_pos(k, logn);
+            ntt_pair(pw[r], qq, c->fold, base + at);
+            ntt_pair(ipw[r], qq, c->fold, base + 2 * n + at);
         }
         DevPrime& dp = primes[id];
         dp.m = c->mods[id];
+        fold_consts(qq, dp.f);
         const u64* dbase = c->d_tables + (size_t)id * 4 * n;
         dp.tw = reinterpret_cast<const ulonglong2*>(dbase);
         dp.itw = reinterpret_cast<const ulonglong2*>(dbase + 2 * n);
-        dp.n_inv = invmod((u64)n % qq, qq);
-        dp.n_inv_p = shoup(dp.n_inv, qq);
+        u64 ni[2];
+        ntt_pair(invmod((u64)n % qq, qq), qq, c->fold, ni);
+        dp.n_inv = make_ulonglong2(ni[0], ni[1]);
+        dp.im = pw[n / 2];
+        dp.im_p = shoup(dp.im, qq);
         dp.r64 = (u64)(((unsigned __int128)1 << 64) % qq);
         dp.r64p = shoup(dp.r64, qq);
         dp.inv64 = (u64)((((unsigned __int128)1) << 64) / qq);

@@ -1,0 +1,58 @@
+"""Transforms in both arithmetics (folded products for primes next to a power of two, Shoup products
+for others) at the ends of their ranges: every one-CTA ring size, the two-pass ring in every
+launch variant, and residues at the extremes (all q - 1, 0 / q - 1 alternating), where the lazy
+values are largest.  Integers: compared bit for bit with the oracle."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+# (log_n, q0_bits, scale_bits, p_bits): primes 2^k +- small qualify for folding up to 60 bits; one
+# 61-bit (or below 33-bit) prime puts the whole context on Shoup products
+CASES = [(n, 60, 42, 60) for n in (7, 8, 9, 10, 11, 12, 13, 16)] + \
+        [(12, 50, 34, 57), (16, 55, 36, 56), (12, 61, 40, 60), (16, 60, 42, 61), (8, 45, 30, 45)]
+
+
+@pytest.mark.parametrize("log_n,q0,sc,pb", CASES)
+def test_transform_extremes_bitexact(log_n, q0, sc, pb):
+    from oracle import _clib as C
+    from oracle import params as PP
+    from paper_2312_04356_gb300 import build
+    from paper_2312_04356_gb300 import ckks as K
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    d = dict(log_n=log_n, n_q=4, dnum=1, n_p=1, q0_bits=q0, scale_bits=sc, p_bits=pb, boot_bits=0, n_boot=0, h=0,
+             sigma=3.2)
+    P = PP.Params(log_n, 4, 1, q0, sc, pb, h=0, n_p=1)
+    ctx = K.ckks_ctx_create(d, 1, torch.cuda.current_stream().cuda_stream)
+    q, p, _, _ = K.ckks_ctx_info(ctx)
+    mods = q + p
+    assert mods == list(P.q) + list(P.p)
+    n, ids = 1 << log_n, list(range(len(mods))) * 4
+    g = np.random.default_rng(3)
+    rows = []
+    for fill in ("top", "alternate", "random", "impulse"):
+        for m in mods:
+            if fill == "top":
+                r = np.full(n, m - 1, dtype=np.uint64)
+            elif fill == "alternate":
+                r = np.where(np.arange(n) % 2 == 0, 0, m - 1).astype(np.uint64)
+            elif fill == "random":
+                r = g.integers(0, m, n, dtype=np.uint64)
+            else:
+                r = np.zeros(n, dtype=np.uint64)
+                r[-1] = m - 1
+            rows.append(r)
+    x = np.stack(rows)
+    psi = (list(P.psi_q) + list(P.psi_p)) * 4
+    fwd = C.ntt_forward(x, mods * 4, psi, log_n)
+    inv = C.ntt_inverse(x, mods * 4, psi, log_n)
+    for variant in range(-1, 6) if log_n == 16 else [-1]:
+        K.ckks_ctx_set_ntt_variant(ctx, variant)
+        for call, want in ((K.ckks_ntt_forward, fwd), (K.ckks_ntt_inverse, inv)):
+            dev = torch.from_numpy(x.view(np.int64).copy()).cuda()
+            call(ctx, dev.data_ptr(), len(ids), ids)
+            torch.cuda.synchronize()
+            assert (dev.cpu().numpy().view(np.uint64) == want).all(), (variant, call.__name__)
