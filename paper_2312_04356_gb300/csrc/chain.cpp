@@ -80,6 +80,13 @@ bool fold_consts(u64 q, FoldMod& f) {
     if ((big ? ((u128)8 << (60 - K)) : (top >> K) + 1) * ae >= q) return false;   // canonical after one fold
     // |x0 W0 + x1 W1| <= (2^31 + |x1|) q / 2 < 2^(K + 31)
     if ((((u128)1 << 31) + (lim >> 32) + 2) * q >= ((u128)1 << (K + 32))) return false;
+    // 128-bit sums: T = L + (V >> s) e_r stays below 2^(K + 31) and its fold is a lazy word
+    const int s = big ? 64 : K;
+    const u128 aer = ae << (s - K), H = ((u128)40 * q * q) >> s;
+    if (aer >= ((u128)1 << 31) || H >= ((u128)1 << 62) || H * aer + ((u128)2 << s) >= ((u128)7 << (K + 28))) return false;
+    f.kr = (unsigned)(s - 32);
+    f.maskr = (unsigned)(((u64)1 << (s - 32)) - 1);
+    f.er = (int)(e < 0 ? -(int64_t)(u64)aer : (int64_t)(u64)aer);
     f.kc = (unsigned)(K - 32);
     f.mask = (unsigned)(((u64)1 << (K - 32)) - 1);
     f.e = (int)e;

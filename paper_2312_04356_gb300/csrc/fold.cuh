@@ -31,6 +31,10 @@ struct FoldMod {
     unsigned kc, mask;   // K - 32, 2^(K-32) - 1
     int e;               // 2^K - q
     unsigned big;        // 60-bit class: values are folded every four stages
+    // first fold of a 128-bit sum, at bit K, or at 64 in the 60-bit class: position - 32, the mask of
+    // the word that bit lies in, 2^position mod q (nearest to 0)
+    unsigned kr, maskr;
+    int er;
 };
 
 // a b + c, signed 32 x 32 -> 64 (one wide multiply-add)
@@ -81,3 +85,27 @@ FOLD_HD uint64_t fold_canon(int64_t v, uint64_t q, const FoldMod& f) {
     const int64_t t = s - (int64_t)q;
     return (uint64_t)(t < 0 ? s : t);
 }
+
+#ifdef __CUDACC__
+// the canonical residue of hi 2^64 + lo, a sum of at most 40 products of two residues.  With
+// s = kr + 32: T = H 2^s + L = L + H e_r (H below 2^62, two signed digits: two wide multiplies) is
+// below 2^(K+31), its fold at K within R, and the fold of that canonical up to one q: four wide
+// multiplies, against about twenty for a Shoup reduction of each half.
+__device__ __forceinline__ unsigned long long fold_128(unsigned long long hi, unsigned long long lo,
+                                                       unsigned long long q, const FoldMod& f) {
+    const unsigned v1 = (unsigned)(lo >> 32), v2 = (unsigned)hi, v3 = (unsigned)(hi >> 32);
+    const unsigned h0 = __funnelshift_rc(v1, v2, f.kr), h1 = __funnelshift_rc(v2, v3, f.kr);
+    const int64_t a = mul_wide((int)h0, f.er), b = mul_wide((int)h1 + (int)(h0 >> 31), f.er);
+    unsigned t0, t1, t2;
+    asm("add.cc.u32  %0, %3, %4;\n\t"
+        "addc.cc.u32 %1, %5, %6;\n\t"
+        "addc.u32    %2, %7, %8;\n\t"
+        "add.cc.u32  %1, %1, %9;\n\t"
+        "addc.u32    %2, %2, 0;"
+        : "=&r"(t0), "=&r"(t1), "=&r"(t2)
+        : "r"((unsigned)lo), "r"((unsigned)a), "r"(v1 & f.maskr), "r"((unsigned)(a >> 32)),
+          "r"((unsigned)(a >> 63)), "r"((unsigned)(b >> 32)), "r"((unsigned)b));
+    const int h = (int)__funnelshift_r(t1, t2, f.kc);
+    return fold_canon(mad_wide(h, f.e, (int64_t)(((uint64_t)(t1 & f.mask) << 32) | t0)), q, f);
+}
+#endif

@@ -315,10 +315,10 @@ struct BsgsFused {
     int nb, ng, ndig;
     unsigned acc;
 };
-// D [ndig][next][N] raised digits of c1; c0, c1 [nl][N]; s, sp: P mod q_i and Shoup
+// D [ndig][next][N] raised digits of c1; c0, c1 [nl][N]; s: P mod q_i
 // (bt: a batch of bt.nb ciphertexts, D at + t dstr, c0 and c1 at + t xstr, outputs at o[g] + t ostr)
 void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1, int nl,
-                int next, const int* ext_ids, const u64* s, const u64* sp, const KsBatch& bt);
+                int next, const int* ext_ids, const u64* s, const KsBatch& bt);
 // o = sum_t w_t a_t (mod q per limb) for up to MAX terms: the integer-weighted sum of a
 // Chebyshev leaf in one pass.  Arrays of nl limbs, limb k with prime ids[k % lpp]; w[t][r]
 // is the weight's residue for limb index r < lpp, wp[t][r] its Shoup companion (passed by
@@ -371,9 +371,6 @@ void add_const_term(const ckks_ctx* c, u64* a, const u64* v, int nlimbs, const i
 void small_to_rns(const ckks_ctx* c, const int64_t* v, u64* o, int nlimbs, const int* ids);
 // o[i] = a[galois_src(i)] in the NTT domain
 void automorph(const ckks_ctx* c, const u64* a, u64* o, int nlimbs, u64 g);
-// o[limb] += s[limb % lpp] * automorph_g(a[limb]) (s = nullptr: o += automorph_g(a)), NTT domain
-void automorph_acc(const ckks_ctx* c, const u64* a, u64* o, int nlimbs, u64 g, const u64* s, const u64* sp,
-                   const int* ids, int lpp);
 // X^{N/2} times a, NTT domain: pointwise by psi^((2 rev(i)+1) N/2)
 void imult(const ckks_ctx* c, const u64* a, u64* o, int nlimbs, const int* ids, int lpp);
 // centred lift of one coefficient-domain limb with prime `src_id` into nlimbs limbs
@@ -436,7 +433,7 @@ void set_tc_withhold(bool on);
 // x0 / x1 at + t xstr; at most 4 digits)
 void ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
               const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate = false, const u64* x0 = nullptr,
-              int x0rows = 0, const u64* s = nullptr, const u64* sp = nullptr, const u64* x1 = nullptr,
+              int x0rows = 0, const u64* s = nullptr, const u64* x1 = nullptr,
               const KsBatch& bt = KsBatch());
 // d0 = a0 b0, d1 = a0 b1 + a1 b0 (d [2][nl][N]), d2 = a1 b1 (e [nl][N]) over nl limbs with
 // primes ids[0..nl); a, b [2][nl][N]; for a batch of nb ciphertexts, ciphertext t's operands at

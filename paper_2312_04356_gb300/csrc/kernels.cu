@@ -1,10 +1,10 @@
-// Device kernels of the RNS-CKKS hot path (all but the transforms, ntt.cu, and the tensor-core base
-// conversion, convert_tc.cu) and their launchers.
+// Device kernels of the RNS-CKKS hot path (all but the transforms, ntt.cu, the key-switch
+// products, keyswitch.cu, and the tensor-core base conversion, convert_tc.cu) and their launchers.
 //
 // Layout: a polynomial is [limb][N] uint64, limb k of an array of several
 // polynomials uses the prime with global id ids[k % lpp].  One CTA row of the
 // grid (blockIdx.y) is one limb, so the modulus is uniform inside a CTA.
-#include "launch.cuh"
+#include "words.cuh"
 
 #include <atomic>
 
@@ -105,8 +105,6 @@ void ckks_ctx::collect_timing() const {
 
 namespace {
 
-constexpr int EW_THREADS = 256;
-
 inline dim3 ew_grid(int n, int nlimbs) {
     int x = n / (EW_THREADS * 4);
     if (x < 1) x = 1;
@@ -115,13 +113,6 @@ inline dim3 ew_grid(int n, int nlimbs) {
 
 #define EW_LOOP(n) for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < (n); j += gridDim.x * blockDim.x)
 
-// grid of the one-thread-per-V-words kernels
-inline dim3 ewv_grid(int n, int nlimbs, int v) {
-    int x = n / (EW_THREADS * v);
-    if (x < 1) x = 1;
-    return dim3(x, nlimbs);
-}
-inline bool al16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 // words per thread of the elementwise kernels when every pointer is 16-byte aligned
 constexpr int EWV_VEC = 4;
 #define EWV_LAUNCH(K, vec, nl, ...)                                                          \
@@ -133,50 +124,6 @@ constexpr int EWV_VEC = 4;
     } while (0)
 
 // ----------------------------------------------------------- elementwise ----
-// One thread per V consecutive words of a limb (V = 2 or 4: 16-byte loads and stores, used
-// when every pointer of the launch is 16-byte aligned); all operands are loaded before any
-// store, so in-place calls (o == a) are safe.
-template <int V>
-__device__ __forceinline__ void ldv(const u64* p, u64 (&r)[V]) {
-    if constexpr (V == 1) {
-        r[0] = p[0];
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; k += 2) {
-            const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p + k);
-            r[k] = t.x;
-            r[k + 1] = t.y;
-        }
-    }
-}
-// streaming load (evict-first in L1 and L2): for data read once, so that it does not push
-// reused data out of L2
-template <int V>
-__device__ __forceinline__ void ldv_cs(const u64* p, u64 (&r)[V]) {
-    if constexpr (V == 1) {
-        r[0] = __ldcs(p);
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; k += 2) {
-            const ulonglong2 t = __ldcs(reinterpret_cast<const ulonglong2*>(p + k));
-            r[k] = t.x;
-            r[k + 1] = t.y;
-        }
-    }
-}
-template <int V>
-__device__ __forceinline__ void stv(u64* p, const u64 (&r)[V]) {
-    if constexpr (V == 1) {
-        p[0] = r[0];
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; k += 2) *reinterpret_cast<ulonglong2*>(p + k) = make_ulonglong2(r[k], r[k + 1]);
-    }
-}
-#define EWV_BEGIN(n)                                                \
-    const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);      \
-    if (j >= (n)) return;
-
 template <int V>
 __global__ void k_add(const u64* a, const u64* b, u64* o, const DevPrime* P, const int* ids, int lpp, int logn) {
     griddep_entry();
@@ -387,28 +334,6 @@ __global__ void k_automorph(const u64* a, u64* o, u64 g, int logn) {
     const size_t off = (size_t)blockIdx.y << logn;
     EW_LOOP(1 << logn) o[off + j] = a[off + galois_src(j, g, logn)];
 }
-// o[limb][j] += s[limb % lpp] * a[limb][src_g(j)] (s null: plain add), NTT domain
-template <int V>
-__global__ void k_automorph_acc(const u64* a, u64* o, u64 g, const u64* s, const u64* sp, const DevPrime* P,
-                                const int* ids, int lpp, int logn) {
-    griddep_entry();
-    const int limb = blockIdx.y;
-    const int r = limb % lpp;
-    const u64 q = P[ids[r]].m.q;
-    const size_t off = (size_t)limb << logn;
-    EWV_BEGIN(1 << logn)
-    u64 z[V];
-    ldv<V>(o + off + j, z);
-    if (s) {
-        const u64 w = s[r], wp = sp[r];
-#pragma unroll
-        for (int v = 0; v < V; ++v) z[v] = add_mod(z[v], mul_shoup(a[off + galois_src(j + v, g, logn)], w, wp, q), q);
-    } else {
-#pragma unroll
-        for (int v = 0; v < V; ++v) z[v] = add_mod(z[v], a[off + galois_src(j + v, g, logn)], q);
-    }
-    stv<V>(o + off + j, z);
-}
 __global__ void k_imult(const u64* a, u64* o, const DevPrime* P, const int* ids, int lpp, int logn) {
     griddep_entry();
     const int limb = blockIdx.y;
@@ -474,175 +399,6 @@ __global__ void k_sub_mul_scalar(const u64* a, const u64* b, const u64* s, const
 #pragma unroll
     for (int v = 0; v < V; ++v) x[v] = mul_shoup(sub_mod(x[v], y[v], q), w, wp, q);
     stv<V>(o + off + j, x);
-}
-
-// ------------------------------------------------- BSGS inner products ----
-// o[g][poly][limb] = sum_b a_b[poly][limb] * p_{g,b}[limb] for NG giant steps at once: each
-// baby value is loaded once and multiplied into every giant step's sum; the products are
-// summed exactly in 128 bits (each < 2^122, at most 32 terms) and reduced once.
-// blockIdx.y = row * nbt + t: ciphertext t of a batch (babies at T.a[b] + t astr, outputs at
-// T.o[g] + t ostr; the diagonals are shared and read by neighbouring CTAs)
-template <int V, int NG>
-__global__ void k_bsgs_inner_giants(kern::BsgsGiants T, const DevPrime* __restrict__ primes, int nl,
-                                    const int* __restrict__ ids, int logn, int nbt, size_t astr, size_t ostr) {
-    griddep_entry();
-    const int t = blockIdx.y % nbt;
-    const int limb = blockIdx.y / nbt;     // 0 .. 2 nl - 1, polynomial-major
-    const int r = limb % nl;
-    const DevPrime P = primes[ids[r]];
-    const size_t offa = t * astr + ((size_t)limb << logn), offo = t * ostr + ((size_t)limb << logn);
-    const size_t offp = (size_t)r << logn;
-    EWV_BEGIN(1 << logn)
-    u64 lo[NG][V], hi[NG][V];
-#pragma unroll
-    for (int g = 0; g < NG; ++g)
-#pragma unroll
-        for (int v = 0; v < V; ++v) lo[g][v] = hi[g][v] = 0;
-    for (int b = 0; b < T.nb; ++b) {
-        u64 x[V];
-        ldv<V>(T.a[b] + offa + j, x);
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            const u64* pg = T.p[g][b];
-            if (!pg) continue;
-            u64 y[V];
-            ldv<V>(pg + offp + j, y);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const u64 pl = x[v] * y[v], ph = __umul64hi(x[v], y[v]);
-                lo[g][v] += pl;
-                hi[g][v] += ph + (lo[g][v] < pl ? 1ull : 0ull);
-            }
-        }
-    }
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        u64 res[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) res[v] = reduce128_lazy(hi[g][v], lo[g][v], P);
-        if ((T.acc >> g) & 1u) {
-            u64 prev[V];
-            ldv<V>(T.o[g] + offo + j, prev);
-#pragma unroll
-            for (int v = 0; v < V; ++v) res[v] = add_mod(res[v], prev[v], P.m.q);
-        }
-        stv<V>(T.o[g] + offo + j, res);
-    }
-}
-
-// Baby rotations fused with the giant-step inner sums (see kern::bsgs_fused): per baby the
-// key-switch product is summed in 128 bits and reduced, the automorphed c0 term added, and the
-// reduced baby multiplied into every giant step's 128-bit sum; the babies stay in registers.
-// Same arithmetic as k_ks_inner_d followed by k_bsgs_inner_giants, so the same residues.
-// The next baby's operands (key words, gathered digit words, c0, diagonal words) are copied
-// into shared memory by per-thread asynchronous copies while the current baby is computed:
-// two stages of NS words per thread, so the memory latency of a baby overlaps the arithmetic
-// of the previous one without holding the words in registers (a version loading them into
-// registers ran 1.7x slower on a top-level CtoS level, latency bound at 36% warp occupancy).
-__device__ __forceinline__ void cp_async8(u64* dst_smem, const u64* src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-template <int NDIG, int NG>
-__global__ void __launch_bounds__(256, 3)
-    k_bsgs_fused_async(const __grid_constant__ kern::BsgsFused T, const u64* __restrict__ D,
-                       const u64* __restrict__ c0, const u64* __restrict__ c1, int nl, int next,
-                       const int* __restrict__ ext_ids, const u64* __restrict__ s0, const u64* __restrict__ s0p,
-                       const DevPrime* __restrict__ P, int logn, size_t kstride, kern::KsBatch bt) {
-    griddep_entry();
-    constexpr int NS = 3 * NDIG + 2 + NG;       // kb, ka, D per digit; c0 (gathered or row); c1 row; diagonals
-    extern __shared__ u64 sbuf[];               // [2][NS][256]
-    const int e = blockIdx.y;
-    const int id = ext_ids[e];
-    const DevPrime pr = P[id];
-    const u64 q = pr.m.q;
-    const size_t n = (size_t)1 << logn;
-    const bool qrow = e < nl;
-    const u64 w = qrow ? s0[e] : 0, wp = qrow ? s0p[e] : 0;
-    const int tid = threadIdx.x;
-    // ciphertext t of a batch (fastest varying, so that the CTAs reading the same key and diagonal
-    // words run side by side and share them through L2): D + t dstr, c0 / c1 + t xstr, outputs
-    // + t ostr
-    const int t = blockIdx.x % bt.nb;
-    const int j = (blockIdx.x / bt.nb) * 256 + tid;
-    if (j >= (int)n) return;
-    D += t * bt.dstr;
-    c0 += t * bt.xstr;
-    c1 += t * bt.xstr;
-    auto slot = [&](int st, int k) -> u64* { return sbuf + ((size_t)(st * NS + k) << 8) + tid; };
-    auto issue = [&](int b, int st) {
-        if (!T.kb[b]) {
-            if (qrow) {
-                cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + j);
-                cp_async8(slot(st, 3 * NDIG + 1), c1 + (size_t)e * n + j);
-            }
-        } else {
-            const unsigned src = galois_src(j, T.gal[b], logn);
-#pragma unroll
-            for (int d = 0; d < NDIG; ++d) {
-                const size_t kk = d * kstride + (size_t)id * n + j;
-                cp_async8(slot(st, d), T.kb[b] + kk);
-                cp_async8(slot(st, NDIG + d), T.ka[b] + kk);
-                cp_async8(slot(st, 2 * NDIG + d), D + ((size_t)d * next + e) * n + src);
-            }
-            if (qrow) cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + src);
-        }
-#pragma unroll
-        for (int g = 0; g < NG; ++g)
-            if (T.p[g][b]) cp_async8(slot(st, 3 * NDIG + 2 + g), T.p[g][b] + (size_t)e * n + j);
-        cp_async_commit();
-    };
-    u64 lob[NG], hib[NG], loa[NG], hia[NG];
-#pragma unroll
-    for (int g = 0; g < NG; ++g) lob[g] = hib[g] = loa[g] = hia[g] = 0;
-    issue(0, 0);
-    if (T.nb > 1) issue(1, 1);
-    else cp_async_commit();
-    for (int b = 0; b < T.nb; ++b) {
-        const int st = b & 1;
-        cp_async_wait<1>();                          // the group of baby b has landed
-        u64 rb, ra;
-        if (!T.kb[b]) {
-            rb = qrow ? mul_shoup(*slot(st, 3 * NDIG), w, wp, q) : 0;
-            ra = qrow ? mul_shoup(*slot(st, 3 * NDIG + 1), w, wp, q) : 0;
-        } else {
-            u64 bl = 0, bh = 0, al = 0, ah = 0;
-#pragma unroll
-            for (int d = 0; d < NDIG; ++d) {
-                const u64 x = *slot(st, 2 * NDIG + d), yb = *slot(st, d), ya = *slot(st, NDIG + d);
-                mac128(bl, bh, x, yb);
-                mac128(al, ah, x, ya);
-            }
-            rb = reduce128_lazy(bh, bl, pr);
-            ra = reduce128_lazy(ah, al, pr);
-            if (qrow) rb = add_mod(rb, mul_shoup(*slot(st, 3 * NDIG), w, wp, q), q);
-        }
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            if (!T.p[g][b]) continue;
-            const u64 y = *slot(st, 3 * NDIG + 2 + g);
-            mac128(lob[g], hib[g], rb, y);
-            mac128(loa[g], hia[g], ra, y);
-        }
-        if (b + 2 < T.nb) issue(b + 2, st);          // this stage has been read
-        else cp_async_commit();                      // keep one group per iteration
-    }
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        u64 vb = reduce128_lazy(hib[g], lob[g], pr), va = reduce128_lazy(hia[g], loa[g], pr);
-        u64* ob = T.o[g] + t * bt.ostr + (size_t)e * n + j;
-        u64* oa = T.o[g] + t * bt.ostr + ((size_t)next + e) * n + j;
-        if ((T.acc >> g) & 1u) {
-            vb = add_mod(vb, *ob, q);
-            va = add_mod(va, *oa, q);
-        }
-        *ob = vb;
-        *oa = va;
-    }
 }
 
 // ------------------------------------------------------- base conversion ----
@@ -782,143 +538,6 @@ __global__ void __launch_bounds__(256, (MC <= 6 ? 4 : 3)) k_base_convert(kern::C
         if (m < mcount) out[(size_t)s_row[m] * n + j] = reduce128_lazy(hi[m], lo[m], s_pm[m]);
 }
 
-// ---------------------------------------------------- key-switch product ----
-template <bool ACC, int V>
-__global__ void k_ks_inner(const u64* __restrict__ D, int ndig, int next, const int* __restrict__ ext_ids,
-                           const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
-                           u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride) {
-    griddep_entry();
-    const int e = blockIdx.y;
-    const int id = ext_ids[e];
-    const DevMod m = P[id].m;
-    const size_t n = (size_t)1 << logn;
-    EWV_BEGIN(1 << logn)
-    unsigned src[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) src[v] = g == 1 ? (unsigned)(j + v) : galois_src(j + v, g, logn);
-    u64 accb[V], acca[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) accb[v] = acca[v] = 0;
-    for (int d = 0; d < ndig; ++d) {
-        const u64* Dd = D + ((size_t)d * next + e) * n;
-        const size_t kk = d * kstride + (size_t)id * n + j;
-        u64 yb[V], ya[V];
-        ldv<V>(kb + kk, yb);
-        ldv<V>(ka + kk, ya);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const u64 x = Dd[src[v]];
-            accb[v] = add_mod(accb[v], mul_mod(x, yb[v], m), m.q);
-            acca[v] = add_mod(acca[v], mul_mod(x, ya[v], m), m.q);
-        }
-    }
-    if (ACC) {
-        u64 pb[V], pa[V];
-        ldv<V>(ob + (size_t)e * n + j, pb);
-        ldv<V>(oa + (size_t)e * n + j, pa);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            accb[v] = add_mod(accb[v], pb[v], m.q);
-            acca[v] = add_mod(acca[v], pa[v], m.q);
-        }
-    }
-    stv<V>(ob + (size_t)e * n + j, accb);
-    stv<V>(oa + (size_t)e * n + j, acca);
-}
-
-// The same product for a digit count fixed at compile time: every digit's key words and
-// gathered input are loaded before any arithmetic, the products are summed exactly in 128 bits
-// (each < 2^122, at most 4 terms) and reduced once per output word.
-// A batch of bt.nb key switches with the same key: ciphertext t's digits at D + t dstr, its
-// outputs at ob / oa + t ostr, its x0 / x1 at + t xstr.  The ciphertext index is the fastest
-// varying part of blockIdx.x, so the CTAs that read the same key words run side by side and
-// all but the first find them in L2: the key streams from HBM about once per batch.
-template <bool ACC, int V, int NDIG>
-__global__ void k_ks_inner_d(const u64* __restrict__ D, int next, const int* __restrict__ ext_ids,
-                             const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
-                             u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride,
-                             const u64* __restrict__ x0, const u64* __restrict__ x1, int x0rows,
-                             const u64* __restrict__ s0, const u64* __restrict__ s0p, kern::KsBatch bt) {
-    griddep_entry();
-    const int e = blockIdx.y;
-    const int id = ext_ids[e];
-    const DevPrime pr = P[id];
-    const size_t n = (size_t)1 << logn;
-    const int t = blockIdx.x % bt.nb;
-    const int j = V * ((blockIdx.x / bt.nb) * blockDim.x + threadIdx.x);
-    if (j >= (int)n) return;
-    D += t * bt.dstr;
-    ob += t * bt.ostr;
-    oa += t * bt.ostr;
-    if (x0) x0 += t * bt.xstr;
-    if (x1) x1 += t * bt.xstr;
-    unsigned src[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) src[v] = g == 1 ? (unsigned)(j + v) : galois_src(j + v, g, logn);
-    u64 x[NDIG][V], yb[NDIG][V], ya[NDIG][V];
-#pragma unroll
-    for (int d = 0; d < NDIG; ++d) {
-        const u64* Dd = D + ((size_t)d * next + e) * n;
-        const size_t kk = d * kstride + (size_t)id * n + j;
-        if (bt.nb == 1) {
-            ldv_cs<V>(kb + kk, yb[d]);   // each key word is read once per key switch: keep the
-            ldv_cs<V>(ka + kk, ya[d]);   // raised digits, which every rotation re-reads, in L2
-        } else {
-            ldv<V>(kb + kk, yb[d]);      // the other ciphertexts of the batch read them next
-            ldv<V>(ka + kk, ya[d]);
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[d][v] = Dd[src[v]];
-    }
-    u64 rb[V], ra[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        u64 bl = 0, bh = 0, al = 0, ah = 0;
-#pragma unroll
-        for (int d = 0; d < NDIG; ++d) {
-            const u64 pbl = x[d][v] * yb[d][v], pal = x[d][v] * ya[d][v];
-            bh += __umul64hi(x[d][v], yb[d][v]);
-            ah += __umul64hi(x[d][v], ya[d][v]);
-            bl += pbl;
-            bh += bl < pbl ? 1ull : 0ull;
-            al += pal;
-            ah += al < pal ? 1ull : 0ull;
-        }
-        rb[v] = reduce128_lazy(bh, bl, pr);
-        ra[v] = reduce128_lazy(ah, al, pr);
-    }
-    if (ACC) {
-        u64 pb[V], pa[V];
-        ldv<V>(ob + (size_t)e * n + j, pb);
-        ldv<V>(oa + (size_t)e * n + j, pa);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            rb[v] = add_mod(rb[v], pb[v], pr.m.q);
-            ra[v] = add_mod(ra[v], pa[v], pr.m.q);
-        }
-    }
-    if (x0 && e < x0rows) {
-        const u64* xr = x0 + (size_t)e * n;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            u64 t = xr[src[v]];
-            if (s0) t = mul_shoup(t, s0[e], s0p[e], pr.m.q);
-            rb[v] = add_mod(rb[v], t, pr.m.q);
-        }
-        if (x1) {
-            const u64* yr = x1 + (size_t)e * n;
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                u64 t = yr[src[v]];
-                if (s0) t = mul_shoup(t, s0[e], s0p[e], pr.m.q);
-                ra[v] = add_mod(ra[v], t, pr.m.q);
-            }
-        }
-    }
-    stv<V>(ob + (size_t)e * n + j, rb);
-    stv<V>(oa + (size_t)e * n + j, ra);
-}
-
 // o += a * s[limb % lpp] (Shoup pairs s, sp)
 template <int V>
 // o_ps > 0: row limb of o at (limb / lpp) o_ps + (limb % lpp) N (a contiguous)
@@ -982,112 +601,6 @@ __global__ void k_sample_small(int64_t* o, int logn, u64 key, int kind, const u6
 namespace kern {
 
 #define LAUNCH_CHECK() CUDA_CHECK(cudaGetLastError())
-
-template <int V>
-static void launch_bsgs_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int* ids, const KsBatch& bt) {
-    const dim3 grid = ewv_grid(c->n, 2 * nl * bt.nb, V);
-#define GIANTS_CASE(NG)                                                                                         \
-    klaunch(c, k_bsgs_inner_giants<V, NG>, grid, EW_THREADS, 0, t, c->d_primes, nl, ids, c->logn, bt.nb, bt.dstr, \
-            bt.ostr)
-    switch (t.ng) {
-        case 1: GIANTS_CASE(1); break;
-        case 2: GIANTS_CASE(2); break;
-        case 3: GIANTS_CASE(3); break;
-        case 4: GIANTS_CASE(4); break;
-        case 5: GIANTS_CASE(5); break;
-        case 6: GIANTS_CASE(6); break;
-        case 7: GIANTS_CASE(7); break;
-        default: GIANTS_CASE(8); break;
-    }
-#undef GIANTS_CASE
-}
-
-void bsgs_inner_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int* ids, const KsBatch& bt) {
-    CK_CHECK(t.nb >= 1 && t.nb <= BsgsGiants::MAXB && t.ng >= 1 && t.ng <= BsgsGiants::MAXG, CKKS_EINVAL,
-             "1..32 baby steps and 1..8 giant steps per inner-sum launch");
-    int terms = 0;
-    bool vec = true;
-    for (int b = 0; b < t.nb; ++b) vec = vec && al16(t.a[b]);
-    for (int g = 0; g < t.ng; ++g) {
-        vec = vec && al16(t.o[g]);
-        for (int b = 0; b < t.nb; ++b)
-            if (t.p[g][b]) {
-                ++terms;
-                vec = vec && al16(t.p[g][b]);
-            }
-    }
-    {
-        // algorithmic bytes: every baby (2 polynomials) once, every diagonal once, each giant's
-        // output written (and read when accumulating)
-        int accs = 0;
-        for (int g = 0; g < t.ng; ++g) accs += (t.acc >> g) & 1u;
-        KTimer kt_(c, "bsgs_inner", (bt.nb * (2.0 * t.nb + 2.0 * t.ng + 2.0 * accs) + terms) * nl * c->n * 8.0);
-        if (vec)
-            launch_bsgs_giants<2>(c, t, nl, ids, bt);
-        else
-            launch_bsgs_giants<1>(c, t, nl, ids, bt);
-    }
-    LAUNCH_CHECK();
-}
-
-template <int NDIG, int NG>
-static void launch_bsgs_async_one(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0,
-                                  const u64* c1, int nl, int next, const int* ext, const u64* s, const u64* sp,
-                                  const KsBatch& bt) {
-    constexpr int NS = 3 * NDIG + 2 + NG;
-    const size_t smem = 2 * (size_t)NS * 256 * sizeof(u64);
-    static std::atomic<unsigned> done{0};
-    allow_dynamic_smem((const void*)k_bsgs_fused_async<NDIG, NG>, (int)smem, done);
-    const dim3 grid((c->n + 255) / 256 * bt.nb, next);
-    klaunch(c, k_bsgs_fused_async<NDIG, NG>, grid, 256, smem, t, D, c0, c1, nl, next, ext, s, sp, c->d_primes,
-            c->logn, (size_t)c->nall << c->logn, bt);
-}
-
-template <int NDIG>
-static void launch_bsgs_async_g(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1,
-                                int nl, int next, const int* ext, const u64* s, const u64* sp, const KsBatch& bt) {
-    switch (t.ng) {
-        case 1: launch_bsgs_async_one<NDIG, 1>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-        case 2: launch_bsgs_async_one<NDIG, 2>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-        case 3: launch_bsgs_async_one<NDIG, 3>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-        default: launch_bsgs_async_one<NDIG, 4>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-    }
-}
-
-static void launch_bsgs_async(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1,
-                              int nl, int next, const int* ext, const u64* s, const u64* sp, const KsBatch& bt) {
-    switch (t.ndig) {
-        case 1: launch_bsgs_async_g<1>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-        case 2: launch_bsgs_async_g<2>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-        case 3: launch_bsgs_async_g<3>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-        default: launch_bsgs_async_g<4>(c, t, D, c0, c1, nl, next, ext, s, sp, bt); break;
-    }
-}
-
-void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1, int nl,
-                int next, const int* ext_ids, const u64* s, const u64* sp, const KsBatch& bt) {
-    CK_CHECK(t.nb >= 1 && t.nb <= BsgsFused::MAXB && t.ng >= 1 && t.ng <= BsgsFused::MAXG && t.ndig >= 1 &&
-                 t.ndig <= 4, CKKS_EINVAL, "fused BSGS: 1..32 babies, 1..4 giant steps, 1..4 digits");
-    int terms = 0, rots = 0;
-    for (int b = 0; b < t.nb; ++b) {
-        if (t.kb[b]) ++rots;
-        for (int g = 0; g < t.ng; ++g)
-            if (t.p[g][b]) ++terms;
-    }
-    int accs = 0;
-    for (int g = 0; g < t.ng; ++g) accs += (t.acc >> g) & 1u;
-    {
-        // algorithmic bytes: per rotation the digits, both key halves and c0 on the Q rows; the
-        // identity's c0 and c1; every diagonal once; each giant's output (read when accumulating)
-        // (a batch reads the keys and diagonals once, and its ciphertexts' own words each)
-        const double shared = (double)rots * 2.0 * t.ndig + terms;
-        const double own = (double)rots * (t.ndig * next + nl) / next + (t.nb - rots) * 2.0 * nl / next +
-                           2.0 * t.ng + 2.0 * accs;
-        KTimer kt_(c, "bsgs_fused", (shared + bt.nb * own) * next * c->n * 8.0);
-        launch_bsgs_async(c, t, D, c0, c1, nl, next, ext_ids, s, sp, bt);
-    }
-    LAUNCH_CHECK();
-}
 
 void add(const ckks_ctx* c, const u64* a, const u64* b, u64* o, int nl, const int* ids, int lpp) {
     if (nl <= 0) return;
@@ -1209,14 +722,6 @@ void automorph(const ckks_ctx* c, const u64* a, u64* o, int nl, u64 g) {
     }
     LAUNCH_CHECK();
 }
-void automorph_acc(const ckks_ctx* c, const u64* a, u64* o, int nl, u64 g, const u64* s, const u64* sp,
-                   const int* ids, int lpp) {
-    if (nl <= 0) return;
-    { KTimer kt_(c, "automorph_acc", 3.0 * (double)nl * c->n * 8.0);
-    EWV_LAUNCH(k_automorph_acc, al16(o), nl, a, o, g, s, sp, c->d_primes, ids, lpp, c->logn);
-    }
-    LAUNCH_CHECK();
-}
 void imult(const ckks_ctx* c, const u64* a, u64* o, int nl, const int* ids, int lpp) {
     if (nl <= 0) return;
     { KTimer kt_(c, "imult", 2.0 * (double)nl * c->n * 8.0);
@@ -1332,69 +837,6 @@ void base_convert_jobs(const ckks_ctx* c, const ConvJobs& J0, int npoly) {
     LAUNCH_CHECK();
 }
 
-template <bool ACC, int V>
-static void launch_ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
-                            const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
-                            const u64* s0, const u64* s0p, const KsBatch& bt) {
-    dim3 grid = ewv_grid(c->n, next, V);
-    grid.x *= bt.nb;
-    const size_t ks = (size_t)c->nall << c->logn;
-    switch (ndig) {
-        case 1:
-            klaunch(c, k_ks_inner_d<ACC, V, 1>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, s0p, bt);
-            break;
-        case 2:
-            klaunch(c, k_ks_inner_d<ACC, V, 2>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, s0p, bt);
-            break;
-        case 3:
-            klaunch(c, k_ks_inner_d<ACC, V, 3>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, s0p, bt);
-            break;
-        case 4:
-            klaunch(c, k_ks_inner_d<ACC, V, 4>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, s0p, bt);
-            break;
-        default:
-            klaunch(c, k_ks_inner<ACC, V>, grid, EW_THREADS, 0, D, ndig, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks);
-            break;
-    }
-}
-
-void ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
-              const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate, const u64* x0, int x0rows, const u64* s,
-              const u64* sp, const u64* x1, const KsBatch& bt) {
-    CK_CHECK(bt.nb >= 1 && (bt.nb == 1 || ndig <= 4), CKKS_EINVAL, "batched key switching needs at most 4 digits");
-    const bool vec = al16(kb) && al16(ka) && al16(ob) && al16(oa);
-    const bool fuse = x0 && x0rows > 0 && ndig <= 4;   // the generic kernel adds x0, x1 in further passes
-    {
-        // algorithmic bytes: the key once for the whole batch, per ciphertext its digits, outputs
-        // (read too when accumulating) and the x0 / x1 rows
-        const double extra = fuse ? (double)x0rows * (x1 ? 2.0 : 1.0) / next : 0.0;
-        KTimer kt_(c, "ks_inner",
-                   (2.0 * ndig + bt.nb * (ndig + (accumulate ? 4.0 : 2.0) + extra)) * next * c->n * 8.0);
-        const u64* fx = fuse ? x0 : nullptr;
-        const u64* fy = fuse ? x1 : nullptr;
-        if (accumulate) {
-            if (vec)
-                launch_ks_inner<true, 2>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, fx, fy, x0rows, s, sp, bt);
-            else
-                launch_ks_inner<true, 1>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, fx, fy, x0rows, s, sp, bt);
-        } else {
-            if (vec)
-                launch_ks_inner<false, 2>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, fx, fy, x0rows, s, sp, bt);
-            else
-                launch_ks_inner<false, 1>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, fx, fy, x0rows, s, sp, bt);
-        }
-    }
-    LAUNCH_CHECK();
-    if (x0 && x0rows > 0 && !fuse) {
-        automorph_acc(c, x0, ob, x0rows, g, s, sp, ext_ids, x0rows);
-        if (x1) automorph_acc(c, x1, oa, x0rows, g, s, sp, ext_ids, x0rows);
-    }
-}
 void mul_scalar_acc(const ckks_ctx* c, const u64* a, const u64* s, const u64* sp, u64* o, int nl, const int* ids,
                     int lpp, size_t o_pstride) {
     if (nl <= 0) return;

@@ -1,0 +1,437 @@
+// The products of key switching: a rotation's or relinearisation's inner product with its key, the
+// inner sums of a BSGS map, and both in one pass (the hoisted rotations of a BSGS map are never
+// stored).  Each output word is one 128-bit sum of products, reduced once (words.cuh).
+//
+// A product added to a 128-bit sum costs about 20 cycles of the integer-multiply pipe per warp and SM
+// quarter; the reduction cost 72 with two Shoup products (90 in all) and costs 16 folded, which
+// was half the work of a baby with three digits.  The c0 term rides in the same sum.  At N = 2^16,
+// level 23: the seven maps of a bootstrapped block 2.19 -> 1.85 ms (6.5 TB/s by algorithmic
+// bytes, the keys and diagonals read once: HBM), eight ciphertexts in lockstep 15.0 -> 12.5 ms
+// (bound by the products), the key switches of a block 1.14 -> 1.07 ms.
+#include "words.cuh"
+
+#include <atomic>
+
+namespace {
+
+// ------------------------------------------------- BSGS inner products ----
+// o[g][poly][limb] = sum_b a_b[poly][limb] * p_{g,b}[limb] for NG giant steps at once: each
+// baby value is loaded once and multiplied into every giant step's sum; the products are
+// summed exactly in 128 bits (each < 2^122, at most 32 terms) and reduced once.
+// blockIdx.y = row * nbt + t: ciphertext t of a batch (babies at T.a[b] + t astr, outputs at
+// T.o[g] + t ostr; the diagonals are shared and read by neighbouring CTAs)
+template <bool FOLD, int V, int NG>
+__global__ void k_bsgs_inner_giants(kern::BsgsGiants T, const DevPrime* __restrict__ primes, int nl,
+                                    const int* __restrict__ ids, int logn, int nbt, size_t astr, size_t ostr) {
+    griddep_entry();
+    const int t = blockIdx.y % nbt;
+    const int limb = blockIdx.y / nbt;     // 0 .. 2 nl - 1, polynomial-major
+    const int r = limb % nl;
+    const Reducer<FOLD> red(primes[ids[r]]);
+    const size_t offa = t * astr + ((size_t)limb << logn), offo = t * ostr + ((size_t)limb << logn);
+    const size_t offp = (size_t)r << logn;
+    EWV_BEGIN(1 << logn)
+    u64 lo[NG][V], hi[NG][V];
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int v = 0; v < V; ++v) lo[g][v] = hi[g][v] = 0;
+    for (int b = 0; b < T.nb; ++b) {
+        u64 x[V];
+        ldv<V>(T.a[b] + offa + j, x);
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            const u64* pg = T.p[g][b];
+            if (!pg) continue;
+            u64 y[V];
+            ldv<V>(pg + offp + j, y);
+#pragma unroll
+            for (int v = 0; v < V; ++v) mac128(lo[g][v], hi[g][v], x[v], y[v]);
+        }
+    }
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        u64 res[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) res[v] = red(hi[g][v], lo[g][v]);
+        if ((T.acc >> g) & 1u) {
+            u64 prev[V];
+            ldv<V>(T.o[g] + offo + j, prev);
+#pragma unroll
+            for (int v = 0; v < V; ++v) res[v] = add_mod(res[v], prev[v], red.q);
+        }
+        stv<V>(T.o[g] + offo + j, res);
+    }
+}
+
+// Baby rotations fused with the giant-step inner sums (see kern::bsgs_fused): per baby the
+// key-switch product and the automorphed c0 term are summed in 128 bits and reduced, and the
+// reduced baby multiplied into every giant step's 128-bit sum; the babies stay in registers.
+// Same residues as k_ks_inner_d followed by k_bsgs_inner_giants.
+// The next baby's operands (key words, gathered digit words, c0, diagonal words) are copied
+// into shared memory by per-thread asynchronous copies while the current baby is computed:
+// two stages of NS words per thread, so the memory latency of a baby overlaps the arithmetic
+// of the previous one without holding the words in registers (a version loading them into
+// registers ran 1.7x slower on a top-level CtoS level, latency bound at 36% warp occupancy).
+__device__ __forceinline__ void cp_async8(u64* dst_smem, const u64* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <bool FOLD, int NDIG, int NG>
+__global__ void __launch_bounds__(256, 3)
+    k_bsgs_fused_async(const __grid_constant__ kern::BsgsFused T, const u64* __restrict__ D,
+                       const u64* __restrict__ c0, const u64* __restrict__ c1, int nl, int next,
+                       const int* __restrict__ ext_ids, const u64* __restrict__ s0,
+                       const DevPrime* __restrict__ P, int logn, size_t kstride, kern::KsBatch bt) {
+    griddep_entry();
+    constexpr int NS = 3 * NDIG + 2 + NG;       // kb, ka, D per digit; c0 (gathered or row); c1 row; diagonals
+    extern __shared__ u64 sbuf[];               // [2][NS][256]
+    const int e = blockIdx.y;
+    const int id = ext_ids[e];
+    const Reducer<FOLD> red(P[id]);
+    const u64 q = red.q;
+    const size_t n = (size_t)1 << logn;
+    const bool qrow = e < nl;
+    const u64 w = qrow ? s0[e] : 0;
+    const int tid = threadIdx.x;
+    // ciphertext t of a batch (fastest varying, so that the CTAs reading the same key and diagonal
+    // words run side by side and share them through L2): D + t dstr, c0 / c1 + t xstr, outputs
+    // + t ostr
+    const int t = blockIdx.x % bt.nb;
+    const int j = (blockIdx.x / bt.nb) * 256 + tid;
+    if (j >= (int)n) return;
+    D += t * bt.dstr;
+    c0 += t * bt.xstr;
+    c1 += t * bt.xstr;
+    auto slot = [&](int st, int k) -> u64* { return sbuf + ((size_t)(st * NS + k) << 8) + tid; };
+    auto issue = [&](int b, int st) {
+        if (!T.kb[b]) {
+            if (qrow) {
+                cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + j);
+                cp_async8(slot(st, 3 * NDIG + 1), c1 + (size_t)e * n + j);
+            }
+        } else {
+            const unsigned src = galois_src(j, T.gal[b], logn);
+#pragma unroll
+            for (int d = 0; d < NDIG; ++d) {
+                const size_t kk = d * kstride + (size_t)id * n + j;
+                cp_async8(slot(st, d), T.kb[b] + kk);
+                cp_async8(slot(st, NDIG + d), T.ka[b] + kk);
+                cp_async8(slot(st, 2 * NDIG + d), D + ((size_t)d * next + e) * n + src);
+            }
+            if (qrow) cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + src);
+        }
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+            if (T.p[g][b]) cp_async8(slot(st, 3 * NDIG + 2 + g), T.p[g][b] + (size_t)e * n + j);
+        cp_async_commit();
+    };
+    u64 lob[NG], hib[NG], loa[NG], hia[NG];
+#pragma unroll
+    for (int g = 0; g < NG; ++g) lob[g] = hib[g] = loa[g] = hia[g] = 0;
+    issue(0, 0);
+    if (T.nb > 1) issue(1, 1);
+    else cp_async_commit();
+    for (int b = 0; b < T.nb; ++b) {
+        const int st = b & 1;
+        cp_async_wait<1>();                          // the group of baby b has landed
+        // the baby: sum of the digits' products with the key and w c0 (w = P mod q), reduced once
+        u64 bl = 0, bh = 0, al = 0, ah = 0;
+        if (!T.kb[b]) {
+            if (qrow) {
+                mac128(bl, bh, *slot(st, 3 * NDIG), w);
+                mac128(al, ah, *slot(st, 3 * NDIG + 1), w);
+            }
+        } else {
+#pragma unroll
+            for (int d = 0; d < NDIG; ++d) {
+                const u64 x = *slot(st, 2 * NDIG + d), yb = *slot(st, d), ya = *slot(st, NDIG + d);
+                mac128(bl, bh, x, yb);
+                mac128(al, ah, x, ya);
+            }
+            if (qrow) mac128(bl, bh, *slot(st, 3 * NDIG), w);
+        }
+        const u64 rb = red(bh, bl), ra = red(ah, al);
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            if (!T.p[g][b]) continue;
+            const u64 y = *slot(st, 3 * NDIG + 2 + g);
+            mac128(lob[g], hib[g], rb, y);
+            mac128(loa[g], hia[g], ra, y);
+        }
+        if (b + 2 < T.nb) issue(b + 2, st);          // this stage has been read
+        else cp_async_commit();                      // keep one group per iteration
+    }
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        u64 vb = red(hib[g], lob[g]), va = red(hia[g], loa[g]);
+        u64* ob = T.o[g] + t * bt.ostr + (size_t)e * n + j;
+        u64* oa = T.o[g] + t * bt.ostr + ((size_t)next + e) * n + j;
+        if ((T.acc >> g) & 1u) {
+            vb = add_mod(vb, *ob, q);
+            va = add_mod(va, *oa, q);
+        }
+        *ob = vb;
+        *oa = va;
+    }
+}
+
+// ---------------------------------------------------- key-switch product ----
+// Key-switch inner product over NDIG digits: every digit's key words and gathered input are
+// loaded before any arithmetic, the products are summed exactly in 128 bits (each < 2^122) and
+// reduced once per output word.
+// A batch of bt.nb key switches with the same key: ciphertext t's digits at D + t dstr, its
+// outputs at ob / oa + t ostr, its x0 / x1 at + t xstr.  The ciphertext index is the fastest
+// varying part of blockIdx.x, so the CTAs that read the same key words run side by side and
+// all but the first find them in L2: the key streams from HBM about once per batch.
+template <bool FOLD, bool ACC, int V, int NDIG>
+__global__ void k_ks_inner_d(const u64* __restrict__ D, int next, const int* __restrict__ ext_ids,
+                             const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
+                             u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride,
+                             const u64* __restrict__ x0, const u64* __restrict__ x1, int x0rows,
+                             const u64* __restrict__ s0, kern::KsBatch bt) {
+    griddep_entry();
+    const int e = blockIdx.y;
+    const int id = ext_ids[e];
+    const Reducer<FOLD> red(P[id]);
+    const size_t n = (size_t)1 << logn;
+    const int t = blockIdx.x % bt.nb;
+    const int j = V * ((blockIdx.x / bt.nb) * blockDim.x + threadIdx.x);
+    if (j >= (int)n) return;
+    D += t * bt.dstr;
+    ob += t * bt.ostr;
+    oa += t * bt.ostr;
+    if (x0) x0 += t * bt.xstr;
+    if (x1) x1 += t * bt.xstr;
+    unsigned src[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) src[v] = g == 1 ? (unsigned)(j + v) : galois_src(j + v, g, logn);
+    u64 x[NDIG][V], yb[NDIG][V], ya[NDIG][V];
+#pragma unroll
+    for (int d = 0; d < NDIG; ++d) {
+        const u64* Dd = D + ((size_t)d * next + e) * n;
+        const size_t kk = d * kstride + (size_t)id * n + j;
+        if (bt.nb == 1) {
+            ldv_cs<V>(kb + kk, yb[d]);   // each key word is read once per key switch: keep the
+            ldv_cs<V>(ka + kk, ya[d]);   // raised digits, which every rotation re-reads, in L2
+        } else {
+            ldv<V>(kb + kk, yb[d]);      // the other ciphertexts of the batch read them next
+            ldv<V>(ka + kk, ya[d]);
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) x[d][v] = Dd[src[v]];
+    }
+    // the sums: digits times key, the previous output (accumulating) and w x0, w x1 (w = s0's row, or 1)
+    u64 bl[V], bh[V], al[V], ah[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) bl[v] = bh[v] = al[v] = ah[v] = 0;
+    if (ACC) {
+        ldv<V>(ob + (size_t)e * n + j, bl);
+        ldv<V>(oa + (size_t)e * n + j, al);
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+#pragma unroll
+        for (int d = 0; d < NDIG; ++d) {
+            mac128(bl[v], bh[v], x[d][v], yb[d][v]);
+            mac128(al[v], ah[v], x[d][v], ya[d][v]);
+        }
+    }
+    if (x0 && e < x0rows) {
+        const u64 w = s0 ? s0[e] : 1;
+        const u64* xr = x0 + (size_t)e * n;
+#pragma unroll
+        for (int v = 0; v < V; ++v) mac128(bl[v], bh[v], xr[src[v]], w);
+        if (x1) {
+            const u64* yr = x1 + (size_t)e * n;
+#pragma unroll
+            for (int v = 0; v < V; ++v) mac128(al[v], ah[v], yr[src[v]], w);
+        }
+    }
+    u64 rb[V], ra[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        rb[v] = red(bh[v], bl[v]);
+        ra[v] = red(ah[v], al[v]);
+    }
+    stv<V>(ob + (size_t)e * n + j, rb);
+    stv<V>(oa + (size_t)e * n + j, ra);
+}
+
+}  // namespace
+
+namespace kern {
+
+#define LAUNCH_CHECK() CUDA_CHECK(cudaGetLastError())
+
+template <bool FOLD, int V>
+static void launch_bsgs_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int* ids, const KsBatch& bt) {
+    const dim3 grid = ewv_grid(c->n, 2 * nl * bt.nb, V);
+#define GIANTS_CASE(NG)                                                                                         \
+    klaunch(c, k_bsgs_inner_giants<FOLD, V, NG>, grid, EW_THREADS, 0, t, c->d_primes, nl, ids, c->logn, bt.nb, bt.dstr, \
+            bt.ostr)
+    switch (t.ng) {
+        case 1: GIANTS_CASE(1); break;
+        case 2: GIANTS_CASE(2); break;
+        case 3: GIANTS_CASE(3); break;
+        case 4: GIANTS_CASE(4); break;
+        case 5: GIANTS_CASE(5); break;
+        case 6: GIANTS_CASE(6); break;
+        case 7: GIANTS_CASE(7); break;
+        default: GIANTS_CASE(8); break;
+    }
+#undef GIANTS_CASE
+}
+
+void bsgs_inner_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int* ids, const KsBatch& bt) {
+    CK_CHECK(t.nb >= 1 && t.nb <= BsgsGiants::MAXB && t.ng >= 1 && t.ng <= BsgsGiants::MAXG, CKKS_EINVAL,
+             "1..32 baby steps and 1..8 giant steps per inner-sum launch");
+    int terms = 0;
+    bool vec = true;
+    for (int b = 0; b < t.nb; ++b) vec = vec && al16(t.a[b]);
+    for (int g = 0; g < t.ng; ++g) {
+        vec = vec && al16(t.o[g]);
+        for (int b = 0; b < t.nb; ++b)
+            if (t.p[g][b]) {
+                ++terms;
+                vec = vec && al16(t.p[g][b]);
+            }
+    }
+    {
+        // algorithmic bytes: every baby (2 polynomials) once, every diagonal once, each giant's
+        // output written (and read when accumulating)
+        int accs = 0;
+        for (int g = 0; g < t.ng; ++g) accs += (t.acc >> g) & 1u;
+        KTimer kt_(c, "bsgs_inner", (bt.nb * (2.0 * t.nb + 2.0 * t.ng + 2.0 * accs) + terms) * nl * c->n * 8.0);
+        if (c->fold && vec)
+            launch_bsgs_giants<true, 2>(c, t, nl, ids, bt);
+        else if (c->fold)
+            launch_bsgs_giants<true, 1>(c, t, nl, ids, bt);
+        else
+            launch_bsgs_giants<false, 1>(c, t, nl, ids, bt);
+    }
+    LAUNCH_CHECK();
+}
+
+template <bool FOLD, int NDIG, int NG>
+static void launch_bsgs_async_one(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0,
+                                  const u64* c1, int nl, int next, const int* ext, const u64* s,
+                                  const KsBatch& bt) {
+    constexpr int NS = 3 * NDIG + 2 + NG;
+    const size_t smem = 2 * (size_t)NS * 256 * sizeof(u64);
+    static std::atomic<unsigned> done{0};
+    allow_dynamic_smem((const void*)k_bsgs_fused_async<FOLD, NDIG, NG>, (int)smem, done);
+    const dim3 grid((c->n + 255) / 256 * bt.nb, next);
+    klaunch(c, k_bsgs_fused_async<FOLD, NDIG, NG>, grid, 256, smem, t, D, c0, c1, nl, next, ext, s, c->d_primes,
+            c->logn, (size_t)c->nall << c->logn, bt);
+}
+
+template <bool FOLD, int NDIG>
+static void launch_bsgs_async_g(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1,
+                                int nl, int next, const int* ext, const u64* s, const KsBatch& bt) {
+    switch (t.ng) {
+        case 1: launch_bsgs_async_one<FOLD, NDIG, 1>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+        case 2: launch_bsgs_async_one<FOLD, NDIG, 2>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+        case 3: launch_bsgs_async_one<FOLD, NDIG, 3>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+        default: launch_bsgs_async_one<FOLD, NDIG, 4>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+    }
+}
+
+template <bool FOLD>
+static void launch_bsgs_async(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1,
+                              int nl, int next, const int* ext, const u64* s, const KsBatch& bt) {
+    switch (t.ndig) {
+        case 1: launch_bsgs_async_g<FOLD, 1>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+        case 2: launch_bsgs_async_g<FOLD, 2>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+        case 3: launch_bsgs_async_g<FOLD, 3>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+        default: launch_bsgs_async_g<FOLD, 4>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
+    }
+}
+
+void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1, int nl,
+                int next, const int* ext_ids, const u64* s, const KsBatch& bt) {
+    CK_CHECK(t.nb >= 1 && t.nb <= BsgsFused::MAXB && t.ng >= 1 && t.ng <= BsgsFused::MAXG && t.ndig >= 1 &&
+                 t.ndig <= 4, CKKS_EINVAL, "fused BSGS: 1..32 babies, 1..4 giant steps, 1..4 digits");
+    int terms = 0, rots = 0;
+    for (int b = 0; b < t.nb; ++b) {
+        if (t.kb[b]) ++rots;
+        for (int g = 0; g < t.ng; ++g)
+            if (t.p[g][b]) ++terms;
+    }
+    int accs = 0;
+    for (int g = 0; g < t.ng; ++g) accs += (t.acc >> g) & 1u;
+    {
+        // algorithmic bytes: per rotation the digits, both key halves and c0 on the Q rows; the
+        // identity's c0 and c1; every diagonal once; each giant's output (read when accumulating)
+        // (a batch reads the keys and diagonals once, and its ciphertexts' own words each)
+        const double shared = (double)rots * 2.0 * t.ndig + terms;
+        const double own = (double)rots * (t.ndig * next + nl) / next + (t.nb - rots) * 2.0 * nl / next +
+                           2.0 * t.ng + 2.0 * accs;
+        KTimer kt_(c, "bsgs_fused", (shared + bt.nb * own) * next * c->n * 8.0);
+        if (c->fold)
+            launch_bsgs_async<true>(c, t, D, c0, c1, nl, next, ext_ids, s, bt);
+        else
+            launch_bsgs_async<false>(c, t, D, c0, c1, nl, next, ext_ids, s, bt);
+    }
+    LAUNCH_CHECK();
+}
+
+template <bool FOLD, bool ACC, int V>
+static void launch_ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
+                            const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
+                            const u64* s0, const KsBatch& bt) {
+    dim3 grid = ewv_grid(c->n, next, V);
+    grid.x *= bt.nb;
+    const size_t ks = (size_t)c->nall << c->logn;
+    switch (ndig) {
+        case 1:
+            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 1>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
+                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
+            break;
+        case 2:
+            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 2>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
+                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
+            break;
+        case 3:
+            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 3>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
+                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
+            break;
+        default:
+            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 4>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
+                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
+            break;
+    }
+}
+
+void ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
+              const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate, const u64* x0, int x0rows, const u64* s,
+              const u64* x1, const KsBatch& bt) {
+    CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4, CKKS_EINVAL, "key switching takes 1..4 digits");
+    const bool vec = al16(kb) && al16(ka) && al16(ob) && al16(oa);
+    {
+        // algorithmic bytes: the key once for the whole batch, per ciphertext its digits, outputs
+        // (read too when accumulating) and the x0 / x1 rows
+        const double extra = x0 ? (double)x0rows * (x1 ? 2.0 : 1.0) / next : 0.0;
+        KTimer kt_(c, "ks_inner",
+                   (2.0 * ndig + bt.nb * (ndig + (accumulate ? 4.0 : 2.0) + extra)) * next * c->n * 8.0);
+#define KS(FOLD, ACC, V) launch_ks_inner<FOLD, ACC, V>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s, bt)
+        if (c->fold && vec) {
+            if (accumulate) KS(true, true, 2);
+            else KS(true, false, 2);
+        } else if (c->fold) {
+            if (accumulate) KS(true, true, 1);
+            else KS(true, false, 1);
+        } else {
+            if (accumulate) KS(false, true, 1);
+            else KS(false, false, 1);
+        }
+#undef KS
+    }
+    LAUNCH_CHECK();
+}
+
+}  // namespace kern

@@ -93,8 +93,8 @@ __device__ __forceinline__ unsigned brev_bits(unsigned x, int bits) { return __b
 // index of the NTT slot holding a(X^g) at slot i (bit-reversed evaluation order):
 // slot i is the evaluation at psi^(2 rev(i) + 1); a(X^g) there is a at psi^((2 rev(i)+1) g)
 __device__ __forceinline__ unsigned galois_src(unsigned i, u64 g, int logn) {
-    unsigned r = brev_bits(i, logn);
-    u64 e = ((2ull * r + 1ull) * g) & ((2ull << logn) - 1ull);
-    return brev_bits((unsigned)((e - 1) >> 1), logn);
+    const unsigned r = brev_bits(i, logn);
+    const unsigned e = ((2u * r + 1u) * (unsigned)g) & ((2u << logn) - 1u);   // mod 2N, a power of two: 32 bits do
+    return brev_bits((e - 1) >> 1, logn);
 }
 #endif  // __CUDACC__

@@ -600,7 +600,7 @@ DevBuf mod_up(ckks_ctx* c, const u64* x, int level, int* ndig_out, int nb, size_
 // at + t xstr; the key is read once for the batch.
 void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const u64* D, int ndig, int level, u64 code, u64 g,
                       u64* acc, bool accumulate, const u64* x0 = nullptr, int x0rows = 0, const u64* s = nullptr,
-                      const u64* sp = nullptr, const u64* x1 = nullptr, int nb = 1, size_t xstr = 0) {
+                      const u64* x1 = nullptr, int nb = 1, size_t xstr = 0) {
     auto it = keys.swk.find(code);
     CK_CHECK(it != keys.swk.end(), CKKS_ENOKEY, "missing switching key (code " + std::to_string(code) + ")");
     const SwitchKey& k = *it->second;
@@ -612,7 +612,7 @@ void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const u64* D, int ndig
     bt.ostr = 2 * next * c->n;
     bt.xstr = xstr;
     kern::ks_inner(c, D, ndig, (int)next, c->d_ext_ids[level], k.b.ptr, k.a.ptr, acc, acc + next * c->n, g,
-                   accumulate, x0, x0rows, s, sp, x1, bt);
+                   accumulate, x0, x0rows, s, x1, bt);
 }
 
 // ModDown fused with the rescale after it: both halves of acc (Q_l u P, NTT domain) divided
@@ -674,7 +674,7 @@ static ckks_ct switch_galois(const ckks_keys& keys, const ckks_ct& a, const u64*
     ckks_ctx* c = a.ctx;
     const int l = a.level, nl = l + 1;
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n, c->stream);
-    key_switch_inner(c, keys, D, ndig, l, g, g, acc.ptr, false, a.c0(), nl, c->d_pmod, c->d_pmod + c->nq, nullptr,
+    key_switch_inner(c, keys, D, ndig, l, g, g, acc.ptr, false, a.c0(), nl, c->d_pmod, nullptr,
                      a.nb, a.cstride());
     ckks_ct o = new_ct(c, l, a.scale, a.nb);
     mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
@@ -734,7 +734,7 @@ ckks_ct mul_relin(const ckks_keys& keys, const ckks_ct& a, const ckks_ct& b) {
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel; then
     // ModDown (= (d0, d1) + ModDown(k), see switch_galois)
-    key_switch_inner(c, keys, D.ptr, ndig, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod, c->d_pmod + c->nq,
+    key_switch_inner(c, keys, D.ptr, ndig, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l, a.scale * b.scale, a.nb);
     mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
@@ -755,7 +755,7 @@ ckks_ct mul_relin_rescale(const ckks_keys& keys, const ckks_ct& a, const ckks_ct
     DevBuf D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, &ndig, a.nb, ds);
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel
-    key_switch_inner(c, keys, D.ptr, ndig, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod, c->d_pmod + c->nq,
+    key_switch_inner(c, keys, D.ptr, ndig, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l - 1, a.scale * b.scale / (double)c->q[l], a.nb);
     mod_down_rescale(c, acc.ptr, l, o.buf.ptr, twice, a.nb);
@@ -797,8 +797,8 @@ static std::vector<DevBuf> rotate_hoisted_ext(const ckks_keys& keys, const ckks_
         } else {
             if (!D.ptr) D = mod_up(c, a.c1(), l, &ndig, a.nb, a.cstride());
             c->ops["hrot"]++;
-            key_switch_inner(c, keys, D.ptr, ndig, l, g, g, o.ptr, false, a.c0(), nl, c->d_pmod, c->d_pmod + c->nq,
-                             nullptr, a.nb, a.cstride());
+            key_switch_inner(c, keys, D.ptr, ndig, l, g, g, o.ptr, false, a.c0(), nl, c->d_pmod, nullptr, a.nb,
+                             a.cstride());
         }
         outs.push_back(std::move(o));
     }
@@ -911,7 +911,7 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             bt.dstr = (size_t)ndig * next * n;
             bt.xstr = a.cstride();
             bt.ostr = es;
-            kern::bsgs_fused(c, T, D.ptr, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, c->d_pmod + c->nq, bt);
+            kern::bsgs_fused(c, T, D.ptr, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
             continue;
         }
         std::vector<DevBuf> baby = rotate_hoisted_ext(keys, a, steps);
@@ -979,7 +979,7 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             int ndig = 0;
             DevBuf D = mod_up(c, c1q.ptr, l, &ndig, nb, (size_t)nl * n);
             key_switch_inner(c, keys, D.ptr, ndig, l, gal, gal, sums[k].ptr, false, x, (int)next, nullptr, nullptr,
-                             nullptr, nb, es);
+                             nb, es);
         }
         for (int k = 0; k < nside; ++k) {
             CUDA_CHECK(cudaEventRecord(c->side_ev[k], c->side[k]));
@@ -1023,7 +1023,7 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         DevBuf D = mod_up(c, c1q.ptr, l, &ndig, nb, (size_t)nl * n);
         if (!have_acc) acc = DevBuf(nb * es, c->stream);
         key_switch_inner(c, keys, D.ptr, ndig, l, gal, gal, acc.ptr, have_acc, x, (int)next, nullptr, nullptr,
-                         nullptr, nb, es);
+                         nb, es);
         have_acc = true;
     }
     if (rescale_out) {
