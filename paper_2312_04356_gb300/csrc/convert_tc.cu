@@ -16,10 +16,12 @@
 // the final word's low 23 bits are D itself, from which the value of sum_b 2^(8b) D_{m,b} is
 // assembled and reduced mod p_m (with, for an exact table, the
 // rounded correction v (Q mod p_m) of the integer-pipe kernel, Halevi-Polyakov-Shoup 2019).
-// Every output goes to a forward NTT.  For N = 2^16 the words are left congruent but below 4p
-// (the radix-16 transform's lazy butterflies take such inputs and end canonical); otherwise they
-// are the canonical residues.  Either way the transformed words equal the integer-pipe
-// kernel's.
+// The kernel is bound by this epilogue on the integer pipes.  Contexts whose primes lie next to a
+// power of two (fold.cuh) add the correction to the assembled sum and fold it once (one wide
+// multiply); a Shoup product by 2^24, and another for the correction, remain for other primes.
+// Every output goes to a forward NTT, which takes the folded words as they are (signed, within
+// 2^K + 2^43); a Shoup context's words are canonical.  Either way the transformed words equal the
+// integer-pipe kernel's.
 //
 // A CTA takes 128 coefficients per tile (MMA M = 128, one TMEM lane per coefficient) for one
 // output group of S <= 16 outputs (N = 8 S <= 128 TMEM columns, four CTAs per SM fill the
@@ -186,6 +188,26 @@ __device__ __forceinline__ u64 chunk_reduce_lazy(const unsigned* w, u64 p, u64 r
     return lo + ((hi << 24) - __umul64hi(hi, r24p) * p);   // lo + [0, 2p) < 3p
 }
 
+// the same sum plus v corr (v < 2^5, corr < p), folded at bit K: D_{2k} + 2^8 D_{2k+1} < 2^32 in one shift
+// and two additions (the word's high byte 0x4B leaves by the shift or is subtracted), two such
+// words 16 bits apart, and the two halves as c 2^32 + (32 bits of a).  A 42- or 48-bit prime's table
+// entries have no chunks above bit 49, so the sum stays below 2^64 (2^80 at 60 bits) and its part
+// above bit K below 2^20.
+template <bool EXACT>
+__device__ __forceinline__ int64_t chunk_fold(const unsigned* w, const ConvOut& f, unsigned v) {
+    constexpr unsigned OFF = 0x4B000000u;
+    const unsigned e0 = (w[1] << 8) + (w[0] - OFF), e1 = (w[3] << 8) + (w[2] - OFF);
+    const unsigned e2 = (w[5] << 8) + (w[4] - OFF), e3 = (w[7] << 8) + (w[6] - OFF);
+    u64 a = ((u64)e1 << 16) + e0, c = ((u64)e3 << 16) + e2;
+    if (EXACT) {
+        a += (u64)v * (unsigned)f.corr;
+        c += (u64)v * (unsigned)(f.corr >> 32);
+    }
+    c += a >> 32;
+    const int h = (int)__funnelshift_r((unsigned)c, (unsigned)(c >> 32), f.kc);
+    return mad_wide(h, f.e, (int64_t)(((u64)((unsigned)c & f.mask) << 32) | (unsigned)a));
+}
+
 // TPR threads per coefficient row (CTA = 128 TPR threads): thread (r, h) writes the chunks of
 // the inputs i = h (mod TPR) of row r and finishes the output pairs p = h (mod TPR) of row r;
 // warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31, the rows of its threads.  With
@@ -194,17 +216,18 @@ __device__ __forceinline__ u64 chunk_reduce_lazy(const unsigned* w, u64 p, u64 r
 // EXACT / PRE: every job of the launch has an exact table / prescaled inputs.  The
 // accumulators of a tile are set to 2^23 before its first MMA, so that each holds 2^23 + D
 // (exact: below 2^24) and its bit pattern exposes D directly.
-template <int MAXIN, int TPR, bool EXACT, bool PRE, bool LAZY>
+// FOLD: the context's primes qualify for folding.
+template <int MAXIN, int TPR, bool EXACT, bool PRE, bool FOLD>
 __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
     k_base_convert_tc(kern::ConvJobs J, const DevPrime* __restrict__ P, int logn, int tiles) {
-    constexpr bool lazy = LAZY;
     griddep_entry();
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     __shared__ __align__(8) u64 s_bar[2];   // [0]: B image landed, [1]: MMAs of the tile done
     __shared__ unsigned s_taddr;
     __shared__ u64 s_qi[TC_MAXIN], s_qinv[TC_MAXIN], s_qinvp[TC_MAXIN];
     __shared__ u64 s_invm[TC_MAXIN];
-    __shared__ int s_invs[TC_MAXIN];
+    __shared__ int s_pre[TC_MAXIN], s_post[TC_MAXIN];
+    __shared__ ConvOut s_f[TC_MAXS];
     __shared__ u64 s_p[TC_MAXS], s_r24p[TC_MAXS], s_corr[TC_MAXS], s_corrp[TC_MAXS];
     __shared__ int s_row[TC_MAXS];
 
@@ -228,25 +251,48 @@ __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
     u64* xs = reinterpret_cast<u64*>(sB + S * sbo);
     const unsigned bytesB = (unsigned)S * sbo;
 
+    const size_t n = (size_t)1 << logn;
+    const u64* in = job.in + blockIdx.y * job.in_pstride;
+    u64* out = job.out + blockIdx.y * job.out_pstride;
+    const int ntiles = (int)(n / TC_M);
+    const int t0 = blockIdx.x * tiles, t1 = min(ntiles, t0 + tiles);
+    // the first tile's inputs are in flight during the set-up
+    constexpr int NX = MAXIN / TPR;   // this thread's inputs: i = k TPR + h
+    u64 x[NX];
+#pragma unroll
+    for (int k = 0; k < NX; ++k)
+        if (k * TPR + h < nin && t0 < t1) x[k] = in[(size_t)(k * TPR + h) * n + (size_t)t0 * TC_M + row];
     if (tid < nin) {
-        s_qi[tid] = P[job.in_ids[tid]].m.q;
-        s_qinv[tid] = job.qinv[tid];
-        s_qinvp[tid] = job.qinv[nin + tid];
-        s_invm[tid] = exact ? job.inv_q[tid] : 0;
-        s_invs[tid] = exact ? (int)job.inv_q[nin + tid] : 64;
+        if (!PRE) {
+            s_qi[tid] = P[job.in_ids[tid]].m.q;
+            s_qinv[tid] = job.qinv[tid];
+            s_qinvp[tid] = job.qinv[nin + tid];
+        }
+        if (exact) {
+            const int sh = (int)job.inv_q[nin + tid];
+            s_invm[tid] = job.inv_q[tid];
+            s_pre[tid] = max(65 - sh, 0);
+            s_post[tid] = max(sh - 64, 1);
+        }
     }
     if (tid < mcount) {
-        s_p[tid] = P[job.out_ids[m0 + tid]].m.q;
-        s_r24p[tid] = job.tcr[m0 + tid];
-        s_row[tid] = job.out_rows[m0 + tid];
-        s_corr[tid] = exact ? job.corr[m0 + tid] : 0;
-        s_corrp[tid] = exact ? job.corr[job.nout + m0 + tid] : 0;
+        if constexpr (FOLD) {
+            s_f[tid] = job.outs[m0 + tid];
+        } else {
+            s_p[tid] = P[job.out_ids[m0 + tid]].m.q;
+            s_r24p[tid] = job.tcr[m0 + tid];
+            s_row[tid] = job.out_rows[m0 + tid];
+            s_corr[tid] = exact ? job.corr[m0 + tid] : 0;
+            s_corrp[tid] = exact ? job.corr[job.nout + m0 + tid] : 0;
+        }
     }
     const unsigned barB = smem_u32(&s_bar[0]), barM = smem_u32(&s_bar[1]);
     if (tid == 0) {
         mbar_init(barB, 1);
         mbar_init(barM, 1);
         mbar_init_fence();
+        mbar_expect_tx(barB, bytesB);
+        bulk_g2s(smem_u32(sB), job.tcb + (size_t)m0 * nin2 * 64, bytesB, barB);
     }
     __syncwarp();
     if (warp == 0) {
@@ -257,16 +303,7 @@ __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
     __syncthreads();
     tc_fence_after();
     const unsigned taddr = s_taddr;
-    if (tid == 0) {
-        mbar_expect_tx(barB, bytesB);
-        bulk_g2s(smem_u32(sB), job.tcb + (size_t)m0 * nin2 * 64, bytesB, barB);
-    }
 
-    const size_t n = (size_t)1 << logn;
-    const u64* in = job.in + blockIdx.y * job.in_pstride;
-    u64* out = job.out + blockIdx.y * job.out_pstride;
-    const int ntiles = (int)(n / TC_M);
-    const int t0 = blockIdx.x * tiles, t1 = min(ntiles, t0 + tiles);
     const unsigned idesc = idesc_f16_f32(TC_M, 8 * S);
     const unsigned aaddr = smem_u32(sA), baddr = smem_u32(sB);
     const unsigned tlane = taddr + ((unsigned)((warp & 3) * 32) << 16);
@@ -274,11 +311,6 @@ __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
     bool ok = true, b_ready = false;
     unsigned phase = 0;
 
-    constexpr int NX = MAXIN / TPR;   // this thread's inputs: i = k TPR + h
-    u64 x[NX];
-#pragma unroll
-    for (int k = 0; k < NX; ++k)
-        if (k * TPR + h < nin && t0 < t1) x[k] = in[(size_t)(k * TPR + h) * n + (size_t)t0 * TC_M + row];
     for (int t = t0; t < t1; ++t) {
         const size_t j = (size_t)t * TC_M + row;
         u64 f = 0;
@@ -288,7 +320,7 @@ __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
             if (i < nin) {
                 const u64 xh = PRE ? x[k] : mul_shoup(x[k], s_qinv[i], s_qinvp[i], s_qi[i]);
                 if (exact) {
-                    if (TPR == 1) f += conv_round_term(xh, s_invm[i], s_invs[i]);
+                    if (TPR == 1) f += conv_round_term_hi(xh, s_invm[i], s_pre[i], s_post[i]);
                     else xs[i * TC_M + row] = xh;
                 }
                 *reinterpret_cast<uint4*>(arow + i * 128) = chunks_f16(xh);
@@ -320,7 +352,7 @@ __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
         }
         __syncwarp();
         if (TPR > 1 && exact) {
-            for (int i = 0; i < nin; ++i) f += conv_round_term(xs[i * TC_M + row], s_invm[i], s_invs[i]);
+            for (int i = 0; i < nin; ++i) f += conv_round_term_hi(xs[i * TC_M + row], s_invm[i], s_pre[i], s_post[i]);
         }
         const u64 v = exact ? conv_round_finish(f) : 0;
         // the next tile's inputs are in flight while the MMAs and this tile's epilogue run
@@ -343,17 +375,18 @@ __global__ void __launch_bounds__(TC_M * TPR, TC_CTAS_PER_SM)
             for (int e = 0; e < 2; ++e) {
                 const int m = 2 * p + e;
                 if (m >= mcount) continue;   // only the last group of a table can be short
-                const u64 pm = s_p[m];
-                u64 y = chunk_reduce_lazy(r + 8 * e, pm, s_r24p[m]);
-                if (lazy) {
-                    // the forward NTT of N = 2^16 takes inputs below 4p
-                    if (exact) y += mul_shoup(v, s_corr[m], s_corrp[m], pm);
+                if constexpr (FOLD) {
+                    const ConvOut fo = s_f[m];
+                    *reinterpret_cast<int64_t*>(reinterpret_cast<char*>(out + j) + fo.off) =
+                        chunk_fold<EXACT>(r + 8 * e, fo, (unsigned)v);
                 } else {
+                    const u64 pm = s_p[m];
+                    u64 y = chunk_reduce_lazy(r + 8 * e, pm, s_r24p[m]);
                     if (y >= 2 * pm) y -= 2 * pm;
                     if (y >= pm) y -= pm;
                     if (exact) y = add_mod(y, mul_shoup(v, s_corr[m], s_corrp[m], pm), pm);
+                    out[(size_t)s_row[m] * n + j] = y;
                 }
-                out[(size_t)s_row[m] * n + j] = y;
             }
         }
         tc_fence_before();
@@ -415,32 +448,30 @@ bool conv_tc_eligible(const ckks_ctx* c, const ConvJobs& J) {
     return J.n > 0;
 }
 
-template <int MAXIN, int TPR, bool EXACT, bool PRE, bool LAZY>
+template <int MAXIN, int TPR, bool EXACT, bool PRE, bool FOLD>
 static void launch_tc(const ckks_ctx* c, const ConvJobs& J, dim3 grid, unsigned smem, int per) {
     // the attribute is set once per device for the largest operand tiles (K = 128, S = 16)
     constexpr int SMEM_MAX = TC_M * TC_MAXIN * 16 + TC_MAXS * TC_MAXIN * 128 + TC_M * TC_MAXIN * 8;
     static std::atomic<unsigned> done{0};
-    allow_dynamic_smem((const void*)k_base_convert_tc<MAXIN, TPR, EXACT, PRE, LAZY>, SMEM_MAX, done);
-    klaunch(c, k_base_convert_tc<MAXIN, TPR, EXACT, PRE, LAZY>, grid, TC_M * TPR, smem, J, c->d_primes, c->logn, per);
+    allow_dynamic_smem((const void*)k_base_convert_tc<MAXIN, TPR, EXACT, PRE, FOLD>, SMEM_MAX, done);
+    klaunch(c, k_base_convert_tc<MAXIN, TPR, EXACT, PRE, FOLD>, grid, TC_M * TPR, smem, J, c->d_primes, c->logn, per);
 }
 
-template <int MAXIN, int TPR, bool LAZY>
+template <int MAXIN, int TPR, bool FOLD>
 static void launch_tc_flags(const ckks_ctx* c, const ConvJobs& J, dim3 grid, unsigned smem, int per, bool exact,
                             bool pre) {
     if (exact) {
-        if (pre) launch_tc<MAXIN, TPR, true, true, LAZY>(c, J, grid, smem, per);
-        else launch_tc<MAXIN, TPR, true, false, LAZY>(c, J, grid, smem, per);
+        if (pre) launch_tc<MAXIN, TPR, true, true, FOLD>(c, J, grid, smem, per);
+        else launch_tc<MAXIN, TPR, true, false, FOLD>(c, J, grid, smem, per);
     } else {
-        if (pre) launch_tc<MAXIN, TPR, false, true, LAZY>(c, J, grid, smem, per);
-        else launch_tc<MAXIN, TPR, false, false, LAZY>(c, J, grid, smem, per);
+        if (pre) launch_tc<MAXIN, TPR, false, true, FOLD>(c, J, grid, smem, per);
+        else launch_tc<MAXIN, TPR, false, false, FOLD>(c, J, grid, smem, per);
     }
 }
-// every conversion output goes to a forward NTT; for N = 2^16 its lazy butterflies take inputs
-// below 4p, so the words are left in [0, 4p) there (canonical for the generic NTT)
 template <int MAXIN, int TPR>
-static void launch_tc_lazy(const ckks_ctx* c, const ConvJobs& J, dim3 grid, unsigned smem, int per, bool exact,
+static void launch_tc_fold(const ckks_ctx* c, const ConvJobs& J, dim3 grid, unsigned smem, int per, bool exact,
                            bool pre) {
-    if (c->logn == 16) launch_tc_flags<MAXIN, TPR, true>(c, J, grid, smem, per, exact, pre);
+    if (c->fold) launch_tc_flags<MAXIN, TPR, true>(c, J, grid, smem, per, exact, pre);
     else launch_tc_flags<MAXIN, TPR, false>(c, J, grid, smem, per, exact, pre);
 }
 
@@ -484,11 +515,11 @@ void base_convert_tc_jobs(const ckks_ctx* c, const ConvJobs& J0, int npoly) {
     KTimer kt_(c, "base_convert", bytes);
     const bool two = c->conv_tc_tpr == 2;
     if (maxin <= 8) {
-        if (two) launch_tc_lazy<8, 2>(c, J, grid, smem, per, exact, pre);
-        else launch_tc_lazy<8, 1>(c, J, grid, smem, per, exact, pre);
+        if (two) launch_tc_fold<8, 2>(c, J, grid, smem, per, exact, pre);
+        else launch_tc_fold<8, 1>(c, J, grid, smem, per, exact, pre);
     } else {
-        if (two) launch_tc_lazy<16, 2>(c, J, grid, smem, per, exact, pre);
-        else launch_tc_lazy<16, 1>(c, J, grid, smem, per, exact, pre);
+        if (two) launch_tc_fold<16, 2>(c, J, grid, smem, per, exact, pre);
+        else launch_tc_fold<16, 1>(c, J, grid, smem, per, exact, pre);
     }
 }
 

@@ -47,6 +47,15 @@ struct DevPrime {
     u64 inv64;               // floor(2^64 / q): Shoup companion of 1, reduces any 64-bit word
 };
 
+// What the tensor-core conversion needs of one output (ckks_ctx::fold): folding constants, the byte
+// offset of its row and, for an exact table, -(prod q_i) mod p
+struct alignas(16) ConvOut {
+    unsigned kc, mask;
+    int e;
+    unsigned off;
+    u64 corr, pad;
+};
+
 // Base-conversion table: inputs (prime ids in_ids, count nin) -> outputs (out_ids, nout).
 //   xhat_i = x_i * qhat_inv[i] mod q_i ; y_m = sum_i xhat_i * qhat_mod[m*nin + i] mod p_m
 struct ConvTab {
@@ -71,6 +80,7 @@ struct ConvTab {
     // tc_nin2, outputs to tc_groups groups of tc_S (even, <= 16)
     unsigned short* d_tcb = nullptr;
     u64* d_tcr = nullptr;        // floor(2^88 / p_m) [nout]: Shoup companion of 2^24 mod p_m
+    ConvOut* d_outs = nullptr;   // [nout]
     int tc_nin2 = 0, tc_S = 0, tc_groups = 0;
 };
 
@@ -276,6 +286,7 @@ struct ScalarVec {
 // (length lpp = limbs per polynomial); limb k of a multi-polynomial array uses ids[k % lpp].
 namespace kern {
 // pstride: words between consecutive polynomials of lpp limbs (0 = lpp * N, contiguous)
+// (contexts with ckks_ctx::fold: the inputs may be signed words within 4 q that are only congruent)
 void ntt_forward(const ckks_ctx* c, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride = 0);
 // forward NTT of an arbitrary list of limbs: limb i at data + off[i] * N with prime ids[i] (N = 2^16);
 // for nb copies of the list, copy t at data + t * bstride
@@ -393,6 +404,7 @@ struct ConvJob {
     u64* out;
     const int *in_ids, *out_ids, *out_rows;
     const u64 *qinv, *qmod;
+    const ConvOut* outs;
     const u64* inv_q;      // non-null: subtract v Q, v = round(sum_i xhat_i / q_i) (centred remainder)
     const u64* corr;
     int nin, nout, ngroups;

@@ -770,6 +770,7 @@ void add_conv_job(ConvJobs& J, const ConvTab& t, const u64* in, u64* out, size_t
     j.qinv = t.d_qhat_inv;
     j.qmod = t.d_qhat_mod;
     j.inv_q = t.d_inv_q;
+    j.outs = t.d_outs;
     j.corr = t.d_corr;
     j.nin = t.nin;
     j.nout = t.nout;

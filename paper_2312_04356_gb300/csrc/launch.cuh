@@ -61,4 +61,9 @@ __device__ __forceinline__ u64 conv_round_term(u64 xh, u64 m, int sh) {
     const u64 lo = xh * m, hi = __umul64hi(xh, m);
     return sh >= 64 ? hi >> (sh - 64) : (hi << (64 - sh)) | (lo >> sh);
 }
+// the same term from the high product alone: shifting xh left by pre first makes the shift right at
+// least 65 (pre = max(65 - sh, 0), post = max(sh - 64, 1)); xh 2^pre < 2^61
+__device__ __forceinline__ u64 conv_round_term_hi(u64 xh, u64 m, int pre, int post) {
+    return __umul64hi(xh << pre, m) >> post;
+}
 __device__ __forceinline__ u64 conv_round_finish(u64 s) { return (s + (1ull << 57)) >> 58; }

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(NTT_THREADS)
         }
         int sid = sid0 + s;
         size_t j = ((size_t)(sid >> logT1) << log2T0) + ((size_t)k << logT1) + (sid & (T1 - 1));
-        sm[k * stride + s] = a[j];
+        sm[k * stride + s] = !INV && s0 == 0 ? ar.canon(a[j]) : a[j];
     }
     __syncthreads();
 

@@ -115,6 +115,7 @@ static std::unique_ptr<ConvTab> make_conv_tab(ckks_ctx* c, const std::vector<int
                                                              t->tc_groups, r24p));
         if (t->d_tcb) t->d_tcr = dev_upload_persistent(r24p);
     }
+    std::vector<ConvOut> outs(t->nout);
     if (exact) {
         // 1/q_i = M_i 2^-(64 + b_i): the rounding term in fixed point (kern: conv_round)
         std::vector<u64> invq(2 * t->nin);
@@ -132,9 +133,21 @@ static std::unique_ptr<ConvTab> make_conv_tab(ckks_ctx* c, const std::vector<int
             for (int k = 0; k < t->nin; ++k) v = mulmod(v, c->mod_of[in_ids[k]] % pm, pm);
             corr[m] = v ? pm - v : 0;
             corr[t->nout + m] = shoup(corr[m], pm);
+            outs[m].corr = corr[m];
         }
         t->d_inv_q = dev_upload_persistent(invq);
         t->d_corr = dev_upload_persistent(corr);
+    }
+    if (c->fold) {
+        for (int m = 0; m < t->nout; ++m) {
+            FoldMod f;
+            fold_consts(c->mod_of[out_ids[m]], f);
+            outs[m].kc = f.kc;
+            outs[m].mask = f.mask;
+            outs[m].e = f.e;
+            outs[m].off = (unsigned)out_rows[m] << (c->logn + 3);
+        }
+        t->d_outs = dev_upload_persistent(outs);
     }
     return t;
 }
@@ -191,6 +204,9 @@ static void free_tab(ConvTab* t) {
     cudaFree(t->d_qhat_mod);
     if (t->d_inv_q) cudaFree(t->d_inv_q);
     if (t->d_corr) cudaFree(t->d_corr);
+    cudaFree(t->d_tcb);
+    cudaFree(t->d_tcr);
+    cudaFree(t->d_outs);
     cudaFree(t->d_iscale);
 }
 

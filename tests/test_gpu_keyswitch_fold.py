@@ -1,6 +1,7 @@
 """Key-switch products in both reductions (folded 128-bit sums, Shoup products) over the digit
 counts and both BSGS kernels: rotations, HMult and a BSGS map bit-exact against the oracle."""
-import numpy as np
+import gc
+
 import pytest
 
 import workloads as WL
@@ -10,18 +11,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-# every digit count; a 61-bit base prime puts the
-# context on Shoup products
-@pytest.mark.parametrize("q0,dnum,n_q", [(60, 1, 4), (60, 2, 4), (60, 4, 4), (61, 1, 4), (61, 3, 5), (61, 4, 4)])
-def test_key_switch_bitexact(q0, dnum, n_q):
+# every digit count; a 61-bit base prime puts the context on Shoup products; N = 2^13 transforms the
+# conversions' lazy outputs in the general shared-memory pass
+@pytest.mark.parametrize("log_n,q0,dnum,n_q", [(10, 60, 1, 4), (10, 60, 2, 4), (10, 60, 4, 4), (10, 61, 1, 4),
+                                               (10, 61, 3, 5), (10, 61, 4, 4), (13, 60, 2, 4)])
+def test_key_switch_bitexact(log_n, q0, dnum, n_q):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2312_04356_gb300 import build
     build.build()
-    WL.PARAMS["fold_test"] = dict(log_n=10, n_q=n_q, dnum=dnum, n_p=0, q0_bits=q0, scale_bits=42, p_bits=60, boot_bits=0,
-                                  n_boot=0, h=0, sigma=3.2)
+    WL.PARAMS["fold_test"] = dict(log_n=log_n, n_q=n_q, dnum=dnum, n_p=0, q0_bits=q0, scale_bits=42, p_bits=60,
+                                  boot_bits=0, n_boot=0, h=0, sigma=3.2)
     try:
-        m = 512
+        m = 1 << (log_n - 1)
         K, o, ctx, keys = make_pair("fold_test", 31, rotations=list(range(1, 9)) + [m - 4, m - 8])
         P, lev = o.P, o.P.L
         ct = o.encrypt(o.encode_pt(WL.slots(1, m, 0.5), lev, P.delta[lev]), 1)
@@ -33,5 +35,8 @@ def test_key_switch_bitexact(q0, dnum, n_q):
         for B in (4, 1):            # 3 giant steps (fused kernel), 9 (stored babies)
             plan = o.make_plan(diags, 0, 1, 9, lev, P.delta[lev], B=B)
             assert_ct_equal(K, ctx, K.ckks_bsgs(ctx, keys, gct, import_plan(K, ctx, plan)), o.bsgs(ct, plan), "BSGS B=%d" % B)
+        K.ckks_sync(ctx)
     finally:
         del WL.PARAMS["fold_test"]
+        K = o = ctx = keys = ct = gct = g = w = plan = None
+        gc.collect()        # the device memory goes back here, not in the middle of a later test
