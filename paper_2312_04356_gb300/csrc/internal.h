@@ -114,6 +114,10 @@ struct DevBuf {
     void reset();
 };
 
+namespace kern {
+struct ScaleTab;
+}
+
 struct ckks_ctx {
     ckks_params P;
     int logn = 0, n = 0, nq = 0, L = 0, alpha = 0, np = 0, nall = 0, n_circuit = 0;
@@ -148,10 +152,11 @@ struct ckks_ctx {
     u64* d_tables = nullptr;
     u64* d_gauss = nullptr;
     int* d_iota = nullptr;                   // 0..nall-1
-    u64* d_pinv = nullptr;                   // P^{-1} mod q_i [nq], Shoup [nq]
-    u64* d_qlinv = nullptr;                  // q_l^{-1} mod q_i [nq][nq], Shoup [nq][nq]
+    // constants per row: residues, Shoup companions, ntt_pair pairs, one block after another
+    u64* d_pinv = nullptr;                   // P^{-1} mod q_i [nq]
+    u64* d_qlinv = nullptr;                  // q_l^{-1} mod q_i [nq][nq]
     std::vector<u64> h_qlinv;                // host copy of the residues [nq][nq]
-    u64* d_pqlinv = nullptr;                 // (P q_l)^{-1} mod q_i [nq][nq], Shoup [nq][nq]
+    u64* d_pqlinv = nullptr;                 // (P q_l)^{-1} mod q_i [nq][nq]
     u64* d_pqlinv2 = nullptr;                // the same times 2 (products doubled in the tail)
     u64* d_pmod = nullptr;                   // P mod q_i [nq], Shoup [nq]
     std::vector<int*> d_ext_ids;             // per level: [0..l] + specials
@@ -187,6 +192,8 @@ struct ckks_ctx {
     mutable std::vector<cudaEvent_t> event_pool;
     mutable std::map<std::string, KStat> kstats;   // name -> launches, ms, algorithmic bytes
     void collect_timing() const;
+
+    kern::ScaleTab scale_tab(const u64* tab, size_t words, size_t row) const;
 
     std::vector<std::vector<int>> digits(int level) const;
     std::vector<int> ext_ids(int level) const;
@@ -288,6 +295,32 @@ namespace kern {
 // pstride: words between consecutive polynomials of lpp limbs (0 = lpp * N, contiguous)
 // (contexts with ckks_ctx::fold: the inputs may be signed words within 4 q that are only congruent)
 void ntt_forward(const ckks_ctx* c, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride = 0);
+// per-row constants in every form the kernels take: residues, Shoup companions, ntt_pair pairs
+// (pair: contexts with ckks_ctx::fold)
+struct ScaleTab {
+    const u64 *w, *wp;
+    const ulonglong2* pair;
+};
+// the rows of polynomial p are the centred lift of the coefficient-domain row src + p * src_pstride
+// with prime src_id
+struct NttLift {
+    const u64* src;
+    size_t src_pstride;
+    int src_id;
+};
+// the transform x leaves as (a - x) s, or a ks - x s (ks: residues and Shoup companions per row); row k of a
+// at a + (k / lpp) * a_pstride + (k % lpp) N
+struct NttTail {
+    const u64* a;
+    size_t a_pstride;
+    ScaleTab s;
+    const ScalarVec* ks;
+};
+// forward NTT of out ([nlimbs / lpp][lpp][N], row k with prime ids[k % lpp] = k % lpp), its input
+// replaced by a lift and / or its output passed through a tail, both optional; lift->src and tail->a
+// must not overlap out
+void ntt_forward_fused(const ckks_ctx* c, u64* out, int nlimbs, const int* ids, int lpp, const NttLift* lift,
+                       const NttTail* tail);
 // forward NTT of an arbitrary list of limbs: limb i at data + off[i] * N with prime ids[i] (N = 2^16);
 // for nb copies of the list, copy t at data + t * bstride
 void ntt_forward_list(const ckks_ctx* c, u64* data, int nlimbs, const int* off, const int* ids, int nb = 1,

@@ -4,8 +4,8 @@
 // graph without the memory-pool nodes, real-time serving loops that forbid cudaMalloc
 // because it can synchronise the device, or hosts that hand the library a fixed memory
 // budget.  ckks_rescale_noalloc gives them the rescale of ckks_rescale with its scratch
-// (the dropped limb in the coefficient domain and its centred lift into every other
-// limb) taken from one file-scope device array instead of the stream-ordered pool.
+// (the dropped limb in the coefficient domain) taken from one file-scope device array
+// instead of the stream-ordered pool.
 #include <mutex>
 #include <unordered_map>
 
@@ -13,7 +13,8 @@
 
 namespace {
 
-// 2^22 words = 32 MiB: the lift needs (2 level + 2) N words, i.e. levels up to 31 at N = 2^16.
+// 2^22 words = 32 MiB.  A call is admitted while (2 level + 2) N fits (levels up to 31 at N = 2^16); it uses
+// the first 2 N words, the output array holding the lift while it is transformed.
 constexpr size_t kScratchWords = (size_t)1 << 22;
 __device__ __align__(256) u64 g_rescale_scratch[kScratchWords];
 
@@ -59,21 +60,15 @@ extern "C" int ckks_rescale_noalloc(ckks_ctx* ctx, const uint64_t* d_in, int lev
                      std::to_string(kScratchWords) + " (lower the level or use ckks_rescale)");
         const size_t nl = (size_t)level + 1;
         const u64* in0 = reinterpret_cast<const u64*>(d_in);
-        const u64* in1 = in0 + nl * n;
         u64* out0 = reinterpret_cast<u64*>(d_out);
         CK_CHECK(out0 + 2 * level * n <= in0 || in0 + 2 * nl * n <= out0, CKKS_EINVAL,
                  "d_out must not overlap d_in");
-        u64* scratch = scratch_for_current_device(ctx->stream);
-        u64* last = scratch;            // [2][N]: the dropped limb of c0 and c1
-        u64* lift = scratch + 2 * n;    // [2][level][N]
-        CUDA_CHECK(cudaMemcpyAsync(last, in0 + (size_t)level * n, n * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        CUDA_CHECK(cudaMemcpyAsync(last + n, in1 + (size_t)level * n, n * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        kern::ntt_inverse(ctx, last, 2, ctx->d_iota + level, 1);
-        kern::lift_centred(ctx, last, level, lift, 2 * level, ctx->d_iota, level, n);   // both polynomials
-        kern::ntt_forward(ctx, lift, 2 * level, ctx->d_iota, level);
-        const u64* s = ctx->d_qlinv + (size_t)level * ctx->nq;
-        const u64* sp = ctx->d_qlinv + (size_t)ctx->nq * ctx->nq + (size_t)level * ctx->nq;
-        kern::sub_mul_scalar(ctx, in0, lift, s, sp, out0, 2 * level, ctx->d_iota, level, (size_t)nl * n);
+        u64* last = scratch_for_current_device(ctx->stream);   // [2][N]: the dropped limb of c0 and c1
+        kern::ntt_inverse_from(ctx, in0 + (size_t)level * n, nl * n, last, 2, ctx->d_iota + level, 1, n, nullptr);
+        const kern::NttLift lift{last, n, level};
+        const kern::NttTail tail{in0, nl * n, ctx->scale_tab(ctx->d_qlinv, (size_t)ctx->nq * ctx->nq, (size_t)level * ctx->nq),
+                                 nullptr};
+        kern::ntt_forward_fused(ctx, out0, 2 * level, ctx->d_iota, level, &lift, &tail);
         ctx->ops["rescale"]++;
     } catch (const CkksError& e) {
         ctx->err = e.msg;

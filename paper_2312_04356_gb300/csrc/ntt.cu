@@ -119,17 +119,55 @@ __device__ __forceinline__ void inv_stages(u64 (&x)[16], const AR& ar, const ulo
     }
 }
 
-// Input of the inverse transform's first pass when it is not the data array itself (SRC
-// kernels): row k reads src + (k / lpp) * src_pstride + (k % lpp) N and the result goes to the
-// data array, so the input is left as it is (no copy before an out-of-place transform).
-// scaled replaces the final factor N^{-1} by the pair w, e.g. k N^{-1} to multiply the result by the
+// What a transform reads or writes besides the data array (X kernels).
+// Inverse, first pass: row k reads src + (k / lpp) * src_pstride + (k % lpp) N and the result goes to the
+// data array, so the input is left as it is (no copy before an out-of-place transform); scaled
+// replaces the final factor N^{-1} by the pair w, e.g. k N^{-1} to multiply the result by the
 // integer k.
+// Forward, first pass: every row of polynomial p is the centred lift of the one row
+// src + p * src_pstride with modulus lift_q (a signed word is what the lazy butterflies take; one
+// fold brings a wider source prime's word into range).
 struct NttSrc {
     const u64* src;
     size_t src_pstride;
     bool scaled;
     ulonglong2 w;
+    u64 lift_q;
 };
+// Forward, last pass: row k receives (a - x) s, or a ks - x s when has_k, instead of the transform x; row k
+// of a at a + (k / lpp) a_pstride + (k % lpp) N, s and ks as ntt_pair pairs per row k % lpp.
+// Against a lift kernel before and a tail kernel after the transform (each a pass over every limb):
+// block 8.94 -> 8.51 ms, 8 ciphertexts in lockstep 62.0 -> 58.6 ms, composite ReLU 6.83 -> 6.14 ms.
+// a's 16 words have to be loaded before the first store: left between the stores they were 16
+// dependent round trips, and the fused pass was slower than the two kernels (9.50 ms).
+struct NttTailArgs {
+    const u64* a;
+    size_t a_pstride;
+    const ulonglong2* s;
+    int has_k;
+    ulonglong2 ks[ScalarVec::MAX];
+};
+template <bool TAIL>
+struct NttArgs {
+    typedef NttSrc type;
+};
+template <>
+struct NttArgs<true> {
+    typedef NttTailArgs type;
+};
+// the centred residue of v mod lq as a signed word, folded
+__device__ __forceinline__ u64 lift_word(u64 v, u64 lq, const FoldMod& f) {
+    return (u64)fold_word((int64_t)(v > (lq >> 1) ? v - lq : v), f);
+}
+// the tail of one word; x lazy
+__device__ __forceinline__ u64 tail_word(u64 a, u64 x, const NttTailArgs& tl, ulonglong2 s, int r, u64 q,
+                                         const FoldMod& f) {
+    if (tl.has_k) {
+        const ulonglong2 ks = tl.ks[r];
+        return fold_canon(fold_mul((int64_t)a, ks.x, ks.y, f) - fold_mul((int64_t)x, s.x, s.y, f), q, f);
+    }
+    return fold_canon(fold_mul((int64_t)(a - x), s.x, s.y, f), q, f);
+}
 // the inverse transform's final factor of row r
 __device__ __forceinline__ ulonglong2 out_factor(const DevPrime* P, const u64* osc, int r, const NttSrc& io) {
     if (io.scaled) return io.w;
@@ -236,12 +274,13 @@ __device__ __forceinline__ int sk(int t, int i, int p) {
 }
 __device__ __forceinline__ int spad(int k) { return k + (k >> 4); }
 
-template <class AR, bool INV, int LOGN>
+template <class AR, bool INV, int LOGN, bool TAIL = false>
 __global__ void __launch_bounds__(1 << (LOGN - 4))
     k_ntt_one(u64* __restrict__ data, const DevPrime* __restrict__ primes, const int* __restrict__ ids, int lpp,
-              size_t pstride, const u64* __restrict__ osc, NttSrc io) {
+              size_t pstride, const u64* __restrict__ osc, const __grid_constant__ NttSrc io,
+              const __grid_constant__ typename NttArgs<TAIL>::type tl) {
     griddep_entry();
-    constexpr int N = 1 << LOGN, NR = (LOGN + 3) / 4, TAIL = LOGN - 4 * (NR - 1);   // rounds, stages of the last
+    constexpr int N = 1 << LOGN, NR = (LOGN + 3) / 4, LAST = LOGN - 4 * (NR - 1);   // rounds, stages of the last
     __shared__ u64 sm[N + N / 16];
     const int limb = blockIdx.y;
     const int r = limb % lpp;
@@ -251,8 +290,14 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
     const int t = threadIdx.x;
     u64 x[16];
     if (!INV) {
+        if (io.lift_q) {
+            const u64* src = io.src + (size_t)(limb / lpp) * io.src_pstride;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = a[sk<LOGN>(t, i, LOGN - 4)];
+            for (int i = 0; i < 16; ++i) x[i] = lift_word(src[sk<LOGN>(t, i, LOGN - 4)], io.lift_q, ar.f);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = a[sk<LOGN>(t, i, LOGN - 4)];
+        }
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr) {
             const int p = rr < NR - 1 ? LOGN - 4 - 4 * rr : 0, s0 = 4 * rr;
@@ -267,14 +312,27 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
             }
             auto widx = [&](int s, int i) { return (1 << (s0 + s)) + (sk<LOGN>(t, i, p) >> (LOGN - s0 - s)); };
             if (rr < NR - 1) fwd_stages<4>(x, ar, P->tw, widx);
-            else fwd_stages<TAIL>(x, ar, P->tw, widx);
+            else fwd_stages<LAST>(x, ar, P->tw, widx);
         }
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sm[spad(16 * t + i)] = ar.canon(x[i]);
-        __syncthreads();
+        for (int i = 0; i < 16; ++i) sm[spad(16 * t + i)] = TAIL ? x[i] : ar.canon(x[i]);
+        if constexpr (TAIL) {
+            const u64* A = tl.a + (size_t)(limb / lpp) * tl.a_pstride + ((size_t)r << LOGN);
+            const ulonglong2 s = tl.s[r];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) a[i * (N / 16) + t] = sm[spad(i * (N / 16) + t)];
+            for (int i = 0; i < 16; ++i) x[i] = __ldg(A + i * (N / 16) + t);
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int j = i * (N / 16) + t;
+                a[j] = tail_word(x[i], sm[spad(j)], tl, s, r, ar.q, ar.f);
+            }
+        } else {
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) a[i * (N / 16) + t] = sm[spad(i * (N / 16) + t)];
+        }
     } else {
         const u64* src = io.src ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << LOGN) : a;
 #pragma unroll
@@ -288,7 +346,7 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
             auto widx = [&](int s, int i) { return (1 << (s0 + s)) + (sk<LOGN>(t, i, p) >> (LOGN - s0 - s)); };
             if (rr == 0) inv_stages<true, 4>(x, ar, P->itw, widx);
             else if (rr < NR - 1) inv_stages<false, 4>(x, ar, P->itw, widx);
-            else inv_stages<false, TAIL>(x, ar, P->itw, widx);
+            else inv_stages<false, LAST>(x, ar, P->itw, widx);
             if (rr > 0) {
                 const int pn = LOGN - 4 * rr;           // register bits of the next round
                 __syncthreads();
@@ -342,12 +400,12 @@ __device__ __forceinline__ void inv_round(u64 (&x)[16], int t, int hi, int s0, c
 // COL: sub-problems are columns (s0 = 0, T1 = 256, element j = k*256 + lo), threads with
 //      consecutive tid take consecutive columns.  ROW: sub-problems are contiguous rows
 //      (s0 = 8, T1 = 1, j = hi*256 + k), consecutive tid take consecutive k.
-template <class AR, bool COL, bool INV, int SUBS, int MINB, bool SRC = false>
+template <class AR, bool COL, bool INV, int SUBS, int MINB, bool X = false>
 __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ data, const DevPrime* __restrict__ primes,
                                                     const int* __restrict__ ids, int lpp, size_t pstride,
                                                     const int* __restrict__ loff, const u64* __restrict__ osc,
-                                                    NttSrc io) {
-    static_assert(!SRC || (INV && !COL), "only the inverse transform's first pass reads a separate source");
+                                                    const __grid_constant__ typename NttArgs<X && !INV && !COL>::type io) {
+    static_assert(!X || !(INV && COL), "the inverse's last pass has no X form");
     griddep_entry();
     __shared__ u64 sm[SUBS * f_stride<SUBS>];
     const int limb = blockIdx.y;
@@ -365,8 +423,14 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
     auto gidx = [&](int k) -> size_t { return COL ? ((size_t)k << 8) + sub : ((size_t)sub << 8) + k; };
 
     if (!INV) {
+        if constexpr (X && !INV && COL) {
+            const u64* src = io.src + (size_t)(limb / lpp) * io.src_pstride;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = a[gidx(t + 16 * i)];
+            for (int i = 0; i < 16; ++i) x[i] = lift_word(src[gidx(t + 16 * i)], io.lift_q, ar.f);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = a[gidx(t + 16 * i)];
+        }
         fwd_round<false>(x, t, hi, s0, P->tw, ar);
 #pragma unroll
         for (int i = 0; i < 16; ++i) sm[f_slot<SUBS>(sp, t + 16 * i)] = x[i];
@@ -379,20 +443,34 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
             for (int i = 0; i < 16; ++i) a[gidx(16 * t + i)] = x[i];     // lazy
         } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = ar.canon(x[i]);
+            for (int i = 0; i < 16; ++i)
+                if (!X) x[i] = ar.canon(x[i]);
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < 16; ++i) sm[f_slot<SUBS>(sp, 16 * t + i)] = x[i];
-            __syncthreads();
+            if constexpr (X && !INV && !COL) {
+                // all of a's words in flight at once (loads cannot pass the stores below)
+                const u64* A = io.a + (size_t)(limb / lpp) * io.a_pstride + ((size_t)r << 16);
+                const ulonglong2 s = io.s[r];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = sm[f_slot<SUBS>(sp, t + 16 * i)];
+                for (int i = 0; i < 16; ++i) x[i] = __ldg(A + gidx(t + 16 * i));
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    a[gidx(t + 16 * i)] = tail_word(x[i], sm[f_slot<SUBS>(sp, t + 16 * i)], io, s, r, ar.q, ar.f);
+            } else {
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = sm[f_slot<SUBS>(sp, t + 16 * i)];
+            }
         }
     } else {
         if (COL) {
 #pragma unroll
             for (int i = 0; i < 16; ++i) x[i] = a[gidx(16 * t + i)];
         } else {
-            const u64* sr = SRC ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << 16) : a;
+            const u64* sr = a;
+            if constexpr (X && INV) sr = io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << 16);
 #pragma unroll
             for (int i = 0; i < 16; ++i) sm[f_slot<SUBS>(sp, t + 16 * i)] = sr[gidx(t + 16 * i)];
             __syncthreads();
@@ -407,7 +485,7 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
 #pragma unroll
         for (int i = 0; i < 16; ++i) x[i] = sm[f_slot<SUBS>(sp, t + 16 * i)];
         inv_round<false, COL>(x, t, hi, s0, P->itw, ar);
-        if (COL) {
+        if constexpr (COL && INV) {
             const ulonglong2 ni = out_factor(P, osc, r, io);
 #pragma unroll
             for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = ar.scale(x[i], ni);
@@ -658,16 +736,19 @@ enum NttVariant {
     NTT_MIX = 0, NTT_V16 = 1, NTT_V4 = 2, NTT_V4_R80 = 3, NTT_X4 = 4, NTT_CL = 5, NTT_NVARIANTS = 6
 };
 
-template <bool COL, bool INV, bool SRC = false>
+template <bool COL, bool INV, bool X = false>
 void launch_ntt16_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const int* ids, int lpp,
-                          size_t pstride, const int* loff, const u64* osc, const NttSrc& io) {
+                          size_t pstride, const int* loff, const u64* osc,
+                          const typename NttArgs<X && !INV && !COL>::type& io) {
 #define NTT16(AR, SUBS, MINB)                                                                      \
-    klaunch(cx, k_ntt16<AR, COL, INV, SUBS, MINB, SRC>, dim3(256 / SUBS, nlimbs), 16 * SUBS, 0,    \
+    klaunch(cx, k_ntt16<AR, COL, INV, SUBS, MINB, X>, dim3(256 / SUBS, nlimbs), 16 * SUBS, 0,      \
             data, cx->d_primes, ids, lpp, pstride, loff, osc, io)
-    if (!cx->fold) {
-        if (v == NTT_V16) NTT16(ArShoup, 16, 3);
-        else NTT16(ArShoup, 4, 8);
-        return;
+    if constexpr (!X || INV) {
+        if (!cx->fold) {
+            if (v == NTT_V16) NTT16(ArShoup, 16, 3);
+            else NTT16(ArShoup, 4, 8);
+            return;
+        }
     }
     switch (v) {
         case NTT_MIX:
@@ -678,8 +759,9 @@ void launch_ntt16_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, cons
         case NTT_V4: NTT16(ArFold, 4, 8); break;
         case NTT_V4_R80: NTT16(ArFold, 4, 12); break;
         default:
-            klaunch(cx, k_ntt16s<ArFold, COL, INV, SRC>, dim3(256 / 4, nlimbs), 256, 0,
-                    data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
+            if constexpr (!X || INV)
+                klaunch(cx, k_ntt16s<ArFold, COL, INV, X>, dim3(256 / 4, nlimbs), 256, 0,
+                        data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
             break;
     }
 #undef NTT16
@@ -744,13 +826,14 @@ void launch_ntt_transform(const ckks_ctx* cx, u64* data, int nlimbs, const int* 
 // N = 2^8 .. 2^12 of a fold context: the whole limb in one CTA
 inline bool ntt_one_cta(const ckks_ctx* cx) { return cx->fold && cx->logn >= 8 && cx->logn <= 12; }
 
-template <bool INV>
+template <bool INV, bool TAIL = false>
 void launch_ntt_one(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
-                    const u64* osc = nullptr, const NttSrc& io = NttSrc{}) {
+                    const u64* osc = nullptr, const NttSrc& io = NttSrc{},
+                    const typename NttArgs<TAIL>::type& tl = typename NttArgs<TAIL>::type{}) {
     KTimer kt_(cx, INV ? "ntt_inv" : "ntt_fwd", 2.0 * nlimbs * cx->n * 8.0);
 #define ONE(LOGN)                                                                                                   \
-    klaunch(cx, k_ntt_one<ArFold, INV, LOGN>, dim3(1, nlimbs), 1 << (LOGN - 4), 0, data, cx->d_primes, ids, lpp, \
-            pstride, osc, io)
+    klaunch(cx, k_ntt_one<ArFold, INV, LOGN, TAIL>, dim3(1, nlimbs), 1 << (LOGN - 4), 0, data, cx->d_primes, ids,   \
+            lpp, pstride, osc, io, tl)
     switch (cx->logn) {
         case 8: ONE(8); break;
         case 9: ONE(9); break;
@@ -811,6 +894,65 @@ void ntt_forward(const ckks_ctx* c, u64* data, int nlimbs, const int* ids, int l
         return;
     }
     for (const PassPlan& p : ntt_passes(c->logn)) launch_pass<false>(c, data, nlimbs, ids, lpp, pstride, p, 0);
+    LAUNCH_CHECK();
+}
+
+// out = the transform of `in` through the tail (NttLift, NttTail).  Where the transform's passes
+// have the lift and the tail built in (a fold context whose variant is made of k_ntt16 passes, or
+// the one-CTA rings) that is all; elsewhere the lift, the transform in place and the tail run one
+// after another.
+void ntt_forward_fused(const ckks_ctx* c, u64* out, int nlimbs, const int* ids, int lpp, const NttLift* lift,
+                       const NttTail* tail) {
+    if (nlimbs <= 0) return;
+    CK_CHECK(lpp >= 1 && nlimbs % lpp == 0, CKKS_EINVAL, "whole polynomials only");
+    const size_t n = c->n, ps = (size_t)lpp * n;
+    const int v = c->logn == 16 ? ntt_pick(c, nlimbs) : -1;
+    const bool one = ntt_one_cta(c);
+    if (!c->fold || lpp > ScalarVec::MAX || (!one && (c->logn != 16 || v > NTT_V4_R80))) {
+        if (lift) lift_centred(c, lift->src, lift->src_id, out, nlimbs, ids, lpp, lift->src_pstride);
+        ntt_forward(c, out, nlimbs, ids, lpp);
+        if (tail && tail->ks)
+            sub_mul2_scalar(c, tail->a, out, *tail->ks, tail->s.w, tail->s.wp, out, nlimbs, ids, lpp, tail->a_pstride);
+        else if (tail)
+            sub_mul_scalar(c, tail->a, out, tail->s.w, tail->s.wp, out, nlimbs, ids, lpp, tail->a_pstride);
+        return;
+    }
+    NttSrc io{};
+    if (lift) {
+        io.src = lift->src;
+        io.src_pstride = lift->src_pstride;
+        io.lift_q = c->mod_of[lift->src_id];
+    }
+    NttTailArgs tl;
+    if (tail) {
+        tl.a = tail->a;
+        tl.a_pstride = tail->a_pstride;
+        tl.s = tail->s.pair;
+        tl.has_k = tail->ks != nullptr;
+        if (tail->ks)
+            for (int i = 0; i < lpp; ++i) {
+                u64 w[2];
+                hostmath::ntt_pair(tail->ks->v[i], c->q[i], true, w);
+                tl.ks[i] = make_ulonglong2(w[0], w[1]);
+            }
+    }
+    if (one) {
+        if (tail) launch_ntt_one<false, true>(c, out, nlimbs, ids, lpp, ps, nullptr, io, tl);
+        else launch_ntt_one<false>(c, out, nlimbs, ids, lpp, ps, nullptr, io);
+        LAUNCH_CHECK();
+        return;
+    }
+    const double bytes = (double)nlimbs * n * 8.0;
+    {
+        KTimer kt_(c, "ntt_fwd", bytes);
+        if (lift) launch_ntt16_variant<true, false, true>(c, v, out, nlimbs, ids, lpp, ps, nullptr, nullptr, io);
+        else launch_ntt16_variant<true, false>(c, v, out, nlimbs, ids, lpp, ps, nullptr, nullptr, io);
+    }
+    {
+        KTimer kt_(c, "ntt_fwd", bytes);
+        if (tail) launch_ntt16_variant<false, false, true>(c, v, out, nlimbs, ids, lpp, ps, nullptr, nullptr, tl);
+        else launch_ntt16_variant<false, false>(c, v, out, nlimbs, ids, lpp, ps, nullptr, nullptr, io);
+    }
     LAUNCH_CHECK();
 }
 
@@ -894,7 +1036,7 @@ void ntt_inverse_from(const ckks_ctx* c, const u64* src, size_t src_pstride, u64
     CK_CHECK(!scaled || (lpp == 1 && osc == nullptr && pstride == c->n), CKKS_EINVAL,
              "an integer factor needs one contiguous row per polynomial and no output scale table");
     if (c->logn == 16 || ntt_one_cta(c)) {
-        NttSrc io{src, src_pstride, scaled, {}};
+        NttSrc io{src, src_pstride, scaled, {}, 0};
         if (scaled) {
             const u64 q = c->mod_of[k_id];
             u64 w[2];

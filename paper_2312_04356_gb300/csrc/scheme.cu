@@ -63,6 +63,11 @@ std::vector<std::vector<int>> ckks_ctx::digits(int level) const {
     return out;
 }
 
+// the rows from `row` on of a constant table of `words` residues (ckks_ctx::d_pinv ...)
+kern::ScaleTab ckks_ctx::scale_tab(const u64* tab, size_t words, size_t row) const {
+    return {tab + row, tab + words + row, reinterpret_cast<const ulonglong2*>(tab + 2 * words) + row};
+}
+
 std::vector<int> ckks_ctx::ext_ids(int level) const {
     std::vector<int> v;
     for (int i = 0; i <= level; ++i) v.push_back(i);
@@ -349,6 +354,13 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
             pqlinv2[(size_t)l * c->nq + i] = v2;
             pqlinv2[(size_t)c->nq * c->nq + (size_t)l * c->nq + i] = shoup(v2, c->q[i]);
         }
+    // third block: the pairs (row k of a table has prime k mod nq)
+    for (std::vector<u64>* t : {&pinv, &qlinv, &pqlinv, &pqlinv2}) {
+        const size_t words = t->size() / 2;
+        t->resize(4 * words);
+        if (c->fold)
+            for (size_t k = 0; k < words; ++k) ntt_pair((*t)[k], c->q[k % c->nq], true, t->data() + 2 * words + 2 * k);
+    }
     c->d_pinv = dev_upload_persistent(pinv);
     c->d_qlinv = dev_upload_persistent(qlinv);
     c->h_qlinv.assign(qlinv.begin(), qlinv.begin() + (size_t)c->nq * c->nq);
@@ -493,36 +505,36 @@ ckks_ct imult(const ckks_ct& a) {
     return o;
 }
 
-// rescale(mul_int(a, k)) without materialising a k: the dropped limbs are scaled by k while
-// they are copied out, and the tail computes a_i (k q_l^{-1}) - lift_i q_l^{-1} (the same
-// residues as (k a_i - lift_i) q_l^{-1}); like rescale(mul_int(a, k)) the scale becomes
-// a.scale / q_l (callers track the integer factor themselves).
-ckks_ct rescale_mul(const ckks_ct& a, long long k) {
+// rescale(mul_int(a, kk)) without materialising a kk: the dropped limbs are scaled by kk by the
+// inverse transform's last factor, and the forward transform's tail computes a_i (kk q_l^{-1}) -
+// lift_i q_l^{-1} (the same residues as (kk a_i - lift_i) q_l^{-1}); like rescale(mul_int(a, kk)) the
+// scale becomes a.scale / q_l (callers track the integer factor themselves).
+ckks_ct rescale_mul(const ckks_ct& a, long long kk) {
     ckks_ctx* c = a.ctx;
     const int l = a.level;
     CK_CHECK(l >= 1, CKKS_ELEVEL, "cannot rescale a level-0 ciphertext");
     CK_CHECK(l <= ScalarVec::MAX, CKKS_EINVAL, "too many limbs for a by-value scalar vector");
     c->ops["rescale"]++;
     const size_t n = c->n;
-    // k times the last limb of every polynomial (c0, c1 of each ciphertext: 2 nb rows (l + 1) N
+    // kk times the last limb of every polynomial (c0, c1 of each ciphertext: 2 nb rows (l + 1) N
     // apart), to the coefficient domain; then its centred lift to the other l primes, back to
     // the NTT domain
     const int np_ = 2 * a.nb;
     DevBuf last((size_t)np_ * n, c->stream);
     kern::ntt_inverse_from(c, a.c0() + (size_t)l * n, (size_t)(l + 1) * n, last.ptr, np_, c->d_iota + l, 1, n,
-                           nullptr, from_signed(k, c->q[l]), l);
-    DevBuf lift((size_t)np_ * l * n, c->stream);
-    kern::lift_centred(c, last.ptr, l, lift.ptr, np_ * l, c->d_iota, l, n);     // every polynomial
-    kern::ntt_forward(c, lift.ptr, np_ * l, c->d_iota, l);
+                           nullptr, from_signed(kk, c->q[l]), l);
     ckks_ct o = new_ct(c, l - 1, a.scale / (double)c->q[l], a.nb);
     ScalarVec s1;
-    for (int i = 0; i < l; ++i) {
-        s1.v[i] = mulmod(from_signed(k, c->q[i]), c->h_qlinv[(size_t)l * c->nq + i], c->q[i]);
-        s1.vp[i] = shoup(s1.v[i], c->q[i]);
-    }
-    const u64* s2 = c->d_qlinv + (size_t)l * c->nq;
-    const u64* s2p = c->d_qlinv + (size_t)c->nq * c->nq + (size_t)l * c->nq;
-    kern::sub_mul2_scalar(c, a.c0(), lift.ptr, s1, s2, s2p, o.c0(), np_ * l, c->d_iota, l, (size_t)(l + 1) * n);
+    if (kk != 1)
+        for (int i = 0; i < l; ++i) {
+            s1.v[i] = mulmod(from_signed(kk, c->q[i]), c->h_qlinv[(size_t)l * c->nq + i], c->q[i]);
+            s1.vp[i] = shoup(s1.v[i], c->q[i]);
+        }
+    const size_t words = (size_t)c->nq * c->nq;
+    const kern::NttLift lift{last.ptr, n, l};
+    const kern::NttTail tail{a.c0(), (size_t)(l + 1) * n, c->scale_tab(c->d_qlinv, words, (size_t)l * c->nq),
+                             kk != 1 ? &s1 : nullptr};
+    kern::ntt_forward_fused(c, o.c0(), np_ * l, c->d_iota, l, &lift, &tail);
     return o;
 }
 
@@ -564,8 +576,8 @@ ckks_ct mod_raise(const ckks_ct& a) {
     DevBuf coef((size_t)np_ * n, c->stream);
     kern::ntt_inverse_from(c, a.c0(), n, coef.ptr, np_, c->d_iota, 1, n, nullptr);
     ckks_ct o = new_ct(c, c->L, a.scale, a.nb);
-    kern::lift_centred(c, coef.ptr, 0, o.buf.ptr, np_ * c->nq, c->d_iota, c->nq, n);   // row k from source k / nq
-    kern::ntt_forward(c, o.buf.ptr, np_ * c->nq, c->d_iota, c->nq);
+    const kern::NttLift lift{coef.ptr, n, 0};            // row k from source k / nq
+    kern::ntt_forward_fused(c, o.buf.ptr, np_ * c->nq, c->d_iota, c->nq, &lift, nullptr);
     return o;
 }
 
@@ -643,13 +655,10 @@ void mod_down_rescale(ckks_ctx* c, u64* acc, int level, u64* out, bool twice, in
     const int* pid = c->d_ext_ids[level] + l;      // q_l, then the special primes
     const ConvTab& tab_c = c->mdrs_tab(l);
     kern::ntt_inverse(c, acc + (size_t)l * n, npoly * np1, pid, np1, next * n, tab_c.d_iscale);
-    DevBuf conv((size_t)npoly * l * n, c->stream);
-    kern::base_convert(c, tab_c, acc + (size_t)l * n, n, conv.ptr, n, npoly, next * n, (size_t)l * n, true);
-    kern::ntt_forward(c, conv.ptr, npoly * l, c->d_iota, l);
+    kern::base_convert(c, tab_c, acc + (size_t)l * n, n, out, n, npoly, next * n, (size_t)l * n, true);
     const u64* tab = twice ? c->d_pqlinv2 : c->d_pqlinv;     // twice: 2 x the result, same pass
-    const u64* s = tab + (size_t)l * c->nq;
-    const u64* sp = tab + (size_t)c->nq * c->nq + (size_t)l * c->nq;
-    kern::sub_mul_scalar(c, acc, conv.ptr, s, sp, out, npoly * l, c->d_iota, l, next * n);
+    const kern::NttTail tail{acc, next * n, c->scale_tab(tab, (size_t)c->nq * c->nq, (size_t)l * c->nq), nullptr};
+    kern::ntt_forward_fused(c, out, npoly * l, c->d_iota, l, nullptr, &tail);
 }
 
 // acc (Q_l u P) += P x on the Q rows, x [nb][2][l+1][N], acc [nb][2][next][N]
@@ -667,12 +676,9 @@ static void mod_down(ckks_ctx* c, u64* acc, int level, u64* out, int nb = 1) {
     const int* pid = c->d_ext_ids[level] + nl;
     const ConvTab& tab_c = c->moddown_tab(level);
     kern::ntt_inverse(c, acc + (size_t)nl * n, npoly * c->np, pid, c->np, (size_t)next * n, tab_c.d_iscale);
-    DevBuf conv((size_t)npoly * nl * n, c->stream);
-    kern::base_convert(c, tab_c, acc + (size_t)nl * n, n, conv.ptr, n, npoly, (size_t)next * n, (size_t)nl * n,
-                       true);
-    kern::ntt_forward(c, conv.ptr, npoly * nl, c->d_iota, nl);
-    kern::sub_mul_scalar(c, acc, conv.ptr, c->d_pinv, c->d_pinv + c->nq, out, npoly * nl, c->d_iota, nl,
-                         (size_t)next * n);
+    kern::base_convert(c, tab_c, acc + (size_t)nl * n, n, out, n, npoly, (size_t)next * n, (size_t)nl * n, true);
+    const kern::NttTail tail{acc, (size_t)next * n, c->scale_tab(c->d_pinv, c->nq, 0), nullptr};
+    kern::ntt_forward_fused(c, out, npoly * nl, c->d_iota, nl, nullptr, &tail);
 }
 
 u64 galois_of_step(const ckks_ctx* c, long long r) {
@@ -787,10 +793,9 @@ static void mod_down_poly(ckks_ctx* c, u64* x, int level, u64* out, int nb = 1, 
     if (xstride == 0) xstride = ((size_t)nl + c->np) * n;
     const ConvTab& tab_c = c->moddown_tab(level);
     kern::ntt_inverse(c, x + (size_t)nl * n, nb * c->np, c->d_ext_ids[level] + nl, c->np, xstride, tab_c.d_iscale);
-    DevBuf conv((size_t)nb * nl * n, c->stream);
-    kern::base_convert(c, tab_c, x + (size_t)nl * n, n, conv.ptr, n, nb, xstride, (size_t)nl * n, true);
-    kern::ntt_forward(c, conv.ptr, nb * nl, c->d_iota, nl);
-    kern::sub_mul_scalar(c, x, conv.ptr, c->d_pinv, c->d_pinv + c->nq, out, nb * nl, c->d_iota, nl, xstride);
+    kern::base_convert(c, tab_c, x + (size_t)nl * n, n, out, n, nb, xstride, (size_t)nl * n, true);
+    const kern::NttTail tail{x, xstride, c->scale_tab(c->d_pinv, c->nq, 0), nullptr};
+    kern::ntt_forward_fused(c, out, nb * nl, c->d_iota, nl, nullptr, &tail);
 }
 
 // rot_r(a) for every r in steps kept over Q_l u P before ModDown (double hoisting), each

@@ -1,5 +1,6 @@
 """Key-switch products in both reductions (folded 128-bit sums, Shoup products) over the digit
-counts and both BSGS kernels: rotations, HMult and a BSGS map bit-exact against the oracle."""
+counts and both BSGS kernels, and the lifts and tails inside the transforms or beside them:
+rotations, HMult, rescales, ModRaise and a BSGS map bit-exact against the oracle."""
 import gc
 
 import pytest
@@ -31,6 +32,10 @@ def test_key_switch_bitexact(log_n, q0, dnum, n_q):
         for s, g, w in zip([1, 7], K.ckks_rotate_hoisted(ctx, keys, gct, [1, 7]), o.rotate_hoisted(ct, [1, 7])):
             assert_ct_equal(K, ctx, g, w, "HRot %d" % s)
         assert_ct_equal(K, ctx, K.ckks_mul_relin(ctx, keys, gct, gct), o.mul_relin(ct, ct), "HMult")
+        assert_ct_equal(K, ctx, K.ckks_rescale(ctx, gct), o.rescale(ct), "rescale")
+        assert_ct_equal(K, ctx, K.ckks_level_down(ctx, gct, 1), o.level_down(ct, 1), "level_down")
+        c0 = o.mod_drop(ct, 0)
+        assert_ct_equal(K, ctx, K.ckks_mod_raise(ctx, import_ct(K, ctx, c0)), o.mod_raise(c0), "ModRaise")
         diags = {i: WL.slots(40 + i, m) for i in range(9)}
         for B in (4, 1):            # 3 giant steps (fused kernel), 9 (stored babies)
             plan = o.make_plan(diags, 0, 1, 9, lev, P.delta[lev], B=B)
