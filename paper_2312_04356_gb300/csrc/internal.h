@@ -343,6 +343,14 @@ struct KsBatch {
     int nb = 1;
     size_t dstr = 0, ostr = 0, xstr = 0;
 };
+// Where row e of raised digit d lies.  ModUp writes only the rows it converts; a digit's own rows
+// (e in [d alpha, (d + 1) alpha), e < nl) are the polynomial it was raised from, read where that lies.
+struct Digits {
+    const u64* D;        // [ndig][next][N]; ciphertext t of a batch at + t KsBatch::dstr
+    const u64* own;      // [nl][N]; ciphertext t at + t own_str
+    size_t own_str;
+    int nl, alpha;
+};
 // (bt: a batch of bt.nb ciphertexts, babies at a[b] + t dstr, outputs at o[g] + t ostr)
 void bsgs_inner_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int* ids, const KsBatch& bt);
 // Baby rotations and giant-step inner sums in one pass, the babies never stored: for every
@@ -359,9 +367,9 @@ struct BsgsFused {
     int nb, ng, ndig;
     unsigned acc;
 };
-// D [ndig][next][N] raised digits of c1; c0, c1 [nl][N]; s: P mod q_i
+// D: raised digits of c1; c0, c1 [nl][N]; s: P mod q_i
 // (bt: a batch of bt.nb ciphertexts, D at + t dstr, c0 and c1 at + t xstr, outputs at o[g] + t ostr)
-void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1, int nl,
+void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0, const u64* c1, int nl,
                 int next, const int* ext_ids, const u64* s, const KsBatch& bt);
 // o = sum_t w_t a_t (mod q per limb) for up to MAX terms: the integer-weighted sum of a
 // Chebyshev leaf in one pass.  Arrays of nl limbs, limb k with prime ids[k % lpp]; w[t][r]
@@ -468,7 +476,7 @@ unsigned take_device_faults();
 unsigned peek_device_faults();   // the same count, not cleared
 // test hook: withhold the tensor-core conversion's MMAs so that its bounded waits run out
 void set_tc_withhold(bool on);
-// key-switch inner product: D [ndig][next][N], key rows krow[e] of [ndig][nall][N];
+// key-switch inner product: raised digits D, key rows krow[e] of [ndig][nall][N];
 // ob/oa [next][N] = sum_d D_d(sigma_g) * key_d ; g = 1 means no automorphism
 // x0 (optional, rows [x0rows][N] with the primes of the first x0rows extended limbs): ob row e
 // += s[e] * x0[e](sigma_g) for e < x0rows (s null: unscaled), the automorphed c0 term of a
@@ -476,7 +484,7 @@ void set_tc_withhold(bool on);
 // P-lifted d0, d1 of a relinearisation, g = 1)
 // (bt: a batch of bt.nb ciphertexts switched with the same key, D at + t dstr, ob / oa at + t ostr,
 // x0 / x1 at + t xstr; at most 4 digits)
-void ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
+void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
               const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate = false, const u64* x0 = nullptr,
               int x0rows = 0, const u64* s = nullptr, const u64* x1 = nullptr,
               const KsBatch& bt = KsBatch());

@@ -14,6 +14,13 @@
 
 namespace {
 
+// row e of digit d of ciphertext t (the CTA's e is fixed, so this is uniform)
+__device__ __forceinline__ const u64* digit_row(const kern::Digits& D, int d, int e, int t, int next, size_t dstr,
+                                                int logn) {
+    if (e < D.nl && e / D.alpha == d) return D.own + t * D.own_str + ((size_t)e << logn);
+    return D.D + t * dstr + (((size_t)d * next + e) << logn);
+}
+
 // ------------------------------------------------- BSGS inner products ----
 // o[g][poly][limb] = sum_b a_b[poly][limb] * p_{g,b}[limb] for NG giant steps at once: each
 // baby value is loaded once and multiplied into every giant step's sum; the products are
@@ -83,7 +90,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 template <bool FOLD, int NDIG, int NG>
 __global__ void __launch_bounds__(256, 3)
-    k_bsgs_fused_async(const __grid_constant__ kern::BsgsFused T, const u64* __restrict__ D,
+    k_bsgs_fused_async(const __grid_constant__ kern::BsgsFused T, const __grid_constant__ kern::Digits D,
                        const u64* __restrict__ c0, const u64* __restrict__ c1, int nl, int next,
                        const int* __restrict__ ext_ids, const u64* __restrict__ s0,
                        const DevPrime* __restrict__ P, int logn, size_t kstride, kern::KsBatch bt) {
@@ -104,7 +111,9 @@ __global__ void __launch_bounds__(256, 3)
     const int t = blockIdx.x % bt.nb;
     const int j = (blockIdx.x / bt.nb) * 256 + tid;
     if (j >= (int)n) return;
-    D += t * bt.dstr;
+    const u64* Dr[NDIG];
+#pragma unroll
+    for (int d = 0; d < NDIG; ++d) Dr[d] = digit_row(D, d, e, t, next, bt.dstr, logn);
     c0 += t * bt.xstr;
     c1 += t * bt.xstr;
     auto slot = [&](int st, int k) -> u64* { return sbuf + ((size_t)(st * NS + k) << 8) + tid; };
@@ -121,7 +130,7 @@ __global__ void __launch_bounds__(256, 3)
                 const size_t kk = d * kstride + (size_t)id * n + j;
                 cp_async8(slot(st, d), T.kb[b] + kk);
                 cp_async8(slot(st, NDIG + d), T.ka[b] + kk);
-                cp_async8(slot(st, 2 * NDIG + d), D + ((size_t)d * next + e) * n + src);
+                cp_async8(slot(st, 2 * NDIG + d), Dr[d] + src);
             }
             if (qrow) cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + src);
         }
@@ -189,7 +198,7 @@ __global__ void __launch_bounds__(256, 3)
 // varying part of blockIdx.x, so the CTAs that read the same key words run side by side and
 // all but the first find them in L2: the key streams from HBM about once per batch.
 template <bool FOLD, bool ACC, int V, int NDIG>
-__global__ void k_ks_inner_d(const u64* __restrict__ D, int next, const int* __restrict__ ext_ids,
+__global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, const int* __restrict__ ext_ids,
                              const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
                              u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride,
                              const u64* __restrict__ x0, const u64* __restrict__ x1, int x0rows,
@@ -202,7 +211,6 @@ __global__ void k_ks_inner_d(const u64* __restrict__ D, int next, const int* __r
     const int t = blockIdx.x % bt.nb;
     const int j = V * ((blockIdx.x / bt.nb) * blockDim.x + threadIdx.x);
     if (j >= (int)n) return;
-    D += t * bt.dstr;
     ob += t * bt.ostr;
     oa += t * bt.ostr;
     if (x0) x0 += t * bt.xstr;
@@ -213,7 +221,7 @@ __global__ void k_ks_inner_d(const u64* __restrict__ D, int next, const int* __r
     u64 x[NDIG][V], yb[NDIG][V], ya[NDIG][V];
 #pragma unroll
     for (int d = 0; d < NDIG; ++d) {
-        const u64* Dd = D + ((size_t)d * next + e) * n;
+        const u64* Dd = digit_row(D, d, e, t, next, bt.dstr, logn);
         const size_t kk = d * kstride + (size_t)id * n + j;
         if (bt.nb == 1) {
             ldv_cs<V>(kb + kk, yb[d]);   // each key word is read once per key switch: keep the
@@ -318,7 +326,7 @@ void bsgs_inner_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int
 }
 
 template <bool FOLD, int NDIG, int NG>
-static void launch_bsgs_async_one(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0,
+static void launch_bsgs_async_one(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0,
                                   const u64* c1, int nl, int next, const int* ext, const u64* s,
                                   const KsBatch& bt) {
     constexpr int NS = 3 * NDIG + 2 + NG;
@@ -331,7 +339,7 @@ static void launch_bsgs_async_one(const ckks_ctx* c, const BsgsFused& t, const u
 }
 
 template <bool FOLD, int NDIG>
-static void launch_bsgs_async_g(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1,
+static void launch_bsgs_async_g(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0, const u64* c1,
                                 int nl, int next, const int* ext, const u64* s, const KsBatch& bt) {
     switch (t.ng) {
         case 1: launch_bsgs_async_one<FOLD, NDIG, 1>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
@@ -342,7 +350,7 @@ static void launch_bsgs_async_g(const ckks_ctx* c, const BsgsFused& t, const u64
 }
 
 template <bool FOLD>
-static void launch_bsgs_async(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1,
+static void launch_bsgs_async(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0, const u64* c1,
                               int nl, int next, const int* ext, const u64* s, const KsBatch& bt) {
     switch (t.ndig) {
         case 1: launch_bsgs_async_g<FOLD, 1>(c, t, D, c0, c1, nl, next, ext, s, bt); break;
@@ -352,7 +360,7 @@ static void launch_bsgs_async(const ckks_ctx* c, const BsgsFused& t, const u64* 
     }
 }
 
-void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* c0, const u64* c1, int nl,
+void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0, const u64* c1, int nl,
                 int next, const int* ext_ids, const u64* s, const KsBatch& bt) {
     CK_CHECK(t.nb >= 1 && t.nb <= BsgsFused::MAXB && t.ng >= 1 && t.ng <= BsgsFused::MAXG && t.ndig >= 1 &&
                  t.ndig <= 4, CKKS_EINVAL, "fused BSGS: 1..32 babies, 1..4 giant steps, 1..4 digits");
@@ -381,7 +389,7 @@ void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const u64* D, const u64* 
 }
 
 template <bool FOLD, bool ACC, int V>
-static void launch_ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
+static void launch_ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
                             const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
                             const u64* s0, const KsBatch& bt) {
     dim3 grid = ewv_grid(c->n, next, V);
@@ -407,7 +415,7 @@ static void launch_ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next,
     }
 }
 
-void ks_inner(const ckks_ctx* c, const u64* D, int ndig, int next, const int* ext_ids, const u64* kb,
+void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
               const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate, const u64* x0, int x0rows, const u64* s,
               const u64* x1, const KsBatch& bt) {
     CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4, CKKS_EINVAL, "key switching takes 1..4 digits");

@@ -487,15 +487,17 @@ ckks_ct mul_int(const ckks_ct& a, long long v) {
     return o;
 }
 
-ckks_ct add_const(const ckks_ct& a, double cst) {
+ckks_ct add_const(const ckks_ct& a, double cst) { return add_const(copy_ct(a), cst); }
+
+ckks_ct add_const(ckks_ct&& o, double cst) {
+    const ckks_ct& a = o;
     ckks_ctx* c = a.ctx;
     const int nl = a.level + 1;
     long long v = llround_away(cst * a.scale);
     ScalarVec sv;
     for (int i = 0; i < nl; ++i) sv.v[i] = from_signed(v, c->q[i]);
-    ckks_ct o = copy_ct(a);
     kern::add_scalar_v(c, o.c0(), sv, nl * a.nb, c->d_iota, nl, a.cstride());    // c0 of each ciphertext
-    return o;
+    return std::move(o);
 }
 
 ckks_ct imult(const ckks_ct& a) {
@@ -568,6 +570,17 @@ ckks_ct level_down(const ckks_ct& a, int level) {
     return x;
 }
 
+ckks_ct level_down(ckks_ct&& a, int level) {
+    if (level == a.level) return std::move(a);
+    return level_down(static_cast<const ckks_ct&>(a), level);
+}
+
+// a itself when it is at that level, else its level_down, held in tmp
+static const ckks_ct& at_level(const ckks_ct& a, int level, ckks_ct& tmp) {
+    if (level == a.level) return a;
+    return tmp = level_down(a, level);
+}
+
 ckks_ct mod_raise(const ckks_ct& a) {
     ckks_ctx* c = a.ctx;
     CK_CHECK(a.level == 0, CKKS_EINVAL, "ModRaise needs a level-0 ciphertext");
@@ -582,9 +595,16 @@ ckks_ct mod_raise(const ckks_ct& a) {
 }
 
 // ------------------------------------------------------- key switching -----
-// D: [ndig][next][N], NTT domain; for a batch, x of ciphertext t at x + t xstride and D
-// [nb][ndig][next][N]
-DevBuf mod_up(ckks_ctx* c, const u64* x, int level, int* ndig_out, int nb, size_t xstride) {
+// The polynomial x (NTT domain, [l+1][N]; ciphertext t of a batch at x + t xstride) raised to Q_l u P
+// per digit: the converted rows of [nb][ndig][next][N] and x itself, which holds each digit's own
+// rows (kern::Digits).  x must outlive the key switches that read the digits.
+struct Raised {
+    DevBuf D;
+    const u64* x = nullptr;
+    size_t xstride = 0;
+    int ndig = 1;
+};
+Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride = 0) {
     const size_t n = c->n;
     const int nl = level + 1;
     const int next = nl + c->np;
@@ -595,38 +615,39 @@ DevBuf mod_up(ckks_ctx* c, const u64* x, int level, int* ndig_out, int nb, size_
     DevBuf coef((size_t)nb * nl * n, c->stream);
     kern::ntt_inverse_from(c, x, xstride, coef.ptr, nb * nl, c->d_iota, nl, (size_t)nl * n,
                            c->d_modup_iscale[level]);   // prescaled
-    DevBuf D((size_t)nb * dstr, c->stream);
+    Raised r;
+    r.D = DevBuf((size_t)nb * dstr, c->stream);
+    r.x = x;
+    r.xstride = xstride;
+    r.ndig = ndig;
     const int* ext = c->d_ext_ids[level];
     kern::ConvJobs jobs;
     jobs.n = 0;
     for (int d = 0; d < ndig; ++d)
         kern::add_conv_job(jobs, c->modup_tab(level, d), coef.ptr + (size_t)dig[d].front() * n,
-                           D.ptr + (size_t)d * next * n, (size_t)nl * n, dstr, true);
+                           r.D.ptr + (size_t)d * next * n, (size_t)nl * n, dstr, true);
     kern::base_convert_jobs(c, jobs, nb);
-    for (int d = 0; d < ndig; ++d) {
-        u64* Dd = D.ptr + (size_t)d * next * n;
-        const int lo = dig[d].front(), hi = dig[d].back() + 1;
-        CUDA_CHECK(cudaMemcpy2DAsync(Dd + (size_t)lo * n, dstr * 8, x + (size_t)lo * n, xstride * 8,
-                                     (size_t)(hi - lo) * n * 8, nb, cudaMemcpyDeviceToDevice, c->stream));
-        if (c->logn != 16) {
-            if (lo > 0) kern::ntt_forward(c, Dd, nb * lo, ext, lo, dstr);
-            if (next > hi) kern::ntt_forward(c, Dd + (size_t)hi * n, nb * (next - hi), ext + hi, next - hi, dstr);
-        }
-    }
-    if (c->logn == 16)   // every converted row of every digit of every ciphertext in one launch
-        kern::ntt_forward_list(c, D.ptr, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb,
+    if (c->logn == 16) {   // every converted row of every digit of every ciphertext in one launch
+        kern::ntt_forward_list(c, r.D.ptr, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb,
                                dstr);
-    *ndig_out = ndig;
-    return D;
+        return r;
+    }
+    for (int d = 0; d < ndig; ++d) {
+        u64* Dd = r.D.ptr + (size_t)d * next * n;
+        const int lo = dig[d].front(), hi = dig[d].back() + 1;
+        if (lo > 0) kern::ntt_forward(c, Dd, nb * lo, ext, lo, dstr);
+        if (next > hi) kern::ntt_forward(c, Dd + (size_t)hi * n, nb * (next - hi), ext + hi, next - hi, dstr);
+    }
+    return r;
 }
 
 // inner product with switching key `code` (automorphism g applied to D on the fly) over
 // Q_l u P: acc [2][next][N], NTT domain; `accumulate` adds to what acc holds.  With x0, the
 // first x0rows rows of acc's first half also receive s x0(sigma_g) (s null: x0(sigma_g)), the
 // automorphed c0 term of a rotation, in the same kernel.
-// For a batch of nb ciphertexts: D [nb][ndig][next][N], acc [nb][2][next][N], x0 / x1 of ciphertext t
+// For a batch of nb ciphertexts: acc [nb][2][next][N], x0 / x1 of ciphertext t
 // at + t xstr; the key is read once for the batch.
-void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const u64* D, int ndig, int level, u64 code, u64 g,
+void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int level, u64 code, u64 g,
                       u64* acc, bool accumulate, const u64* x0 = nullptr, int x0rows = 0, const u64* s = nullptr,
                       const u64* x1 = nullptr, int nb = 1, size_t xstr = 0) {
     auto it = keys.swk.find(code);
@@ -636,10 +657,10 @@ void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const u64* D, int ndig
     const size_t next = (size_t)level + 1 + c->np;
     kern::KsBatch bt;
     bt.nb = nb;
-    bt.dstr = (size_t)ndig * next * c->n;
+    bt.dstr = (size_t)D.ndig * next * c->n;
     bt.ostr = 2 * next * c->n;
     bt.xstr = xstr;
-    kern::ks_inner(c, D, ndig, (int)next, c->d_ext_ids[level], k.b.ptr, k.a.ptr, acc, acc + next * c->n, g,
+    kern::ks_inner(c, kern::Digits{D.D.ptr, D.x, D.xstride, level + 1, c->alpha}, D.ndig, (int)next, c->d_ext_ids[level], k.b.ptr, k.a.ptr, acc, acc + next * c->n, g,
                    accumulate, x0, x0rows, s, x1, bt);
 }
 
@@ -692,11 +713,11 @@ u64 galois_of_step(const ckks_ctx* c, long long r) {
 // P c0(sigma_g) added on the Q rows in the same kernel, then ModDown: ModDown(P x + k) = x +
 // ModDown(k) exactly (P x vanishes on the P rows), so this is automorph(c0) + ModDown(k) in
 // fewer passes.
-static ckks_ct switch_galois(const ckks_keys& keys, const ckks_ct& a, const u64* D, int ndig, u64 g) {
+static ckks_ct switch_galois(const ckks_keys& keys, const ckks_ct& a, const Raised& D, u64 g) {
     ckks_ctx* c = a.ctx;
     const int l = a.level, nl = l + 1;
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n, c->stream);
-    key_switch_inner(c, keys, D, ndig, l, g, g, acc.ptr, false, a.c0(), nl, c->d_pmod, nullptr,
+    key_switch_inner(c, keys, D, l, g, g, acc.ptr, false, a.c0(), nl, c->d_pmod, nullptr,
                      a.nb, a.cstride());
     ckks_ct o = new_ct(c, l, a.scale, a.nb);
     mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
@@ -707,17 +728,16 @@ std::vector<ckks_ct> rotate_hoisted(const ckks_keys& keys, const ckks_ct& a, con
     ckks_ctx* c = a.ctx;
     const int l = a.level;
     std::vector<ckks_ct> outs;
-    DevBuf D;
-    int ndig = 0;
+    Raised D;
     for (long long r : steps) {
         const u64 g = galois_of_step(c, r);
         if (g == 1) {
             outs.push_back(copy_ct(a));
             continue;
         }
-        if (!D.ptr) D = mod_up(c, a.c1(), l, &ndig, a.nb, a.cstride());
+        if (!D.x) D = mod_up(c, a.c1(), l, a.nb, a.cstride());
         c->ops["hrot"]++;
-        outs.push_back(switch_galois(keys, a, D.ptr, ndig, g));
+        outs.push_back(switch_galois(keys, a, D, g));
     }
     return outs;
 }
@@ -729,9 +749,8 @@ ckks_ct rotate(const ckks_keys& keys, const ckks_ct& a, long long r) {
 
 ckks_ct conjugate(const ckks_keys& keys, const ckks_ct& a) {
     ckks_ctx* c = a.ctx;
-    int ndig = 0;
-    DevBuf D = mod_up(c, a.c1(), a.level, &ndig, a.nb, a.cstride());
-    return switch_galois(keys, a, D.ptr, ndig, 2ULL * c->n - 1);
+    const Raised D = mod_up(c, a.c1(), a.level, a.nb, a.cstride());
+    return switch_galois(keys, a, D, 2ULL * c->n - 1);
 }
 
 // tensor product of a batch: d [nb][3][l+1][N] (d0, d1, d2 of each ciphertext)
@@ -751,12 +770,11 @@ ckks_ct mul_relin(const ckks_keys& keys, const ckks_ct& a, const ckks_ct& b) {
     const int l = a.level, nl = l + 1;
     const size_t n = c->n, ds = 3 * (size_t)nl * n;
     DevBuf d = tensor_batch(a, b);
-    int ndig = 0;
-    DevBuf D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, &ndig, a.nb, ds);
+    const Raised D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, a.nb, ds);
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel; then
     // ModDown (= (d0, d1) + ModDown(k), see switch_galois)
-    key_switch_inner(c, keys, D.ptr, ndig, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
+    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l, a.scale * b.scale, a.nb);
     mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
@@ -773,11 +791,10 @@ ckks_ct mul_relin_rescale(const ckks_keys& keys, const ckks_ct& a, const ckks_ct
     const int l = a.level, nl = l + 1;
     const size_t n = c->n, ds = 3 * (size_t)nl * n;
     DevBuf d = tensor_batch(a, b);                 // d0, d1, d2 of each ciphertext
-    int ndig = 0;
-    DevBuf D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, &ndig, a.nb, ds);
+    const Raised D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, a.nb, ds);
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel
-    key_switch_inner(c, keys, D.ptr, ndig, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
+    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l - 1, a.scale * b.scale / (double)c->q[l], a.nb);
     mod_down_rescale(c, acc.ptr, l, o.buf.ptr, twice, a.nb);
@@ -807,8 +824,7 @@ static std::vector<DevBuf> rotate_hoisted_ext(const ckks_keys& keys, const ckks_
     const int l = a.level, nl = l + 1;
     const size_t n = c->n, next = (size_t)nl + c->np;
     std::vector<DevBuf> outs;
-    DevBuf D;
-    int ndig = 0;
+    Raised D;
     for (long long r : steps) {
         const u64 g = galois_of_step(c, r);
         DevBuf o((size_t)a.nb * 2 * next * n, c->stream);      // [nb][2][next][N]
@@ -816,9 +832,9 @@ static std::vector<DevBuf> rotate_hoisted_ext(const ckks_keys& keys, const ckks_
             CUDA_CHECK(cudaMemsetAsync(o.ptr, 0, (size_t)a.nb * 2 * next * n * 8, c->stream));
             lift_p(c, a.buf.ptr, o.ptr, l, a.nb);
         } else {
-            if (!D.ptr) D = mod_up(c, a.c1(), l, &ndig, a.nb, a.cstride());
+            if (!D.x) D = mod_up(c, a.c1(), l, a.nb, a.cstride());
             c->ops["hrot"]++;
-            key_switch_inner(c, keys, D.ptr, ndig, l, g, g, o.ptr, false, a.c0(), nl, c->d_pmod, nullptr, a.nb,
+            key_switch_inner(c, keys, D, l, g, g, o.ptr, false, a.c0(), nl, c->d_pmod, nullptr, a.nb,
                              a.cstride());
         }
         outs.push_back(std::move(o));
@@ -884,15 +900,14 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         if ((int)used_b.size() <= kern::BsgsFused::MAXB && (int)gs.size() <= kern::BsgsFused::MAXG &&
             c->digits(l).size() <= 4) {
             // babies and inner sums in one kernel: the baby rotations are never stored
-            DevBuf D;
-            int ndig = 1;
+            Raised D;
             bool any_rot = false;
             for (long long r : steps) any_rot = any_rot || r != 0;
-            if (any_rot) D = mod_up(c, a.c1(), l, &ndig, nb, a.cstride());
+            if (any_rot) D = mod_up(c, a.c1(), l, nb, a.cstride());
             kern::BsgsFused T;
             T.nb = (int)used_b.size();
             T.ng = (int)gs.size();
-            T.ndig = ndig;
+            T.ndig = D.ndig;
             T.acc = 0;
             for (int i = 0; i < T.nb; ++i) {
                 if (steps[i] == 0) {
@@ -929,10 +944,10 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             }
             kern::KsBatch bt;
             bt.nb = nb;
-            bt.dstr = (size_t)ndig * next * n;
+            bt.dstr = (size_t)D.ndig * next * n;
             bt.xstr = a.cstride();
             bt.ostr = es;
-            kern::bsgs_fused(c, T, D.ptr, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
+            kern::bsgs_fused(c, T, kern::Digits{D.D.ptr, D.x, D.xstride, nl, c->alpha}, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
             continue;
         }
         std::vector<DevBuf> baby = rotate_hoisted_ext(keys, a, steps);
@@ -997,9 +1012,8 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             c->ops["hrot"]++;
             DevBuf c1q((size_t)nb * nl * n, c->stream);
             mod_down_poly(c, x + next * n, l, c1q.ptr, nb, es);
-            int ndig = 0;
-            DevBuf D = mod_up(c, c1q.ptr, l, &ndig, nb, (size_t)nl * n);
-            key_switch_inner(c, keys, D.ptr, ndig, l, gal, gal, sums[k].ptr, false, x, (int)next, nullptr, nullptr,
+            const Raised D = mod_up(c, c1q.ptr, l, nb, (size_t)nl * n);
+            key_switch_inner(c, keys, D, l, gal, gal, sums[k].ptr, false, x, (int)next, nullptr, nullptr,
                              nb, es);
         }
         for (int k = 0; k < nside; ++k) {
@@ -1040,10 +1054,9 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         c->ops["hrot"]++;
         DevBuf c1q((size_t)nb * nl * n, c->stream);
         mod_down_poly(c, x + next * n, l, c1q.ptr, nb, es);
-        int ndig = 0;
-        DevBuf D = mod_up(c, c1q.ptr, l, &ndig, nb, (size_t)nl * n);
+        const Raised D = mod_up(c, c1q.ptr, l, nb, (size_t)nl * n);
         if (!have_acc) acc = DevBuf(nb * es, c->stream);
-        key_switch_inner(c, keys, D.ptr, ndig, l, gal, gal, acc.ptr, have_acc, x, (int)next, nullptr, nullptr,
+        key_switch_inner(c, keys, D, l, gal, gal, acc.ptr, have_acc, x, (int)next, nullptr, nullptr,
                          nb, es);
         have_acc = true;
     }
@@ -1098,30 +1111,24 @@ static int poly_out_level(const ckks_ctx* c, int level, int depth) {
 // T_(k mod 2 ? 1 : 0), operands brought to a common level by level_down.
 struct ChebPowers {
     const ckks_keys* keys;
-    std::map<int, ckks_ct> T;
+    const ckks_ct* x;                 // T_1, the caller's
+    std::map<int, ckks_ct> T;         // T_2, ...
+    const ckks_ct& get(int k) const { return k == 1 ? *x : T.at(k); }
     std::map<std::pair<int, int>, ckks_ct> cache;
     const ckks_ct& at(int k, int lev) {
-        const ckks_ct& t = T.at(k);
+        const ckks_ct& t = get(k);
         if (t.level == lev) return t;
         auto key = std::make_pair(k, lev);
         auto it = cache.find(key);
         if (it == cache.end()) it = cache.emplace(key, level_down(t, lev)).first;
         return it->second;
     }
-    void need(int k) {
-        if (T.count(k)) return;
-        const int a = k / 2, b = k - k / 2;
-        need(a);
-        need(b);
-        if (a != b) need(b - a);
-        T[k] = product(k);
-    }
     // T_k from T_a, T_b (and T_(b-a)), which must exist
     ckks_ct product(int k) {
         const int a = k / 2, b = k - k / 2;
-        const int m = prod_level(T.at(a).ctx, std::min(T.at(a).level, T.at(b).level));
+        const int m = prod_level(get(a).ctx, std::min(get(a).level, get(b).level));
         ckks_ct t = mul_relin_rescale(*keys, at(a, m), at(b, m), true);     // 2 T_a T_b
-        return (a == b) ? add_const(t, -1.0) : sub(t, at(b - a, m - 1));
+        return (a == b) ? add_const(std::move(t), -1.0) : sub(t, at(b - a, m - 1));
     }
     // several T_k at once: the products taken at the same level run as one lockstep batch
     // (one relinearisation key read, every launch over all of them); same residues as product(k)
@@ -1129,7 +1136,7 @@ struct ChebPowers {
         std::map<int, std::vector<int>> by_level;
         for (int k : ks) {
             const int a = k / 2, b = k - k / 2;
-            by_level[prod_level(T.at(a).ctx, std::min(T.at(a).level, T.at(b).level))].push_back(k);
+            by_level[prod_level(get(a).ctx, std::min(get(a).level, get(b).level))].push_back(k);
         }
         for (auto& kv : by_level) {
             const int m = kv.first;
@@ -1147,14 +1154,14 @@ struct ChebPowers {
             for (size_t i = 0; i < g.size(); ++i) {
                 const int k = g[i], a = k / 2, b = k - k / 2;
                 ckks_ct t = take_ct(prod, (int)i);
-                T[k] = (a == b) ? add_const(t, -1.0) : sub(t, at(b - a, m - 1));
+                T[k] = (a == b) ? add_const(std::move(t), -1.0) : sub(t, at(b - a, m - 1));
             }
         }
     }
     // the level_downs product(k) reads, made ahead (so that products can run side by side)
     void warm(int k) {
         const int a = k / 2, b = k - k / 2;
-        const int m = prod_level(T.at(a).ctx, std::min(T.at(a).level, T.at(b).level));
+        const int m = prod_level(get(a).ctx, std::min(get(a).level, get(b).level));
         at(a, m);
         at(b, m);
         if (a != b) at(b - a, m - 1);
@@ -1173,7 +1180,7 @@ struct PolyVal {
 // leaves of one polynomial share it), multiplied by llround(c_k s_c), s_c = Delta_target
 // q_(target+1) / scale, summed and rescaled once.
 static PolyVal cheb_leaf(ChebPowers& pw, const std::vector<double>& c) {
-    ckks_ctx* ctx = pw.T.at(1).ctx;
+    ckks_ctx* ctx = pw.get(1).ctx;
     PolyVal out;
     std::vector<int> ks;
     for (int k = 1; k < (int)c.size(); ++k)
@@ -1184,7 +1191,7 @@ static PolyVal cheb_leaf(ChebPowers& pw, const std::vector<double>& c) {
         return out;
     }
     int lev = 1 << 30;
-    for (int k : ks) lev = std::min(lev, pw.T.at(k).level);
+    for (int k : ks) lev = std::min(lev, pw.get(k).level);
     const int target = lev - 1;
     CK_CHECK((int)ks.size() <= kern::LinComb::MAX, CKKS_EINVAL, "Chebyshev leaf with more than 16 terms");
     kern::LinComb L;
@@ -1200,12 +1207,12 @@ static PolyVal cheb_leaf(ChebPowers& pw, const std::vector<double>& c) {
         }
         ++L.n;
     }
-    const int nb = pw.T.at(1).nb;
+    const int nb = pw.get(1).nb;
     ckks_ct acc = new_ct(ctx, lev, 0.0, nb);
     kern::lincomb(ctx, L, acc.buf.ptr, 2 * (lev + 1) * nb, ctx->d_iota, lev + 1);
     acc = rescale(acc);
     acc.scale = ctx->delta[target];
-    out.ct = add_const(acc, c[0]);
+    out.ct = add_const(std::move(acc), c[0]);
     return out;
 }
 
@@ -1227,7 +1234,7 @@ ckks_ct cheb_eval(const ckks_keys& keys, const ckks_ct& x, const std::vector<dou
     for (int n = b; n <= d; n *= 2) giants.push_back(n);
     ChebPowers pw;
     pw.keys = &keys;
-    pw.T[1] = copy_ct(x);
+    pw.x = &x;
     // The leaves (pieces of degree < b) depend only on the baby steps T_1..T_(b-1): collect them
     // in the order the Chebyshev division below visits them.
     auto trim = [](std::vector<double>& c) {
@@ -1327,7 +1334,7 @@ ckks_ct cheb_eval(const ckks_keys& keys, const ckks_ct& x, const std::vector<dou
     for (const auto& c : leaves) {
         int lev = 1 << 30;
         for (int k = 1; k < (int)c.size(); ++k)
-            if (c[k] != 0.0) lev = std::min(lev, pw.T.at(k).level);
+            if (c[k] != 0.0) lev = std::min(lev, pw.get(k).level);
         for (int k = 1; k < (int)c.size(); ++k)
             if (c[k] != 0.0) pw.at(k, lev);
     }
@@ -1383,13 +1390,13 @@ ckks_ct cheb_eval(const ckks_keys& keys, const ckks_ct& x, const std::vector<dou
     for (auto& nd : nodes)
         if (nd.leaf >= 0) nd.val = std::move(leaf_vals[nd.leaf]);
     auto prod_lev = [&](const Node& nd) {
-        const ckks_ct& Tn = pw.T.at(nd.n);
+        const ckks_ct& Tn = pw.get(nd.n);
         return prod_level(Tn.ctx, std::min(nodes[nd.q].val.ct.level, Tn.level));
     };
     auto combine = [&](Node& nd) -> PolyVal {
         PolyVal& Q = nodes[nd.q].val;
         PolyVal& R = nodes[nd.r].val;
-        const ckks_ct& Tn = pw.T.at(nd.n);
+        const ckks_ct& Tn = pw.get(nd.n);
         ckks_ctx* ctx = Tn.ctx;
         ckks_ct prod;
         bool hp = false;
@@ -1403,18 +1410,20 @@ ckks_ct cheb_eval(const ckks_keys& keys, const ckks_ct& x, const std::vector<dou
             }
         } else {
             const int lev = prod_lev(nd);
-            prod = mul_relin_rescale(keys, level_down(Q.ct, lev), pw.at(nd.n, lev));
+            ckks_ct tmp;
+            prod = mul_relin_rescale(keys, at_level(Q.ct, lev, tmp), pw.at(nd.n, lev));
             hp = true;
         }
         PolyVal out;
         if (R.is_const) {
             if (!hp) return std::move(R);
-            out.ct = add_const(prod, R.cst);
+            out.ct = add_const(std::move(prod), R.cst);
             return out;
         }
         if (!hp) return std::move(R);
         const int lev = std::min(prod.level, R.ct.level);
-        out.ct = add(level_down(prod, lev), level_down(R.ct, lev));
+        ckks_ct t0, t1;
+        out.ct = add(at_level(prod, lev, t0), at_level(R.ct, lev, t1));
         return out;
     };
     for (int h = 1; h <= nodes[root].height; ++h) {
@@ -1452,7 +1461,7 @@ ckks_ct cheb_eval(const ckks_keys& keys, const ckks_ct& x, const std::vector<dou
     PolyVal res = std::move(nodes[root].val);
     CK_CHECK(!res.is_const, CKKS_EINVAL, "polynomial evaluates to a constant");
     CK_CHECK(res.ct.level >= want, CKKS_ELEVEL, "polynomial evaluation ended below its level budget");
-    return level_down(res.ct, want);
+    return level_down(std::move(res.ct), want);
 }
 
 // HActivation as a composite polynomial: y = s_k(...s_1(x)) by chained Chebyshev
@@ -1463,7 +1472,8 @@ ckks_ct eval_relu(const ckks_keys& keys, const ckks_ct& x, const std::vector<std
     for (size_t i = 1; i < stages.size(); ++i) y = cheb_eval(keys, y, stages[i]);
     const int lev = prod_level(x.ctx, y.level);
     CK_CHECK(lev >= 1, CKKS_ELEVEL, "not enough levels for the final product");
-    return mul_relin_rescale(keys, level_down(x, lev), level_down(y, lev));
+    ckks_ct tx, ty;
+    return mul_relin_rescale(keys, at_level(x, lev, tx), at_level(y, lev, ty));
 }
 
 // alpha x + beta: x times llround(alpha Delta_(l-1) q_l / scale), rescaled onto the canonical
@@ -1474,7 +1484,7 @@ ckks_ct affine(const ckks_ct& x, double alpha, double beta) {
     CK_CHECK(l >= 1, CKKS_ELEVEL, "not enough levels for the change of variable");
     ckks_ct y = rescale_mul(x, llround_away(alpha * (c->delta[l - 1] * (double)c->q[l]) / x.scale));
     y.scale = c->delta[l - 1];
-    return add_const(y, beta);
+    return add_const(std::move(y), beta);
 }
 
 // p(x) on [a, b]: y = (2x - a - b) / (b - a) (no level for [-1, 1]), a power-basis p re-expressed
@@ -1492,7 +1502,7 @@ ckks_ct eval_mod(const ckks_keys& keys, const ckks_ct& x, const std::vector<doub
     ckks_ct y = cheb_eval(keys, x, coeffs);
     for (int i = 0; i < r; ++i) {
         y = mul_relin_rescale(keys, y, y, true);     // 2 y^2
-        y = add_const(y, -1.0);
+        y = add_const(std::move(y), -1.0);
     }
     return y;
 }

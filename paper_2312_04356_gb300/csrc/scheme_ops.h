@@ -20,9 +20,8 @@ ckks_ct rescale_mul(const ckks_ct& a, long long k);
 ckks_ct mod_drop(const ckks_ct& a, int level);
 ckks_ct level_down(const ckks_ct& a, int level);
 ckks_ct mod_raise(const ckks_ct& a);
-// per digit, the polynomial x (NTT domain, [l+1][N]) raised to Q_l u P: [ndig][next][N]; for a
-// batch, nb polynomials at x + t xstride -> [nb][ndig][next][N]
-DevBuf mod_up(ckks_ctx* c, const u64* x, int level, int* ndig_out, int nb = 1, size_t xstride = 0);
+ckks_ct add_const(ckks_ct&& a, double cst);      // in place
+ckks_ct level_down(ckks_ct&& a, int level);      // no copy when a is at that level
 
 u64 galois_of_step(const ckks_ctx* c, long long r);
 std::vector<ckks_ct> rotate_hoisted(const ckks_keys& keys, const ckks_ct& a, const std::vector<long long>& steps);
