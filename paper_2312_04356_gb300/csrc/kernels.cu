@@ -113,14 +113,26 @@ inline dim3 ew_grid(int n, int nlimbs) {
 
 #define EW_LOOP(n) for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < (n); j += gridDim.x * blockDim.x)
 
-// words per thread of the elementwise kernels when every pointer is 16-byte aligned
+// words per thread of the elementwise kernels when every pointer is 16-byte aligned and a CTA's
+// words lie in one limb
 constexpr int EWV_VEC = 4;
 #define EWV_LAUNCH(K, vec, nl, ...)                                                          \
     do {                                                                                     \
-        if (vec)                                                                             \
+        if ((vec) && c->n >= EWV_VEC * EW_THREADS)                                           \
             klaunch(c, K<EWV_VEC>, ewv_grid(c->n, (nl), EWV_VEC), EW_THREADS, 0, __VA_ARGS__); \
         else                                                                                 \
             klaunch(c, K<1>, ewv_grid(c->n, (nl), 1), EW_THREADS, 0, __VA_ARGS__);        \
+    } while (0)
+// the same for kernels that reduce products
+#define EWV_LAUNCH_RED(K, V, vec, zdim, nl, ...)                                             \
+    do {                                                                                     \
+        const bool vec_ = (vec) && c->n >= (V) * EW_THREADS;                                 \
+        dim3 grid_ = ewv_grid(c->n, (nl), vec_ ? (V) : 1);                                   \
+        grid_.z = (zdim);                                                                    \
+        if (vec_ && c->fold) klaunch(c, K<V, true>, grid_, EW_THREADS, 0, __VA_ARGS__);      \
+        else if (vec_) klaunch(c, K<V, false>, grid_, EW_THREADS, 0, __VA_ARGS__);           \
+        else if (c->fold) klaunch(c, K<1, true>, grid_, EW_THREADS, 0, __VA_ARGS__);         \
+        else klaunch(c, K<1, false>, grid_, EW_THREADS, 0, __VA_ARGS__);                     \
     } while (0)
 
 // ----------------------------------------------------------- elementwise ----
@@ -167,12 +179,12 @@ __global__ void k_neg(const u64* a, u64* o, const DevPrime* P, const int* ids, i
 }
 // bmod > 0: b is broadcast, row limb % bmod of b multiplies row limb of a (one plaintext times
 // every polynomial of a batch of ciphertexts)
-template <int V>
+template <int V, bool FOLD>
 __global__ void k_mul(const u64* a, const u64* b, u64* o, const DevPrime* P, const int* ids, int lpp, int logn,
                       int bmod) {
     griddep_entry();
     const int limb = blockIdx.y;
-    const DevMod m = P[ids[limb % lpp]].m;
+    const Reducer<FOLD> red(P[ids[limb % lpp]]);
     const size_t off = (size_t)limb << logn;
     const size_t boff = (size_t)(bmod ? limb % bmod : limb) << logn;
     EWV_BEGIN(1 << logn)
@@ -180,18 +192,18 @@ __global__ void k_mul(const u64* a, const u64* b, u64* o, const DevPrime* P, con
     ldv<V>(a + off + j, x);
     ldv<V>(b + boff + j, y);
 #pragma unroll
-    for (int v = 0; v < V; ++v) x[v] = mul_mod(x[v], y[v], m);
+    for (int v = 0; v < V; ++v) x[v] = red.mul(x[v], y[v]);
     stv<V>(o + off + j, x);
 }
 // tensor product of two ciphertexts: d0 = a0 b0, d1 = a0 b1 + a1 b0 (d [2][nl][N]), d2 = a1 b1
 // (e [nl][N]); a, b [2][nl][N]; one pass over the nl limbs
 // blockIdx.z: ciphertext t of a batch, its operands at a + t abs, b + t abs, d + t dbs, e + t ebs
-template <int V>
+template <int V, bool FOLD>
 __global__ void k_tensor(const u64* a, const u64* b, u64* d, u64* e, const DevPrime* P, const int* ids, int nl,
                          int logn, size_t abs, size_t dbs, size_t ebs) {
     griddep_entry();
     const int limb = blockIdx.y;
-    const DevMod m = P[ids[limb]].m;
+    const Reducer<FOLD> red(P[ids[limb]]);
     const size_t off = (size_t)limb << logn, ps = (size_t)nl << logn;
     a += blockIdx.z * abs;
     b += blockIdx.z * abs;
@@ -205,19 +217,22 @@ __global__ void k_tensor(const u64* a, const u64* b, u64* d, u64* e, const DevPr
     ldv<V>(b + ps + off + j, b1);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        d0[v] = mul_mod(a0[v], b0[v], m);
-        d1[v] = add_mod(mul_mod(a0[v], b1[v], m), mul_mod(a1[v], b0[v], m), m.q);
-        d2[v] = mul_mod(a1[v], b1[v], m);
+        d0[v] = red.mul(a0[v], b0[v]);
+        u64 lo = 0, hi = 0;
+        mac128(lo, hi, a0[v], b1[v]);
+        mac128(lo, hi, a1[v], b0[v]);
+        d1[v] = red(hi, lo);
+        d2[v] = red.mul(a1[v], b1[v]);
     }
     stv<V>(d + off + j, d0);
     stv<V>(d + ps + off + j, d1);
     stv<V>(e + off + j, d2);
 }
-template <int V>
+template <int V, bool FOLD>
 __global__ void k_mul_acc(const u64* a, const u64* b, u64* o, const DevPrime* P, const int* ids, int lpp, int logn) {
     griddep_entry();
     const int limb = blockIdx.y;
-    const DevMod m = P[ids[limb % lpp]].m;
+    const Reducer<FOLD> red(P[ids[limb % lpp]]);
     const size_t off = (size_t)limb << logn;
     EWV_BEGIN(1 << logn)
     u64 x[V], y[V], z[V];
@@ -225,7 +240,7 @@ __global__ void k_mul_acc(const u64* a, const u64* b, u64* o, const DevPrime* P,
     ldv<V>(b + off + j, y);
     ldv<V>(o + off + j, z);
 #pragma unroll
-    for (int v = 0; v < V; ++v) z[v] = add_mod(z[v], mul_mod(x[v], y[v], m), m.q);
+    for (int v = 0; v < V; ++v) z[v] = add_mod(z[v], red.mul(x[v], y[v]), red.q);
     stv<V>(o + off + j, z);
 }
 template <int V>
@@ -626,30 +641,23 @@ void neg(const ckks_ctx* c, const u64* a, u64* o, int nl, const int* ids, int lp
 void mul(const ckks_ctx* c, const u64* a, const u64* b, u64* o, int nl, const int* ids, int lpp, int bmod) {
     if (nl <= 0) return;
     { KTimer kt_(c, "mul", (bmod ? 2.0 + (double)bmod / nl : 3.0) * (double)nl * c->n * 8.0);
-    EWV_LAUNCH(k_mul, al16(a) && al16(b) && al16(o), nl, a, b, o, c->d_primes, ids, lpp, c->logn, bmod);
+    EWV_LAUNCH_RED(k_mul, EWV_VEC, al16(a) && al16(b) && al16(o), 1, nl, a, b, o, c->d_primes, ids, lpp, c->logn, bmod);
     }
     LAUNCH_CHECK();
 }
 void tensor(const ckks_ctx* c, const u64* a, const u64* b, u64* d, u64* e, int nl, const int* ids, int nb,
             size_t ab_bstride, size_t d_bstride, size_t e_bstride) {
     if (nl <= 0 || nb <= 0) return;
-    const bool vec = al16(a) && al16(b) && al16(d) && al16(e);
-    dim3 grid = ewv_grid(c->n, nl, vec ? 2 : 1);
-    grid.z = nb;
     { KTimer kt_(c, "tensor", 7.0 * (double)nl * nb * c->n * 8.0);
-    if (vec)
-        klaunch(c, k_tensor<2>, grid, EW_THREADS, 0, a, b, d, e, c->d_primes, ids, nl, c->logn, ab_bstride, d_bstride,
-                e_bstride);
-    else
-        klaunch(c, k_tensor<1>, grid, EW_THREADS, 0, a, b, d, e, c->d_primes, ids, nl, c->logn, ab_bstride, d_bstride,
-                e_bstride);
+    EWV_LAUNCH_RED(k_tensor, 2, al16(a) && al16(b) && al16(d) && al16(e), nb, nl, a, b, d, e, c->d_primes, ids, nl,
+                   c->logn, ab_bstride, d_bstride, e_bstride);
     }
     LAUNCH_CHECK();
 }
 void mul_acc(const ckks_ctx* c, const u64* a, const u64* b, u64* o, int nl, const int* ids, int lpp) {
     if (nl <= 0) return;
     { KTimer kt_(c, "mul_acc", 4.0 * (double)nl * c->n * 8.0);
-    EWV_LAUNCH(k_mul_acc, al16(a) && al16(b) && al16(o), nl, a, b, o, c->d_primes, ids, lpp, c->logn);
+    EWV_LAUNCH_RED(k_mul_acc, EWV_VEC, al16(a) && al16(b) && al16(o), 1, nl, a, b, o, c->d_primes, ids, lpp, c->logn);
     }
     LAUNCH_CHECK();
 }
