@@ -50,6 +50,11 @@ void ntt_pair(u64 w, u64 q, bool fold, u64* out2) {
     }
 }
 
+void ntt_out_factor(u64 f, u64 w, u64 q, bool fold, u64* out4) {
+    ntt_pair(f, q, fold, out4);
+    ntt_pair(mulmod(f, w, q), q, fold, out4 + 2);
+}
+
 int ntt_tw_pos(int idx, int logn) {
     if (logn != 16 || idx < 2) return idx;
     int sg = 0;

@@ -41,7 +41,7 @@ struct DevPrime {
     // transform constants as the pairs of hostmath::ntt_pair
     const ulonglong2* tw;    // psi^rev(k), k < N   (forward, Cooley-Tukey)
     const ulonglong2* itw;   // psi^-rev(k)          (inverse, Gentleman-Sande)
-    ulonglong2 n_inv;
+    ulonglong2 n_inv, n_inv_w;   // N^{-1}, and times the last inverse stage's twiddle
     u64 im, im_p;            // psi^(N/2) and its Shoup companion
     u64 r64, r64p;           // 2^64 mod q and its Shoup companion (128-bit lazy sums)
     u64 inv64;               // floor(2^64 / q): Shoup companion of 1, reduces any 64-bit word
@@ -70,7 +70,7 @@ struct ConvTab {
     // p_m - (prod q_i mod p_m) [nout] followed by its Shoup companions [nout]
     u64* d_inv_q = nullptr;
     u64* d_corr = nullptr;
-    // N^{-1} qhat_i^{-1} mod q_i as pairs (hostmath::ntt_pair), [nin][2]: the factor an inverse NTT
+    // N^{-1} qhat_i^{-1} mod q_i as hostmath::ntt_out_factor gives it, [nin][4]: the factor an inverse NTT
     // ends with when its output feeds this conversion directly (prescaled inputs)
     u64* d_iscale = nullptr;
     // tensor-core form (kern::base_convert_jobs with ctx->conv_tc): the table split into 8-bit
@@ -124,6 +124,7 @@ struct ckks_ctx {
     bool mods_below_2_60 = false;    // every modulus < 2^60 (enables the split base conversion)
     bool fold = false;               // every modulus qualifies for fold.cuh
     std::vector<u64> q, p, psi;      // psi indexed by prime id
+    std::vector<u64> ipsi_half;      // psi^-(N/2) by prime id
     std::vector<u64> mod_of;         // modulus by prime id
     std::vector<double> delta;
     std::vector<DevMod> mods;        // by prime id
@@ -165,7 +166,7 @@ struct ckks_ctx {
     std::vector<int*> d_modup_off, d_modup_pid;
     std::vector<int> modup_nrows;
     // per level: for each of the l + 1 rows of a ModUp input, N^{-1} qhat^{-1} of its digit's
-    // conversion (pairs, [l+1][2]), the inverse NTT's final factor for prescaled inputs
+    // conversion ([l+1][4]), the inverse NTT's final factor for prescaled inputs
     std::vector<u64*> d_modup_iscale;
     std::map<std::pair<int, int>, std::unique_ptr<ConvTab>> modup_tabs;  // (level, digit)
     std::map<int, std::unique_ptr<ConvTab>> moddown_tabs;               // level
@@ -384,7 +385,7 @@ struct LinComb {
 };
 void lincomb(const ckks_ctx* c, const LinComb& t, u64* o, int nl, const int* ids, int lpp);
 void autotune_ntt(ckks_ctx* c, int reps);
-// (osc: per row r = k % lpp a Shoup pair (w, w') at osc[2r], osc[2r + 1] that replaces the final
+// (osc: per row r = k % lpp the four words of hostmath::ntt_out_factor at osc[4r] that replace the final
 // factor N^{-1}, e.g. N^{-1} qhat^{-1} for a base conversion that reads the output prescaled)
 void ntt_inverse(const ckks_ctx* c, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride = 0,
                  const u64* osc = nullptr);
@@ -512,6 +513,9 @@ u64 shoup(u64 w, u64 q);
 bool fold_consts(u64 q, FoldMod& f);
 // a transform constant w as the kernels take it: fold.cuh's packed digits, else w and its Shoup companion
 void ntt_pair(u64 w, u64 q, bool fold, u64* out2);
+// an inverse transform's final factor f as the kernels take it: the pairs of f and f w, w = psi^-(N/2) the
+// one twiddle of the last stage
+void ntt_out_factor(u64 f, u64 w, u64 q, bool fold, u64* out4);
 // position of twiddle idx (2^stage + group) in a prime's table: in order, but for N = 2^16 the last
 // four stages of each eight-stage pass are transposed within a sub-problem (ntt.cu)
 int ntt_tw_pos(int idx, int logn);

@@ -43,6 +43,8 @@ struct ArShoup {
         x = s;
     }
     __device__ __forceinline__ u64 sum_out(u64 v) const { return v; }
+    __device__ __forceinline__ u64 sum(u64 x, u64 y) const { return x + y; }          // below 4 q
+    __device__ __forceinline__ u64 diff(u64 x, u64 y) const { return x - y + q2; }
     __device__ __forceinline__ u64 scale(u64 v, ulonglong2 w) const { return mul_shoup(v, w.x, w.y, q); }
 };
 
@@ -60,9 +62,9 @@ struct ArFold {
     __device__ __forceinline__ u64 open(u64 v) const { return (u64)fold_word((int64_t)v, f); }
     template <int U>
     __device__ __forceinline__ void fwd(u64& x, u64& y, ulonglong2 w) const {
-        const u64 r = (u64)fold_mul((int64_t)y, w.x, w.y, f);
-        y = x - r;
-        x = x + r;
+        const u64 s = x + (u64)fold_mul((int64_t)y, w.x, w.y, f);
+        y = 2 * x - s;       // x - r; in this form both results land in place, without register moves
+        x = s;
     }
     __device__ __forceinline__ u64 canon(u64 v) const { return fold_canon((int64_t)v, q, f); }
     __device__ __forceinline__ void inv(u64& x, u64& y, ulonglong2 w) const {
@@ -71,9 +73,16 @@ struct ArFold {
         y = (u64)fold_mul((int64_t)d, w.x, w.y, f);
     }
     __device__ __forceinline__ u64 sum_out(u64 v) const { return (u64)fold_word((int64_t)v, f); }
+    __device__ __forceinline__ u64 sum(u64 x, u64 y) const { return x + y; }
+    __device__ __forceinline__ u64 diff(u64 x, u64 y) const { return x - y; }
     __device__ __forceinline__ u64 scale(u64 v, ulonglong2 w) const {
         return fold_canon(fold_mul((int64_t)v, w.x, w.y, f), q, f);
     }
+};
+
+// the inverse transform's final factor f and f times the last stage's twiddle
+struct OutFactor {
+    ulonglong2 f, fw;
 };
 
 // S stages on 16 register values, stage s pairing i with i + 2^(S-1-s); widx(s, i) is the twiddle
@@ -99,17 +108,24 @@ __device__ __forceinline__ void fwd_stages(u64 (&x)[16], const AR& ar, const ulo
     }
 }
 
-// the S stages in reverse order; LAST: a scaling follows, so the sums need not be folded
+// the S stages in reverse order.  LAST: the transform's last stage (one twiddle) carries the output
+// factor: sums are scaled by out.f, differences by out.fw = f w, and the results are canonical.
 template <bool LAST, int S, class AR, class F>
-__device__ __forceinline__ void inv_stages(u64 (&x)[16], const AR& ar, const ulonglong2* __restrict__ itw, F widx) {
+__device__ __forceinline__ void inv_stages(u64 (&x)[16], const AR& ar, const ulonglong2* __restrict__ itw, F widx,
+                                           const OutFactor& out = OutFactor{}) {
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         const int is = 1 << j;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             if (i & is) continue;
-            const ulonglong2 w = __ldg(itw + widx(S - 1 - j, i));
-            ar.inv(x[i], x[i + is], w);
+            if (LAST && j == S - 1) {
+                const u64 s = ar.sum(x[i], x[i + is]), d = ar.diff(x[i], x[i + is]);
+                x[i] = ar.scale(s, out.f);
+                x[i + is] = ar.scale(d, out.fw);
+            } else {
+                ar.inv(x[i], x[i + is], __ldg(itw + widx(S - 1 - j, i)));
+            }
         }
         if (j == S - 1 ? !LAST : j == 1 && ar.folds()) {
 #pragma unroll
@@ -122,8 +138,8 @@ __device__ __forceinline__ void inv_stages(u64 (&x)[16], const AR& ar, const ulo
 // What a transform reads or writes besides the data array (X kernels).
 // Inverse, first pass: row k reads src + (k / lpp) * src_pstride + (k % lpp) N and the result goes to the
 // data array, so the input is left as it is (no copy before an out-of-place transform); scaled
-// replaces the final factor N^{-1} by the pair w, e.g. k N^{-1} to multiply the result by the
-// integer k.
+// replaces the final factor N^{-1} by w (w2: times the last twiddle), e.g. k N^{-1} to multiply the
+// result by the integer k.
 // Forward, first pass: every row of polynomial p is the centred lift of the one row
 // src + p * src_pstride with modulus lift_q (a signed word is what the lazy butterflies take; one
 // fold brings a wider source prime's word into range).
@@ -131,7 +147,7 @@ struct NttSrc {
     const u64* src;
     size_t src_pstride;
     bool scaled;
-    ulonglong2 w;
+    ulonglong2 w, w2;
     u64 lift_q;
 };
 // Forward, last pass: row k receives (a - x) s, or a ks - x s when has_k, instead of the transform x; row k
@@ -168,10 +184,12 @@ __device__ __forceinline__ u64 tail_word(u64 a, u64 x, const NttTailArgs& tl, ul
     }
     return fold_canon(fold_mul((int64_t)(a - x), s.x, s.y, f), q, f);
 }
-// the inverse transform's final factor of row r
-__device__ __forceinline__ ulonglong2 out_factor(const DevPrime* P, const u64* osc, int r, const NttSrc& io) {
-    if (io.scaled) return io.w;
-    return osc ? make_ulonglong2(osc[2 * r], osc[2 * r + 1]) : P->n_inv;
+// the inverse transform's final factor of row r (osc: [rows][f, f w])
+__device__ __forceinline__ OutFactor out_factor(const DevPrime* P, const u64* osc, int r, const NttSrc& io) {
+    if (io.scaled) return OutFactor{io.w, io.w2};
+    if (!osc) return OutFactor{P->n_inv, P->n_inv_w};
+    const ulonglong2* o = reinterpret_cast<const ulonglong2*>(osc) + 2 * r;
+    return OutFactor{o[0], o[1]};
 }
 
 // ---- any ring: c consecutive stages from s0 in shared memory, one barrier per stage.  Only index
@@ -246,7 +264,7 @@ __global__ void __launch_bounds__(NTT_THREADS)
     }
 
     // the inverse transform's final factor: N^{-1}, or per row a caller-given pair
-    const ulonglong2 ni = out_factor(P, osc, limb % lpp, NttSrc{});
+    const ulonglong2 ni = out_factor(P, osc, limb % lpp, NttSrc{}).f;
     for (int e = threadIdx.x; e < total; e += blockDim.x) {
         int s, k;
         if (T1 == 1) {
@@ -344,7 +362,7 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
         for (int rr = NR - 1; rr >= 0; --rr) {
             const int p = rr < NR - 1 ? LOGN - 4 - 4 * rr : 0, s0 = 4 * rr;
             auto widx = [&](int s, int i) { return (1 << (s0 + s)) + (sk<LOGN>(t, i, p) >> (LOGN - s0 - s)); };
-            if (rr == 0) inv_stages<true, 4>(x, ar, P->itw, widx);
+            if (rr == 0) inv_stages<true, 4>(x, ar, P->itw, widx, out_factor(P, osc, r, io));
             else if (rr < NR - 1) inv_stages<false, 4>(x, ar, P->itw, widx);
             else inv_stages<false, LAST>(x, ar, P->itw, widx);
             if (rr > 0) {
@@ -357,9 +375,8 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
                 for (int i = 0; i < 16; ++i) x[i] = sm[spad(sk<LOGN>(t, i, pn))];
             }
         }
-        const ulonglong2 ni = out_factor(P, osc, r, io);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) a[sk<LOGN>(t, i, LOGN - 4)] = ar.scale(x[i], ni);
+        for (int i = 0; i < 16; ++i) a[sk<LOGN>(t, i, LOGN - 4)] = x[i];
     }
 }
 
@@ -389,12 +406,12 @@ __device__ __forceinline__ void fwd_round(u64 (&x)[16], int t, int hi, int s0, c
 }
 template <bool ROUND_B, bool LAST, class AR>
 __device__ __forceinline__ void inv_round(u64 (&x)[16], int t, int hi, int s0, const ulonglong2* __restrict__ itw,
-                                          const AR& ar) {
+                                          const AR& ar, const OutFactor& out = OutFactor{}) {
     inv_stages<LAST, 4>(x, ar, itw, [&](int s, int i) {
         const int u = (ROUND_B ? 4 : 0) + s;
         const int base = (1 << (s0 + u)) + (hi << u);
         return ROUND_B ? base + t + 16 * (i >> (4 - s)) : base + (i >> (4 - s));
-    });
+    }, out);
 }
 
 // COL: sub-problems are columns (s0 = 0, T1 = 256, element j = k*256 + lo), threads with
@@ -484,15 +501,10 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 16; ++i) x[i] = sm[f_slot<SUBS>(sp, t + 16 * i)];
-        inv_round<false, COL>(x, t, hi, s0, P->itw, ar);
-        if constexpr (COL && INV) {
-            const ulonglong2 ni = out_factor(P, osc, r, io);
+        if constexpr (COL && INV) inv_round<false, true>(x, t, hi, s0, P->itw, ar, out_factor(P, osc, r, io));
+        else inv_round<false, false>(x, t, hi, s0, P->itw, ar);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = ar.scale(x[i], ni);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = x[i];     // lazy
-        }
+        for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = x[i];     // canonical (COL), lazy (ROW)
     }
 }
 
@@ -594,13 +606,19 @@ __global__ void __launch_bounds__(256) k_ntt16s(u64* __restrict__ data, const De
                 ar.inv(x[0], x[1], w0);
                 ar.inv(x[2], x[3], w1);
             }
-            // stage u: pairs (0, 2), (1, 3)
-            {
+            // stage u: pairs (0, 2), (1, 3); the transform's last carries the output factor
+            if (rr == 0 && COL) {
+                const OutFactor out = out_factor(P, osc, r, io);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const u64 s = ar.sum(x[i], x[i + 2]), d = ar.diff(x[i], x[i + 2]);
+                    x[i] = ar.scale(s, out.f);
+                    x[i + 2] = ar.scale(d, out.fw);
+                }
+            } else {
                 const ulonglong2 w = __ldg(P->itw + (1 << (s0 + u)) + (hi << u) + tw_pos(u, k0 >> (8 - u)));
                 ar.inv(x[0], x[2], w);
                 ar.inv(x[1], x[3], w);
-            }
-            if (rr > 0 || !COL) {
                 x[0] = ar.sum_out(x[0]);
                 x[1] = ar.sum_out(x[1]);
             }
@@ -608,13 +626,9 @@ __global__ void __launch_bounds__(256) k_ntt16s(u64* __restrict__ data, const De
                 __syncthreads();
 #pragma unroll
                 for (int i = 0; i < 4; ++i) sm[f_slot<4>(sp, ks[i])] = x[i];
-            } else if (COL) {
-                const ulonglong2 ni = out_factor(P, osc, r, io);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[gidx(ks[i])] = ar.scale(x[i], ni);
             } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) a[gidx(ks[i])] = x[i];     // lazy
+                for (int i = 0; i < 4; ++i) a[gidx(ks[i])] = x[i];     // canonical (COL), lazy (ROW)
             }
         }
     }
@@ -715,10 +729,9 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(CL_THREADS, 2)
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 16; ++i) x[i] = sm[f_slot<CL_SUBS>(spc, tc + 16 * i)];
-        inv_round<false, true>(x, tc, 0, 0, P->itw, ar);
-        const ulonglong2 ni = out_factor(P, osc, r, io);
+        inv_round<false, true>(x, tc, 0, 0, P->itw, ar, out_factor(P, osc, r, io));
 #pragma unroll
-        for (int i = 0; i < 16; ++i) a[((size_t)(tc + 16 * i) << 8) + col] = ar.scale(x[i], ni);
+        for (int i = 0; i < 16; ++i) a[((size_t)(tc + 16 * i) << 8) + col] = x[i];
     }
 }
 
@@ -1036,12 +1049,14 @@ void ntt_inverse_from(const ckks_ctx* c, const u64* src, size_t src_pstride, u64
     CK_CHECK(!scaled || (lpp == 1 && osc == nullptr && pstride == c->n), CKKS_EINVAL,
              "an integer factor needs one contiguous row per polynomial and no output scale table");
     if (c->logn == 16 || ntt_one_cta(c)) {
-        NttSrc io{src, src_pstride, scaled, {}, 0};
+        NttSrc io{src, src_pstride, scaled, {}, {}, 0};
         if (scaled) {
             const u64 q = c->mod_of[k_id];
-            u64 w[2];
-            hostmath::ntt_pair(hostmath::mulmod(kres, hostmath::invmod((u64)c->n % q, q), q), q, c->fold, w);
+            u64 w[4];
+            hostmath::ntt_out_factor(hostmath::mulmod(kres, hostmath::invmod((u64)c->n % q, q), q), c->ipsi_half[k_id], q,
+                                     c->fold, w);
             io.w = make_ulonglong2(w[0], w[1]);
+            io.w2 = make_ulonglong2(w[2], w[3]);
         }
         if (c->logn == 16) launch_ntt_transform<true>(c, data, nlimbs, ids, lpp, pstride, nullptr, osc, io);
         else launch_ntt_one<true>(c, data, nlimbs, ids, lpp, pstride, osc, io);

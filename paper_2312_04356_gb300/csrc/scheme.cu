@@ -101,10 +101,10 @@ static std::unique_ptr<ConvTab> make_conv_tab(ckks_ctx* c, const std::vector<int
         }
     }
     // N^{-1} qhat_i^{-1}: the inverse NTT that produces this conversion's inputs ends with it
-    std::vector<u64> isc(2 * t->nin);
+    std::vector<u64> isc(4 * t->nin);
     for (int i = 0; i < t->nin; ++i) {
         const u64 qi = c->mod_of[in_ids[i]];
-        ntt_pair(mulmod(invmod((u64)c->n % qi, qi), qinv[i], qi), qi, c->fold, &isc[2 * i]);
+        ntt_out_factor(mulmod(invmod((u64)c->n % qi, qi), qinv[i], qi), c->ipsi_half[in_ids[i]], qi, c->fold, &isc[4 * i]);
     }
     t->d_iscale = dev_upload_persistent(isc);
     std::vector<int> ids_rows = out_ids;
@@ -305,9 +305,11 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
         const u64* dbase = c->d_tables + (size_t)id * 4 * n;
         dp.tw = reinterpret_cast<const ulonglong2*>(dbase);
         dp.itw = reinterpret_cast<const ulonglong2*>(dbase + 2 * n);
-        u64 ni[2];
-        ntt_pair(invmod((u64)n % qq, qq), qq, c->fold, ni);
+        c->ipsi_half.push_back(ipw[n / 2]);
+        u64 ni[4];
+        ntt_out_factor(invmod((u64)n % qq, qq), ipw[n / 2], qq, c->fold, ni);
         dp.n_inv = make_ulonglong2(ni[0], ni[1]);
+        dp.n_inv_w = make_ulonglong2(ni[2], ni[3]);
         dp.im = pw[n / 2];
         dp.im_p = shoup(dp.im, qq);
         dp.r64 = (u64)(((unsigned __int128)1 << 64) % qq);
@@ -389,7 +391,7 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
         // digit's N^{-1} qhat^{-1}
         std::vector<u64> isc;
         for (int d = 0; d < (int)dig.size(); ++d) {
-            std::vector<u64> h(2 * dig[d].size());
+            std::vector<u64> h(4 * dig[d].size());
             CUDA_CHECK(cudaMemcpy(h.data(), c->modup_tab(l, d).d_iscale, h.size() * 8, cudaMemcpyDeviceToHost));
             isc.insert(isc.end(), h.begin(), h.end());
         }
