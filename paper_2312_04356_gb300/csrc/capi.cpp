@@ -75,48 +75,7 @@ void encode_complex(ckks_ctx* c, const std::vector<cplx>& z, int level, double s
     CK_CHECK(level >= 0 && level <= c->L, CKKS_EINVAL, "level out of range");
     std::vector<cplx> zz(z);
     zz.resize(c->n / 2, cplx(0, 0));
-    upload_coeffs(c, round_coeffs(fp64::encode_slots(zz, c->n), scale), level, scale, out, ext);
-}
-
-// limbs (host, coefficient domain, [nl][N]) -> centred values / scale, by Garner's mixed radix
-std::vector<double> crt_centred(const ckks_ctx* c, const std::vector<u64>& limbs, int nl) {
-    const size_t n = c->n;
-    std::vector<double> out(n);
-    // inverse of prod_{k<i} q_k mod q_i
-    std::vector<u64> pinv(nl);
-    for (int i = 0; i < nl; ++i) {
-        u64 pr = 1;
-        for (int k = 0; k < i; ++k) pr = mulmod(pr, c->q[k] % c->q[i], c->q[i]);
-        pinv[i] = i ? invmod(pr, c->q[i]) : 1;
-    }
-    std::vector<u64> v(nl);
-    for (size_t j = 0; j < n; ++j) {
-        bool neg = false;
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int i = 0; i < nl; ++i) {
-                u64 qi = c->q[i];
-                u64 r = limbs[(size_t)i * n + j];
-                if (neg) r = r ? qi - r : 0;
-                // v_i = (r - sum_{t<i} v_t prod_{k<t} q_k) * (prod_{k<i} q_k)^{-1} mod q_i
-                u64 acc = 0, pr = 1;
-                for (int t = 0; t < i; ++t) {
-                    acc = (acc + mulmod(v[t] % qi, pr, qi)) % qi;
-                    pr = mulmod(pr, c->q[t] % qi, qi);
-                }
-                u64 diff = r >= acc ? r - acc : r + qi - acc;
-                v[i] = mulmod(diff, pinv[i], qi);
-            }
-            if (pass == 0 && v[nl - 1] > (c->q[nl - 1] - 1) / 2) {
-                neg = true;
-                continue;
-            }
-            break;
-        }
-        double x = 0.0;
-        for (int i = nl - 1; i >= 0; --i) x = x * (double)c->q[i] + (double)v[i];
-        out[j] = neg ? -x : x;
-    }
-    return out;
+    upload_coeffs(c, round_coeffs(fp64::encode_slots(zz, c->n, &c->roots), scale), level, scale, out, ext);
 }
 
 std::vector<u64> download(ckks_ctx* c, const u64* dev, size_t words) {
@@ -124,6 +83,21 @@ std::vector<u64> download(ckks_ctx* c, const u64* dev, size_t words) {
     CUDA_CHECK(cudaMemcpyAsync(h.data(), dev, words * 8, cudaMemcpyDeviceToHost, c->stream));
     CUDA_CHECK(cudaStreamSynchronize(c->stream));
     return h;
+}
+
+// the plaintext's centred coefficients divided by its scale (exact CRT on the device)
+std::vector<double> decoded_coeffs(ckks_ctx* c, const ckks_pt* pt) {
+    CK_CHECK(pt->level >= 0, CKKS_EINVAL, "empty plaintext");
+    const int nl = pt->level + 1;
+    const size_t n = c->n;
+    DevBuf t((size_t)nl * n, c->stream), x(n, c->stream);
+    kern::ntt_inverse_from(c, pt->buf.ptr, (size_t)nl * n, t.ptr, nl, c->d_iota, nl, 0, nullptr);
+    kern::garner(c, t.ptr, reinterpret_cast<double*>(x.ptr), nl);
+    std::vector<double> f(n);
+    CUDA_CHECK(cudaMemcpyAsync(f.data(), x.ptr, n * 8, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_CHECK(cudaStreamSynchronize(c->stream));
+    for (double& v : f) v /= pt->scale;
+    return f;
 }
 
 ckks_ptset* make_plan(ckks_ctx* c, const fp64::Diag& D, int a0, int step, int count, int level, double scale,
@@ -549,7 +523,7 @@ int ckks_encode(ckks_ctx* ctx, const double* re, const double* im, int n, int le
             CK_CHECK(n >= 0 && n <= N, CKKS_EINVAL, "too many values");
             std::vector<double> m(N, 0.0);
             for (int j = 0; j < n; ++j) m[j] = re[j];
-            encode_complex(ctx, fp64::real_cins_slots(m.data(), C, slice_len), level, scale, out);
+            encode_complex(ctx, fp64::real_cins_slots(m.data(), C, slice_len, &ctx->roots), level, scale, out);
         } else {
             CK_THROW(CKKS_EINVAL, "unknown encoding kind");
         }
@@ -562,19 +536,13 @@ int ckks_decode(ckks_ctx* ctx, const ckks_pt* pt, int kind, int slice_len, doubl
         REQ(pt);
         REQ(re);
         const int N = ctx->n;
-        const int nl = pt->level + 1;
-        DevBuf t((size_t)nl * N, ctx->stream);
-        CUDA_CHECK(cudaMemcpyAsync(t.ptr, pt->buf.ptr, (size_t)nl * N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        kern::ntt_inverse(ctx, t.ptr, nl, ctx->d_iota, nl);
-        std::vector<u64> h = download(ctx, t.ptr, (size_t)nl * N);
-        std::vector<double> f = crt_centred(ctx, h, nl);
-        for (double& x : f) x /= pt->scale;
+        std::vector<double> f = decoded_coeffs(ctx, pt);
         if (kind == CKKS_COEFF) {
             CK_CHECK(n <= N, CKKS_EINVAL, "n above N");
             for (int j = 0; j < n; ++j) re[j] = f[j];
         } else if (kind == CKKS_SLOT) {
             CK_CHECK(n <= N / 2, CKKS_EINVAL, "n above N/2");
-            std::vector<cplx> z = fp64::decode_slots(f, N);
+            std::vector<cplx> z = fp64::decode_slots(f, N, &ctx->roots);
             for (int j = 0; j < n; ++j) {
                 re[j] = z[j].real();
                 if (im) im[j] = z[j].imag();
@@ -582,7 +550,7 @@ int ckks_decode(ckks_ctx* ctx, const ckks_pt* pt, int kind, int slice_len, doubl
         } else if (kind == CKKS_CINS_REAL) {
             CK_CHECK(slice_len >= 2 && (slice_len & (slice_len - 1)) == 0 && slice_len <= N, CKKS_EINVAL,
                      "bad slice_len");
-            std::vector<double> m = fp64::cins_to_reals(fp64::decode_slots(f, N), N / slice_len, slice_len);
+            std::vector<double> m = fp64::cins_to_reals(fp64::decode_slots(f, N, &ctx->roots), N / slice_len, slice_len, &ctx->roots);
             for (int j = 0; j < n && j < N; ++j) re[j] = m[j];
         } else {
             CK_THROW(CKKS_EINVAL, "unknown encoding kind");
@@ -605,7 +573,7 @@ int ckks_encode_image(ckks_ctx* ctx, const double* img, int c, int w0, int w, in
             for (int r = 0; r < w0; ++r)
                 for (int col = 0; col < w0; ++col)
                     m[(size_t)i * two_l + r * w + col] = img[((size_t)i * w0 + r) * w0 + col];
-        encode_complex(ctx, fp64::real_cins_slots(m.data(), C, two_l), level, scale, out);
+        encode_complex(ctx, fp64::real_cins_slots(m.data(), C, two_l, &ctx->roots), level, scale, out);
     });
 }
 
@@ -618,16 +586,11 @@ int ckks_decode_image(ckks_ctx* ctx, const ckks_pt* pt, int from_coeff, int c, i
         CK_CHECK(w >= 2 && (w & (w - 1)) == 0 && w * w <= N && w0 >= 1 && w0 <= w, CKKS_EINVAL, "bad w / w0");
         const int two_l = w * w, C = N / two_l;
         CK_CHECK(c >= 1 && c <= C, CKKS_EINVAL, "channels do not fit in one ciphertext");
-        const int nl = pt->level + 1;
-        DevBuf t((size_t)nl * N, ctx->stream);
-        CUDA_CHECK(cudaMemcpyAsync(t.ptr, pt->buf.ptr, (size_t)nl * N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        kern::ntt_inverse(ctx, t.ptr, nl, ctx->d_iota, nl);
-        std::vector<double> f = crt_centred(ctx, download(ctx, t.ptr, (size_t)nl * N), nl);
-        for (double& x : f) x /= pt->scale;
+        std::vector<double> f = decoded_coeffs(ctx, pt);
         int cbits = 0;
         while ((1 << cbits) < C) ++cbits;
         std::vector<double> m;
-        if (!from_coeff) m = fp64::cins_to_reals(fp64::decode_slots(f, N), C, two_l);
+        if (!from_coeff) m = fp64::cins_to_reals(fp64::decode_slots(f, N, &ctx->roots), C, two_l, &ctx->roots);
         for (int i = 0; i < c; ++i) {
             unsigned rv = 0, x = (unsigned)i;
             for (int b = 0; b < cbits; ++b) {

@@ -26,8 +26,23 @@ static cplx root_of_unity(long long e, long long m) {
     return cplx(cos(th), sin(th));
 }
 
+std::vector<cplx> roots_2n(int n) {
+    std::vector<cplx> r(2 * (size_t)n);
+    for (size_t e = 0; e < r.size(); ++e) r[e] = root_of_unity((long long)e, 2LL * n);
+    return r;
+}
+
+// exp(2 pi i e / m): looked up when a table is given and covers m (the angle 2 pi e / m has the same bits
+// when e and m carry a common power of two, so the entry equals the direct value)
+static inline cplx root_at(const std::vector<cplx>* R, long long e, long long m) {
+    if (!R || (long long)R->size() < m) return root_of_unity(e, m);
+    e %= m;
+    if (e < 0) e += m;
+    return (*R)[(size_t)(e * ((long long)R->size() / m))];
+}
+
 // in-place iterative radix-2 FFT; sign -1: sum_k a_k e^{-2 pi i jk/n}, sign +1: e^{+...}
-static void fft(std::vector<cplx>& a, int sign) {
+static void fft(std::vector<cplx>& a, int sign, const std::vector<cplx>* R) {
     const int n = (int)a.size();
     for (int i = 1, j = 0; i < n; ++i) {
         int bit = n >> 1;
@@ -37,7 +52,7 @@ static void fft(std::vector<cplx>& a, int sign) {
     }
     for (int len = 2; len <= n; len <<= 1) {
         std::vector<cplx> w(len / 2);
-        for (int k = 0; k < len / 2; ++k) w[k] = root_of_unity(sign * (long long)k, len);
+        for (int k = 0; k < len / 2; ++k) w[k] = root_at(R, sign * (long long)k, len);
         for (int i = 0; i < n; i += len)
             for (int k = 0; k < len / 2; ++k) {
                 cplx u = a[i + k], v = a[i + k + len / 2] * w[k];
@@ -64,18 +79,18 @@ static inline int odd_index(long long e, int n) {
     return (int)((e - 1) / 2);
 }
 
-std::vector<cplx> decode_slots(const std::vector<double>& f, int n) {
+std::vector<cplx> decode_slots(const std::vector<double>& f, int n, const std::vector<cplx>* R) {
     // y_m = f(zeta^(2m+1)) = sum_k (f_k zeta^k) e^{2 pi i m k / N}
     std::vector<cplx> g(n);
-    for (int k = 0; k < n; ++k) g[k] = f[k] * root_of_unity(k, 2LL * n);
-    fft(g, +1);
+    for (int k = 0; k < n; ++k) g[k] = f[k] * root_at(R, k, 2LL * n);
+    fft(g, +1, R);
     std::vector<long long> rg = rot_group(n);
     std::vector<cplx> z(n / 2);
     for (int j = 0; j < n / 2; ++j) z[j] = g[odd_index(rg[j], n)];
     return z;
 }
 
-std::vector<double> encode_slots(const std::vector<cplx>& z, int n) {
+std::vector<double> encode_slots(const std::vector<cplx>& z, int n, const std::vector<cplx>* R) {
     // values at zeta^(5^j) are z_j, at zeta^(-5^j) their conjugates; invert the evaluation
     std::vector<cplx> y(n, cplx(0, 0));
     std::vector<long long> rg = rot_group(n);
@@ -83,9 +98,9 @@ std::vector<double> encode_slots(const std::vector<cplx>& z, int n) {
         y[odd_index(rg[j], n)] = z[j];
         y[odd_index(-rg[j], n)] = std::conj(z[j]);
     }
-    fft(y, -1);
+    fft(y, -1, R);
     std::vector<double> f(n);
-    for (int k = 0; k < n; ++k) f[k] = (y[k] / (double)n * root_of_unity(-(long long)k, 2LL * n)).real();
+    for (int k = 0; k < n; ++k) f[k] = (y[k] / (double)n * root_at(R, -(long long)k, 2LL * n)).real();
     return f;
 }
 
@@ -211,23 +226,23 @@ int boot_bsgs_B(int count) {
 }
 
 // --------------------------------------------------------------- CinS ------
-std::vector<cplx> real_cins_slots(const double* m, int C, int two_l) {
+std::vector<cplx> real_cins_slots(const double* m, int C, int two_l, const std::vector<cplx>* R) {
     const int ell = two_l / 2;
     std::vector<cplx> z((size_t)C * ell);
     for (int i = 0; i < C; ++i) {
         std::vector<double> sl(m + (size_t)i * two_l, m + (size_t)(i + 1) * two_l);
-        std::vector<cplx> d = decode_slots(sl, two_l);   // DFT'_{2l}: the subring's embedding
+        std::vector<cplx> d = decode_slots(sl, two_l, R);   // DFT'_{2l}: the subring's embedding
         std::copy(d.begin(), d.end(), z.begin() + (size_t)i * ell);
     }
     return z;
 }
 
-std::vector<double> cins_to_reals(const std::vector<cplx>& z, int C, int two_l) {
+std::vector<double> cins_to_reals(const std::vector<cplx>& z, int C, int two_l, const std::vector<cplx>* R) {
     const int ell = two_l / 2;
     std::vector<double> out((size_t)C * two_l);
     for (int i = 0; i < C; ++i) {
         std::vector<cplx> sl(z.begin() + (size_t)i * ell, z.begin() + (size_t)(i + 1) * ell);
-        std::vector<double> f = encode_slots(sl, two_l);
+        std::vector<double> f = encode_slots(sl, two_l, R);
         std::copy(f.begin(), f.end(), out.begin() + (size_t)i * two_l);
     }
     return out;

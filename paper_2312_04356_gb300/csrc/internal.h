@@ -149,6 +149,8 @@ struct ckks_ctx {
     // allocator (PyTorch's) reuses a freed block on the stream it was allocated on, so every
     // buffer must be used on that one stream
     bool use_side_streams() const { return side_streams_on && alloc.alloc == nullptr; }
+    std::vector<cplx> roots;                 // fp64::roots_2n(N): the client side's FFT twiddles
+    u64* d_garner = nullptr;                 // kern::garner's table [nq][nq] of Shoup pairs
     DevPrime* d_primes = nullptr;
     u64* d_tables = nullptr;
     u64* d_gauss = nullptr;
@@ -434,6 +436,9 @@ void lift_centred(const ckks_ctx* c, const u64* src, int src_id, u64* o, int nli
 // a_pstride, row k of a is at a + (k / lpp) * a_pstride + (k % lpp) * N (b and out contiguous)
 void sub_mul_scalar(const ckks_ctx* c, const u64* a, const u64* b, const u64* s, const u64* sp, u64* o,
                     int nlimbs, const int* ids, int lpp, size_t a_pstride = 0);
+// exact CRT of nl coefficient-domain limbs (q_0 .. q_{nl-1}, overwritten): out[j] = the centred value in
+// FP64, from its mixed-radix digits (Garner)
+void garner(const ckks_ctx* c, u64* limbs, double* out, int nl);
 // fast base conversion, coefficient domain: in [nin][N] (limb stride in_stride words),
 // out rows written at out + out_row[m]*N
 // (prescaled: the inputs already carry the factor qhat_i^{-1}, see ConvTab::d_iscale)
@@ -535,8 +540,10 @@ void gauss_table(double sigma, u64* t39);
 
 // FP64 encoding and plan construction (fp64.cpp)
 namespace fp64 {
-std::vector<double> encode_slots(const std::vector<cplx>& z, int n);       // -> N real coeffs
-std::vector<cplx> decode_slots(const std::vector<double>& f, int n);       // -> N/2 slots
+// R (optional): roots_2n of a ring at least as large, in place of a sine and cosine per twiddle
+std::vector<cplx> roots_2n(int n);                                         // exp(2 pi i e / 2N), e < 2N
+std::vector<double> encode_slots(const std::vector<cplx>& z, int n, const std::vector<cplx>* R = nullptr);   // -> N real coeffs
+std::vector<cplx> decode_slots(const std::vector<double>& f, int n, const std::vector<cplx>* R = nullptr);   // -> N/2 slots
 typedef std::map<int, std::vector<cplx>> Diag;                            // offset -> vector
 Diag s_product(const std::vector<int>& strides, int m, bool inverse);
 std::vector<std::vector<int>> split_groups(const std::vector<int>& stages, int levels);
@@ -546,8 +553,8 @@ std::vector<cplx> dwconv_kernel_slots(const double* K, int c, int f, int w, int 
 Diag decompose_diag(int w, int m);
 Diag fc_stoc_diagonals(const double* M, int n_out, int n_in, int n);
 std::vector<double> decompose_kernels(const double* W, int cout, int cin, int f, int C, int t, int* f_out);
-std::vector<cplx> real_cins_slots(const double* m, int C, int two_l);
-std::vector<double> cins_to_reals(const std::vector<cplx>& z, int C, int two_l);
+std::vector<cplx> real_cins_slots(const double* m, int C, int two_l, const std::vector<cplx>* R = nullptr);
+std::vector<double> cins_to_reals(const std::vector<cplx>& z, int C, int two_l, const std::vector<cplx>* R = nullptr);
 std::vector<double> cheb_interp_cos(double K, int r, int deg);
 std::vector<double> power_to_cheb(const std::vector<double>& c, double alpha, double beta);
 int default_bsgs_B(int count);

@@ -233,6 +233,7 @@ ckks_ctx::~ckks_ctx() {
     cudaFree(d_primes);
     cudaFree(d_tables);
     cudaFree(d_gauss);
+    cudaFree(d_garner);
     cudaFree(d_pinv);
     cudaFree(d_qlinv);
     cudaFree(d_pqlinv);
@@ -363,6 +364,19 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
         if (c->fold)
             for (size_t k = 0; k < words; ++k) ntt_pair((*t)[k], c->q[k % c->nq], true, t->data() + 2 * words + 2 * k);
     }
+    c->roots = fp64::roots_2n(n);
+    // prod_{k<t} q_k mod q_i (t < i) and (prod_{k<i} q_k)^{-1} mod q_i, Shoup pairs
+    std::vector<u64> gar(2 * (size_t)c->nq * c->nq, 0);
+    for (int i = 0; i < c->nq; ++i) {
+        u64 pr = 1 % c->q[i];
+        for (int t = 0; t <= i; ++t) {
+            const u64 v = t < i ? pr : invmod(pr, c->q[i]);
+            gar[2 * ((size_t)i * c->nq + t)] = v;
+            gar[2 * ((size_t)i * c->nq + t) + 1] = shoup(v, c->q[i]);
+            if (t < i) pr = mulmod(pr, c->q[t] % c->q[i], c->q[i]);
+        }
+    }
+    c->d_garner = dev_upload_persistent(gar);
     c->d_pinv = dev_upload_persistent(pinv);
     c->d_qlinv = dev_upload_persistent(qlinv);
     c->h_qlinv.assign(qlinv.begin(), qlinv.begin() + (size_t)c->nq * c->nq);
