@@ -737,14 +737,15 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(CL_THREADS, 2)
 
 // Launch shapes (identical results).  NTT_MIX, the default at every size, takes the best shape of
 // each pass: 8 columns per COL CTA (64-byte runs; 4 columns leave half of every 64-byte access
-// unused, 14.3 against 10.3 us just to read and write 62 limbs in that pattern) and 4 rows per ROW
-// CTA (rows are contiguous, and CTAs of two warps fill the last wave best).  us per pass with the
-// CTA's sub-problems x least resident CTAs, 62 / 248 limbs: forward COL 8x6 22.7 / 69, 16x3
-// 23.5 / 72, 4x8 24.8 / 76; forward ROW 4x8 25.4 / 85, 8x4 26.3 / 87, 16x3 30.4 / 99; inverse
-// ROW 4x12 22.7 / 76, 4x8 23.6 / 80, 16x3 24.8 / 82; inverse COL 8x4 28.2 / 91, 4x8 29.5 / 93,
-// 16x3 29.4 / 99; below 16 limbs they agree within 1 us of 8 to 12.  (Each figure holds about
-// 4 us of the two events around the launch.)  ckks_autotune times every shape per limb-count class.
-// ArShoup contexts have NTT_V16 and NTT_V4 only.
+// unused, 14.3 against 10.3 us just to read and write 62 limbs in that pattern) and 2 or 4 rows
+// per ROW CTA (rows are contiguous, and CTAs of one or two warps fill the last wave best).  us per
+// pass with the CTA's sub-problems x least resident CTAs, 62 / 368 limbs: forward COL 8x6 22.7 / 98,
+// 16x3 23.9 / 104; forward ROW 2x20 25.0 / 115, 4x8 25.8 / 120; inverse ROW 4x12 22.8 / 105, 4x8
+// 23.3 / 113; inverse COL 8x5 26.2 / 119, 8x4 26.8 / 123, 16x3 28.7 / 137; below 16 limbs they agree
+// within 1 us of 8 to 12.  (Each figure holds about 4 us of the two events around the launch.)
+// What is left between these and the butterflies alone (31 cycles per warp and SM quarter: 75 us for
+// 368 limbs) are the loads of data and twiddles that other warps do not cover.  ckks_autotune times
+// every shape per limb-count class.  ArShoup contexts have NTT_V16 and NTT_V4 only.
 enum NttVariant {
     NTT_MIX = 0, NTT_V16 = 1, NTT_V4 = 2, NTT_V4_R80 = 3, NTT_X4 = 4, NTT_CL = 5, NTT_NVARIANTS = 6
 };
@@ -765,8 +766,9 @@ void launch_ntt16_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, cons
     }
     switch (v) {
         case NTT_MIX:
-            if constexpr (COL) NTT16(ArFold, 8, INV ? 4 : 6);
-            else NTT16(ArFold, 4, INV ? 12 : 8);
+            if constexpr (COL) NTT16(ArFold, 8, INV ? 5 : 6);
+            else if constexpr (INV) NTT16(ArFold, 4, 12);
+            else NTT16(ArFold, 2, 20);
             break;
         case NTT_V16: NTT16(ArFold, 16, 3); break;
         case NTT_V4: NTT16(ArFold, 4, 8); break;
