@@ -318,6 +318,11 @@ struct NttTail {
     size_t a_pstride;
     ScaleTab s;
     const ScalarVec* ks;
+    // not null: the result goes to outs[i] for polynomials i per_out .. (i + 1) per_out - 1 (contiguous
+    // rows, at most MAX_OUTS of them) and the transformed array is only worked in
+    static constexpr int MAX_OUTS = 16;
+    u64* const* outs = nullptr;
+    int per_out = 0;
 };
 // forward NTT of out ([nlimbs / lpp][lpp][N], row k with prime ids[k % lpp] = k % lpp), its input
 // replaced by a lift and / or its output passed through a tail, both optional; lift->src and tail->a

@@ -161,7 +161,13 @@ struct NttTailArgs {
     size_t a_pstride;
     const ulonglong2* s;
     int has_k;
+    int per_out;           // 0: in place, else polynomials per entry of outs
+    u64* outs[kern::NttTail::MAX_OUTS];
     ulonglong2 ks[ScalarVec::MAX];
+    // row r (of lpp) of polynomial p
+    __device__ __forceinline__ u64* row(u64* data_row, int p, int r, int lpp, int logn) const {
+        return per_out ? outs[p / per_out] + (((size_t)(p % per_out) * lpp + r) << logn) : data_row;
+    }
 };
 template <bool TAIL>
 struct NttArgs {
@@ -338,13 +344,14 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
         if constexpr (TAIL) {
             const u64* A = tl.a + (size_t)(limb / lpp) * tl.a_pstride + ((size_t)r << LOGN);
             const ulonglong2 s = tl.s[r];
+            u64* o = tl.row(a, limb / lpp, r, lpp, LOGN);
 #pragma unroll
             for (int i = 0; i < 16; ++i) x[i] = __ldg(A + i * (N / 16) + t);
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 const int j = i * (N / 16) + t;
-                a[j] = tail_word(x[i], sm[spad(j)], tl, s, r, ar.q, ar.f);
+                o[j] = tail_word(x[i], sm[spad(j)], tl, s, r, ar.q, ar.f);
             }
         } else {
             __syncthreads();
@@ -469,12 +476,13 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
                 // all of a's words in flight at once (loads cannot pass the stores below)
                 const u64* A = io.a + (size_t)(limb / lpp) * io.a_pstride + ((size_t)r << 16);
                 const ulonglong2 s = io.s[r];
+                u64* o = io.row(a, limb / lpp, r, lpp, 16);
 #pragma unroll
                 for (int i = 0; i < 16; ++i) x[i] = __ldg(A + gidx(t + 16 * i));
                 __syncthreads();
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    a[gidx(t + 16 * i)] = tail_word(x[i], sm[f_slot<SUBS>(sp, t + 16 * i)], io, s, r, ar.q, ar.f);
+                    o[gidx(t + 16 * i)] = tail_word(x[i], sm[f_slot<SUBS>(sp, t + 16 * i)], io, s, r, ar.q, ar.f);
             } else {
                 __syncthreads();
 #pragma unroll
@@ -926,10 +934,16 @@ void ntt_forward_fused(const ckks_ctx* c, u64* out, int nlimbs, const int* ids, 
     if (!c->fold || lpp > ScalarVec::MAX || (!one && (c->logn != 16 || v > NTT_V4_R80))) {
         if (lift) lift_centred(c, lift->src, lift->src_id, out, nlimbs, ids, lpp, lift->src_pstride);
         ntt_forward(c, out, nlimbs, ids, lpp);
-        if (tail && tail->ks)
-            sub_mul2_scalar(c, tail->a, out, *tail->ks, tail->s.w, tail->s.wp, out, nlimbs, ids, lpp, tail->a_pstride);
-        else if (tail)
-            sub_mul_scalar(c, tail->a, out, tail->s.w, tail->s.wp, out, nlimbs, ids, lpp, tail->a_pstride);
+        if (!tail) return;
+        const int per = tail->outs ? tail->per_out : nlimbs / lpp;        // polynomials per output array
+        for (int p0 = 0; p0 < nlimbs / lpp; p0 += per) {
+            const u64* A = tail->a + p0 * tail->a_pstride;
+            u64 *x = out + p0 * ps, *o = tail->outs ? tail->outs[p0 / per] : x;
+            if (tail->ks)
+                sub_mul2_scalar(c, A, x, *tail->ks, tail->s.w, tail->s.wp, o, per * lpp, ids, lpp, tail->a_pstride);
+            else
+                sub_mul_scalar(c, A, x, tail->s.w, tail->s.wp, o, per * lpp, ids, lpp, tail->a_pstride);
+        }
         return;
     }
     NttSrc io{};
@@ -944,6 +958,11 @@ void ntt_forward_fused(const ckks_ctx* c, u64* out, int nlimbs, const int* ids, 
         tl.a_pstride = tail->a_pstride;
         tl.s = tail->s.pair;
         tl.has_k = tail->ks != nullptr;
+        tl.per_out = tail->outs ? tail->per_out : 0;
+        CK_CHECK(!tail->outs || (tail->per_out >= 1 && nlimbs <= NttTail::MAX_OUTS * tail->per_out * lpp), CKKS_EINVAL,
+                 "too many outputs for one tail");
+        if (tail->outs)
+            for (int i = 0; i * tail->per_out * lpp < nlimbs; ++i) tl.outs[i] = tail->outs[i];
         if (tail->ks)
             for (int i = 0; i < lpp; ++i) {
                 u64 w[2];

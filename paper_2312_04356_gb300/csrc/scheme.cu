@@ -707,18 +707,29 @@ static void lift_p(ckks_ctx* c, const u64* x, u64* acc, int level, int nb = 1) {
     kern::mul_scalar_acc(c, x, c->d_pmod, c->d_pmod + c->nq, acc, 2 * nl * nb, c->d_iota, nl, next * c->n);
 }
 
-// ModDown of both halves of acc: [nb][2][next][N] -> out [nb][2][l+1][N]
-static void mod_down(ckks_ctx* c, u64* acc, int level, u64* out, int nb = 1) {
+// ModDown of both halves of `count` sums acc [count][nb][2][next][N] -> outs[i] [nb][2][l+1][N]
+static void mod_down(ckks_ctx* c, u64* acc, int level, u64* const* outs, int count, int nb) {
     const size_t n = c->n;
-    const int nl = level + 1, npoly = 2 * nb;
+    const int nl = level + 1, npoly = 2 * nb * count;
     const int next = nl + c->np;
     const int* pid = c->d_ext_ids[level] + nl;
     const ConvTab& tab_c = c->moddown_tab(level);
     kern::ntt_inverse(c, acc + (size_t)nl * n, npoly * c->np, pid, c->np, (size_t)next * n, tab_c.d_iscale);
-    kern::base_convert(c, tab_c, acc + (size_t)nl * n, n, out, n, npoly, (size_t)next * n, (size_t)nl * n, true);
-    const kern::NttTail tail{acc, (size_t)next * n, c->scale_tab(c->d_pinv, c->nq, 0), nullptr};
-    kern::ntt_forward_fused(c, out, npoly * nl, c->d_iota, nl, nullptr, &tail);
+    DevBuf conv;                      // a single output array is worked in itself
+    u64* work = outs[0];
+    if (count > 1) {
+        conv = DevBuf((size_t)npoly * nl * n, c->stream);
+        work = conv.ptr;
+    }
+    kern::base_convert(c, tab_c, acc + (size_t)nl * n, n, work, n, npoly, (size_t)next * n, (size_t)nl * n, true);
+    kern::NttTail tail{acc, (size_t)next * n, c->scale_tab(c->d_pinv, c->nq, 0), nullptr};
+    if (count > 1) {
+        tail.outs = outs;
+        tail.per_out = 2 * nb;
+    }
+    kern::ntt_forward_fused(c, work, npoly * nl, c->d_iota, nl, nullptr, &tail);
 }
+static void mod_down(ckks_ctx* c, u64* acc, int level, u64* out, int nb = 1) { mod_down(c, acc, level, &out, 1, nb); }
 
 u64 galois_of_step(const ckks_ctx* c, long long r) {
     const long long m = c->n / 2;
@@ -727,35 +738,49 @@ u64 galois_of_step(const ckks_ctx* c, long long r) {
     return powmod(5, (u64)r, 2ULL * c->n);
 }
 
-// rot_g(a) for every ciphertext of a: the key switch of the automorphed raised digits D of c1 with
-// P c0(sigma_g) added on the Q rows in the same kernel, then ModDown: ModDown(P x + k) = x +
+// rot_g(a) for every g and every ciphertext of a: the key switches of the automorphed raised digits D
+// of c1 with P c0(sigma_g) added on the Q rows in the same kernel, then ModDown: ModDown(P x + k) = x +
 // ModDown(k) exactly (P x vanishes on the P rows), so this is automorph(c0) + ModDown(k) in
-// fewer passes.
-static ckks_ct switch_galois(const ckks_keys& keys, const ckks_ct& a, const Raised& D, u64 g) {
+// fewer passes.  Several rotations are brought down together (eight rotations at level 9, summed:
+// 621 -> 515 us).
+static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& a, const Raised& D,
+                                          const std::vector<u64>& gs) {
     ckks_ctx* c = a.ctx;
     const int l = a.level, nl = l + 1;
-    DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n, c->stream);
-    key_switch_inner(c, keys, D, l, g, g, acc.ptr, false, a.c0(), nl, c->d_pmod, nullptr,
-                     a.nb, a.cstride());
-    ckks_ct o = new_ct(c, l, a.scale, a.nb);
-    mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
-    return o;
+    const size_t es = (size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n;
+    const size_t group = std::min((size_t)kern::NttTail::MAX_OUTS, (size_t)std::max(1, 8 / a.nb));
+    std::vector<ckks_ct> outs;
+    for (size_t k0 = 0; k0 < gs.size(); k0 += group) {
+        const size_t cnt = std::min(group, gs.size() - k0);
+        DevBuf acc(cnt * es, c->stream);
+        std::vector<u64*> o;
+        for (size_t k = 0; k < cnt; ++k) {
+            key_switch_inner(c, keys, D, l, gs[k0 + k], gs[k0 + k], acc.ptr + k * es, false, a.c0(), nl, c->d_pmod, nullptr,
+                             a.nb, a.cstride());
+            outs.push_back(new_ct(c, l, a.scale, a.nb));
+            o.push_back(outs.back().buf.ptr);
+        }
+        mod_down(c, acc.ptr, l, o.data(), (int)cnt, a.nb);
+    }
+    return outs;
 }
 
 std::vector<ckks_ct> rotate_hoisted(const ckks_keys& keys, const ckks_ct& a, const std::vector<long long>& steps) {
     ckks_ctx* c = a.ctx;
-    const int l = a.level;
-    std::vector<ckks_ct> outs;
-    Raised D;
+    std::vector<u64> gs;
     for (long long r : steps) {
         const u64 g = galois_of_step(c, r);
-        if (g == 1) {
-            outs.push_back(copy_ct(a));
-            continue;
-        }
-        if (!D.x) D = mod_up(c, a.c1(), l, a.nb, a.cstride());
-        c->ops["hrot"]++;
-        outs.push_back(switch_galois(keys, a, D, g));
+        if (g != 1) gs.push_back(g);
+    }
+    std::vector<ckks_ct> rot, outs;
+    if (!gs.empty()) {
+        c->ops["hrot"] += (long)gs.size();
+        rot = switch_galois(keys, a, mod_up(c, a.c1(), a.level, a.nb, a.cstride()), gs);
+    }
+    size_t k = 0;
+    for (long long r : steps) {
+        if (galois_of_step(c, r) == 1) outs.push_back(copy_ct(a));
+        else outs.push_back(std::move(rot[k++]));
     }
     return outs;
 }
@@ -768,7 +793,8 @@ ckks_ct rotate(const ckks_keys& keys, const ckks_ct& a, long long r) {
 ckks_ct conjugate(const ckks_keys& keys, const ckks_ct& a) {
     ckks_ctx* c = a.ctx;
     const Raised D = mod_up(c, a.c1(), a.level, a.nb, a.cstride());
-    return switch_galois(keys, a, D, 2ULL * c->n - 1);
+    std::vector<ckks_ct> o = switch_galois(keys, a, D, {2ULL * c->n - 1});
+    return std::move(o[0]);
 }
 
 // tensor product of a batch: d [nb][3][l+1][N] (d0, d1, d2 of each ciphertext)

@@ -6,7 +6,7 @@ import gc
 import pytest
 
 import workloads as WL
-from tests.pairs import assert_ct_equal, import_ct, import_plan, make_pair
+from tests.pairs import assert_ct_equal, gpu_ctx, import_ct, import_plan, make_pair
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -45,3 +45,29 @@ def test_key_switch_bitexact(log_n, q0, dnum, n_q):
         del WL.PARAMS["fold_test"]
         K = o = ctx = keys = ct = gct = g = w = plan = None
         gc.collect()        # the device memory goes back here, not in the middle of a later test
+
+
+# rotations brought down together against each alone: two pass kernels (N = 2^16), one CTA a limb and
+# the general transform with separate tails; an identity, a repeated step and more than one group
+@pytest.mark.parametrize("log_n,q0", [(16, 60), (10, 60), (13, 60), (10, 61)])
+def test_hoisted_rotations_together_match_single(log_n, q0):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_04356_gb300 import build
+    build.build()
+    WL.PARAMS["fold_test"] = dict(log_n=log_n, n_q=3, dnum=2, n_p=0, q0_bits=q0, scale_bits=42, p_bits=60,
+                                  boot_bits=0, n_boot=0, h=0, sigma=3.2)
+    try:
+        from paper_2312_04356_gb300 import ckks as K
+        ctx = gpu_ctx("fold_test", 33)
+        keys = K.ckks_keygen(ctx, list(range(1, 9)), False)
+        ct = K.ckks_encrypt(ctx, keys, K.ckks_encode(ctx, WL.slots(1, 1 << (log_n - 1), 0.5), 2, 2.0 ** 42), 1)
+        steps = [3, 0, 1, 2, 4, 5, 6, 7, 8, 3]
+        for s, got in zip(steps, K.ckks_rotate_hoisted(ctx, keys, ct, steps)):
+            want = K.ckks_rotate_hoisted(ctx, keys, ct, [s])[0] if s else ct
+            assert (K.ckks_ct_export_rns(ctx, got) == K.ckks_ct_export_rns(ctx, want)).all(), s
+        K.ckks_sync(ctx)
+    finally:
+        del WL.PARAMS["fold_test"]
+        K = ctx = keys = ct = got = want = None
+        gc.collect()
