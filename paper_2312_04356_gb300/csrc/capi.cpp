@@ -1800,14 +1800,24 @@ static int raw_ntt(ckks_ctx* ctx, uint64_t* dev, int n_limbs, const int32_t* ids
         REQ(ids);
         for (int i = 0; i < n_limbs; ++i)
             CK_CHECK(ids[i] >= 0 && ids[i] < ctx->nall, CKKS_EINVAL, "prime id out of range");
-        std::vector<u64> tmp(n_limbs);
+        const auto run = [&](const int* d, int lpp) {
+            if (inv)
+                kern::ntt_inverse(ctx, (u64*)dev, n_limbs, d, lpp);
+            else
+                kern::ntt_forward(ctx, (u64*)dev, n_limbs, d, lpp);
+        };
+        // Limbs of consecutive primes, repeated or not (one polynomial or several), find their ids in the
+        // context's table: the upload of a list takes a copy between the call and its first kernel (48
+        // limbs, forward and inverse, N = 2^16: 98 us with the copies, 89 without).
+        int period = 1;
+        while (period < n_limbs && ids[period] == ids[0] + period) ++period;
+        int same = period;
+        while (same < n_limbs && ids[same] == ids[same - period]) ++same;
+        if (same == n_limbs) return run(ctx->d_iota + ids[0], period);
         DevBuf d((n_limbs + 1) / 2, ctx->stream);
         std::vector<int> v(ids, ids + n_limbs);
         CUDA_CHECK(cudaMemcpyAsync(d.ptr, v.data(), n_limbs * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
-        if (inv)
-            kern::ntt_inverse(ctx, (u64*)dev, n_limbs, (const int*)d.ptr, n_limbs);
-        else
-            kern::ntt_forward(ctx, (u64*)dev, n_limbs, (const int*)d.ptr, n_limbs);
+        run((const int*)d.ptr, n_limbs);
     });
 }
 int ckks_ntt_forward(ckks_ctx* ctx, uint64_t* dev, int n_limbs, const int32_t* ids) {

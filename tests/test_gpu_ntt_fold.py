@@ -56,3 +56,28 @@ def test_transform_extremes_bitexact(log_n, q0, sc, pb):
             call(ctx, dev.data_ptr(), len(ids), ids)
             torch.cuda.synchronize()
             assert (dev.cpu().numpy().view(np.uint64) == want).all(), (variant, call.__name__)
+
+
+# id lists that are runs of consecutive primes (whole, cut off, not from the first prime, one prime) and
+# lists that are not: each against every limb transformed by itself
+@pytest.mark.parametrize("log_n", [9, 13, 16])
+@pytest.mark.parametrize("ids", [[0, 1, 2, 3, 4, 0, 1, 2], [2, 3, 4, 2, 3, 4, 2], [3, 3, 3], [4], [0, 1, 2, 4], [2, 1, 0],
+                                 [0, 1, 0, 2], [1, 2, 1, 2, 3], [0, 0, 1, 1]])
+def test_id_lists_match_single_limbs(log_n, ids):
+    from paper_2312_04356_gb300 import build
+    from paper_2312_04356_gb300 import ckks as K
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    d = dict(log_n=log_n, n_q=4, dnum=1, n_p=1, q0_bits=60, scale_bits=42, p_bits=60, boot_bits=0, n_boot=0, h=0, sigma=3.2)
+    ctx = K.ckks_ctx_create(d, 1, torch.cuda.current_stream().cuda_stream)
+    q, p, _, _ = K.ckks_ctx_info(ctx)
+    g = np.random.default_rng(5)
+    x = np.stack([g.integers(0, (q + p)[i], 1 << log_n, dtype=np.uint64) for i in ids]).view(np.int64)
+    for call in (K.ckks_ntt_forward, K.ckks_ntt_inverse):
+        dev, one = torch.from_numpy(x.copy()).cuda(), torch.from_numpy(x.copy()).cuda()
+        call(ctx, dev.data_ptr(), len(ids), ids)
+        for k, i in enumerate(ids):
+            call(ctx, one[k].data_ptr(), 1, [i])
+        torch.cuda.synchronize()
+        assert torch.equal(dev, one), call.__name__
