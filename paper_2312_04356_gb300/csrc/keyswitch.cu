@@ -88,14 +88,19 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <bool FOLD, int NDIG, int NG>
-__global__ void __launch_bounds__(256, 3)
+// NC ciphertexts of a batch per thread: the key, diagonal and automorphism index of an element serve
+// all of them, so NC = 2 moves 18 words per baby and element for two ciphertexts (3 digits, 4 giant
+// steps) where NC = 1 moves 28.  Eight ciphertexts at the
+// top level, six sums of a block: 12.59 -> 11.84 ms.
+template <bool FOLD, int NDIG, int NG, int NC>
+__global__ void __launch_bounds__(256, NC == 1 ? 3 : 2)
     k_bsgs_fused_async(const __grid_constant__ kern::BsgsFused T, const __grid_constant__ kern::Digits D,
                        const u64* __restrict__ c0, const u64* __restrict__ c1, int nl, int next,
                        const int* __restrict__ ext_ids, const u64* __restrict__ s0,
                        const DevPrime* __restrict__ P, int logn, size_t kstride, kern::KsBatch bt) {
     griddep_entry();
-    constexpr int NS = 3 * NDIG + 2 + NG;       // kb, ka, D per digit; c0 (gathered or row); c1 row; diagonals
+    // words of a stage: kb, ka per digit, diagonals; then per ciphertext D per digit, c0 (gathered or row), c1 row
+    constexpr int OWN = 2 * NDIG + NG, NS = OWN + NC * (NDIG + 2);
     extern __shared__ u64 sbuf[];               // [2][NS][256]
     const int e = blockIdx.y;
     const int id = ext_ids[e];
@@ -105,23 +110,29 @@ __global__ void __launch_bounds__(256, 3)
     const bool qrow = e < nl;
     const u64 w = qrow ? s0[e] : 0;
     const int tid = threadIdx.x;
-    // ciphertext t of a batch (fastest varying, so that the CTAs reading the same key and diagonal
-    // words run side by side and share them through L2): D + t dstr, c0 / c1 + t xstr, outputs
+    // ciphertexts t .. t + NC - 1 of a batch (fastest varying, so that the CTAs reading the same key and
+    // diagonal words run side by side and share them through L2): D + t dstr, c0 / c1 + t xstr, outputs
     // + t ostr
-    const int t = blockIdx.x % bt.nb;
-    const int j = (blockIdx.x / bt.nb) * 256 + tid;
+    const int groups = bt.nb / NC, t = blockIdx.x % groups * NC;
+    const int j = (blockIdx.x / groups) * 256 + tid;
     if (j >= (int)n) return;
-    const u64* Dr[NDIG];
+    const u64* Dr[NC][NDIG];
 #pragma unroll
-    for (int d = 0; d < NDIG; ++d) Dr[d] = digit_row(D, d, e, t, next, bt.dstr, logn);
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int d = 0; d < NDIG; ++d) Dr[c][d] = digit_row(D, d, e, t + c, next, bt.dstr, logn);
     c0 += t * bt.xstr;
     c1 += t * bt.xstr;
     auto slot = [&](int st, int k) -> u64* { return sbuf + ((size_t)(st * NS + k) << 8) + tid; };
+    auto own = [&](int st, int c, int k) -> u64* { return slot(st, OWN + c * (NDIG + 2) + k); };
     auto issue = [&](int b, int st) {
         if (!T.kb[b]) {
             if (qrow) {
-                cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + j);
-                cp_async8(slot(st, 3 * NDIG + 1), c1 + (size_t)e * n + j);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    cp_async8(own(st, c, NDIG), c0 + c * bt.xstr + (size_t)e * n + j);
+                    cp_async8(own(st, c, NDIG + 1), c1 + c * bt.xstr + (size_t)e * n + j);
+                }
             }
         } else {
             const unsigned src = galois_src(j, T.gal[b], logn);
@@ -130,18 +141,24 @@ __global__ void __launch_bounds__(256, 3)
                 const size_t kk = d * kstride + (size_t)id * n + j;
                 cp_async8(slot(st, d), T.kb[b] + kk);
                 cp_async8(slot(st, NDIG + d), T.ka[b] + kk);
-                cp_async8(slot(st, 2 * NDIG + d), Dr[d] + src);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) cp_async8(own(st, c, d), Dr[c][d] + src);
             }
-            if (qrow) cp_async8(slot(st, 3 * NDIG), c0 + (size_t)e * n + src);
+            if (qrow) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) cp_async8(own(st, c, NDIG), c0 + c * bt.xstr + (size_t)e * n + src);
+            }
         }
 #pragma unroll
         for (int g = 0; g < NG; ++g)
-            if (T.p[g][b]) cp_async8(slot(st, 3 * NDIG + 2 + g), T.p[g][b] + (size_t)e * n + j);
+            if (T.p[g][b]) cp_async8(slot(st, 2 * NDIG + g), T.p[g][b] + (size_t)e * n + j);
         cp_async_commit();
     };
-    u64 lob[NG], hib[NG], loa[NG], hia[NG];
+    u64 lob[NC][NG], hib[NC][NG], loa[NC][NG], hia[NC][NG];
 #pragma unroll
-    for (int g = 0; g < NG; ++g) lob[g] = hib[g] = loa[g] = hia[g] = 0;
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int g = 0; g < NG; ++g) lob[c][g] = hib[c][g] = loa[c][g] = hia[c][g] = 0;
     issue(0, 0);
     if (T.nb > 1) issue(1, 1);
     else cp_async_commit();
@@ -149,44 +166,54 @@ __global__ void __launch_bounds__(256, 3)
         const int st = b & 1;
         cp_async_wait<1>();                          // the group of baby b has landed
         // the baby: sum of the digits' products with the key and w c0 (w = P mod q), reduced once
-        u64 bl = 0, bh = 0, al = 0, ah = 0;
-        if (!T.kb[b]) {
-            if (qrow) {
-                mac128(bl, bh, *slot(st, 3 * NDIG), w);
-                mac128(al, ah, *slot(st, 3 * NDIG + 1), w);
-            }
-        } else {
+        u64 rb[NC], ra[NC];
 #pragma unroll
-            for (int d = 0; d < NDIG; ++d) {
-                const u64 x = *slot(st, 2 * NDIG + d), yb = *slot(st, d), ya = *slot(st, NDIG + d);
-                mac128(bl, bh, x, yb);
-                mac128(al, ah, x, ya);
+        for (int c = 0; c < NC; ++c) {
+            u64 bl = 0, bh = 0, al = 0, ah = 0;
+            if (!T.kb[b]) {
+                if (qrow) {
+                    mac128(bl, bh, *own(st, c, NDIG), w);
+                    mac128(al, ah, *own(st, c, NDIG + 1), w);
+                }
+            } else {
+#pragma unroll
+                for (int d = 0; d < NDIG; ++d) {
+                    const u64 x = *own(st, c, d), yb = *slot(st, d), ya = *slot(st, NDIG + d);
+                    mac128(bl, bh, x, yb);
+                    mac128(al, ah, x, ya);
+                }
+                if (qrow) mac128(bl, bh, *own(st, c, NDIG), w);
             }
-            if (qrow) mac128(bl, bh, *slot(st, 3 * NDIG), w);
+            rb[c] = red(bh, bl);
+            ra[c] = red(ah, al);
         }
-        const u64 rb = red(bh, bl), ra = red(ah, al);
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
             if (!T.p[g][b]) continue;
-            const u64 y = *slot(st, 3 * NDIG + 2 + g);
-            mac128(lob[g], hib[g], rb, y);
-            mac128(loa[g], hia[g], ra, y);
+            const u64 y = *slot(st, 2 * NDIG + g);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                mac128(lob[c][g], hib[c][g], rb[c], y);
+                mac128(loa[c][g], hia[c][g], ra[c], y);
+            }
         }
         if (b + 2 < T.nb) issue(b + 2, st);          // this stage has been read
         else cp_async_commit();                      // keep one group per iteration
     }
 #pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        u64 vb = red(hib[g], lob[g]), va = red(hia[g], loa[g]);
-        u64* ob = T.o[g] + t * bt.ostr + (size_t)e * n + j;
-        u64* oa = T.o[g] + t * bt.ostr + ((size_t)next + e) * n + j;
-        if ((T.acc >> g) & 1u) {
-            vb = add_mod(vb, *ob, q);
-            va = add_mod(va, *oa, q);
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            u64 vb = red(hib[c][g], lob[c][g]), va = red(hia[c][g], loa[c][g]);
+            u64* ob = T.o[g] + (t + c) * bt.ostr + (size_t)e * n + j;
+            u64* oa = T.o[g] + (t + c) * bt.ostr + ((size_t)next + e) * n + j;
+            if ((T.acc >> g) & 1u) {
+                vb = add_mod(vb, *ob, q);
+                va = add_mod(va, *oa, q);
+            }
+            *ob = vb;
+            *oa = va;
         }
-        *ob = vb;
-        *oa = va;
-    }
 }
 
 // ---------------------------------------------------- key-switch product ----
@@ -197,7 +224,9 @@ __global__ void __launch_bounds__(256, 3)
 // outputs at ob / oa + t ostr, its x0 / x1 at + t xstr.  The ciphertext index is the fastest
 // varying part of blockIdx.x, so the CTAs that read the same key words run side by side and
 // all but the first find them in L2: the key streams from HBM about once per batch.
-template <bool FOLD, bool ACC, int V, int NDIG>
+// NC of its ciphertexts share a thread and with it the key words and the automorphism.  Eight ciphertexts,
+// the 49 of a block: 5.86 -> 5.71 ms (4.7 TB/s of algorithmic bytes).
+template <bool FOLD, bool ACC, int V, int NDIG, int NC>
 __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, const int* __restrict__ ext_ids,
                              const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
                              u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride,
@@ -208,20 +237,19 @@ __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, c
     const int id = ext_ids[e];
     const Reducer<FOLD> red(P[id]);
     const size_t n = (size_t)1 << logn;
-    const int t = blockIdx.x % bt.nb;
-    const int j = V * ((blockIdx.x / bt.nb) * blockDim.x + threadIdx.x);
+    const int groups = bt.nb / NC, t = blockIdx.x % groups * NC;
+    const int j = V * ((blockIdx.x / groups) * blockDim.x + threadIdx.x);
     if (j >= (int)n) return;
-    ob += t * bt.ostr;
-    oa += t * bt.ostr;
-    if (x0) x0 += t * bt.xstr;
-    if (x1) x1 += t * bt.xstr;
+    ob += t * bt.ostr + (size_t)e * n + j;
+    oa += t * bt.ostr + (size_t)e * n + j;
+    if (x0) x0 += t * bt.xstr + (size_t)e * n;
+    if (x1) x1 += t * bt.xstr + (size_t)e * n;
     unsigned src[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) src[v] = g == 1 ? (unsigned)(j + v) : galois_src(j + v, g, logn);
-    u64 x[NDIG][V], yb[NDIG][V], ya[NDIG][V];
+    u64 x[NC][NDIG][V], yb[NDIG][V], ya[NDIG][V];
 #pragma unroll
     for (int d = 0; d < NDIG; ++d) {
-        const u64* Dd = digit_row(D, d, e, t, next, bt.dstr, logn);
         const size_t kk = d * kstride + (size_t)id * n + j;
         if (bt.nb == 1) {
             ldv_cs<V>(kb + kk, yb[d]);   // each key word is read once per key switch: keep the
@@ -231,43 +259,56 @@ __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, c
             ldv<V>(ka + kk, ya[d]);
         }
 #pragma unroll
-        for (int v = 0; v < V; ++v) x[d][v] = Dd[src[v]];
+        for (int c = 0; c < NC; ++c) {
+            const u64* Dd = digit_row(D, d, e, t + c, next, bt.dstr, logn);
+#pragma unroll
+            for (int v = 0; v < V; ++v) x[c][d][v] = Dd[src[v]];
+        }
     }
     // the sums: digits times key, the previous output (accumulating) and w x0, w x1 (w = s0's row, or 1)
-    u64 bl[V], bh[V], al[V], ah[V];
+    u64 bl[NC][V], bh[NC][V], al[NC][V], ah[NC][V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) bl[v] = bh[v] = al[v] = ah[v] = 0;
-    if (ACC) {
-        ldv<V>(ob + (size_t)e * n + j, bl);
-        ldv<V>(oa + (size_t)e * n + j, al);
-    }
+    for (int c = 0; c < NC; ++c) {
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-#pragma unroll
-        for (int d = 0; d < NDIG; ++d) {
-            mac128(bl[v], bh[v], x[d][v], yb[d][v]);
-            mac128(al[v], ah[v], x[d][v], ya[d][v]);
+        for (int v = 0; v < V; ++v) bl[c][v] = bh[c][v] = al[c][v] = ah[c][v] = 0;
+        if (ACC) {
+            ldv<V>(ob + c * bt.ostr, bl[c]);
+            ldv<V>(oa + c * bt.ostr, al[c]);
         }
     }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+#pragma unroll
+            for (int d = 0; d < NDIG; ++d) {
+                mac128(bl[c][v], bh[c][v], x[c][d][v], yb[d][v]);
+                mac128(al[c][v], ah[c][v], x[c][d][v], ya[d][v]);
+            }
+        }
     if (x0 && e < x0rows) {
         const u64 w = s0 ? s0[e] : 1;
-        const u64* xr = x0 + (size_t)e * n;
 #pragma unroll
-        for (int v = 0; v < V; ++v) mac128(bl[v], bh[v], xr[src[v]], w);
-        if (x1) {
-            const u64* yr = x1 + (size_t)e * n;
+        for (int c = 0; c < NC; ++c) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) mac128(al[v], ah[v], yr[src[v]], w);
+            for (int v = 0; v < V; ++v) mac128(bl[c][v], bh[c][v], x0[c * bt.xstr + src[v]], w);
+            if (x1) {
+#pragma unroll
+                for (int v = 0; v < V; ++v) mac128(al[c][v], ah[c][v], x1[c * bt.xstr + src[v]], w);
+            }
         }
     }
-    u64 rb[V], ra[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-        rb[v] = red(bh[v], bl[v]);
-        ra[v] = red(ah[v], al[v]);
+    for (int c = 0; c < NC; ++c) {
+        u64 rb[V], ra[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            rb[v] = red(bh[c][v], bl[c][v]);
+            ra[v] = red(ah[c][v], al[c][v]);
+        }
+        stv<V>(ob + c * bt.ostr, rb);
+        stv<V>(oa + c * bt.ostr, ra);
     }
-    stv<V>(ob + (size_t)e * n + j, rb);
-    stv<V>(oa + (size_t)e * n + j, ra);
 }
 
 }  // namespace
@@ -325,17 +366,44 @@ void bsgs_inner_giants(const ckks_ctx* c, const BsgsGiants& t, int nl, const int
     LAUNCH_CHECK();
 }
 
+// the digits from ciphertext k of a batch on
+static Digits digits_from(Digits D, size_t k, size_t dstr) {
+    D.D += k * dstr;
+    D.own += k * D.own_str;
+    return D;
+}
+
+template <bool FOLD, int NDIG, int NG, int NC>
+static void launch_bsgs_async_nc(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0,
+                                 const u64* c1, int nl, int next, const int* ext, const u64* s, const KsBatch& bt) {
+    constexpr int NS = 2 * NDIG + NG + NC * (NDIG + 2);
+    const size_t smem = 2 * (size_t)NS * 256 * sizeof(u64);
+    static std::atomic<unsigned> done{0};
+    allow_dynamic_smem((const void*)k_bsgs_fused_async<FOLD, NDIG, NG, NC>, (int)smem, done);
+    const dim3 grid((c->n + 255) / 256 * (bt.nb / NC), next);
+    klaunch(c, k_bsgs_fused_async<FOLD, NDIG, NG, NC>, grid, 256, smem, t, D, c0, c1, nl, next, ext, s, c->d_primes,
+            c->logn, (size_t)c->nall << c->logn, bt);
+}
+
+// the ciphertexts of a batch in pairs, the last of an odd number by itself
 template <bool FOLD, int NDIG, int NG>
 static void launch_bsgs_async_one(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u64* c0,
                                   const u64* c1, int nl, int next, const int* ext, const u64* s,
                                   const KsBatch& bt) {
-    constexpr int NS = 3 * NDIG + 2 + NG;
-    const size_t smem = 2 * (size_t)NS * 256 * sizeof(u64);
-    static std::atomic<unsigned> done{0};
-    allow_dynamic_smem((const void*)k_bsgs_fused_async<FOLD, NDIG, NG>, (int)smem, done);
-    const dim3 grid((c->n + 255) / 256 * bt.nb, next);
-    klaunch(c, k_bsgs_fused_async<FOLD, NDIG, NG>, grid, 256, smem, t, D, c0, c1, nl, next, ext, s, c->d_primes,
-            c->logn, (size_t)c->nall << c->logn, bt);
+    const int pairs = bt.nb / 2;
+    if (pairs) {
+        KsBatch b2 = bt;
+        b2.nb = 2 * pairs;
+        launch_bsgs_async_nc<FOLD, NDIG, NG, 2>(c, t, D, c0, c1, nl, next, ext, s, b2);
+    }
+    if (bt.nb & 1) {
+        const size_t k = bt.nb - 1;
+        BsgsFused t1 = t;
+        for (int g = 0; g < t.ng; ++g) t1.o[g] += k * bt.ostr;
+        KsBatch b1 = bt;
+        b1.nb = 1;
+        launch_bsgs_async_nc<FOLD, NDIG, NG, 1>(c, t1, digits_from(D, k, bt.dstr), c0 + k * bt.xstr, c1 + k * bt.xstr, nl, next, ext, s, b1);
+    }
 }
 
 template <bool FOLD, int NDIG>
@@ -388,30 +456,40 @@ void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u6
     LAUNCH_CHECK();
 }
 
+template <bool FOLD, bool ACC, int V, int NC>
+static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
+                               const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
+                               const u64* s0, const KsBatch& bt) {
+    dim3 grid = ewv_grid(c->n, next, V);
+    grid.x *= bt.nb / NC;
+    const size_t ks = (size_t)c->nall << c->logn;
+#define KS_CASE(NDIG)                                                                                                  \
+    klaunch(c, k_ks_inner_d<FOLD, ACC, V, NDIG, NC>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes, \
+            c->logn, g, ks, x0, x1, x0rows, s0, bt)
+    switch (ndig) {
+        case 1: KS_CASE(1); break;
+        case 2: KS_CASE(2); break;
+        case 3: KS_CASE(3); break;
+        default: KS_CASE(4); break;
+    }
+#undef KS_CASE
+}
+
+// the ciphertexts of a batch in pairs, the last of an odd number by itself
 template <bool FOLD, bool ACC, int V>
 static void launch_ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
                             const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
                             const u64* s0, const KsBatch& bt) {
-    dim3 grid = ewv_grid(c->n, next, V);
-    grid.x *= bt.nb;
-    const size_t ks = (size_t)c->nall << c->logn;
-    switch (ndig) {
-        case 1:
-            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 1>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
-            break;
-        case 2:
-            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 2>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
-            break;
-        case 3:
-            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 3>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
-            break;
-        default:
-            klaunch(c, k_ks_inner_d<FOLD, ACC, V, 4>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,
-                    c->logn, g, ks, x0, x1, x0rows, s0, bt);
-            break;
+    KsBatch part = bt;
+    part.nb = bt.nb & ~1;
+    if (part.nb)
+        launch_ks_inner_nc<FOLD, ACC, V, 2>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s0, part);
+    if (bt.nb & 1) {
+        const size_t k = part.nb;
+        part.nb = 1;
+        launch_ks_inner_nc<FOLD, ACC, V, 1>(c, digits_from(D, k, bt.dstr), ndig, next, ext_ids, kb, ka, ob + k * bt.ostr,
+                                            oa + k * bt.ostr, g, x0 ? x0 + k * bt.xstr : x0, x1 ? x1 + k * bt.xstr : x1,
+                                            x0rows, s0, part);
     }
 }
 

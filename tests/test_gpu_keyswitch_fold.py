@@ -71,3 +71,28 @@ def test_hoisted_rotations_together_match_single(log_n, q0):
         del WL.PARAMS["fold_test"]
         K = ctx = keys = ct = got = want = None
         gc.collect()
+
+
+# batches share key words between pairs of ciphertexts; an odd number leaves one over.  Both reductions,
+# the block's accumulated key switches and (cin = 16, w0 = 2) the stored babies
+@pytest.mark.parametrize("B", [1, 2, 5])
+@pytest.mark.parametrize("q0", [60, 61])
+@pytest.mark.parametrize("spec", [WL.CONV["cfg2_small"], dict(cin=16, cout=16, w0=2, f=3, weight="gauss")])
+def test_batched_pairs_match_single(B, q0, spec):
+    from tests.test_gpu_batch import _setup
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_04356_gb300 import build
+    build.build()
+    WL.PARAMS["fold_test"] = dict(WL.PARAMS["cfg2_small"], q0_bits=q0)
+    try:
+        d = _setup("fold_test", 57, spec, B, oracle_keys=False)
+        K, ctx, keys = d["K"], d["ctx"], d["keys"]
+        outs = K.ckks_block_batched(ctx, keys, d["gcts"], d["gplan"], d["bt"])
+        for c, out in zip(d["gcts"], outs):
+            one = K.ckks_block(ctx, keys, c, d["gplan"], d["bt"])
+            assert (K.ckks_ct_export_rns(ctx, out) == K.ckks_ct_export_rns(ctx, one)).all()
+    finally:
+        del WL.PARAMS["fold_test"]
+        d = K = ctx = keys = outs = c = out = one = None
+        gc.collect()
