@@ -1,5 +1,6 @@
 // extern "C" entry points (include/ckks.h).  Each call catches every C++ error and
 // returns a status code; ckks_last_error(ctx) keeps the message.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -39,6 +40,30 @@ int guard(const ckks_ctx* c, F&& f) {
         if (c) const_cast<ckks_ctx*>(c)->err = e.what();
         return CKKS_EINVAL;
     }
+}
+
+// The device address of `bytes` of host memory that kernels may read and write (pinned, mapped, one
+// allocation), or null.
+u64* device_view(const void* host, size_t bytes) {
+    using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Query query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return (Query)f;
+    }();
+    if (!query) return nullptr;
+    unsigned type = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* to[4] = {&type, &dev, &start, &size};
+    if (query(4, what, to, (CUdeviceptr)host) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || dev == 0 || dev % 8 || dev < start || dev - start + bytes > size) return nullptr;
+    return (u64*)dev;
 }
 
 #define REQ(p) CK_CHECK((p) != nullptr, CKKS_EINVAL, #p " is NULL")
@@ -416,8 +441,13 @@ int ckks_ct_import_rns(ckks_ctx* ctx, const uint64_t* host, int level, double sc
         CK_CHECK(level >= 0 && level <= ctx->L, CKKS_EINVAL, "level out of range");
         ckks_ct o = ops::new_ct(ctx, level, scale);
         const size_t words = 2 * (size_t)(level + 1) * ctx->n;
-        CUDA_CHECK(cudaMemcpyAsync(o.buf.ptr, host, words * 8, cudaMemcpyHostToDevice, ctx->stream));
-        kern::ntt_forward(ctx, o.buf.ptr, 2 * (level + 1), ctx->d_iota, level + 1);
+        const u64* view = kern::ntt_host_io(ctx, 2 * (level + 1)) ? device_view(host, words * 8) : nullptr;
+        if (view) {
+            kern::ntt_forward_from_host(ctx, view, o.buf.ptr, 2 * (level + 1), ctx->d_iota, level + 1);
+        } else {
+            CUDA_CHECK(cudaMemcpyAsync(o.buf.ptr, host, words * 8, cudaMemcpyHostToDevice, ctx->stream));
+            kern::ntt_forward(ctx, o.buf.ptr, 2 * (level + 1), ctx->d_iota, level + 1);
+        }
         assign(out, std::move(o));
     });
 }
@@ -442,9 +472,18 @@ int ckks_ct_export_rns(ckks_ctx* ctx, const ckks_ct* ct, uint64_t* host) {
         CK_CHECK(ct->level >= 0, CKKS_EINVAL, "empty ciphertext");
         const int nl = ct->level + 1;
         const size_t words = 2 * (size_t)nl * ctx->n;
-        DevBuf t(words, ctx->stream);
-        kern::ntt_inverse_from(ctx, ct->buf.ptr, (size_t)nl * ctx->n, t.ptr, 2 * nl, ctx->d_iota, nl, 0, nullptr);
-        CUDA_CHECK(cudaMemcpyAsync(host, t.ptr, words * 8, cudaMemcpyDeviceToHost, ctx->stream));
+        // pinned memory takes the words from the transform's last pass: no copy after it, and the link works
+        // while limbs are still transformed (HMult, rescale and export of 15 limbs: 294 -> 287 us; a
+        // convolution of a 4096-coefficient ring, import to export: 168 -> 159 us)
+        u64* view = kern::ntt_host_io(ctx, 2 * nl) ? device_view(host, words * 8) : nullptr;
+        DevBuf t;
+        if (!view || ctx->logn == 16) t = DevBuf(words, ctx->stream);
+        if (view) {
+            kern::ntt_inverse_to_host(ctx, ct->buf.ptr, (size_t)nl * ctx->n, t.ptr, view, 2 * nl, ctx->d_iota, nl);
+        } else {
+            kern::ntt_inverse_from(ctx, ct->buf.ptr, (size_t)nl * ctx->n, t.ptr, 2 * nl, ctx->d_iota, nl, 0, nullptr);
+            CUDA_CHECK(cudaMemcpyAsync(host, t.ptr, words * 8, cudaMemcpyDeviceToHost, ctx->stream));
+        }
         CUDA_CHECK(cudaStreamSynchronize(ctx->stream));
     });
 }

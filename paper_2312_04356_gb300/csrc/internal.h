@@ -329,6 +329,13 @@ struct NttTail {
 // must not overlap out
 void ntt_forward_fused(const ckks_ctx* c, u64* out, int nlimbs, const int* ids, int lpp, const NttLift* lift,
                        const NttTail* tail);
+// Transforms whose first pass reads, or whose last pass writes, host memory that the device reaches
+// (contiguous limbs), where ntt_host_io says that the context's passes do.  work (N = 2^16 only) is as
+// large as host.
+bool ntt_host_io(const ckks_ctx* c, int nlimbs);
+void ntt_forward_from_host(const ckks_ctx* c, const u64* host, u64* data, int nlimbs, const int* ids, int lpp);
+void ntt_inverse_to_host(const ckks_ctx* c, const u64* src, size_t src_pstride, u64* work, u64* host, int nlimbs,
+                         const int* ids, int lpp);
 // forward NTT of an arbitrary list of limbs: limb i at data + off[i] * N with prime ids[i] (N = 2^16);
 // for nb copies of the list, copy t at data + t * bstride
 void ntt_forward_list(const ckks_ctx* c, u64* data, int nlimbs, const int* off, const int* ids, int nb = 1,

@@ -142,13 +142,16 @@ __device__ __forceinline__ void inv_stages(u64 (&x)[16], const AR& ar, const ulo
 // result by the integer k.
 // Forward, first pass: every row of polynomial p is the centred lift of the one row
 // src + p * src_pstride with modulus lift_q (a signed word is what the lazy butterflies take; one
-// fold brings a wider source prime's word into range).
+// fold brings a wider source prime's word into range); lift_q 0: row k reads src + (k / lpp) src_pstride +
+// (k % lpp) N as it is.
+// Inverse, last pass: dst not null takes row k at dst + k N instead of the data array.
 struct NttSrc {
     const u64* src;
     size_t src_pstride;
     bool scaled;
     ulonglong2 w, w2;
     u64 lift_q;
+    u64* dst;
 };
 // Forward, last pass: row k receives (a - x) s, or a ks - x s when has_k, instead of the transform x; row k
 // of a at a + (k / lpp) a_pstride + (k % lpp) N, s and ks as ntt_pair pairs per row k % lpp.
@@ -319,8 +322,9 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
 #pragma unroll
             for (int i = 0; i < 16; ++i) x[i] = lift_word(src[sk<LOGN>(t, i, LOGN - 4)], io.lift_q, ar.f);
         } else {
+            const u64* src = io.src ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << LOGN) : a;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = a[sk<LOGN>(t, i, LOGN - 4)];
+            for (int i = 0; i < 16; ++i) x[i] = src[sk<LOGN>(t, i, LOGN - 4)];
         }
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr) {
@@ -452,8 +456,10 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
 #pragma unroll
             for (int i = 0; i < 16; ++i) x[i] = lift_word(src[gidx(t + 16 * i)], io.lift_q, ar.f);
         } else {
+            const u64* sr = a;
+            if constexpr (COL && !INV) sr = io.src ? io.src + (size_t)(limb / lpp) * io.src_pstride + ((size_t)r << 16) : a;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = a[gidx(t + 16 * i)];
+            for (int i = 0; i < 16; ++i) x[i] = sr[gidx(t + 16 * i)];
         }
         fwd_round<false>(x, t, hi, s0, P->tw, ar);
 #pragma unroll
@@ -511,6 +517,9 @@ __global__ void __launch_bounds__(16 * SUBS, MINB) k_ntt16(u64* __restrict__ dat
         for (int i = 0; i < 16; ++i) x[i] = sm[f_slot<SUBS>(sp, t + 16 * i)];
         if constexpr (COL && INV) inv_round<false, true>(x, t, hi, s0, P->itw, ar, out_factor(P, osc, r, io));
         else inv_round<false, false>(x, t, hi, s0, P->itw, ar);
+        if constexpr (COL && INV) {
+            if (io.dst) a = io.dst + ((size_t)limb << 16);
+        }
 #pragma unroll
         for (int i = 0; i < 16; ++i) a[gidx(t + 16 * i)] = x[i];     // canonical (COL), lazy (ROW)
     }
@@ -808,14 +817,14 @@ void launch_ntt_cl(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, in
 // One whole N = 2^16 transform with variant v: the cluster kernel, or the two passes (forward:
 // COL then ROW; inverse: ROW then COL).  Algorithmic bytes: one read and one write of the
 // limbs per transform, split evenly over the two passes.
-// (io: a separate source of the inverse's first pass and an output factor, as NttSrc
-// describes)
+// (io: a separate source of the first pass, a separate destination of the inverse's last and an output
+// factor, as NttSrc describes; vcol: another variant for the COL pass)
 template <bool INV>
 void launch_ntt_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
-                        const int* loff, const u64* osc = nullptr, const NttSrc& io = NttSrc{}) {
+                        const int* loff, const u64* osc = nullptr, const NttSrc& io = NttSrc{}, int vcol = -1) {
     const char* nm = INV ? "ntt_inv" : "ntt_fwd";
     const double bytes = 2.0 * nlimbs * cx->n * 8.0;
-    CK_CHECK(INV || !io.src, CKKS_EINVAL, "only the inverse transform reads a separate source");
+    const int vc = vcol >= 0 ? vcol : v;
     if (v == NTT_CL && cx->fold) {
         KTimer kt_(cx, nm, bytes);
         launch_ntt_cl<INV>(cx, data, nlimbs, ids, lpp, pstride, loff, osc, io);
@@ -826,11 +835,11 @@ void launch_ntt_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const 
         if (INV && io.src)     // the inverse's first pass is the ROW pass
             launch_ntt16_variant<false, true, true>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
         else
-            launch_ntt16_variant<!INV, INV>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
+            launch_ntt16_variant<!INV, INV>(cx, INV ? v : vc, data, nlimbs, ids, lpp, pstride, loff, osc, io);
     }
     {
         KTimer kt_(cx, nm, bytes / 2);
-        launch_ntt16_variant<INV, INV>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
+        launch_ntt16_variant<INV, INV>(cx, INV ? vc : v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
     }
 }
 
@@ -1070,7 +1079,7 @@ void ntt_inverse_from(const ckks_ctx* c, const u64* src, size_t src_pstride, u64
     CK_CHECK(!scaled || (lpp == 1 && osc == nullptr && pstride == c->n), CKKS_EINVAL,
              "an integer factor needs one contiguous row per polynomial and no output scale table");
     if (c->logn == 16 || ntt_one_cta(c)) {
-        NttSrc io{src, src_pstride, scaled, {}, {}, 0};
+        NttSrc io{src, src_pstride, scaled, {}, {}, 0, nullptr};
         if (scaled) {
             const u64 q = c->mod_of[k_id];
             u64 w[4];
@@ -1095,6 +1104,38 @@ void ntt_inverse_from(const ckks_ctx* c, const u64* src, size_t src_pstride, u64
                                      cudaMemcpyDeviceToDevice, c->stream));
     }
     ntt_inverse(c, data, nlimbs, ids, lpp, pstride, osc);
+}
+
+bool ntt_host_io(const ckks_ctx* c, int nlimbs) {
+    return ntt_one_cta(c) || (c->logn == 16 && (!c->fold || ntt_pick(c, nlimbs) <= NTT_V4_R80));
+}
+
+// Columns of a COL CTA that touches host memory: the link moves 128-byte runs (16 columns) of a large
+// transfer best (30 limbs out, whole export: 132 us with 64-byte runs, 122 with 128-byte ones, of which
+// the link alone takes about 90); small ones want the CTAs.  8 and 16 columns agree at 4 limbs.
+static int host_columns(int nlimbs) { return nlimbs >= 16 ? (int)NTT_V16 : -1; }
+
+void ntt_forward_from_host(const ckks_ctx* c, const u64* host, u64* data, int nlimbs, const int* ids, int lpp) {
+    const size_t ps = (size_t)lpp * c->n;
+    const NttSrc io{host, ps, false, {}, {}, 0, nullptr};
+    if (c->logn == 16)
+        launch_ntt_variant<false>(c, ntt_pick(c, nlimbs), data, nlimbs, ids, lpp, ps, nullptr, nullptr, io,
+                                  host_columns(nlimbs));
+    else
+        launch_ntt_one<false>(c, data, nlimbs, ids, lpp, ps, nullptr, io);
+    LAUNCH_CHECK();
+}
+
+void ntt_inverse_to_host(const ckks_ctx* c, const u64* src, size_t src_pstride, u64* work, u64* host, int nlimbs,
+                         const int* ids, int lpp) {
+    const size_t ps = (size_t)lpp * c->n;
+    const NttSrc io{src, src_pstride, false, {}, {}, 0, host};
+    if (c->logn == 16)
+        launch_ntt_variant<true>(c, ntt_pick(c, nlimbs), work, nlimbs, ids, lpp, ps, nullptr, nullptr, io,
+                                 host_columns(nlimbs));
+    else
+        launch_ntt_one<true>(c, host, nlimbs, ids, lpp, ps, nullptr, io);
+    LAUNCH_CHECK();
 }
 
 }  // namespace kern

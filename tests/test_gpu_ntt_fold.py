@@ -81,3 +81,39 @@ def test_id_lists_match_single_limbs(log_n, ids):
             call(ctx, one[k].data_ptr(), 1, [i])
         torch.cuda.synchronize()
         assert torch.equal(dev, one), call.__name__
+
+
+# limbs that cross the host boundary in pinned memory (read and written by the transforms) and in pageable
+# memory (copied), whole buffers and parts of one: the same words, and back what went in
+@pytest.mark.parametrize("log_n,q0", [(9, 60), (12, 61), (13, 60), (16, 60), (16, 61)])
+def test_pinned_and_pageable_limbs_agree(log_n, q0):
+    import ctypes
+
+    from paper_2312_04356_gb300 import build
+    from paper_2312_04356_gb300 import ckks as K
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    d = dict(log_n=log_n, n_q=9, dnum=1, n_p=1, q0_bits=q0, scale_bits=42, p_bits=60, boot_bits=0, n_boot=0, h=0, sigma=3.2)
+    ctx = K.ckks_ctx_create(d, 1, torch.cuda.current_stream().cuda_stream)
+    q, _, _, _ = K.ckks_ctx_info(ctx)
+    g = np.random.default_rng(7)
+    pool = torch.zeros((2 * 9 + 2) << log_n, dtype=torch.int64).pin_memory()
+    for level in (0, 3, 8):
+        x = np.stack([[g.integers(0, q[i], 1 << log_n, dtype=np.uint64) for i in range(level + 1)] for _ in range(2)])
+        for variant in (-1, 4) if log_n == 16 else (-1,):
+            K.ckks_ctx_set_ntt_variant(ctx, variant)
+            for skip in (0, 1, 1 << log_n):           # the buffer's start, an odd word, a whole limb further
+                pool.zero_()
+                host = pool[skip:skip + x.size]
+                host.copy_(torch.from_numpy(x.view(np.int64).ravel()))
+                ct, out = K.ckks_ct_create(ctx), pool[skip:skip + x.size]
+                ctx.check(K.lib().ckks_ct_import_rns(ctx, ctypes.c_void_p(host.data_ptr()), level, 2.0 ** 42, ct))
+                K.ckks_sync(ctx)
+                ref = K.ckks_ct_import_rns(ctx, x, level, 2.0 ** 42)
+                assert (K.ckks_ct_export_rns(ctx, ct) == x).all() and (K.ckks_ct_export_rns(ctx, ref) == x).all()
+                out.zero_()
+                ctx.check(K.lib().ckks_ct_export_rns(ctx, ref, ctypes.c_void_p(out.data_ptr())))
+                assert (out.numpy().view(np.uint64).reshape(x.shape) == x).all(), (level, variant, skip)
+                assert not pool[:skip].any() and not pool[skip + x.size:].any(), "words outside the buffer"
+    K.ckks_ctx_set_ntt_variant(ctx, -1)
