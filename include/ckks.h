@@ -164,9 +164,8 @@ int ckks_ctx_set_ntt_choices(ckks_ctx* ctx, const int32_t* choice8);
  * its first memory access, so results are identical either way.  Captured launches are
  * always plain.  on == 0: plain launches everywhere. */
 int ckks_ctx_set_pdl(ckks_ctx* ctx, int on);
-/* Independent work inside one operation (the giant steps of an HMatmul, the Chebyshev
- * leaves, the products of one generation of the Chebyshev power ladder, the division nodes
- * of one height) runs on up to four side streams joined back by events (parallel branches of
+/* Independent work inside one operation (the Chebyshev leaves, the products of one
+ * generation of the Chebyshev power ladder, the division nodes of one height) runs on up to four side streams joined back by events (parallel branches of
  * a captured graph) when on != 0 (the default); on == 0 keeps everything on the context's
  * stream, e.g. so that per-kernel event timing measures each kernel alone.  Results are
  * identical either way. */
@@ -214,7 +213,9 @@ int ckks_ct_create(ckks_ctx* ctx, ckks_ct** out);
 int ckks_ct_destroy(ckks_ct* ct);
 int ckks_ct_info(const ckks_ct* ct, int* level, double* scale);
 int ckks_ct_set_scale(ckks_ct* ct, double scale);
-/* host [2][level+1][N] coefficient domain <-> device (NTT domain inside) */
+/* host [2][level+1][N] coefficient domain <-> device (NTT domain inside).  A host buffer inside one
+ * mapped pinned allocation is read and written by the transforms themselves (it must stay unchanged
+ * until the stream has passed an import, as for an asynchronous copy); any other is copied. */
 int ckks_ct_import_rns(ckks_ctx* ctx, const uint64_t* host, int level, double scale, ckks_ct* out);
 int ckks_ct_export_rns(ckks_ctx* ctx, const ckks_ct* ct, uint64_t* host);
 /* Copies src into dst's existing device buffer (same level required; dst keeps its

@@ -131,8 +131,8 @@ struct ckks_ctx {
     uint64_t seed = 0;
     u64 gauss[39];
     cudaStream_t stream = 0;
-    // side streams for independent work inside one operation (the giant steps of an HMatmul,
-    // the leaves of a Chebyshev evaluation); created on first use
+    // side streams for independent work inside one operation (the leaves and products of a
+    // Chebyshev evaluation); created on first use
     static constexpr int NSIDE = 4;
     cudaStream_t side[NSIDE] = {};
     cudaEvent_t fork_ev = nullptr, side_ev[NSIDE] = {};
@@ -336,7 +336,7 @@ bool ntt_host_io(const ckks_ctx* c, int nlimbs);
 void ntt_forward_from_host(const ckks_ctx* c, const u64* host, u64* data, int nlimbs, const int* ids, int lpp);
 void ntt_inverse_to_host(const ckks_ctx* c, const u64* src, size_t src_pstride, u64* work, u64* host, int nlimbs,
                          const int* ids, int lpp);
-// forward NTT of an arbitrary list of limbs: limb i at data + off[i] * N with prime ids[i] (N = 2^16);
+// forward NTT of an arbitrary list of limbs: limb i at data + off[i] * N with prime ids[i];
 // for nb copies of the list, copy t at data + t * bstride
 void ntt_forward_list(const ckks_ctx* c, u64* data, int nlimbs, const int* off, const int* ids, int nb = 1,
                       size_t bstride = 0);

@@ -209,14 +209,15 @@ constexpr int NTT_THREADS = 256;
 template <class AR, bool INV>
 __global__ void __launch_bounds__(NTT_THREADS)
     k_ntt_pass(u64* __restrict__ data, const DevPrime* __restrict__ primes, const int* __restrict__ ids, int lpp,
-               size_t pstride, int logn, int s0, int c, int logsub, int scale_out, const u64* __restrict__ osc) {
+               size_t pstride, const int* __restrict__ loff, int logn, int s0, int c, int logsub, int scale_out,
+               const u64* __restrict__ osc) {
     griddep_entry();
     extern __shared__ u64 sm[];
     const int limb = blockIdx.y;
     const DevPrime* P = primes + ids[limb % lpp];
     const AR ar(P);
     const u64 q = ar.q;
-    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(limb % lpp) << logn);
+    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(loff ? loff[limb % lpp] : limb % lpp) << logn);
     const int span = 1 << c;
     const int SUB = 1 << logsub;
     const int stride = SUB > 1 ? SUB + 1 : 1;
@@ -304,8 +305,8 @@ __device__ __forceinline__ int spad(int k) { return k + (k >> 4); }
 template <class AR, bool INV, int LOGN, bool TAIL = false>
 __global__ void __launch_bounds__(1 << (LOGN - 4))
     k_ntt_one(u64* __restrict__ data, const DevPrime* __restrict__ primes, const int* __restrict__ ids, int lpp,
-              size_t pstride, const u64* __restrict__ osc, const __grid_constant__ NttSrc io,
-              const __grid_constant__ typename NttArgs<TAIL>::type tl) {
+              size_t pstride, const int* __restrict__ loff, const u64* __restrict__ osc,
+              const __grid_constant__ NttSrc io, const __grid_constant__ typename NttArgs<TAIL>::type tl) {
     griddep_entry();
     constexpr int N = 1 << LOGN, NR = (LOGN + 3) / 4, LAST = LOGN - 4 * (NR - 1);   // rounds, stages of the last
     __shared__ u64 sm[N + N / 16];
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(1 << (LOGN - 4))
     const int r = limb % lpp;
     const DevPrime* P = primes + ids[r];
     const AR ar(P);
-    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)r << LOGN);
+    u64* a = data + (size_t)(limb / lpp) * pstride + ((size_t)(loff ? loff[r] : r) << LOGN);
     const int t = threadIdx.x;
     u64 x[16];
     if (!INV) {
@@ -861,11 +862,12 @@ inline bool ntt_one_cta(const ckks_ctx* cx) { return cx->fold && cx->logn >= 8 &
 template <bool INV, bool TAIL = false>
 void launch_ntt_one(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
                     const u64* osc = nullptr, const NttSrc& io = NttSrc{},
-                    const typename NttArgs<TAIL>::type& tl = typename NttArgs<TAIL>::type{}) {
+                    const typename NttArgs<TAIL>::type& tl = typename NttArgs<TAIL>::type{},
+                    const int* loff = nullptr) {
     KTimer kt_(cx, INV ? "ntt_inv" : "ntt_fwd", 2.0 * nlimbs * cx->n * 8.0);
 #define ONE(LOGN)                                                                                                   \
     klaunch(cx, k_ntt_one<ArFold, INV, LOGN, TAIL>, dim3(1, nlimbs), 1 << (LOGN - 4), 0, data, cx->d_primes, ids,   \
-            lpp, pstride, osc, io, tl)
+            lpp, pstride, loff, osc, io, tl)
     switch (cx->logn) {
         case 8: ONE(8); break;
         case 9: ONE(9); break;
@@ -887,7 +889,7 @@ inline std::vector<PassPlan> ntt_passes(int logn) {
 
 template <bool INV>
 void launch_pass(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride, PassPlan p,
-                 int scale_out, const u64* osc = nullptr) {
+                 int scale_out, const u64* osc = nullptr, const int* loff = nullptr) {
     const int logn = cx->logn;
     int logsub = 12 - p.c;
     if (logsub < 0) logsub = 0;
@@ -899,10 +901,10 @@ void launch_pass(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int 
     dim3 grid(tiles, nlimbs);
     KTimer kt_(cx, INV ? "ntt_inv" : "ntt_fwd", 2.0 * nlimbs * cx->n * 8.0 * p.c / logn);
     if (cx->fold)
-        klaunch(cx, k_ntt_pass<ArFold, INV>, grid, NTT_THREADS, smem, data, cx->d_primes, ids, lpp, pstride, logn,
+        klaunch(cx, k_ntt_pass<ArFold, INV>, grid, NTT_THREADS, smem, data, cx->d_primes, ids, lpp, pstride, loff, logn,
                 p.s0, p.c, logsub, scale_out, osc);
     else
-        klaunch(cx, k_ntt_pass<ArShoup, INV>, grid, NTT_THREADS, smem, data, cx->d_primes, ids, lpp, pstride, logn,
+        klaunch(cx, k_ntt_pass<ArShoup, INV>, grid, NTT_THREADS, smem, data, cx->d_primes, ids, lpp, pstride, loff, logn,
                 p.s0, p.c, logsub, scale_out, osc);
 }
 
@@ -1045,8 +1047,14 @@ void autotune_ntt(ckks_ctx* c, int reps) {
 void ntt_forward_list(const ckks_ctx* c, u64* data, int nlimbs, const int* off, const int* ids, int nb,
                       size_t bstride) {
     if (nlimbs <= 0 || nb <= 0) return;
-    CK_CHECK(c->logn == 16, CKKS_EINVAL, "limb-list NTT needs N = 2^16");
-    launch_ntt_transform<false>(c, data, nlimbs * nb, ids, nlimbs, bstride, off);
+    if (c->logn == 16) {
+        launch_ntt_transform<false>(c, data, nlimbs * nb, ids, nlimbs, bstride, off);
+    } else if (ntt_one_cta(c)) {
+        launch_ntt_one<false>(c, data, nlimbs * nb, ids, nlimbs, bstride, nullptr, NttSrc{}, NttArgs<false>::type{}, off);
+    } else {
+        for (const PassPlan& p : ntt_passes(c->logn))
+            launch_pass<false>(c, data, nlimbs * nb, ids, nlimbs, bstride, p, 0, nullptr, off);
+    }
     LAUNCH_CHECK();
 }
 

@@ -2,13 +2,13 @@
 // BSGS linear maps, the fused CinS conv, Chebyshev evaluation and bootstrapping.
 //
 // Every ciphertext limb lives on the device in the NTT domain.  Host code only
-// sequences kernels (kernels.cu) and prepares constants.  Steps follow the paper's
+// sequences kernels (ntt.cu, keyswitch.cu, convert_tc.cu, kernels.cu) and prepares constants.  Steps follow the paper's
 // Alg. 1 and the hybrid RNS-CKKS it builds on (Sec. 2.1, Sec. 2.4):
 //   key switching: digits of alpha consecutive limbs; ModUp by fast base conversion
 //   without correction; inner product with the key over Q_l u P; ModDown
 //   (c - Conv_{P->Q}([c]_P)) P^{-1}.  Rotations are always hoisted: ModUp(c1) once,
 //   then per step the automorphism is applied to the raised digits inside the inner
-//   product (k_ks_inner gathers through the Galois permutation).
+//   product (k_ks_inner_d gathers through the Galois permutation).
 #include <math.h>
 #include <string.h>
 
@@ -636,24 +636,15 @@ Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride =
     r.x = x;
     r.xstride = xstride;
     r.ndig = ndig;
-    const int* ext = c->d_ext_ids[level];
     kern::ConvJobs jobs;
     jobs.n = 0;
     for (int d = 0; d < ndig; ++d)
         kern::add_conv_job(jobs, c->modup_tab(level, d), coef.ptr + (size_t)dig[d].front() * n,
                            r.D.ptr + (size_t)d * next * n, (size_t)nl * n, dstr, true);
     kern::base_convert_jobs(c, jobs, nb);
-    if (c->logn == 16) {   // every converted row of every digit of every ciphertext in one launch
-        kern::ntt_forward_list(c, r.D.ptr, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb,
-                               dstr);
-        return r;
-    }
-    for (int d = 0; d < ndig; ++d) {
-        u64* Dd = r.D.ptr + (size_t)d * next * n;
-        const int lo = dig[d].front(), hi = dig[d].back() + 1;
-        if (lo > 0) kern::ntt_forward(c, Dd, nb * lo, ext, lo, dstr);
-        if (next > hi) kern::ntt_forward(c, Dd + (size_t)hi * n, nb * (next - hi), ext + hi, next - hi, dstr);
-    }
+    // every converted row of every digit of every ciphertext in one launch (two digits at N = 2^12: one
+    // transform in place of three; a convolution there, import to export: 158 -> 127 us)
+    kern::ntt_forward_list(c, r.D.ptr, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb, dstr);
     return r;
 }
 
