@@ -503,9 +503,22 @@ void set_tc_withhold(bool on);
 // (bt: a batch of bt.nb ciphertexts switched with the same key, D at + t dstr, ob / oa at + t ostr,
 // x0 / x1 at + t xstr; at most 4 digits)
 void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
-              const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate = false, const u64* x0 = nullptr,
-              int x0rows = 0, const u64* s = nullptr, const u64* x1 = nullptr,
-              const KsBatch& bt = KsBatch());
+              const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0 = nullptr, int x0rows = 0,
+              const u64* s = nullptr, const u64* x1 = nullptr, const KsBatch& bt = KsBatch());
+// The key switches of nr rotations by g[k], each of its own polynomial (number k bt.nb + t of D for
+// ciphertext t) with its own key, and x0(sigma_k) on every row (x0 [nr][bt.nb] at stride bt.xstr), summed
+// into ob / oa (added to what they hold when accumulating) without intermediate reductions.
+struct KsRotations {
+    static constexpr int MAXR = 16;
+    // rotations whose products one 128-bit sum holds (40 products, the x0 and the previous words within one)
+    static constexpr int fits(int ndig) { return 39 / ndig < MAXR ? 39 / ndig : MAXR; }
+    int nr = 0;
+    const u64* kb[MAXR];
+    const u64* ka[MAXR];
+    u64 g[MAXR];
+};
+void ks_rotations(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const KsRotations& R,
+                  const u64* x0, u64* ob, u64* oa, bool accumulate, const KsBatch& bt);
 // d0 = a0 b0, d1 = a0 b1 + a1 b0 (d [2][nl][N]), d2 = a1 b1 (e [nl][N]) over nl limbs with
 // primes ids[0..nl); a, b [2][nl][N]; for a batch of nb ciphertexts, ciphertext t's operands at
 // a + t ab_bstride, b + t ab_bstride, d + t d_bstride, e + t e_bstride

@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(256, NC == 1 ? 3 : 2)
 // all but the first find them in L2: the key streams from HBM about once per batch.
 // NC of its ciphertexts share a thread and with it the key words and the automorphism.  Eight ciphertexts,
 // the 49 of a block: 5.86 -> 5.71 ms (4.7 TB/s of algorithmic bytes).
-template <bool FOLD, bool ACC, int V, int NDIG, int NC>
+template <bool FOLD, int V, int NDIG, int NC>
 __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, const int* __restrict__ ext_ids,
                              const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
                              u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride,
@@ -265,17 +265,12 @@ __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, c
             for (int v = 0; v < V; ++v) x[c][d][v] = Dd[src[v]];
         }
     }
-    // the sums: digits times key, the previous output (accumulating) and w x0, w x1 (w = s0's row, or 1)
+    // the sums: digits times key and w x0, w x1 (w = s0's row, or 1)
     u64 bl[NC][V], bh[NC][V], al[NC][V], ah[NC][V];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
+    for (int c = 0; c < NC; ++c)
 #pragma unroll
         for (int v = 0; v < V; ++v) bl[c][v] = bh[c][v] = al[c][v] = ah[c][v] = 0;
-        if (ACC) {
-            ldv<V>(ob + c * bt.ostr, bl[c]);
-            ldv<V>(oa + c * bt.ostr, al[c]);
-        }
-    }
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
@@ -297,6 +292,92 @@ __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, c
                 for (int v = 0; v < V; ++v) mac128(al[c][v], ah[c][v], x1[c * bt.xstr + src[v]], w);
             }
         }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        u64 rb[V], ra[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            rb[v] = red(bh[c][v], bl[c][v]);
+            ra[v] = red(ah[c][v], al[c][v]);
+        }
+        stv<V>(ob + c * bt.ostr, rb);
+        stv<V>(oa + c * bt.ostr, ra);
+    }
+}
+
+// The key switches of several rotations (each with its own key, automorphism and raised polynomial: the
+// rotated giant steps of an HMatmul) summed into one output: rotation k of ciphertext t has the digits
+// of polynomial k nb + t of D and adds x0(sigma_k) of x0 + (k nb + t) xstr on every row.  One 128-bit
+// sum and one reduction for all of them; a launch per rotation read and wrote the output each time.
+// Bound by HBM like k_ks_inner_d: block 8.13 -> 7.98 ms, eight ciphertexts 54.2 -> 53.5 ms, conv at level 1
+// 250 -> 241 us, downsampling layer 12.07 -> 11.81 ms.
+template <bool FOLD, int V, int NDIG, int NC>
+__global__ void k_ks_rotations(const __grid_constant__ kern::KsRotations R, const __grid_constant__ kern::Digits D,
+                               int next, const int* __restrict__ ext_ids, const u64* __restrict__ x0,
+                               u64* __restrict__ ob, u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn,
+                               size_t kstride, bool accumulate, int t0, int groups, kern::KsBatch bt) {
+    griddep_entry();
+    const int e = blockIdx.y;
+    const int id = ext_ids[e];
+    const Reducer<FOLD> red(P[id]);
+    const size_t n = (size_t)1 << logn;
+    const int t = t0 + blockIdx.x % groups * NC;
+    const int j = V * ((blockIdx.x / groups) * blockDim.x + threadIdx.x);
+    if (j >= (int)n) return;
+    ob += t * bt.ostr + (size_t)e * n + j;
+    oa += t * bt.ostr + (size_t)e * n + j;
+    u64 bl[NC][V], bh[NC][V], al[NC][V], ah[NC][V];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) bl[c][v] = bh[c][v] = al[c][v] = ah[c][v] = 0;
+        if (accumulate) {
+            ldv<V>(ob + c * bt.ostr, bl[c]);
+            ldv<V>(oa + c * bt.ostr, al[c]);
+        }
+    }
+    for (int k = 0; k < R.nr; ++k) {
+        unsigned src[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) src[v] = galois_src(j + v, R.g[k], logn);
+        u64 x[NC][NDIG][V], z[NC][V], yb[NDIG][V], ya[NDIG][V];
+#pragma unroll
+        for (int d = 0; d < NDIG; ++d) {
+            const size_t kk = d * kstride + (size_t)id * n + j;
+            if (bt.nb == 1) {
+                ldv_cs<V>(R.kb[k] + kk, yb[d]);
+                ldv_cs<V>(R.ka[k] + kk, ya[d]);
+            } else {
+                ldv<V>(R.kb[k] + kk, yb[d]);
+                ldv<V>(R.ka[k] + kk, ya[d]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const int poly = k * bt.nb + t + c;
+            const u64* xr = x0 + poly * bt.xstr + (size_t)e * n;
+#pragma unroll
+            for (int v = 0; v < V; ++v) z[c][v] = xr[src[v]];
+#pragma unroll
+            for (int d = 0; d < NDIG; ++d) {
+                const u64* Dd = digit_row(D, d, e, poly, next, bt.dstr, logn);
+#pragma unroll
+                for (int v = 0; v < V; ++v) x[c][d][v] = Dd[src[v]];
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                bl[c][v] += z[c][v];
+                bh[c][v] += bl[c][v] < z[c][v];
+#pragma unroll
+                for (int d = 0; d < NDIG; ++d) {
+                    mac128(bl[c][v], bh[c][v], x[c][d][v], yb[d][v]);
+                    mac128(al[c][v], ah[c][v], x[c][d][v], ya[d][v]);
+                }
+            }
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -456,7 +537,7 @@ void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u6
     LAUNCH_CHECK();
 }
 
-template <bool FOLD, bool ACC, int V, int NC>
+template <bool FOLD, int V, int NC>
 static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
                                const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
                                const u64* s0, const KsBatch& bt) {
@@ -464,7 +545,7 @@ static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int
     grid.x *= bt.nb / NC;
     const size_t ks = (size_t)c->nall << c->logn;
 #define KS_CASE(NDIG)                                                                                                  \
-    klaunch(c, k_ks_inner_d<FOLD, ACC, V, NDIG, NC>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes, \
+    klaunch(c, k_ks_inner_d<FOLD, V, NDIG, NC>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,      \
             c->logn, g, ks, x0, x1, x0rows, s0, bt)
     switch (ndig) {
         case 1: KS_CASE(1); break;
@@ -476,46 +557,81 @@ static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int
 }
 
 // the ciphertexts of a batch in pairs, the last of an odd number by itself
-template <bool FOLD, bool ACC, int V>
+template <bool FOLD, int V>
 static void launch_ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
                             const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
                             const u64* s0, const KsBatch& bt) {
     KsBatch part = bt;
     part.nb = bt.nb & ~1;
     if (part.nb)
-        launch_ks_inner_nc<FOLD, ACC, V, 2>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s0, part);
+        launch_ks_inner_nc<FOLD, V, 2>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s0, part);
     if (bt.nb & 1) {
         const size_t k = part.nb;
         part.nb = 1;
-        launch_ks_inner_nc<FOLD, ACC, V, 1>(c, digits_from(D, k, bt.dstr), ndig, next, ext_ids, kb, ka, ob + k * bt.ostr,
+        launch_ks_inner_nc<FOLD, V, 1>(c, digits_from(D, k, bt.dstr), ndig, next, ext_ids, kb, ka, ob + k * bt.ostr,
                                             oa + k * bt.ostr, g, x0 ? x0 + k * bt.xstr : x0, x1 ? x1 + k * bt.xstr : x1,
                                             x0rows, s0, part);
     }
 }
 
 void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
-              const u64* ka, u64* ob, u64* oa, u64 g, bool accumulate, const u64* x0, int x0rows, const u64* s,
+              const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, int x0rows, const u64* s,
               const u64* x1, const KsBatch& bt) {
     CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4, CKKS_EINVAL, "key switching takes 1..4 digits");
     const bool vec = al16(kb) && al16(ka) && al16(ob) && al16(oa);
     {
         // algorithmic bytes: the key once for the whole batch, per ciphertext its digits, outputs
-        // (read too when accumulating) and the x0 / x1 rows
+        // and the x0 / x1 rows
         const double extra = x0 ? (double)x0rows * (x1 ? 2.0 : 1.0) / next : 0.0;
-        KTimer kt_(c, "ks_inner",
-                   (2.0 * ndig + bt.nb * (ndig + (accumulate ? 4.0 : 2.0) + extra)) * next * c->n * 8.0);
-#define KS(FOLD, ACC, V) launch_ks_inner<FOLD, ACC, V>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s, bt)
-        if (c->fold && vec) {
-            if (accumulate) KS(true, true, 2);
-            else KS(true, false, 2);
-        } else if (c->fold) {
-            if (accumulate) KS(true, true, 1);
-            else KS(true, false, 1);
-        } else {
-            if (accumulate) KS(false, true, 1);
-            else KS(false, false, 1);
-        }
+        KTimer kt_(c, "ks_inner", (2.0 * ndig + bt.nb * (ndig + 2.0 + extra)) * next * c->n * 8.0);
+#define KS(FOLD, V) launch_ks_inner<FOLD, V>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s, bt)
+        if (c->fold && vec) KS(true, 2);
+        else if (c->fold) KS(true, 1);
+        else KS(false, 1);
 #undef KS
+    }
+    LAUNCH_CHECK();
+}
+
+template <bool FOLD, int V>
+static void launch_ks_rotations(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids,
+                                const KsRotations& R, const u64* x0, u64* ob, u64* oa, bool accumulate,
+                                const KsBatch& bt) {
+    const dim3 tiles = ewv_grid(c->n, next, V);
+    const size_t ks = (size_t)c->nall << c->logn;
+    // ciphertexts in pairs, the last of an odd number by itself
+#define KSR_CASE(NDIG, NC, T0, GROUPS)                                                                                 \
+    klaunch(c, k_ks_rotations<FOLD, V, NDIG, NC>, dim3(tiles.x * (GROUPS), tiles.y), EW_THREADS, 0, R, D, next, ext_ids, \
+            x0, ob, oa, c->d_primes, c->logn, ks, accumulate, T0, GROUPS, bt)
+#define KSR_NDIG(NDIG)                                                \
+    do {                                                              \
+        if (bt.nb >= 2) KSR_CASE(NDIG, 2, 0, bt.nb / 2);              \
+        if (bt.nb & 1) KSR_CASE(NDIG, 1, bt.nb - 1, 1);               \
+    } while (0)
+    switch (ndig) {
+        case 1: KSR_NDIG(1); break;
+        case 2: KSR_NDIG(2); break;
+        case 3: KSR_NDIG(3); break;
+        default: KSR_NDIG(4); break;
+    }
+#undef KSR_NDIG
+#undef KSR_CASE
+}
+
+void ks_rotations(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const KsRotations& R,
+                  const u64* x0, u64* ob, u64* oa, bool accumulate, const KsBatch& bt) {
+    CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4 && R.nr >= 1 && R.nr <= KsRotations::fits(ndig), CKKS_EINVAL,
+             "key switching takes 1..4 digits and as many rotations as one sum holds");
+    bool vec = al16(ob) && al16(oa);
+    for (int k = 0; k < R.nr; ++k) vec = vec && al16(R.kb[k]) && al16(R.ka[k]);
+    {
+        // algorithmic bytes: the keys once for the whole batch, per ciphertext its digits and x0 rows, and
+        // the outputs (read too when accumulating)
+        KTimer kt_(c, "ks_inner",
+                   (R.nr * 2.0 * ndig + bt.nb * (R.nr * (ndig + 1.0) + (accumulate ? 4.0 : 2.0))) * next * c->n * 8.0);
+        if (c->fold && vec) launch_ks_rotations<true, 2>(c, D, ndig, next, ext_ids, R, x0, ob, oa, accumulate, bt);
+        else if (c->fold) launch_ks_rotations<true, 1>(c, D, ndig, next, ext_ids, R, x0, ob, oa, accumulate, bt);
+        else launch_ks_rotations<false, 1>(c, D, ndig, next, ext_ids, R, x0, ob, oa, accumulate, bt);
     }
     LAUNCH_CHECK();
 }

@@ -649,18 +649,20 @@ Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride =
 }
 
 // inner product with switching key `code` (automorphism g applied to D on the fly) over
-// Q_l u P: acc [2][next][N], NTT domain; `accumulate` adds to what acc holds.  With x0, the
+// Q_l u P: acc [2][next][N], NTT domain.  With x0, the
 // first x0rows rows of acc's first half also receive s x0(sigma_g) (s null: x0(sigma_g)), the
 // automorphed c0 term of a rotation, in the same kernel.
-// `first`: the first of D's polynomials to switch.
 // For a batch of nb ciphertexts: acc [nb][2][next][N], x0 / x1 of ciphertext t
 // at + t xstr; the key is read once for the batch.
-void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int level, u64 code, u64 g,
-                      u64* acc, bool accumulate, const u64* x0 = nullptr, int x0rows = 0, const u64* s = nullptr,
-                      const u64* x1 = nullptr, int nb = 1, size_t xstr = 0, int first = 0) {
+static const SwitchKey& switching_key(const ckks_keys& keys, u64 code) {
     auto it = keys.swk.find(code);
     CK_CHECK(it != keys.swk.end(), CKKS_ENOKEY, "missing switching key (code " + std::to_string(code) + ")");
-    const SwitchKey& k = *it->second;
+    return *it->second;
+}
+void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int level, u64 code, u64 g,
+                      u64* acc, const u64* x0 = nullptr, int x0rows = 0, const u64* s = nullptr,
+                      const u64* x1 = nullptr, int nb = 1, size_t xstr = 0) {
+    const SwitchKey& k = switching_key(keys, code);
     c->ops["keyswitch"]++;
     const size_t next = (size_t)level + 1 + c->np;
     kern::KsBatch bt;
@@ -668,9 +670,38 @@ void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int l
     bt.dstr = (size_t)D.ndig * next * c->n;
     bt.ostr = 2 * next * c->n;
     bt.xstr = xstr;
-    const kern::Digits dig{D.D.ptr + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
+    const kern::Digits dig{D.D.ptr, D.x, D.xstride, level + 1, c->alpha};
     kern::ks_inner(c, dig, D.ndig, (int)next, c->d_ext_ids[level], k.b.ptr, k.a.ptr, acc, acc + next * c->n, g,
-                   accumulate, x0, x0rows, s, x1, bt);
+                   x0, x0rows, s, x1, bt);
+}
+
+// sum over rotations gs[k] of the key switch of D's polynomials k nb .. (k + 1) nb - 1, plus x0(sigma_k) of
+// x0 [k][nb] (stride xstr) on every row of the first half: acc [nb][2][next][N]
+static void key_switch_rotations(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int level,
+                                 const std::vector<u64>& gs, u64* acc, bool accumulate, const u64* x0, int nb,
+                                 size_t xstr) {
+    const size_t next = (size_t)level + 1 + c->np;
+    kern::KsBatch bt;
+    bt.nb = nb;
+    bt.dstr = (size_t)D.ndig * next * c->n;
+    bt.ostr = 2 * next * c->n;
+    bt.xstr = xstr;
+    const size_t per = kern::KsRotations::fits(D.ndig);
+    for (size_t k0 = 0; k0 < gs.size(); k0 += per) {
+        kern::KsRotations R;
+        for (size_t k = k0; k < std::min(gs.size(), k0 + per); ++k) {
+            const SwitchKey& key = switching_key(keys, gs[k]);
+            c->ops["hrot"]++;
+            c->ops["keyswitch"]++;
+            R.kb[R.nr] = key.b.ptr;
+            R.ka[R.nr] = key.a.ptr;
+            R.g[R.nr++] = gs[k];
+        }
+        const size_t first = k0 * nb;
+        const kern::Digits dig{D.D.ptr + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
+        kern::ks_rotations(c, dig, D.ndig, (int)next, c->d_ext_ids[level], R, x0 + first * xstr, acc, acc + next * c->n,
+                           accumulate || k0 > 0, bt);
+    }
 }
 
 // ModDown fused with the rescale after it: both halves of acc (Q_l u P, NTT domain) divided
@@ -746,7 +777,7 @@ static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& 
         DevBuf acc(cnt * es, c->stream);
         std::vector<u64*> o;
         for (size_t k = 0; k < cnt; ++k) {
-            key_switch_inner(c, keys, D, l, gs[k0 + k], gs[k0 + k], acc.ptr + k * es, false, a.c0(), nl, c->d_pmod, nullptr,
+            key_switch_inner(c, keys, D, l, gs[k0 + k], gs[k0 + k], acc.ptr + k * es, a.c0(), nl, c->d_pmod, nullptr,
                              a.nb, a.cstride());
             outs.push_back(new_ct(c, l, a.scale, a.nb));
             o.push_back(outs.back().buf.ptr);
@@ -809,7 +840,7 @@ ckks_ct mul_relin(const ckks_keys& keys, const ckks_ct& a, const ckks_ct& b) {
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel; then
     // ModDown (= (d0, d1) + ModDown(k), see switch_galois)
-    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
+    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l, a.scale * b.scale, a.nb);
     mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
@@ -829,7 +860,7 @@ ckks_ct mul_relin_rescale(const ckks_keys& keys, const ckks_ct& a, const ckks_ct
     const Raised D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, a.nb, ds);
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel
-    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, false, d.ptr, nl, c->d_pmod,
+    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l - 1, a.scale * b.scale / (double)c->q[l], a.nb);
     mod_down_rescale(c, acc.ptr, l, o.buf.ptr, twice, a.nb);
@@ -869,7 +900,7 @@ static std::vector<DevBuf> rotate_hoisted_ext(const ckks_keys& keys, const ckks_
         } else {
             if (!D.x) D = mod_up(c, a.c1(), l, a.nb, a.cstride());
             c->ops["hrot"]++;
-            key_switch_inner(c, keys, D, l, g, g, o.ptr, false, a.c0(), nl, c->d_pmod, nullptr, a.nb,
+            key_switch_inner(c, keys, D, l, g, g, o.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb,
                              a.cstride());
         }
         outs.push_back(std::move(o));
@@ -1038,9 +1069,9 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         }
     }
     // The rotated giant steps: their c1 sums brought down and raised together (one ModDown and one ModUp
-    // over several of them; a lockstep batch fills the launches by itself), then each key-switched into
-    // the sum.  Against one chain of launches per giant step on side streams with a sum of its own:
-    // conv at level 1 342 (one at a time) or 278 (side streams) -> 260 us, downsampling layer 12.2 -> 11.9 ms.
+    // over several of them; a lockstep batch fills the launches by itself), then key-switched into the sum.  Against one chain of launches per giant step on side streams with a sum of its own:
+    // conv at level 1 342 (one at a time) or 278 (side streams) -> 260 us, downsampling layer 12.2 -> 11.9 ms
+    // (further with one key-switch kernel for them all, k_ks_rotations).
     const int group = std::max(1, 16 / nb);
     u64* acc = nrot < nslots ? inner.ptr + (size_t)nrot * nb * es : nullptr;       // the R = 0 giant's sum
     for (int k = nrot + 1; k < nslots; ++k)
@@ -1052,17 +1083,14 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         DevBuf c1q((size_t)gn * nb * nl * n, c->stream);
         mod_down_poly(c, x + next * n, l, c1q.ptr, gn * nb, es);
         const Raised D = mod_up(c, c1q.ptr, l, gn * nb, (size_t)nl * n);
-        for (int k = 0; k < gn; ++k) {
-            const u64 gal = galois_of_step(c, rots[k0 + k]);
-            c->ops["hrot"]++;
-            const bool have = acc != nullptr;
-            if (!have) {
-                acc_buf = DevBuf(nb * es, c->stream);
-                acc = acc_buf.ptr;
-            }
-            key_switch_inner(c, keys, D, l, gal, gal, acc, have, x + (size_t)k * nb * es, (int)next, nullptr, nullptr,
-                             nb, es, k * nb);
+        std::vector<u64> gals;
+        for (int k = 0; k < gn; ++k) gals.push_back(galois_of_step(c, rots[k0 + k]));
+        const bool have = acc != nullptr;
+        if (!have) {
+            acc_buf = DevBuf(nb * es, c->stream);
+            acc = acc_buf.ptr;
         }
+        key_switch_rotations(c, keys, D, l, gals, acc, have, x, nb, es);
     }
     if (rescale_out) {
         ckks_ct o = new_ct(c, l - 1, scale / (double)c->q[l], nb);

@@ -96,3 +96,29 @@ def test_batched_pairs_match_single(B, q0, spec):
         del WL.PARAMS["fold_test"]
         d = K = ctx = keys = outs = c = out = one = None
         gc.collect()
+
+
+# more rotated giant steps than one sum holds (9 at four digits, 13 at three, 16 otherwise) and than are
+# raised together, with and without an unrotated one to add to
+@pytest.mark.parametrize("log_n,q0,dnum,n_q", [(10, 60, 4, 4), (10, 61, 4, 4), (10, 60, 3, 5), (13, 60, 2, 4)])
+@pytest.mark.parametrize("a0", [0, 1])
+def test_many_giant_steps_bitexact(log_n, q0, dnum, n_q, a0):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_04356_gb300 import build
+    build.build()
+    WL.PARAMS["fold_test"] = dict(log_n=log_n, n_q=n_q, dnum=dnum, n_p=0, q0_bits=q0, scale_bits=42, p_bits=60,
+                                  boot_bits=0, n_boot=0, h=0, sigma=3.2)
+    try:
+        m = 1 << (log_n - 1)
+        K, o, ctx, keys = make_pair("fold_test", 35, rotations=list(range(1, 22)))
+        P, lev = o.P, o.P.L
+        ct = o.encrypt(o.encode_pt(WL.slots(1, m, 0.5), lev, P.delta[lev]), 1)
+        plan = o.make_plan({a0 + i: WL.slots(60 + i, m) for i in range(20)}, a0, 1, 20, lev, P.delta[lev], B=1)
+        got = K.ckks_bsgs(ctx, keys, import_ct(K, ctx, ct), import_plan(K, ctx, plan))
+        assert_ct_equal(K, ctx, got, o.bsgs(ct, plan), "20 giant steps from %d" % a0)
+        K.ckks_sync(ctx)
+    finally:
+        del WL.PARAMS["fold_test"]
+        K = o = ctx = keys = ct = got = plan = None
+        gc.collect()
