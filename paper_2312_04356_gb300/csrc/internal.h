@@ -494,20 +494,7 @@ unsigned take_device_faults();
 unsigned peek_device_faults();   // the same count, not cleared
 // test hook: withhold the tensor-core conversion's MMAs so that its bounded waits run out
 void set_tc_withhold(bool on);
-// key-switch inner product: raised digits D, key rows krow[e] of [ndig][nall][N];
-// ob/oa [next][N] = sum_d D_d(sigma_g) * key_d ; g = 1 means no automorphism
-// x0 (optional, rows [x0rows][N] with the primes of the first x0rows extended limbs): ob row e
-// += s[e] * x0[e](sigma_g) for e < x0rows (s null: unscaled), the automorphed c0 term of a
-// rotation, gathered with the same permutation as D; x1 (optional) likewise into oa (the
-// P-lifted d0, d1 of a relinearisation, g = 1)
-// (bt: a batch of bt.nb ciphertexts switched with the same key, D at + t dstr, ob / oa at + t ostr,
-// x0 / x1 at + t xstr; at most 4 digits)
-void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
-              const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0 = nullptr, int x0rows = 0,
-              const u64* s = nullptr, const u64* x1 = nullptr, const KsBatch& bt = KsBatch());
-// The key switches of nr rotations by g[k], each of its own polynomial (number k bt.nb + t of D for
-// ciphertext t) with its own key, and x0(sigma_k) on every row (x0 [nr][bt.nb] at stride bt.xstr), summed
-// into ob / oa (added to what they hold when accumulating) without intermediate reductions.
+// one or several key switches: keys b, a ([ndig][nall][N]) and automorphisms g[k]
 struct KsRotations {
     static constexpr int MAXR = 16;
     // rotations whose products one 128-bit sum holds (40 products, the x0 and the previous words within one)
@@ -516,7 +503,26 @@ struct KsRotations {
     const u64* kb[MAXR];
     const u64* ka[MAXR];
     u64 g[MAXR];
+    void add(const u64* b, const u64* a, u64 gal) {
+        kb[nr] = b;
+        ka[nr] = a;
+        g[nr++] = gal;
+    }
 };
+// key-switch inner products of one polynomial: raised digits D, for every k of R
+// ob/oa + k rstr [next][N] = sum_d D_d(sigma_k) * key_k,d ; g = 1 means no automorphism
+// x0 (optional, rows [x0rows][N] with the primes of the first x0rows extended limbs): ob row e
+// += s[e] * x0[e](sigma_k) for e < x0rows (s null: unscaled), the automorphed c0 term of a
+// rotation, gathered with the same permutation as D; x1 (optional) likewise into oa (the
+// P-lifted d0, d1 of a relinearisation, g = 1)
+// (bt: a batch of bt.nb ciphertexts switched with the same key, D at + t dstr, ob / oa at + t ostr,
+// x0 / x1 at + t xstr; at most 4 digits)
+void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const KsRotations& R, u64* ob,
+              u64* oa, size_t rstr, const u64* x0 = nullptr, int x0rows = 0, const u64* s = nullptr,
+              const u64* x1 = nullptr, const KsBatch& bt = KsBatch());
+// The key switches of R, each of its own polynomial (number k bt.nb + t of D for ciphertext t), and
+// x0(sigma_k) on every row (x0 [nr][bt.nb] at stride bt.xstr), summed into ob / oa (added to what they hold
+// when accumulating) without intermediate reductions.
 void ks_rotations(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const KsRotations& R,
                   const u64* x0, u64* ob, u64* oa, bool accumulate, const KsBatch& bt);
 // d0 = a0 b0, d1 = a0 b1 + a1 b0 (d [2][nl][N]), d2 = a1 b1 (e [nl][N]) over nl limbs with

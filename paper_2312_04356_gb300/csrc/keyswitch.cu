@@ -224,12 +224,13 @@ __global__ void __launch_bounds__(256, NC == 1 ? 3 : 2)
 // outputs at ob / oa + t ostr, its x0 / x1 at + t xstr.  The ciphertext index is the fastest
 // varying part of blockIdx.x, so the CTAs that read the same key words run side by side and
 // all but the first find them in L2: the key streams from HBM about once per batch.
+// Several rotations of one polynomial (blockIdx.z, outputs at ob / oa + z rstr) share a launch.
 // NC of its ciphertexts share a thread and with it the key words and the automorphism.  Eight ciphertexts,
 // the 49 of a block: 5.86 -> 5.71 ms (4.7 TB/s of algorithmic bytes).
 template <bool FOLD, int V, int NDIG, int NC>
 __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, const int* __restrict__ ext_ids,
-                             const u64* __restrict__ kb, const u64* __restrict__ ka, u64* __restrict__ ob,
-                             u64* __restrict__ oa, const DevPrime* __restrict__ P, int logn, u64 g, size_t kstride,
+                             const __grid_constant__ kern::KsRotations R, u64* __restrict__ ob, u64* __restrict__ oa,
+                             size_t rstr, const DevPrime* __restrict__ P, int logn, size_t kstride,
                              const u64* __restrict__ x0, const u64* __restrict__ x1, int x0rows,
                              const u64* __restrict__ s0, kern::KsBatch bt) {
     griddep_entry();
@@ -240,8 +241,9 @@ __global__ void k_ks_inner_d(const __grid_constant__ kern::Digits D, int next, c
     const int groups = bt.nb / NC, t = blockIdx.x % groups * NC;
     const int j = V * ((blockIdx.x / groups) * blockDim.x + threadIdx.x);
     if (j >= (int)n) return;
-    ob += t * bt.ostr + (size_t)e * n + j;
-    oa += t * bt.ostr + (size_t)e * n + j;
+    const u64 *kb = R.kb[blockIdx.z], *ka = R.ka[blockIdx.z], g = R.g[blockIdx.z];
+    ob += blockIdx.z * rstr + t * bt.ostr + (size_t)e * n + j;
+    oa += blockIdx.z * rstr + t * bt.ostr + (size_t)e * n + j;
     if (x0) x0 += t * bt.xstr + (size_t)e * n;
     if (x1) x1 += t * bt.xstr + (size_t)e * n;
     unsigned src[V];
@@ -538,15 +540,16 @@ void bsgs_fused(const ckks_ctx* c, const BsgsFused& t, const Digits& D, const u6
 }
 
 template <bool FOLD, int V, int NC>
-static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
-                               const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
-                               const u64* s0, const KsBatch& bt) {
+static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids,
+                               const KsRotations& R, u64* ob, u64* oa, size_t rstr, const u64* x0, const u64* x1,
+                               int x0rows, const u64* s0, const KsBatch& bt) {
     dim3 grid = ewv_grid(c->n, next, V);
     grid.x *= bt.nb / NC;
+    grid.z = R.nr;
     const size_t ks = (size_t)c->nall << c->logn;
-#define KS_CASE(NDIG)                                                                                                  \
-    klaunch(c, k_ks_inner_d<FOLD, V, NDIG, NC>, grid, EW_THREADS, 0, D, next, ext_ids, kb, ka, ob, oa, c->d_primes,      \
-            c->logn, g, ks, x0, x1, x0rows, s0, bt)
+#define KS_CASE(NDIG)                                                                                                   \
+    klaunch(c, k_ks_inner_d<FOLD, V, NDIG, NC>, grid, EW_THREADS, 0, D, next, ext_ids, R, ob, oa, rstr, c->d_primes,    \
+            c->logn, ks, x0, x1, x0rows, s0, bt)
     switch (ndig) {
         case 1: KS_CASE(1); break;
         case 2: KS_CASE(2); break;
@@ -558,33 +561,38 @@ static void launch_ks_inner_nc(const ckks_ctx* c, const Digits& D, int ndig, int
 
 // the ciphertexts of a batch in pairs, the last of an odd number by itself
 template <bool FOLD, int V>
-static void launch_ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
-                            const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, const u64* x1, int x0rows,
+static void launch_ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids,
+                            const KsRotations& R, u64* ob, u64* oa, size_t rstr, const u64* x0, const u64* x1, int x0rows,
                             const u64* s0, const KsBatch& bt) {
     KsBatch part = bt;
     part.nb = bt.nb & ~1;
-    if (part.nb)
-        launch_ks_inner_nc<FOLD, V, 2>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s0, part);
+    if (part.nb) launch_ks_inner_nc<FOLD, V, 2>(c, D, ndig, next, ext_ids, R, ob, oa, rstr, x0, x1, x0rows, s0, part);
     if (bt.nb & 1) {
         const size_t k = part.nb;
         part.nb = 1;
-        launch_ks_inner_nc<FOLD, V, 1>(c, digits_from(D, k, bt.dstr), ndig, next, ext_ids, kb, ka, ob + k * bt.ostr,
-                                            oa + k * bt.ostr, g, x0 ? x0 + k * bt.xstr : x0, x1 ? x1 + k * bt.xstr : x1,
-                                            x0rows, s0, part);
+        launch_ks_inner_nc<FOLD, V, 1>(c, digits_from(D, k, bt.dstr), ndig, next, ext_ids, R, ob + k * bt.ostr,
+                                       oa + k * bt.ostr, rstr, x0 ? x0 + k * bt.xstr : x0, x1 ? x1 + k * bt.xstr : x1,
+                                       x0rows, s0, part);
     }
 }
 
-void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const u64* kb,
-              const u64* ka, u64* ob, u64* oa, u64 g, const u64* x0, int x0rows, const u64* s,
-              const u64* x1, const KsBatch& bt) {
-    CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4, CKKS_EINVAL, "key switching takes 1..4 digits");
-    const bool vec = al16(kb) && al16(ka) && al16(ob) && al16(oa);
+static bool al16_keys(const KsRotations& R) {
+    bool vec = true;
+    for (int k = 0; k < R.nr; ++k) vec = vec && al16(R.kb[k]) && al16(R.ka[k]);
+    return vec;
+}
+
+void ks_inner(const ckks_ctx* c, const Digits& D, int ndig, int next, const int* ext_ids, const KsRotations& R, u64* ob,
+              u64* oa, size_t rstr, const u64* x0, int x0rows, const u64* s, const u64* x1, const KsBatch& bt) {
+    CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4 && R.nr >= 1 && R.nr <= KsRotations::MAXR, CKKS_EINVAL,
+             "key switching takes 1..4 digits");
+    const bool vec = al16_keys(R) && al16(ob) && al16(oa) && rstr % 2 == 0;
     {
-        // algorithmic bytes: the key once for the whole batch, per ciphertext its digits, outputs
+        // algorithmic bytes: the keys once for the whole batch, per ciphertext its digits, outputs
         // and the x0 / x1 rows
         const double extra = x0 ? (double)x0rows * (x1 ? 2.0 : 1.0) / next : 0.0;
-        KTimer kt_(c, "ks_inner", (2.0 * ndig + bt.nb * (ndig + 2.0 + extra)) * next * c->n * 8.0);
-#define KS(FOLD, V) launch_ks_inner<FOLD, V>(c, D, ndig, next, ext_ids, kb, ka, ob, oa, g, x0, x1, x0rows, s, bt)
+        KTimer kt_(c, "ks_inner", R.nr * (2.0 * ndig + bt.nb * (ndig + 2.0 + extra)) * next * c->n * 8.0);
+#define KS(FOLD, V) launch_ks_inner<FOLD, V>(c, D, ndig, next, ext_ids, R, ob, oa, rstr, x0, x1, x0rows, s, bt)
         if (c->fold && vec) KS(true, 2);
         else if (c->fold) KS(true, 1);
         else KS(false, 1);
@@ -622,8 +630,7 @@ void ks_rotations(const ckks_ctx* c, const Digits& D, int ndig, int next, const 
                   const u64* x0, u64* ob, u64* oa, bool accumulate, const KsBatch& bt) {
     CK_CHECK(bt.nb >= 1 && ndig >= 1 && ndig <= 4 && R.nr >= 1 && R.nr <= KsRotations::fits(ndig), CKKS_EINVAL,
              "key switching takes 1..4 digits and as many rotations as one sum holds");
-    bool vec = al16(ob) && al16(oa);
-    for (int k = 0; k < R.nr; ++k) vec = vec && al16(R.kb[k]) && al16(R.ka[k]);
+    const bool vec = al16_keys(R) && al16(ob) && al16(oa);
     {
         // algorithmic bytes: the keys once for the whole batch, per ciphertext its digits and x0 rows, and
         // the outputs (read too when accumulating)

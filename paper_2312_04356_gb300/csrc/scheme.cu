@@ -648,31 +648,43 @@ Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride =
     return r;
 }
 
-// inner product with switching key `code` (automorphism g applied to D on the fly) over
-// Q_l u P: acc [2][next][N], NTT domain.  With x0, the
-// first x0rows rows of acc's first half also receive s x0(sigma_g) (s null: x0(sigma_g)), the
-// automorphed c0 term of a rotation, in the same kernel.
-// For a batch of nb ciphertexts: acc [nb][2][next][N], x0 / x1 of ciphertext t
-// at + t xstr; the key is read once for the batch.
 static const SwitchKey& switching_key(const ckks_keys& keys, u64 code) {
     auto it = keys.swk.find(code);
     CK_CHECK(it != keys.swk.end(), CKKS_ENOKEY, "missing switching key (code " + std::to_string(code) + ")");
     return *it->second;
 }
-void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int level, u64 code, u64 g,
-                      u64* acc, const u64* x0 = nullptr, int x0rows = 0, const u64* s = nullptr,
-                      const u64* x1 = nullptr, int nb = 1, size_t xstr = 0) {
-    const SwitchKey& k = switching_key(keys, code);
-    c->ops["keyswitch"]++;
+
+// strides of a batch of nb ciphertexts at a level: digits, outputs [2][next][N], x0 / x1
+static kern::KsBatch ks_batch(const ckks_ctx* c, const Raised& D, int level, int nb, size_t xstr) {
     const size_t next = (size_t)level + 1 + c->np;
     kern::KsBatch bt;
     bt.nb = nb;
     bt.dstr = (size_t)D.ndig * next * c->n;
     bt.ostr = 2 * next * c->n;
     bt.xstr = xstr;
+    return bt;
+}
+
+// inner products with the switching keys of `codes` (automorphisms gs applied to D on the fly) over
+// Q_l u P: acc [codes][2][next][N], NTT domain.  With x0, the
+// first x0rows rows of acc's first half also receive s x0(sigma_g) (s null: x0(sigma_g)), the
+// automorphed c0 term of a rotation, in the same kernel.
+// For a batch of nb ciphertexts: acc [codes][nb][2][next][N], x0 / x1 of ciphertext t
+// at + t xstr; the key is read once for the batch.
+void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int level, const std::vector<u64>& codes,
+                      const std::vector<u64>& gs, u64* acc, const u64* x0 = nullptr, int x0rows = 0,
+                      const u64* s = nullptr, const u64* x1 = nullptr, int nb = 1, size_t xstr = 0) {
+    const size_t next = (size_t)level + 1 + c->np;
+    const kern::KsBatch bt = ks_batch(c, D, level, nb, xstr);
+    kern::KsRotations R;
+    for (size_t k = 0; k < codes.size(); ++k) {
+        const SwitchKey& key = switching_key(keys, codes[k]);
+        c->ops["keyswitch"]++;
+        R.add(key.b.ptr, key.a.ptr, gs[k]);
+    }
     const kern::Digits dig{D.D.ptr, D.x, D.xstride, level + 1, c->alpha};
-    kern::ks_inner(c, dig, D.ndig, (int)next, c->d_ext_ids[level], k.b.ptr, k.a.ptr, acc, acc + next * c->n, g,
-                   x0, x0rows, s, x1, bt);
+    kern::ks_inner(c, dig, D.ndig, (int)next, c->d_ext_ids[level], R, acc, acc + next * c->n, nb * bt.ostr, x0, x0rows, s,
+                   x1, bt);
 }
 
 // sum over rotations gs[k] of the key switch of D's polynomials k nb .. (k + 1) nb - 1, plus x0(sigma_k) of
@@ -681,11 +693,7 @@ static void key_switch_rotations(ckks_ctx* c, const ckks_keys& keys, const Raise
                                  const std::vector<u64>& gs, u64* acc, bool accumulate, const u64* x0, int nb,
                                  size_t xstr) {
     const size_t next = (size_t)level + 1 + c->np;
-    kern::KsBatch bt;
-    bt.nb = nb;
-    bt.dstr = (size_t)D.ndig * next * c->n;
-    bt.ostr = 2 * next * c->n;
-    bt.xstr = xstr;
+    const kern::KsBatch bt = ks_batch(c, D, level, nb, xstr);
     const size_t per = kern::KsRotations::fits(D.ndig);
     for (size_t k0 = 0; k0 < gs.size(); k0 += per) {
         kern::KsRotations R;
@@ -693,9 +701,7 @@ static void key_switch_rotations(ckks_ctx* c, const ckks_keys& keys, const Raise
             const SwitchKey& key = switching_key(keys, gs[k]);
             c->ops["hrot"]++;
             c->ops["keyswitch"]++;
-            R.kb[R.nr] = key.b.ptr;
-            R.ka[R.nr] = key.a.ptr;
-            R.g[R.nr++] = gs[k];
+            R.add(key.b.ptr, key.a.ptr, gs[k]);
         }
         const size_t first = k0 * nb;
         const kern::Digits dig{D.D.ptr + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
@@ -763,8 +769,8 @@ u64 galois_of_step(const ckks_ctx* c, long long r) {
 // rot_g(a) for every g and every ciphertext of a: the key switches of the automorphed raised digits D
 // of c1 with P c0(sigma_g) added on the Q rows in the same kernel, then ModDown: ModDown(P x + k) = x +
 // ModDown(k) exactly (P x vanishes on the P rows), so this is automorph(c0) + ModDown(k) in
-// fewer passes.  Several rotations are brought down together (eight rotations at level 9, summed:
-// 621 -> 515 us).
+// fewer passes.  Several rotations are key-switched and brought down together (eight rotations at
+// level 9, summed: 621 -> 476 us).
 static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& a, const Raised& D,
                                           const std::vector<u64>& gs) {
     ckks_ctx* c = a.ctx;
@@ -776,9 +782,9 @@ static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& 
         const size_t cnt = std::min(group, gs.size() - k0);
         DevBuf acc(cnt * es, c->stream);
         std::vector<u64*> o;
+        const std::vector<u64> part(gs.begin() + k0, gs.begin() + k0 + cnt);
+        key_switch_inner(c, keys, D, l, part, part, acc.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb, a.cstride());
         for (size_t k = 0; k < cnt; ++k) {
-            key_switch_inner(c, keys, D, l, gs[k0 + k], gs[k0 + k], acc.ptr + k * es, a.c0(), nl, c->d_pmod, nullptr,
-                             a.nb, a.cstride());
             outs.push_back(new_ct(c, l, a.scale, a.nb));
             o.push_back(outs.back().buf.ptr);
         }
@@ -840,7 +846,7 @@ ckks_ct mul_relin(const ckks_keys& keys, const ckks_ct& a, const ckks_ct& b) {
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel; then
     // ModDown (= (d0, d1) + ModDown(k), see switch_galois)
-    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, d.ptr, nl, c->d_pmod,
+    key_switch_inner(c, keys, D, l, {0}, {1}, acc.ptr, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l, a.scale * b.scale, a.nb);
     mod_down(c, acc.ptr, l, o.buf.ptr, a.nb);
@@ -860,7 +866,7 @@ ckks_ct mul_relin_rescale(const ckks_keys& keys, const ckks_ct& a, const ckks_ct
     const Raised D = mod_up(c, d.ptr + 2 * (size_t)nl * n, l, a.nb, ds);
     DevBuf acc((size_t)a.nb * 2 * ((size_t)nl + c->np) * n, c->stream);
     // relinearisation key switch with P d0, P d1 added on the Q rows in the same kernel
-    key_switch_inner(c, keys, D, l, 0, 1, acc.ptr, d.ptr, nl, c->d_pmod,
+    key_switch_inner(c, keys, D, l, {0}, {1}, acc.ptr, d.ptr, nl, c->d_pmod,
                      d.ptr + (size_t)nl * n, a.nb, ds);
     ckks_ct o = new_ct(c, l - 1, a.scale * b.scale / (double)c->q[l], a.nb);
     mod_down_rescale(c, acc.ptr, l, o.buf.ptr, twice, a.nb);
@@ -900,7 +906,7 @@ static std::vector<DevBuf> rotate_hoisted_ext(const ckks_keys& keys, const ckks_
         } else {
             if (!D.x) D = mod_up(c, a.c1(), l, a.nb, a.cstride());
             c->ops["hrot"]++;
-            key_switch_inner(c, keys, D, l, g, g, o.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb,
+            key_switch_inner(c, keys, D, l, {g}, {g}, o.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb,
                              a.cstride());
         }
         outs.push_back(std::move(o));
