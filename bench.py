@@ -48,10 +48,11 @@ L2_BYTES = 129e6
 # read 146.3 MB + write 3.6 MB.
 KS_DRAM_PER_ALGO_BYTE = (146.3 + 3.6) / (365 * 65536 * 8 / 1e6)
 ROOF_NOTES = {
-    "ntt_fwd": "integer-multiply-pipe bound (fmaheavy 67-74% busy, DRAM 24-35% under ncu): the roofline is that "
-               "pipe's (64 lanes per SM per clock, 16 lane-cycles per 64-bit Shoup butterfly); hbm_view gives "
+    "ntt_fwd": "integer-pipe bound in large launches (70% of the butterflies' own arithmetic at 128 limbs), latency "
+               "bound in small ones: the roofline is the multiply pipe's for Shoup products (64 lanes per SM per "
+               "clock, 16 lane-cycles per 64-bit butterfly; the folded products that run need 10); hbm_view gives "
                "the same launches against HBM",
-    "bsgs_fused": "integer-multiply-pipe bound after asynchronous staging (fmaheavy 77% busy, DRAM 46% under ncu)",
+    "bsgs_fused": "HBM bound with one ciphertext (keys and diagonals streamed once); a batch is bound by the integer pipes",
     "ks_inner": "HBM bound: switching keys streamed once (evict-first), raised digits gathered through the Galois "
                 "permutation; DRAM 55% of peak under ncu with cold caches",
 }
@@ -173,6 +174,8 @@ def peaks():
 # SM sub-partition per clock, 64 per SM: peak butterflies/s = 64 * SMs * clock / 16.  A
 # transform of one limb does 16 stages of N/2 butterflies and has 2 N 8 algorithmic bytes (one
 # read, one write), so the butterflies are the algorithmic bytes / 2 (per pass or per launch).
+# The library's folded products (primes next to a power of two) take 5 wide multiplies, 10 lane-cycles;
+# the line stays that of the Shoup form, so that its fractions compare over time.
 NTT_MUL_LANE_CYCLES_PER_BUTTERFLY = 16
 GB300_SMS = 152
 
