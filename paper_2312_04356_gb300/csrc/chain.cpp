@@ -79,9 +79,11 @@ bool fold_consts(u64 q, FoldMod& f) {
     // folded value of any word, and the two classes' largest lazy value
     const u128 opened = ((u128)1 << K) + (ae << (63 - K));
     const bool big = 17 * R > ((u128)1 << 62);
-    const u128 top = big ? opened + 4 * R : 4 * (u128)q + 16 * R;        // forward
+    // Forward: what a transform takes (residues, lifted words within opened, a conversion's words within
+    // 2^K + 2^16 |e|: 128 chunk products below 2^8 q, folded once), then R a stage.
+    const u128 top = big ? opened + 4 * R : std::max(4 * (u128)q, opened) + 16 * R;
     const u128 inv = big ? 4 * (R > opened ? R : opened) : 16 * (R > opened ? R : opened);
-    if (top > lim || inv > lim) return false;
+    if (top + q > lim || inv > lim) return false;                        // + q: a tail takes a - x
     if ((big ? ((u128)8 << (60 - K)) : (top >> K) + 1) * ae >= q) return false;   // canonical after one fold
     // |x0 W0 + x1 W1| <= (2^31 + |x1|) q / 2 < 2^(K + 31)
     if ((((u128)1 << 31) + (lim >> 32) + 2) * q >= ((u128)1 << (K + 32))) return false;

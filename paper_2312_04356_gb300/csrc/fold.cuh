@@ -1,10 +1,15 @@
 // Modular arithmetic for primes next to a power of two.
 //
-// Every prime the chain construction picks lies next to 2^K: q_0 and the special primes are the
-// largest below 2^60, the scaling primes the nearest to 2^42 or 2^48, so
+// A chain's primes lie next to powers of two: q_0 and the special primes are the largest below theirs,
+// the scaling primes the nearest to the scale.  So
 //     2^K = e (mod q),   e = 2^K - q,   |e| < 2^26,
 // and the part of a number above bit K is brought back ("folded") by one multiplication by a
-// 32-bit constant.  Values are signed 64-bit words that are only congruent to the residue.  A
+// 32-bit constant.  hostmath::fold_consts says which primes qualify: 33 to 60 bits but not 57, and |e| small
+// enough for one fold to make any value of a transform canonical, which is the tighter bound at 33 to 42 bits
+// (|e| below about 2^24.5 at 42 bits, 2^22.7 at 40, 2^18.5 at 36) and lets every |e| < 2^26 through from 43 bits on
+// (2^25 at 58).  The chains of the named parameter sets qualify.  A long chain of primes
+// at 42 bits or less does not: the primes run away from 2^K (N = 2^16, 24 limbs of 42 bits: 7 of 32
+// refused; none at 45 or 48 bits), and one refused prime puts the whole context on Shoup products.  Values are signed 64-bit words that are only congruent to the residue.  A
 // product with a constant w is taken as
 //     x w = x0 W0 + x1 W1 (mod q),   x = x1 2^32 + x0,  W0 = w,  W1 = w 2^32 mod q,
 // with W0, W1 the representatives in [-q/2, q/2] and every low half (x0, the low halves of W0 and
