@@ -19,6 +19,7 @@ namespace {
 // is reduced on odd stages only; an uncorrected stage maps [0, b q) to [0, (b + 2) q), a corrected
 // one, valid for b <= 8, to [0, 6q)), inverse values below 2q.
 struct ArShoup {
+    static constexpr bool LAZY = false;   // in k_ntt_pass
     u64 q, q2;
     __device__ __forceinline__ explicit ArShoup(const DevPrime* P) : q(P->m.q), q2(2 * P->m.q) {}
     __device__ __forceinline__ bool folds() const { return false; }
@@ -55,6 +56,7 @@ struct ArShoup {
 // Inverse: a sum doubles per stage, so a group of four stages ends with its sums folded (16 R < 2^62),
 // and 60-bit primes fold them after two stages as well (4.2 2^60 at most).
 struct ArFold {
+    static constexpr bool LAZY = true;
     u64 q;
     FoldMod f;
     __device__ __forceinline__ explicit ArFold(const DevPrime* P) : q(P->m.q), f(P->f) {}
@@ -204,6 +206,10 @@ __device__ __forceinline__ OutFactor out_factor(const DevPrime* P, const u64* os
 // ---- any ring: c consecutive stages from s0 in shared memory, one barrier per stage.  Only index
 // bits log2(T1)..log2(T0) move (T0 = N >> (s0+1), T1 = N >> (s0+c)), so the limb splits into
 // independent sub-problems of 2^c elements j = hi*2T0 + k*T1 + lo; a CTA stages 2^logsub of them.
+// ArShoup keeps canonical values throughout.  ArFold's are lazy, with the folds of ArFold's ranges:
+// a product made canonical in every butterfly costs more than a Shoup product (N = 2^15, 200 limbs,
+// forward: 238 us, 210 with Shoup products, 198 lazy; N = 2^13, rescale at level 5: 90, 87, 82).
+// A transform of more than sixteen stages (N = 2^17) is folded between its passes.
 constexpr int NTT_THREADS = 256;
 
 template <class AR, bool INV>
@@ -238,7 +244,7 @@ __global__ void __launch_bounds__(NTT_THREADS)
         }
         int sid = sid0 + s;
         size_t j = ((size_t)(sid >> logT1) << log2T0) + ((size_t)k << logT1) + (sid & (T1 - 1));
-        sm[k * stride + s] = !INV && s0 == 0 ? ar.canon(a[j]) : a[j];
+        sm[k * stride + s] = a[j];
     }
     __syncthreads();
 
@@ -257,17 +263,30 @@ __global__ void __launch_bounds__(NTT_THREADS)
             const int widx = (1 << sg) + (int)(j >> (logn - sg));
             u64* px = sm + k * stride + s;
             u64* py = sm + (k + tk) * stride + s;
-            const u64 x = *px, y = *py;
-            // canonical values throughout
-            if (!INV) {
-                const ulonglong2 w = P->tw[widx];
-                const u64 v = ar.scale(y, w);
-                *px = add_mod(x, v, q);
-                *py = sub_mod(x, v, q);
+            u64 x = *px, y = *py;
+            const ulonglong2 w = (INV ? P->itw : P->tw)[widx];
+            if constexpr (!AR::LAZY) {
+                if (!INV) {
+                    const u64 v = ar.scale(y, w);
+                    *px = add_mod(x, v, q);
+                    *py = sub_mod(x, v, q);
+                } else {
+                    *px = add_mod(x, y, q);
+                    *py = ar.scale(sub_mod(x, y, q), w);
+                }
+            } else if (!INV) {
+                if (u % 4 == 0 && (ar.folds() || (u == 0 && s0 + c > 16))) {
+                    x = ar.open(x);
+                    y = ar.open(y);
+                }
+                ar.template fwd<0>(x, y, w);
+                *px = x;
+                *py = y;
             } else {
-                *px = add_mod(x, y, q);
-                const ulonglong2 w = P->itw[widx];
-                *py = ar.scale(sub_mod(x, y, q), w);
+                ar.inv(x, y, w);
+                if (u % 4 == 3 || u == c - 1 || (ar.folds() && u % 2)) x = ar.sum_out(x);
+                *px = x;
+                *py = y;
             }
         }
         __syncthreads();
@@ -288,6 +307,7 @@ __global__ void __launch_bounds__(NTT_THREADS)
         size_t j = ((size_t)(sid >> logT1) << log2T0) + ((size_t)k << logT1) + (sid & (T1 - 1));
         u64 v = sm[k * stride + s];
         if (scale_out) v = ar.scale(v, ni);
+        if (AR::LAZY && !INV && T1 == 1) v = ar.canon(v);
         a[j] = v;
     }
 }
