@@ -144,14 +144,15 @@ int ckks_ctx_reset_counters(ckks_ctx* ctx);
 int ckks_ctx_kernel_stats(ckks_ctx* ctx, char* buf, int cap, int* len);
 
 /* Autotuner: times each NTT launch variant (two passes of 8 stages with 16 values per thread
- * and 8 columns / 4 rows, 16 or 4 sub-problems per CTA at two register budgets, or 4 values
+ * in CTAs of 16 or 4 sub-problems or of the shape each pass likes best, or 4 values
  * per thread; or the whole transform in one launch by a cluster of 8 CTAs that exchange the
  * half-transformed data through distributed shared memory) for limb counts 1, 2, 7, 14, 24, 48,
  * 96, 192 (forward + inverse, `reps` repetitions, 0 = 3) and keeps the fastest per size class for
  * this context.  All variants compute the same residues.  choice8 (may be NULL) receives the
- * chosen variant per class (0: 8 columns / 4 rows per CTA, 1: 16 of either, 2: 4, 3: 4 with at
- * most 80 registers, 4: 4 values per thread, 5: one-launch cluster; -1: default, the same as 0).
- * Only N = 2^16 has variants.  Synchronises the stream. */
+ * chosen variant per class (0: 16 sub-problems per CTA, 2: 4, 3: 4 with fewer registers, 4: 4 values per
+ * thread, 5: one-launch cluster; 1: 8 columns and 2 or 4 rows per CTA in contexts whose primes all lie next
+ * to powers of two, 16 sub-problems with 64 registers in others; -1: the default, 1 in the former and 2 in
+ * the latter).  Only N = 2^16 has variants.  Synchronises the stream. */
 int ckks_autotune(ckks_ctx* ctx, int reps, int32_t* choice8);
 /* Use one NTT variant (0..5 as above) for every size, or -1 for the default rule. */
 int ckks_ctx_set_ntt_variant(ckks_ctx* ctx, int variant);

@@ -773,8 +773,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(CL_THREADS, 2)
     }
 }
 
-// Launch shapes (identical results).  NTT_MIX, the default at every size, takes the best shape of
-// each pass: 8 columns per COL CTA (64-byte runs; 4 columns leave half of every 64-byte access
+// Launch shapes (identical results).  NTT_MIX, the default of fold contexts at every size, takes the best
+// shape of each pass: 8 columns per COL CTA (64-byte runs; 4 columns leave half of every 64-byte access
 // unused, 14.3 against 10.3 us just to read and write 62 limbs in that pattern) and 2 or 4 rows
 // per ROW CTA (rows are contiguous, and CTAs of one or two warps fill the last wave best).  us per
 // pass with the CTA's sub-problems x least resident CTAs, 62 / 368 limbs: forward COL 8x6 22.7 / 98,
@@ -783,41 +783,47 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(CL_THREADS, 2)
 // within 1 us of 8 to 12.  (Each figure holds about 4 us of the two events around the launch.)
 // What is left between these and the butterflies alone (31 cycles per warp and SM quarter: 75 us for
 // 368 limbs) are the loads of data and twiddles that other warps do not cover.  ckks_autotune times
-// every shape per limb-count class.  ArShoup contexts have NTT_V16 and NTT_V4 only.
+// every shape per limb-count class.  Contexts on Shoup products have 16 sub-problems at two register budgets
+// in the places of NTT_V16 and NTT_MIX; their default is NTT_V4 (64 / 200 limbs forward, events included:
+// 62 / 161 us, NTT_V16 65 / 172; inverse 65 / 173 and 66 / 180; a block 9.82 ms, NTT_V16 from 16 limbs on 10.04).
 enum NttVariant {
-    NTT_MIX = 0, NTT_V16 = 1, NTT_V4 = 2, NTT_V4_R80 = 3, NTT_X4 = 4, NTT_CL = 5, NTT_NVARIANTS = 6
+    NTT_V16 = 0, NTT_MIX = 1, NTT_V16_R64 = 1, NTT_V4 = 2, NTT_V4_R80 = 3, NTT_X4 = 4, NTT_CL = 5, NTT_NVARIANTS = 6
 };
+
+template <class AR, bool COL, bool INV, bool X>
+void launch_ntt16_ar(const ckks_ctx* cx, int v, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
+                     const int* loff, const u64* osc, const typename NttArgs<X && !INV && !COL>::type& io) {
+    constexpr bool FOLD = AR::LAZY;
+#define NTT16(SUBS, MINB)                                                                          \
+    klaunch(cx, k_ntt16<AR, COL, INV, SUBS, MINB, X>, dim3(256 / SUBS, nlimbs), 16 * SUBS, 0,      \
+            data, cx->d_primes, ids, lpp, pstride, loff, osc, io)
+    switch (v) {
+        case NTT_V16: NTT16(16, 3); break;
+        case NTT_MIX:
+            if constexpr (!FOLD) NTT16(16, 4);
+            else if constexpr (COL) NTT16(8, INV ? 5 : 6);
+            else if constexpr (INV) NTT16(4, 12);
+            else NTT16(2, 20);
+            break;
+        case NTT_V4: NTT16(4, 8); break;
+        case NTT_V4_R80: NTT16(4, 12); break;
+        default:
+            if constexpr (!X || INV)
+                klaunch(cx, k_ntt16s<AR, COL, INV, X>, dim3(256 / 4, nlimbs), 256, 0,
+                        data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
+            break;
+    }
+#undef NTT16
+}
 
 template <bool COL, bool INV, bool X = false>
 void launch_ntt16_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const int* ids, int lpp,
                           size_t pstride, const int* loff, const u64* osc,
                           const typename NttArgs<X && !INV && !COL>::type& io) {
-#define NTT16(AR, SUBS, MINB)                                                                      \
-    klaunch(cx, k_ntt16<AR, COL, INV, SUBS, MINB, X>, dim3(256 / SUBS, nlimbs), 16 * SUBS, 0,      \
-            data, cx->d_primes, ids, lpp, pstride, loff, osc, io)
-    if constexpr (!X || INV) {
-        if (!cx->fold) {
-            if (v == NTT_V16) NTT16(ArShoup, 16, 3);
-            else NTT16(ArShoup, 4, 8);
-            return;
-        }
+    if constexpr (!X || INV) {      // lifts and tails are built into the folded passes only
+        if (!cx->fold) return launch_ntt16_ar<ArShoup, COL, INV, X>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
     }
-    switch (v) {
-        case NTT_MIX:
-            if constexpr (COL) NTT16(ArFold, 8, INV ? 5 : 6);
-            else if constexpr (INV) NTT16(ArFold, 4, 12);
-            else NTT16(ArFold, 2, 20);
-            break;
-        case NTT_V16: NTT16(ArFold, 16, 3); break;
-        case NTT_V4: NTT16(ArFold, 4, 8); break;
-        case NTT_V4_R80: NTT16(ArFold, 4, 12); break;
-        default:
-            if constexpr (!X || INV)
-                klaunch(cx, k_ntt16s<ArFold, COL, INV, X>, dim3(256 / 4, nlimbs), 256, 0,
-                        data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
-            break;
-    }
-#undef NTT16
+    launch_ntt16_ar<ArFold, COL, INV, X>(cx, v, data, nlimbs, ids, lpp, pstride, loff, osc, io);
 }
 
 inline int ntt_class(int nlimbs) {
@@ -826,12 +832,12 @@ inline int ntt_class(int nlimbs) {
     return c;
 }
 
-template <bool INV>
+template <class AR, bool INV>
 void launch_ntt_cl(const ckks_ctx* cx, u64* data, int nlimbs, const int* ids, int lpp, size_t pstride,
                    const int* loff, const u64* osc, const NttSrc& io) {
     static std::atomic<unsigned> done{0};
-    allow_dynamic_smem((const void*)k_ntt_cl<ArFold, INV>, CL_SMEM_WORDS * (int)sizeof(u64), done);
-    klaunch(cx, k_ntt_cl<ArFold, INV>, dim3(8, nlimbs), CL_THREADS, CL_SMEM_WORDS * sizeof(u64),
+    allow_dynamic_smem((const void*)k_ntt_cl<AR, INV>, CL_SMEM_WORDS * (int)sizeof(u64), done);
+    klaunch(cx, k_ntt_cl<AR, INV>, dim3(8, nlimbs), CL_THREADS, CL_SMEM_WORDS * sizeof(u64),
             data, cx->d_primes, ids, lpp, pstride, loff, osc, io);
 }
 
@@ -846,9 +852,9 @@ void launch_ntt_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const 
     const char* nm = INV ? "ntt_inv" : "ntt_fwd";
     const double bytes = 2.0 * nlimbs * cx->n * 8.0;
     const int vc = vcol >= 0 ? vcol : v;
-    if (v == NTT_CL && cx->fold) {
+    if (v == NTT_CL) {
         KTimer kt_(cx, nm, bytes);
-        launch_ntt_cl<INV>(cx, data, nlimbs, ids, lpp, pstride, loff, osc, io);
+        (cx->fold ? launch_ntt_cl<ArFold, INV> : launch_ntt_cl<ArShoup, INV>)(cx, data, nlimbs, ids, lpp, pstride, loff, osc, io);
         return;
     }
     {
@@ -864,10 +870,10 @@ void launch_ntt_variant(const ckks_ctx* cx, int v, u64* data, int nlimbs, const 
     }
 }
 
-// the variant that transforms of nlimbs limbs use: the tuned one of their size class, else NTT_MIX
+// the variant that transforms of nlimbs limbs use: the tuned one of their size class, else the default
 inline int ntt_pick(const ckks_ctx* cx, int nlimbs) {
     const int v = cx->ntt_choice[ntt_class(nlimbs)];
-    return v >= 0 ? v : NTT_MIX;
+    return v >= 0 ? v : cx->fold ? NTT_MIX : NTT_V4;
 }
 
 template <bool INV>
@@ -1135,20 +1141,22 @@ void ntt_inverse_from(const ckks_ctx* c, const u64* src, size_t src_pstride, u64
 }
 
 bool ntt_host_io(const ckks_ctx* c, int nlimbs) {
-    return ntt_one_cta(c) || (c->logn == 16 && (!c->fold || ntt_pick(c, nlimbs) <= NTT_V4_R80));
+    return ntt_one_cta(c) || (c->logn == 16 && ntt_pick(c, nlimbs) <= NTT_V4_R80);
 }
 
 // Columns of a COL CTA that touches host memory: the link moves 128-byte runs (16 columns) of a large
 // transfer best (30 limbs out, whole export: 132 us with 64-byte runs, 122 with 128-byte ones, of which
-// the link alone takes about 90); small ones want the CTAs.  8 and 16 columns agree at 4 limbs.
-static int host_columns(int nlimbs) { return nlimbs >= 16 ? (int)NTT_V16 : -1; }
+// the link alone takes about 90); small ones want the CTAs.  8 and 16 columns agree at 4 limbs.  The 4
+// columns of Shoup contexts make 32-byte runs, which the link moves worst: they take 16 at every size (4 limbs
+// out: 38 -> 35 us).
+static int host_columns(const ckks_ctx* c, int nlimbs) { return nlimbs >= 16 || !c->fold ? (int)NTT_V16 : -1; }
 
 void ntt_forward_from_host(const ckks_ctx* c, const u64* host, u64* data, int nlimbs, const int* ids, int lpp) {
     const size_t ps = (size_t)lpp * c->n;
     const NttSrc io{host, ps, false, {}, {}, 0, nullptr};
     if (c->logn == 16)
         launch_ntt_variant<false>(c, ntt_pick(c, nlimbs), data, nlimbs, ids, lpp, ps, nullptr, nullptr, io,
-                                  host_columns(nlimbs));
+                                  host_columns(c, nlimbs));
     else
         launch_ntt_one<false>(c, data, nlimbs, ids, lpp, ps, nullptr, io);
     LAUNCH_CHECK();
@@ -1160,7 +1168,7 @@ void ntt_inverse_to_host(const ckks_ctx* c, const u64* src, size_t src_pstride, 
     const NttSrc io{src, src_pstride, false, {}, {}, 0, host};
     if (c->logn == 16)
         launch_ntt_variant<true>(c, ntt_pick(c, nlimbs), work, nlimbs, ids, lpp, ps, nullptr, nullptr, io,
-                                 host_columns(nlimbs));
+                                 host_columns(c, nlimbs));
     else
         launch_ntt_one<true>(c, host, nlimbs, ids, lpp, ps, nullptr, io);
     LAUNCH_CHECK();
