@@ -41,3 +41,27 @@ def test_variants_run_and_agree():
         want = want or got
         for i, (a, b) in enumerate(zip(got, want)):
             assert (a == b).all(), (v, i)
+
+
+def test_conversions_and_shapes_agree():
+    """tensor-core conversions (one and two threads a coefficient) leave lazy words below 4 p; every transform
+    shape takes them to the words that the integer-pipe conversion leads to"""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_04356_gb300 import build
+    from paper_2312_04356_gb300 import ckks as K
+    build.build()
+    d = dict(log_n=16, n_q=6, dnum=2, n_p=0, q0_bits=61, scale_bits=42, p_bits=61, boot_bits=0, n_boot=0, h=0, sigma=3.2)
+    ctx = K.ckks_ctx_create(d, 3, torch.cuda.current_stream().cuda_stream)
+    keys = K.ckks_keygen(ctx, [3], False)
+    ct = K.ckks_encrypt(ctx, keys, K.ckks_encode(ctx, WL.slots(1, 1 << 15, 0.5), 5, 2.0 ** 42), 1)
+    want = None
+    for mode in (0, 1, 2):
+        for v in (-1, 0, 1, 2, 3, 4, 5):
+            K.ckks_ctx_set_tensor_conversion(ctx, mode)
+            K.ckks_ctx_set_ntt_variant(ctx, v)
+            outs = [K.ckks_rotate_hoisted(ctx, keys, ct, [3])[0], K.ckks_mul_relin(ctx, keys, ct, ct)]
+            got = [K.ckks_ct_export_rns(ctx, o) for o in outs]
+            want = want or got
+            for i, (a, b) in enumerate(zip(got, want)):
+                assert (a == b).all(), (mode, v, i)
