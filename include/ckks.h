@@ -121,6 +121,13 @@ typedef void (*ckks_free_fn)(void* user, void* ptr, size_t bytes, void* cuda_str
  * ckks_ctx_create come from cudaMalloc.  A buffer is freed through the allocator that
  * provided it, so the allocator may be changed at any time; `user` is passed back unchanged
  * and must stay valid while buffers from it are alive.
+ * Workspace: rotations of one ciphertext (ckks_rotate_hoisted, up to eight) and the rotated giant
+ * steps of an HMatmul (ckks_bsgs and the layers built on it, up to sixteen polynomials) share
+ * launches in groups.  With nl = level + 1 limbs, next = nl + n_p, d digits, each rotation of a group
+ * takes 2 next + 2 nl limbs of N words beside the d next limbs of digits and the results, each giant
+ * step 2 nl + d next beside the sums (2 next per giant step); a group takes at most 1.25 GiB.  Where an
+ * allocator returns NULL for a group, half as many are tried, down to one at a time, so a budget
+ * has to hold one.
  * Errors: CKKS_EINVAL (only one of alloc / free_fn given). */
 int ckks_ctx_set_allocator(ckks_ctx* ctx, ckks_alloc_fn alloc, ckks_free_fn free_fn, void* user);
 /* Usage of the device's default memory pool (the library's default allocator): stats4 =

@@ -615,12 +615,18 @@ ckks_ct mod_raise(const ckks_ct& a) {
 // per digit: the converted rows of [nb][ndig][next][N] and x itself, which holds each digit's own
 // rows (kern::Digits).  x must outlive the key switches that read the digits.
 struct Raised {
-    DevBuf D;
+    DevBuf buf;              // empty when the caller gave the workspace
+    u64* D = nullptr;
     const u64* x = nullptr;
     size_t xstride = 0;
     int ndig = 1;
 };
-Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride = 0) {
+// words of the workspace of one polynomial: its coefficients and its raised digits
+static size_t mod_up_words(const ckks_ctx* c, int level) {
+    return ((size_t)level + 1 + c->digits(level).size() * (level + 1 + c->np)) * c->n;
+}
+// (ws: nb mod_up_words, or null to allocate)
+Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride = 0, u64* ws = nullptr) {
     const size_t n = c->n;
     const int nl = level + 1;
     const int next = nl + c->np;
@@ -628,23 +634,29 @@ Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride =
     const int ndig = (int)dig.size();
     const size_t dstr = (size_t)ndig * next * n;     // words per ciphertext of D
     if (xstride == 0) xstride = (size_t)nl * n;
-    DevBuf coef((size_t)nb * nl * n, c->stream);
-    kern::ntt_inverse_from(c, x, xstride, coef.ptr, nb * nl, c->d_iota, nl, (size_t)nl * n,
+    DevBuf own;
+    u64* coef = ws;
+    if (!ws) {
+        own = DevBuf((size_t)nb * nl * n, c->stream);
+        coef = own.ptr;
+    }
+    kern::ntt_inverse_from(c, x, xstride, coef, nb * nl, c->d_iota, nl, (size_t)nl * n,
                            c->d_modup_iscale[level]);   // prescaled
     Raised r;
-    r.D = DevBuf((size_t)nb * dstr, c->stream);
+    if (!ws) r.buf = DevBuf((size_t)nb * dstr, c->stream);
+    r.D = ws ? ws + (size_t)nb * nl * n : r.buf.ptr;
     r.x = x;
     r.xstride = xstride;
     r.ndig = ndig;
     kern::ConvJobs jobs;
     jobs.n = 0;
     for (int d = 0; d < ndig; ++d)
-        kern::add_conv_job(jobs, c->modup_tab(level, d), coef.ptr + (size_t)dig[d].front() * n,
-                           r.D.ptr + (size_t)d * next * n, (size_t)nl * n, dstr, true);
+        kern::add_conv_job(jobs, c->modup_tab(level, d), coef + (size_t)dig[d].front() * n,
+                           r.D + (size_t)d * next * n, (size_t)nl * n, dstr, true);
     kern::base_convert_jobs(c, jobs, nb);
     // every converted row of every digit of every ciphertext in one launch (two digits at N = 2^12: one
     // transform in place of three; a convolution there, import to export: 158 -> 127 us)
-    kern::ntt_forward_list(c, r.D.ptr, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb, dstr);
+    kern::ntt_forward_list(c, r.D, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb, dstr);
     return r;
 }
 
@@ -682,7 +694,7 @@ void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int l
         c->ops["keyswitch"]++;
         R.add(key.b.ptr, key.a.ptr, gs[k]);
     }
-    const kern::Digits dig{D.D.ptr, D.x, D.xstride, level + 1, c->alpha};
+    const kern::Digits dig{D.D, D.x, D.xstride, level + 1, c->alpha};
     kern::ks_inner(c, dig, D.ndig, (int)next, c->d_ext_ids[level], R, acc, acc + next * c->n, nb * bt.ostr, x0, x0rows, s,
                    x1, bt);
 }
@@ -704,7 +716,7 @@ static void key_switch_rotations(ckks_ctx* c, const ckks_keys& keys, const Raise
             R.add(key.b.ptr, key.a.ptr, gs[k]);
         }
         const size_t first = k0 * nb;
-        const kern::Digits dig{D.D.ptr + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
+        const kern::Digits dig{D.D + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
         kern::ks_rotations(c, dig, D.ndig, (int)next, c->d_ext_ids[level], R, x0 + first * xstr, acc, acc + next * c->n,
                            accumulate || k0 > 0, bt);
     }
@@ -735,20 +747,16 @@ static void lift_p(ckks_ctx* c, const u64* x, u64* acc, int level, int nb = 1) {
     kern::mul_scalar_acc(c, x, c->d_pmod, c->d_pmod + c->nq, acc, 2 * nl * nb, c->d_iota, nl, next * c->n);
 }
 
-// ModDown of both halves of `count` sums acc [count][nb][2][next][N] -> outs[i] [nb][2][l+1][N]
-static void mod_down(ckks_ctx* c, u64* acc, int level, u64* const* outs, int count, int nb) {
+// ModDown of both halves of `count` sums acc [count][nb][2][next][N] -> outs[i] [nb][2][l+1][N]; several
+// are worked in `work` ([count][nb][2][l+1][N]), a single one in its output
+static void mod_down(ckks_ctx* c, u64* acc, int level, u64* const* outs, int count, int nb, u64* work) {
     const size_t n = c->n;
     const int nl = level + 1, npoly = 2 * nb * count;
     const int next = nl + c->np;
     const int* pid = c->d_ext_ids[level] + nl;
     const ConvTab& tab_c = c->moddown_tab(level);
     kern::ntt_inverse(c, acc + (size_t)nl * n, npoly * c->np, pid, c->np, (size_t)next * n, tab_c.d_iscale);
-    DevBuf conv;                      // a single output array is worked in itself
-    u64* work = outs[0];
-    if (count > 1) {
-        conv = DevBuf((size_t)npoly * nl * n, c->stream);
-        work = conv.ptr;
-    }
+    if (count == 1) work = outs[0];
     kern::base_convert(c, tab_c, acc + (size_t)nl * n, n, work, n, npoly, (size_t)next * n, (size_t)nl * n, true);
     kern::NttTail tail{acc, (size_t)next * n, c->scale_tab(c->d_pinv, c->nq, 0), nullptr};
     if (count > 1) {
@@ -757,7 +765,7 @@ static void mod_down(ckks_ctx* c, u64* acc, int level, u64* const* outs, int cou
     }
     kern::ntt_forward_fused(c, work, npoly * nl, c->d_iota, nl, nullptr, &tail);
 }
-static void mod_down(ckks_ctx* c, u64* acc, int level, u64* out, int nb = 1) { mod_down(c, acc, level, &out, 1, nb); }
+static void mod_down(ckks_ctx* c, u64* acc, int level, u64* out, int nb = 1) { mod_down(c, acc, level, &out, 1, nb, nullptr); }
 
 u64 galois_of_step(const ckks_ctx* c, long long r) {
     const long long m = c->n / 2;
@@ -766,29 +774,51 @@ u64 galois_of_step(const ckks_ctx* c, long long r) {
     return powmod(5, (u64)r, 2ULL * c->n);
 }
 
+// Rotations of one ciphertext (up to 8 / nb), and the rotated giant steps of an HMatmul (up to 16 / nb), share
+// launches.  The workspace of such a group: `item` words each; group: at most how many on entry, how many
+// on return.  An allocator without room for all of them is asked for half as many, down to one, which
+// takes no more memory than a call without groups (an empty buffer: the caller allocates piece by piece).
+// Launches gain from groups at every level (eight rotations at level 1 / 9 / 23 of N = 2^16 one at a time
+// 330 / 514 / 964 us, two to four 209 / 441 / 809, together 206 / 418 / 772; a map of 64 stored babies at level 23
+// 2.64 ms, three at a time 2.40, together 2.29; block 8.50 ms with one, 8.06 with up to 256 MiB, 7.95 with all).
+// The bound is above the largest group of a 24-limb chain of that ring, 16 polynomials of 70 MiB, and cuts
+// those of larger ones.
+constexpr size_t GROUP_WORDS = (size_t)5 << 25;      // 1.25 GiB
+static DevBuf group_workspace(ckks_ctx* c, size_t item, size_t& group) {
+    group = std::min(group, std::max((size_t)1, GROUP_WORDS / item));
+    for (; group > 1; group /= 2) {
+        try {
+            return DevBuf(group * item, c->stream);
+        } catch (const CkksError& e) {
+            if (e.code != CKKS_ENOMEM) throw;
+            cudaGetLastError();
+        }
+    }
+    return DevBuf();
+}
+
 // rot_g(a) for every g and every ciphertext of a: the key switches of the automorphed raised digits D
 // of c1 with P c0(sigma_g) added on the Q rows in the same kernel, then ModDown: ModDown(P x + k) = x +
 // ModDown(k) exactly (P x vanishes on the P rows), so this is automorph(c0) + ModDown(k) in
-// fewer passes.  Several rotations are key-switched and brought down together (eight rotations at
-// level 9, summed: 621 -> 476 us).
+// fewer passes.  Several rotations are key-switched and brought down together (group_workspace).
 static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& a, const Raised& D,
                                           const std::vector<u64>& gs) {
     ckks_ctx* c = a.ctx;
     const int l = a.level, nl = l + 1;
     const size_t es = (size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n;
-    const size_t group = std::min((size_t)kern::NttTail::MAX_OUTS, (size_t)std::max(1, 8 / a.nb));
+    const size_t item = es + (size_t)a.nb * 2 * nl * c->n;
     std::vector<ckks_ct> outs;
+    for (size_t k = 0; k < gs.size(); ++k) outs.push_back(new_ct(c, l, a.scale, a.nb));
+    size_t group = std::min({(size_t)kern::NttTail::MAX_OUTS, (size_t)std::max(1, 8 / a.nb), gs.size()});
+    DevBuf ws = group_workspace(c, item, group);
+    if (!ws.ptr) ws = DevBuf(es, c->stream);
     for (size_t k0 = 0; k0 < gs.size(); k0 += group) {
         const size_t cnt = std::min(group, gs.size() - k0);
-        DevBuf acc(cnt * es, c->stream);
         std::vector<u64*> o;
+        for (size_t k = 0; k < cnt; ++k) o.push_back(outs[k0 + k].buf.ptr);
         const std::vector<u64> part(gs.begin() + k0, gs.begin() + k0 + cnt);
-        key_switch_inner(c, keys, D, l, part, part, acc.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb, a.cstride());
-        for (size_t k = 0; k < cnt; ++k) {
-            outs.push_back(new_ct(c, l, a.scale, a.nb));
-            o.push_back(outs.back().buf.ptr);
-        }
-        mod_down(c, acc.ptr, l, o.data(), (int)cnt, a.nb);
+        key_switch_inner(c, keys, D, l, part, part, ws.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb, a.cstride());
+        mod_down(c, ws.ptr, l, o.data(), (int)cnt, a.nb, ws.ptr + group * es);
     }
     return outs;
 }
@@ -900,10 +930,17 @@ static Babies rotate_hoisted_ext(const ckks_keys& keys, const ckks_ct& a, const 
     ckks_ctx* c = a.ctx;
     const int l = a.level, nl = l + 1;
     const size_t es = (size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n;
+    std::vector<u64> gs;
+    for (long long r : steps) {
+        const u64 g = galois_of_step(c, r);
+        if (g != 1) gs.push_back(g);
+    }
+    Raised D;                  // before the babies: its scratch is given back by then
+    if (!gs.empty()) D = mod_up(c, a.c1(), l, a.nb, a.cstride());
     Babies out;
     out.buf = DevBuf(steps.size() * es, c->stream);
     out.at.resize(steps.size());
-    std::vector<u64> gs;
+    gs.clear();
     for (size_t i = 0; i < steps.size(); ++i) {
         const u64 g = galois_of_step(c, steps[i]);
         if (g == 1) continue;
@@ -918,8 +955,6 @@ static Babies rotate_hoisted_ext(const ckks_keys& keys, const ckks_ct& a, const 
         CUDA_CHECK(cudaMemsetAsync(o, 0, es * 8, c->stream));
         lift_p(c, a.buf.ptr, o, l, a.nb);
     }
-    if (gs.empty()) return out;
-    const Raised D = mod_up(c, a.c1(), l, a.nb, a.cstride());
     for (size_t k0 = 0; k0 < gs.size(); k0 += kern::KsRotations::MAXR) {
         const size_t cnt = std::min((size_t)kern::KsRotations::MAXR, gs.size() - k0);
         const std::vector<u64> part(gs.begin() + k0, gs.begin() + k0 + cnt);
@@ -988,7 +1023,10 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
     int nrot = 0;
     while (nrot < nslots && rots[nrot]) ++nrot;
     CK_CHECK(nslots > 0, CKKS_EINVAL, "empty plaintext set");
-    DevBuf inner((size_t)nslots * nb * es, c->stream);
+    DevBuf inner;             // allocated when the first ModUp has given its scratch back
+    const auto need_inner = [&] {
+        if (!inner.ptr) inner = DevBuf((size_t)nslots * nb * es, c->stream);
+    };
     std::vector<char> written(nslots, 0);
     double scale = 0;
     for (size_t t = 0; t < ins.size(); ++t) {
@@ -1009,6 +1047,7 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             bool any_rot = false;
             for (long long r : steps) any_rot = any_rot || r != 0;
             if (any_rot) D = mod_up(c, a.c1(), l, nb, a.cstride());
+            need_inner();
             kern::BsgsFused T;
             T.nb = (int)used_b.size();
             T.ng = (int)gs.size();
@@ -1052,10 +1091,11 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             bt.dstr = (size_t)D.ndig * next * n;
             bt.xstr = a.cstride();
             bt.ostr = es;
-            kern::bsgs_fused(c, T, kern::Digits{D.D.ptr, D.x, D.xstride, nl, c->alpha}, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
+            kern::bsgs_fused(c, T, kern::Digits{D.D, D.x, D.xstride, nl, c->alpha}, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
             continue;
         }
         const Babies baby = rotate_hoisted_ext(keys, a, steps);
+        need_inner();
         // otherwise: the babies stored, then the inner sums in chunks of up to MAXG giant steps
         // (one pass over the babies per chunk)
         for (size_t k0 = 0; k0 < gs.size(); k0 += kern::BsgsGiants::MAXG) {
@@ -1094,26 +1134,36 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
     // over several of them; a lockstep batch fills the launches by itself), then key-switched into the sum.  Against one chain of launches per giant step on side streams with a sum of its own:
     // conv at level 1 342 (one at a time) or 278 (side streams) -> 260 us, downsampling layer 12.2 -> 11.9 ms
     // (further with one key-switch kernel for them all, k_ks_rotations).
-    const int group = std::max(1, 16 / nb);
     u64* acc = nrot < nslots ? inner.ptr + (size_t)nrot * nb * es : nullptr;       // the R = 0 giant's sum
     for (int k = nrot + 1; k < nslots; ++k)
         kern::add(c, acc, inner.ptr + (size_t)k * nb * es, acc, 2 * (int)next * nb, ext, (int)next);
     DevBuf acc_buf;
-    for (int k0 = 0; k0 < nrot; k0 += group) {
-        const int gn = std::min(group, nrot - k0);
+    if (!acc && nrot > 1) {
+        acc_buf = DevBuf(nb * es, c->stream);
+        acc = acc_buf.ptr;
+    }
+    bool have = nrot < nslots;
+    const size_t c1_words = (size_t)nb * nl * n, item = c1_words + nb * mod_up_words(c, l);
+    size_t group = std::min((size_t)std::max(1, 16 / nb), (size_t)nrot);
+    DevBuf ws = group_workspace(c, item, group);
+    for (int k0 = 0; k0 < nrot; k0 += (int)group) {
+        const int gn = std::min((int)group, nrot - k0);
         u64* x = inner.ptr + (size_t)k0 * nb * es;
-        DevBuf c1q((size_t)gn * nb * nl * n, c->stream);
-        mod_down_poly(c, x + next * n, l, c1q.ptr, gn * nb, es);
-        const Raised D = mod_up(c, c1q.ptr, l, gn * nb, (size_t)nl * n);
+        DevBuf c1_buf;
+        if (!ws.ptr) c1_buf = DevBuf(c1_words, c->stream);
+        u64* c1q = ws.ptr ? ws.ptr : c1_buf.ptr;
+        mod_down_poly(c, x + next * n, l, c1q, gn * nb, es);
+        const Raised D = mod_up(c, c1q, l, gn * nb, (size_t)nl * n, ws.ptr ? ws.ptr + group * c1_words : nullptr);
         std::vector<u64> gals;
         for (int k = 0; k < gn; ++k) gals.push_back(galois_of_step(c, rots[k0 + k]));
-        const bool have = acc != nullptr;
-        if (!have) {
+        if (!acc) {               // a single rotated giant: its ModUp's scratch has been given back
             acc_buf = DevBuf(nb * es, c->stream);
             acc = acc_buf.ptr;
         }
         key_switch_rotations(c, keys, D, l, gals, acc, have, x, nb, es);
+        have = true;
     }
+    ws.reset();
     if (rescale_out) {
         ckks_ct o = new_ct(c, l - 1, scale / (double)c->q[l], nb);
         mod_down_rescale(c, acc, l, o.buf.ptr, false, nb);
