@@ -35,19 +35,32 @@ u64 invmod(u64 a, u64 q) { return powmod(a, q - 2, q); }
 
 u64 shoup(u64 w, u64 q) { return (u64)(((u128)w << 64) / q); }
 
-void ntt_pair(u64 w, u64 q, bool fold, u64* out2) {
-    if (!fold) {
-        out2[0] = w;
-        out2[1] = shoup(w, q);
-        return;
-    }
-    const u64 v[2] = {w, mulmod(w, (1ull << 32) % q, q)};
+// W0 = w and W1 = w 2^32 mod q in balanced form, their signed low digits in the low halves (fold.cuh)
+static void pack_pair(u64 w, u64 w1, u64 q, u64* out2) {
+    const u64 v[2] = {w, w1};
     for (int i = 0; i < 2; ++i) {
         const int64_t s = v[i] > q / 2 ? (int64_t)v[i] - (int64_t)q : (int64_t)v[i];   // balanced
         const int32_t lo = (int32_t)(uint32_t)(u64)s;                                  // signed low digit
         const int64_t hi = (s - lo) / ((int64_t)1 << 32);
         out2[i] = (u64)(uint32_t)lo | ((u64)(uint32_t)(int32_t)hi << 32);
     }
+}
+
+void ntt_pair(u64 w, u64 q, bool fold, u64* out2) {
+    if (fold) {
+        pack_pair(w, mulmod(w, (1ull << 32) % q, q), q, out2);
+        return;
+    }
+    out2[0] = w;
+    out2[1] = shoup(w, q);
+}
+
+NttPairs::NttPairs(u64 q_, bool fold_) : q(q_), c((1ull << 32) % q_), cp(shoup(c, q_)), fold(fold_) {}
+
+void NttPairs::operator()(u64 w, u64* out2) const {
+    if (!fold) return ntt_pair(w, q, false, out2);
+    const u64 w1 = w * c - (u64)(((u128)w * cp) >> 64) * q;     // below 2 q
+    pack_pair(w, w1 >= q ? w1 - q : w1, q, out2);
 }
 
 void ntt_out_factor(u64 f, u64 w, u64 q, bool fold, u64* out4) {

@@ -549,6 +549,14 @@ u64 shoup(u64 w, u64 q);
 bool fold_consts(u64 q, FoldMod& f);
 // a transform constant w as the kernels take it: fold.cuh's packed digits, else w and its Shoup companion
 void ntt_pair(u64 w, u64 q, bool fold, u64* out2);
+// the same for many constants of one prime (a table): no 128-bit division for each of the folded form (the
+// tables of 31 primes at N = 2^16 are 4 million: context creation 154 -> 126 ms)
+struct NttPairs {
+    u64 q, c, cp;            // c = 2^32 mod q and its Shoup companion
+    bool fold;
+    NttPairs(u64 q, bool fold);
+    void operator()(u64 w, u64* out2) const;
+};
 // an inverse transform's final factor f as the kernels take it: the pairs of f and f w, w = psi^-(N/2) the
 // one twiddle of the last stage
 void ntt_out_factor(u64 f, u64 w, u64 q, bool fold, u64* out4);

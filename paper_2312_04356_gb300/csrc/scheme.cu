@@ -294,11 +294,12 @@ ckks_ctx* ctx_create(const ckks_params* P, uint64_t seed, cudaStream_t stream) {
             ipw[e] = mulmod(ipw[e - 1], ipsi, qq);
         }
         u64* base = tables.data() + (size_t)id * 4 * n;
+        const NttPairs pair(qq, c->fold);
         for (int k = 0; k < n; ++k) {
             unsigned r = brev_host(k, logn);
             const size_t at = 2 * (size_t)ntt_tw_pos(k, logn);
-            ntt_pair(pw[r], qq, c->fold, base + at);
-            ntt_pair(ipw[r], qq, c->fold, base + 2 * n + at);
+            pair(pw[r], base + at);
+            pair(ipw[r], base + 2 * n + at);
         }
         DevPrime& dp = primes[id];
         dp.m = c->mods[id];
