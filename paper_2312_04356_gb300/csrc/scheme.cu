@@ -616,48 +616,44 @@ ckks_ct mod_raise(const ckks_ct& a) {
 // per digit: the converted rows of [nb][ndig][next][N] and x itself, which holds each digit's own
 // rows (kern::Digits).  x must outlive the key switches that read the digits.
 struct Raised {
-    DevBuf buf;              // empty when the caller gave the workspace
-    u64* D = nullptr;
+    DevBuf D;
     const u64* x = nullptr;
     size_t xstride = 0;
     int ndig = 1;
 };
-// words of the workspace of one polynomial: its coefficients and its raised digits
-static size_t mod_up_words(const ckks_ctx* c, int level) {
-    return ((size_t)level + 1 + c->digits(level).size() * (level + 1 + c->np)) * c->n;
+// words of a polynomial's coefficients and of its raised digits
+static size_t coef_words(const ckks_ctx* c, int level) { return ((size_t)level + 1) * c->n; }
+static size_t digit_words(const ckks_ctx* c, int level) {
+    return c->digits(level).size() * ((size_t)level + 1 + c->np) * c->n;
 }
-// (ws: nb mod_up_words, or null to allocate)
-Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride = 0, u64* ws = nullptr) {
+// (coef, D: nb times those words, where the caller has allocated them)
+Raised mod_up(ckks_ctx* c, const u64* x, int level, int nb = 1, size_t xstride = 0, DevBuf&& coef_buf = DevBuf(),
+              DevBuf&& D = DevBuf()) {
     const size_t n = c->n;
     const int nl = level + 1;
     const int next = nl + c->np;
+    if (xstride == 0) xstride = (size_t)nl * n;
     std::vector<std::vector<int>> dig = c->digits(level);
     const int ndig = (int)dig.size();
-    const size_t dstr = (size_t)ndig * next * n;     // words per ciphertext of D
-    if (xstride == 0) xstride = (size_t)nl * n;
-    DevBuf own;
-    u64* coef = ws;
-    if (!ws) {
-        own = DevBuf((size_t)nb * nl * n, c->stream);
-        coef = own.ptr;
-    }
-    kern::ntt_inverse_from(c, x, xstride, coef, nb * nl, c->d_iota, nl, (size_t)nl * n,
+    const size_t dstr = (size_t)ndig * next * n;
+    DevBuf coef(std::move(coef_buf));        // given back on return
+    if (!coef.ptr) coef = DevBuf(nb * coef_words(c, level), c->stream);
+    kern::ntt_inverse_from(c, x, xstride, coef.ptr, nb * nl, c->d_iota, nl, (size_t)nl * n,
                            c->d_modup_iscale[level]);   // prescaled
     Raised r;
-    if (!ws) r.buf = DevBuf((size_t)nb * dstr, c->stream);
-    r.D = ws ? ws + (size_t)nb * nl * n : r.buf.ptr;
+    r.D = D.ptr ? std::move(D) : DevBuf(nb * digit_words(c, level), c->stream);
     r.x = x;
     r.xstride = xstride;
     r.ndig = ndig;
     kern::ConvJobs jobs;
     jobs.n = 0;
     for (int d = 0; d < ndig; ++d)
-        kern::add_conv_job(jobs, c->modup_tab(level, d), coef + (size_t)dig[d].front() * n,
-                           r.D + (size_t)d * next * n, (size_t)nl * n, dstr, true);
+        kern::add_conv_job(jobs, c->modup_tab(level, d), coef.ptr + (size_t)dig[d].front() * n,
+                           r.D.ptr + (size_t)d * next * n, (size_t)nl * n, dstr, true);
     kern::base_convert_jobs(c, jobs, nb);
     // every converted row of every digit of every ciphertext in one launch (two digits at N = 2^12: one
     // transform in place of three; a convolution there, import to export: 158 -> 127 us)
-    kern::ntt_forward_list(c, r.D, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb, dstr);
+    kern::ntt_forward_list(c, r.D.ptr, c->modup_nrows[level], c->d_modup_off[level], c->d_modup_pid[level], nb, dstr);
     return r;
 }
 
@@ -695,7 +691,7 @@ void key_switch_inner(ckks_ctx* c, const ckks_keys& keys, const Raised& D, int l
         c->ops["keyswitch"]++;
         R.add(key.b.ptr, key.a.ptr, gs[k]);
     }
-    const kern::Digits dig{D.D, D.x, D.xstride, level + 1, c->alpha};
+    const kern::Digits dig{D.D.ptr, D.x, D.xstride, level + 1, c->alpha};
     kern::ks_inner(c, dig, D.ndig, (int)next, c->d_ext_ids[level], R, acc, acc + next * c->n, nb * bt.ostr, x0, x0rows, s,
                    x1, bt);
 }
@@ -717,7 +713,7 @@ static void key_switch_rotations(ckks_ctx* c, const ckks_keys& keys, const Raise
             R.add(key.b.ptr, key.a.ptr, gs[k]);
         }
         const size_t first = k0 * nb;
-        const kern::Digits dig{D.D + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
+        const kern::Digits dig{D.D.ptr + first * bt.dstr, D.x + first * D.xstride, D.xstride, level + 1, c->alpha};
         kern::ks_rotations(c, dig, D.ndig, (int)next, c->d_ext_ids[level], R, x0 + first * xstr, acc, acc + next * c->n,
                            accumulate || k0 > 0, bt);
     }
@@ -776,26 +772,29 @@ u64 galois_of_step(const ckks_ctx* c, long long r) {
 }
 
 // Rotations of one ciphertext (up to 8 / nb), and the rotated giant steps of an HMatmul (up to 16 / nb), share
-// launches.  The workspace of such a group: `item` words each; group: at most how many on entry, how many
-// on return.  An allocator without room for all of them is asked for half as many, down to one, which
-// takes no more memory than a call without groups (an empty buffer: the caller allocates piece by piece).
+// launches in groups of `group` items, whose workspace (`item` words each) get(group) allocates.  Where an
+// allocator has no room for all of them half as many are tried, down to one, which takes no more memory
+// than a call without groups.
 // Launches gain from groups at every level (eight rotations at level 1 / 9 / 23 of N = 2^16 one at a time
 // 330 / 514 / 964 us, two to four 209 / 441 / 809, together 206 / 418 / 772; a map of 64 stored babies at level 23
 // 2.64 ms, three at a time 2.40, together 2.29; block 8.50 ms with one, 8.06 with up to 256 MiB, 7.95 with all).
 // The bound is above the largest group of a 24-limb chain of that ring, 16 polynomials of 70 MiB, and cuts
 // those of larger ones.
+// get() allocates the pieces one by one, each given back as soon as it is done with: as one allocation per
+// group, the memory that a recorded 27-layer request reserves grew from 9.9 to 11.6 GiB.
 constexpr size_t GROUP_WORDS = (size_t)5 << 25;      // 1.25 GiB
-static DevBuf group_workspace(ckks_ctx* c, size_t item, size_t& group) {
-    group = std::min(group, std::max((size_t)1, GROUP_WORDS / item));
-    for (; group > 1; group /= 2) {
+template <class F>
+static int allocate_group(int group, size_t item, F&& get) {
+    group = (int)std::min((size_t)group, std::max((size_t)1, GROUP_WORDS / item));
+    for (;; group /= 2) {
         try {
-            return DevBuf(group * item, c->stream);
+            get((size_t)group);
+            return group;
         } catch (const CkksError& e) {
-            if (e.code != CKKS_ENOMEM) throw;
+            if (e.code != CKKS_ENOMEM || group == 1) throw;
             cudaGetLastError();
         }
     }
-    return DevBuf();
 }
 
 // rot_g(a) for every g and every ciphertext of a: the key switches of the automorphed raised digits D
@@ -807,19 +806,25 @@ static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& 
     ckks_ctx* c = a.ctx;
     const int l = a.level, nl = l + 1;
     const size_t es = (size_t)a.nb * 2 * ((size_t)nl + c->np) * c->n;
-    const size_t item = es + (size_t)a.nb * 2 * nl * c->n;
+    const size_t work_words = (size_t)a.nb * 2 * nl * c->n;
     std::vector<ckks_ct> outs;
-    for (size_t k = 0; k < gs.size(); ++k) outs.push_back(new_ct(c, l, a.scale, a.nb));
-    size_t group = std::min({(size_t)kern::NttTail::MAX_OUTS, (size_t)std::max(1, 8 / a.nb), gs.size()});
-    DevBuf ws = group_workspace(c, item, group);
-    if (!ws.ptr) ws = DevBuf(es, c->stream);
-    for (size_t k0 = 0; k0 < gs.size(); k0 += group) {
-        const size_t cnt = std::min(group, gs.size() - k0);
+    for (size_t k0 = 0; k0 < gs.size();) {
+        DevBuf acc, work;
+        const int want = (int)std::min({(size_t)kern::NttTail::MAX_OUTS, (size_t)std::max(1, 8 / a.nb), gs.size() - k0});
+        const size_t cnt = allocate_group(want, es + work_words, [&](size_t g) {
+            acc.reset();
+            work.reset();
+            outs.erase(outs.begin() + k0, outs.end());
+            acc = DevBuf(g * es, c->stream);
+            for (size_t k = 0; k < g; ++k) outs.push_back(new_ct(c, l, a.scale, a.nb));
+            if (g > 1) work = DevBuf(g * work_words, c->stream);
+        });
         std::vector<u64*> o;
         for (size_t k = 0; k < cnt; ++k) o.push_back(outs[k0 + k].buf.ptr);
         const std::vector<u64> part(gs.begin() + k0, gs.begin() + k0 + cnt);
-        key_switch_inner(c, keys, D, l, part, part, ws.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb, a.cstride());
-        mod_down(c, ws.ptr, l, o.data(), (int)cnt, a.nb, ws.ptr + group * es);
+        key_switch_inner(c, keys, D, l, part, part, acc.ptr, a.c0(), nl, c->d_pmod, nullptr, a.nb, a.cstride());
+        mod_down(c, acc.ptr, l, o.data(), (int)cnt, a.nb, work.ptr);
+        k0 += cnt;
     }
     return outs;
 }
@@ -1092,7 +1097,7 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
             bt.dstr = (size_t)D.ndig * next * n;
             bt.xstr = a.cstride();
             bt.ostr = es;
-            kern::bsgs_fused(c, T, kern::Digits{D.D, D.x, D.xstride, nl, c->alpha}, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
+            kern::bsgs_fused(c, T, kern::Digits{D.D.ptr, D.x, D.xstride, nl, c->alpha}, a.c0(), a.c1(), nl, (int)next, ext, c->d_pmod, bt);
             continue;
         }
         const Babies baby = rotate_hoisted_ext(keys, a, steps);
@@ -1144,17 +1149,20 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         acc = acc_buf.ptr;
     }
     bool have = nrot < nslots;
-    const size_t c1_words = (size_t)nb * nl * n, item = c1_words + nb * mod_up_words(c, l);
-    size_t group = std::min((size_t)std::max(1, 16 / nb), (size_t)nrot);
-    DevBuf ws = group_workspace(c, item, group);
-    for (int k0 = 0; k0 < nrot; k0 += (int)group) {
-        const int gn = std::min((int)group, nrot - k0);
+    const size_t c1_words = (size_t)nb * nl * n, coef_w = nb * coef_words(c, l), dig_w = nb * digit_words(c, l);
+    for (int k0 = 0, gn; k0 < nrot; k0 += gn) {
+        DevBuf c1q, coef, dig;
+        gn = allocate_group(std::min(std::max(1, 16 / nb), nrot - k0), c1_words + coef_w + dig_w, [&](size_t g) {
+            c1q.reset();
+            coef.reset();
+            dig.reset();
+            c1q = DevBuf(g * c1_words, c->stream);
+            coef = DevBuf(g * coef_w, c->stream);
+            dig = DevBuf(g * dig_w, c->stream);
+        });
         u64* x = inner.ptr + (size_t)k0 * nb * es;
-        DevBuf c1_buf;
-        if (!ws.ptr) c1_buf = DevBuf(c1_words, c->stream);
-        u64* c1q = ws.ptr ? ws.ptr : c1_buf.ptr;
-        mod_down_poly(c, x + next * n, l, c1q, gn * nb, es);
-        const Raised D = mod_up(c, c1q, l, gn * nb, (size_t)nl * n, ws.ptr ? ws.ptr + group * c1_words : nullptr);
+        mod_down_poly(c, x + next * n, l, c1q.ptr, gn * nb, es);
+        const Raised D = mod_up(c, c1q.ptr, l, gn * nb, (size_t)nl * n, std::move(coef), std::move(dig));
         std::vector<u64> gals;
         for (int k = 0; k < gn; ++k) gals.push_back(galois_of_step(c, rots[k0 + k]));
         if (!acc) {               // a single rotated giant: its ModUp's scratch has been given back
@@ -1164,7 +1172,6 @@ ckks_ct bsgs_multi(const ckks_keys& keys, const std::vector<const ckks_ct*>& ins
         key_switch_rotations(c, keys, D, l, gals, acc, have, x, nb, es);
         have = true;
     }
-    ws.reset();
     if (rescale_out) {
         ckks_ct o = new_ct(c, l - 1, scale / (double)c->q[l], nb);
         mod_down_rescale(c, acc, l, o.buf.ptr, false, nb);
