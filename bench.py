@@ -32,29 +32,32 @@ METRIC = "ms per conv2d+bootstrap block at N=2^16"
 # DRAM bytes (read + write) per algorithmic byte of a forward NTT done as two k_ntt16 passes
 # (one read and one write of the limbs per transform are the algorithmic bytes, 268.4 MB for 256
 # limbs): ncu (--set full, one forward transform of 256 limbs at N = 2^16, cold caches) counted
-# 134.4 + 81.0 MB for the first pass and 186.5 + 89.4 MB for the second; traffic of a launch
-# scales with its limbs, so the in-block traffic per launch is this ratio times the launch's
-# algorithmic bytes.
+# 134.4 + 81.0 MB for the first pass and 186.5 + 89.4 MB for the second (the folded passes: 134.4 + 80.6 and
+# 186.5 + 88.6, 0.3% less); traffic of a launch scales with its limbs, so the in-block traffic per launch
+# is this ratio times the launch's algorithmic bytes.
 NTT_FWD_DRAM_PER_ALGO_BYTE = (134.4 + 81.0 + 186.5 + 89.4) / 268.4
 # The same ratio at the block's own launch sizes (at most ~70 limbs, so the whole transform
 # fits in the 129 MB L2): ncu with warm caches (no flush, as in the block) on a 24-limb forward
-# transform counted 0.005 + 0.050 MB (first pass) and 0.082 + 0.025 MB (second pass) of DRAM
-# traffic for 25.2 MB of algorithmic bytes.
+# transform.  For 25.2 MB of algorithmic bytes the passes with Shoup products counted 0.005 + 0.050 MB
+# (first pass) and 0.082 + 0.025 MB (second) of DRAM traffic, the folded passes that the benchmark's
+# chains run 0.014 + 0.021 and 0.205 + 0.091 MB.
 NTT_FWD_DRAM_PER_ALGO_BYTE_IN_L2 = (0.005120 + 0.049920 + 0.082432 + 0.025088) / (2 * 24 * 0.524288)
+NTT_FOLD_FWD_DRAM_PER_ALGO_BYTE_IN_L2 = (0.013568 + 0.021248 + 0.205312 + 0.091136) / (2 * 24 * 0.524288)
 L2_BYTES = 129e6
 # The same ratio for the key-switch inner product, from an ncu capture (cold caches) of one
 # launch at the top level (`--kernel ks`): 3 digits x 31 extended limbs with the automorphed c0
 # term on 24 rows = (3*3 + 2) * 31 + 24 = 365 limbs of algorithmic traffic (191.4 MB); DRAM
-# read 146.3 MB + write 3.6 MB.
+# read 146.3 MB + write 3.6 MB.  (Now: a relinearisation inside the block, level 20, 143.2 + 2.6 MB for 350
+# limbs, 0.79; four rotations in one launch 587.7 + 99.5 MB for 1460 limbs, 0.90.)
 KS_DRAM_PER_ALGO_BYTE = (146.3 + 3.6) / (365 * 65536 * 8 / 1e6)
 ROOF_NOTES = {
     "ntt_fwd": "integer-pipe bound in large launches (70% of the butterflies' own arithmetic at 128 limbs), latency "
-               "bound in small ones: the roofline is the multiply pipe's for Shoup products (64 lanes per SM per "
-               "clock, 16 lane-cycles per 64-bit butterfly; the folded products that run need 10); hbm_view gives "
-               "the same launches against HBM",
+               "bound in small ones: the roofline is the multiply pipe's (64 lanes per SM per clock) for the folded "
+               "products that run, 10 lane-cycles per 64-bit butterfly; shoup_view has the peak of Shoup products (16), "
+               "hbm_view the same launches against HBM",
     "bsgs_fused": "HBM bound with one ciphertext (keys and diagonals streamed once); a batch is bound by the integer pipes",
     "ks_inner": "HBM bound: switching keys streamed once (evict-first), raised digits gathered through the Galois "
-                "permutation; DRAM 55% of peak under ncu with cold caches",
+                "permutation; DRAM 67% of peak under ncu with cold caches (four rotations in one launch)",
 }
 CONFIG = "cfg2"
 
@@ -174,23 +177,28 @@ def peaks():
 # SM sub-partition per clock, 64 per SM: peak butterflies/s = 64 * SMs * clock / 16.  A
 # transform of one limb does 16 stages of N/2 butterflies and has 2 N 8 algorithmic bytes (one
 # read, one write), so the butterflies are the algorithmic bytes / 2 (per pass or per launch).
-# The library's folded products (primes next to a power of two) take 5 wide multiplies, 10 lane-cycles;
-# the line stays that of the Shoup form, so that its fractions compare over time.
+# The folded products that the benchmark's chains run (primes next to a power of two) take 5 wide
+# multiplies, 10 lane-cycles: the headline fraction is against that peak, the Shoup form's stands beside
+# it so that fractions compare over time.
 NTT_MUL_LANE_CYCLES_PER_BUTTERFLY = 16
+NTT_FOLD_LANE_CYCLES_PER_BUTTERFLY = 10
 GB300_SMS = 152
 
 
 def ntt_alu_roofline(kst, pk):
     mhz = pk.get("sm_max_mhz", 2070.0)
     peak = 64.0 * GB300_SMS * mhz * 1e6 / NTT_MUL_LANE_CYCLES_PER_BUTTERFLY / 1e9     # G butterflies/s
+    folded = peak * NTT_MUL_LANE_CYCLES_PER_BUTTERFLY / NTT_FOLD_LANE_CYCLES_PER_BUTTERFLY
+    source = "152 SMs x 64 multiply lanes x %.0f MHz / %%d lane-cycles per 64-bit %%s butterfly (derived)" % mhz
     out = {"bound": "alu", "pipe": "integer multiply (fmaheavy)", "unit": "Gbutterfly/s",
-           "peak": round(peak, 1), "peak_source": "152 SMs x 64 multiply lanes x %.0f MHz / %d lane-cycles "
-           "per 64-bit Shoup butterfly (derived)" % (mhz, NTT_MUL_LANE_CYCLES_PER_BUTTERFLY)}
+           "peak": round(peak, 1), "peak_source": source % (NTT_MUL_LANE_CYCLES_PER_BUTTERFLY, "Shoup"),
+           "peak_folded": round(folded, 1),
+           "peak_folded_source": source % (NTT_FOLD_LANE_CYCLES_PER_BUTTERFLY, "folded")}
     for k in ("ntt_fwd", "ntt_inv"):
         v = kst.get(k)
         if v:
             ach = v["bytes"] / 2.0 / (v["ms"] * 1e-3) / 1e9
-            out[k] = {"achieved": round(ach, 1), "frac": round(ach / peak, 4)}
+            out[k] = {"achieved": round(ach, 1), "frac": round(ach / peak, 4), "frac_folded": round(ach / folded, 4)}
     return out
 
 
@@ -723,14 +731,14 @@ def run_ours(args):
     per_launch = top[1]["bytes"] / top[1]["launches"]
     ratio = {"ntt_fwd": NTT_FWD_DRAM_PER_ALGO_BYTE, "ks_inner": KS_DRAM_PER_ALGO_BYTE}.get(top[0])
     if top[0] == "ntt_fwd" and per_launch < L2_BYTES:      # the average launch's data stays in L2
-        ratio = NTT_FWD_DRAM_PER_ALGO_BYTE_IN_L2
+        ratio = NTT_FOLD_FWD_DRAM_PER_ALGO_BYTE_IN_L2
     traffic = round(ratio * per_launch) if ratio else None
     roof = {"kernel": top[0], "bound": "hbm", "achieved": round(achieved, 1), "peak": pk.get("hbm_gbs"),
             "unit": "GB/s", "frac": round(achieved / pk.get("hbm_gbs"), 4), "traffic": traffic,
             "algorithmic_bytes_per_launch": round(per_launch),
             "traffic_source": ("DRAM bytes per algorithmic byte of the kernel's ncu capture at a launch size "
                                "that fits in L2 (warm caches, as in the block) x this launch's algorithmic bytes"
-                               if ratio == NTT_FWD_DRAM_PER_ALGO_BYTE_IN_L2 else
+                               if ratio == NTT_FOLD_FWD_DRAM_PER_ALGO_BYTE_IN_L2 else
                                "DRAM bytes per algorithmic byte of the kernel's ncu capture x this launch's "
                                "algorithmic bytes") if ratio else None,
             "note": ROOF_NOTES.get(top[0]),
@@ -743,14 +751,16 @@ def run_ours(args):
         # the NTT is bound by the integer multiply pipe: report that roofline, keep the HBM view
         alu = ntt_alu_roofline(kst, pk)
         hbm_view = {k: roof[k] for k in ("achieved", "peak", "unit", "frac", "peak_source")}
-        roof.update({"bound": "alu", "achieved": alu[top[0]]["achieved"], "peak": alu["peak"],
-                     "unit": alu["unit"], "frac": alu[top[0]]["frac"], "peak_source": alu["peak_source"],
+        roof.update({"bound": "alu", "achieved": alu[top[0]]["achieved"], "peak": alu["peak_folded"],
+                     "unit": alu["unit"], "frac": alu[top[0]]["frac_folded"], "peak_source": alu["peak_folded_source"],
+                     "shoup_view": {"peak": alu["peak"], "frac": alu[top[0]]["frac"],
+                                    "peak_source": alu["peak_source"]},
                      "hbm_view": hbm_view})
         net = {k: dict(v, ms=max(1e-6, v["ms"] - v["launches"] * event_us * 1e-3)) for k, v in kst.items()}
         alu_net = ntt_alu_roofline(net, pk)
         roof["net_of_event_overhead"] = {
-            "achieved": alu_net[top[0]]["achieved"], "frac": alu_net[top[0]]["frac"],
-            "event_us_per_launch": round(event_us, 2), "serial_graph_ms": round(serial_ms, 3),
+            "achieved": alu_net[top[0]]["achieved"], "frac": alu_net[top[0]]["frac_folded"],
+            "frac_shoup_peak": alu_net[top[0]]["frac"], "event_us_per_launch": round(event_us, 2), "serial_graph_ms": round(serial_ms, 3),
             "event_timed_sum_ms": round(total, 3),
             "how": "kernel time minus launches x (sum of event-timed kernels - the same block as a graph "
                    "with side streams off) / launches"}
@@ -1373,6 +1383,7 @@ def run_kernel_ntt(args):
                 res[variant][k]["hbm_frac"] = round(res[variant][k]["GBps"] / peaks()["hbm_gbs"], 4)
                 res[variant][k]["Gbutterfly_s"] = alu[k]["achieved"]
                 res[variant][k]["alu_frac"] = alu[k]["frac"]
+                res[variant][k]["alu_frac_folded"] = alu[k]["frac_folded"]
     print(json.dumps({"kernel": "ntt", "limbs": nl, "N": ctx.n, "roundtrip_exact": ok, "per_variant": res}))
 
 
