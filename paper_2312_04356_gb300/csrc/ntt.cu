@@ -781,6 +781,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(CL_THREADS, 2)
 // 16x3 23.9 / 104; forward ROW 2x20 25.0 / 115, 4x8 25.8 / 120; inverse ROW 4x12 22.8 / 105, 4x8
 // 23.3 / 113; inverse COL 8x5 26.2 / 119, 8x4 26.8 / 123, 16x3 28.7 / 137; below 16 limbs they agree
 // within 1 us of 8 to 12.  (Each figure holds about 4 us of the two events around the launch.)
+// The 80-register shapes spill, inverse ROW 4x12 most: 32 bytes a thread; 4x8 has none and is the slower one.
 // What is left between these and the butterflies alone (31 cycles per warp and SM quarter: 75 us for
 // 368 limbs) are the loads of data and twiddles that other warps do not cover.  ckks_autotune times
 // every shape per limb-count class.  Contexts on Shoup products have 16 sub-problems at two register budgets
