@@ -42,8 +42,8 @@ int guard(const ckks_ctx* c, F&& f) {
     }
 }
 
-// The device address of `bytes` of host memory that kernels may read and write (pinned, mapped, one
-// allocation), or null.
+// The device address of `bytes` of host memory that kernels may read and write (pinned, mapped for both, one
+// allocation), or null: a copy engine takes any host memory, a kernel's store outside a mapping faults.
 u64* device_view(const void* host, size_t bytes) {
     using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
     static const Query query = [] {
@@ -58,10 +58,13 @@ u64* device_view(const void* host, size_t bytes) {
     unsigned type = 0;
     CUdeviceptr dev = 0, start = 0;
     size_t size = 0;
-    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
-                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
-    void* to[4] = {&type, &dev, &start, &size};
-    if (query(4, what, to, (CUdeviceptr)host) != CUDA_SUCCESS) return nullptr;
+    unsigned long long access = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                                   CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
+    void* to[5] = {&type, &dev, &start, &size, &access};
+    if (query(5, what, to, (CUdeviceptr)host) != CUDA_SUCCESS) return nullptr;
+    if ((access & CU_MEM_ACCESS_FLAGS_PROT_READWRITE) != CU_MEM_ACCESS_FLAGS_PROT_READWRITE) return nullptr;
     if (type != CU_MEMORYTYPE_HOST || dev == 0 || dev % 8 || dev < start || dev - start + bytes > size) return nullptr;
     return (u64*)dev;
 }
