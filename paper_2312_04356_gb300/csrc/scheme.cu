@@ -800,7 +800,7 @@ static int allocate_group(int group, size_t item, F&& get) {
 // rot_g(a) for every g and every ciphertext of a: the key switches of the automorphed raised digits D
 // of c1 with P c0(sigma_g) added on the Q rows in the same kernel, then ModDown: ModDown(P x + k) = x +
 // ModDown(k) exactly (P x vanishes on the P rows), so this is automorph(c0) + ModDown(k) in
-// fewer passes.  Several rotations are key-switched and brought down together (group_workspace).
+// fewer passes.  Several rotations are key-switched and brought down together (allocate_group).
 static std::vector<ckks_ct> switch_galois(const ckks_keys& keys, const ckks_ct& a, const Raised& D,
                                           const std::vector<u64>& gs) {
     ckks_ctx* c = a.ctx;
